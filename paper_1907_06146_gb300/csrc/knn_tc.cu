@@ -22,6 +22,9 @@
 //               to the row's buffer in global scratch (L2); a warp compacts a full buffer
 //               with a bisection or a register bitonic sort (top-KS, new threshold).  The
 //               row's own column (self) takes one extra slot and is dropped at output.
+// The last block's padding rows start from a bound of -inf: they append and compact
+// nothing.  (As rows of distance 0 they kept every column: a second pass over 11 rows, 245
+// of its 256 rows padding, took 3.44 ms for 79 tiles at KS = 640.)
 // Columns are visited in BN-wide tiles, in id order or (large self-joins) nearest cluster
 // first; in id order "d2 < threshold" also settles equal distances by id, otherwise ties
 // are admitted and settled by the compaction.  (64-column tiles with four TMEM buffers and
@@ -402,7 +405,7 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
     for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
       const int64_t row = rb * BM + row_in_cta;
       const float nx = row < p.na ? p.a_norm[row] : 0.f;
-      float tau = INF;
+      float tau = row < p.na ? INF : -INF;  // a padding row admits nothing
       if (p.tau_in && row < p.na) {
         // a bound from a shorter walk over the same columns: every column at or below it
         // is admitted, so the KS smallest are all kept
@@ -662,7 +665,7 @@ k_knn_tc_wide(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
       const int64_t row = rb * BMW + row_in_cta;
       const float nx = row < p.na ? p.a_norm[row] : 0.f;
-      float tau = INF;
+      float tau = row < p.na ? INF : -INF;  // a padding row admits nothing
       if (p.tau_in && row < p.na) {
         const float t0 = p.tau_in[row];
         tau = t0 + (fabsf(t0) + fabsf(nx)) * p.tau_relax;
