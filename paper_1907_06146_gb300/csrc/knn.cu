@@ -26,35 +26,73 @@ namespace ssg {
 // ---------------------------------------------------------------------------------------
 // Ingest: row norms and facts about the data.
 // ---------------------------------------------------------------------------------------
-__global__ void k_row_stats(const float* __restrict__ X, int64_t n, int d, int ld,
-                            float* __restrict__ norms, unsigned* __restrict__ max_norm_bits,
-                            unsigned* __restrict__ max_abs_bits, int* __restrict__ non_integer,
-                            int* __restrict__ negative) {
-  int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= n) return;
-  const int lane = lane_id();
-  const float* x = X + row * ld;
-  float s = 0.f, mx = 0.f;
+// T lanes per row (T = 8, 16 or 32 by the row's float4 count), STATS_U rows per team in
+// flight; the facts are kept per thread over all its rows and reach memory with one set of
+// atomics per block.  Bound by the read of the rows: 1M x 128 in 0.14 ms (3.7 TB/s), 1.29 ms
+// with a warp per row, 4-byte loads and two atomics to the same two words from every row.
+constexpr int STATS_U = 4;
+template <int T>
+__global__ void __launch_bounds__(256) k_row_stats(
+    const float* __restrict__ X, int64_t n, int ld4, float* __restrict__ norms,
+    unsigned* __restrict__ max_norm_bits, unsigned* __restrict__ max_abs_bits,
+    int* __restrict__ non_integer, int* __restrict__ negative) {
+  __shared__ unsigned s_norm, s_abs;
+  __shared__ int s_bad, s_neg;
+  if (threadIdx.x == 0) {
+    s_norm = s_abs = 0u;
+    s_bad = s_neg = 0;
+  }
+  __syncthreads();
+  const int tl = threadIdx.x % T;
+  const int64_t teams = (int64_t)gridDim.x * (256 / T);
+  float mx = 0.f;
+  unsigned mn = 0u;
   int bad = 0, neg = 0;
-  for (int t = lane; t < d; t += 32) {
-    float v = x[t];
-    s = fmaf(v, v, s);
-    mx = fmaxf(mx, fabsf(v));
-    bad |= (v != rintf(v));
-    neg |= (v < 0.f);
+  for (int64_t r0 = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; r0 < n;
+       r0 += teams * STATS_U) {
+    float s[STATS_U];
+#pragma unroll
+    for (int u = 0; u < STATS_U; ++u) s[u] = 0.f;
+    for (int f = tl; f < ld4; f += T) {
+      float4 v[STATS_U];
+#pragma unroll
+      for (int u = 0; u < STATS_U; ++u) {
+        const int64_t r = r0 + u * teams;
+        v[u] = r < n ? __ldg((const float4*)X + r * ld4 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < STATS_U; ++u) {
+        const float e[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          s[u] = fmaf(e[k], e[k], s[u]);
+          mx = fmaxf(mx, fabsf(e[k]));
+          bad |= (e[k] != rintf(e[k]));
+          neg |= (e[k] < 0.f);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < STATS_U; ++u) {
+#pragma unroll
+      for (int o = T / 2; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o, T);
+      const int64_t r = r0 + u * teams;
+      if (r < n) {
+        if (tl == 0 && norms) norms[r] = s[u];
+        mn = max(mn, __float_as_uint(sqrtf(s[u])));
+      }
+    }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    s += __shfl_xor_sync(0xffffffffu, s, o);
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-    neg |= __shfl_xor_sync(0xffffffffu, neg, o);
-  }
-  if (lane == 0) {
-    if (norms) norms[row] = s;
-    atomicMax(max_norm_bits, __float_as_uint(sqrtf(s)));
-    atomicMax(max_abs_bits, __float_as_uint(mx));
-    if (bad) atomicOr(non_integer, 1);
-    if (neg) atomicOr(negative, 1);
+  atomicMax(&s_norm, mn);
+  atomicMax(&s_abs, __float_as_uint(mx));
+  if (bad) s_bad = 1;
+  if (neg) s_neg = 1;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicMax(max_norm_bits, s_norm);
+    atomicMax(max_abs_bits, s_abs);
+    if (s_bad) atomicOr(non_integer, 1);
+    if (s_neg) atomicOr(negative, 1);
   }
 }
 
@@ -451,8 +489,19 @@ void ingest(const float* X, int64_t n, int d, cudaStream_t st, PaddedRows& out, 
   pad_rows(X, n, d, st, out);
   Scratch<unsigned> facts(4, st);
   SSG_CUDA(cudaMemsetAsync(facts.p, 0, 4 * sizeof(unsigned), st));
-  SSG_LAUNCH(k_row_stats, (unsigned)ceil_div(n, 8), 256, 0, st, out.p, n, d, out.ld, norms,
-             facts.p, facts.p + 1, (int*)facts.p + 2, (int*)facts.p + 3);
+  const int ld4 = out.ld >> 2;
+  unsigned* f = facts.p;
+  auto stats = [&](auto kernel, int T) {
+    const int64_t want = ceil_div(n, (int64_t)(256 / T) * STATS_U);
+    SSG_LAUNCH(kernel, (unsigned)std::min<int64_t>(want, 8 * num_sms()), 256, 0, st, out.p, n, ld4,
+               norms, f, f + 1, (int*)f + 2, (int*)f + 3);
+  };
+  if (ld4 <= 8)
+    stats(k_row_stats<8>, 8);
+  else if (ld4 <= 16)
+    stats(k_row_stats<16>, 16);
+  else
+    stats(k_row_stats<32>, 32);
   unsigned h[4];
   SSG_CUDA(cudaMemcpyAsync(h, facts.p, sizeof(h), cudaMemcpyDeviceToHost, st));
   SSG_CUDA(cudaStreamSynchronize(st));

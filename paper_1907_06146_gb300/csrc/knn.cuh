@@ -3,6 +3,8 @@
 
 #include <vector>
 
+#include <cuda_bf16.h>
+
 #include "common.cuh"
 
 namespace ssg {
@@ -87,6 +89,12 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
                   int64_t nb, int ldb, const float* b_norm, int d, int self, int K,
                   int32_t* out_id, float* out_d2, cudaStream_t st, StageTimer* gemm_timer,
                   int max_tiles = 0, bool approx = false, const TcExtra& ex = TcExtra());
+
+// bf16 copy of n padded rows (16-byte aligned, stride ld a multiple of 4) in rows of dp
+// values, a multiple of 64; see k_to_bf16 for the options.
+void rows_to_bf16(const float* X, int64_t n, int d, int ld, __nv_bfloat16* Y, int dp,
+                  const int32_t* perm, const float* norm_in, float* norm_out, const float* mu,
+                  int pairs, cudaStream_t st);
 
 // Launch parameters of the certified bf16 kNN (ssg_build_opts.tune_table).
 struct KnnTune {

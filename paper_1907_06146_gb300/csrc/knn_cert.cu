@@ -29,17 +29,27 @@
 
 namespace ssg {
 
-// Column sums in fp64: block (32, 8), column blockIdx.x * 32 + tx, rows strided over y.
+// Column sums: block (32, 8), column blockIdx.x * 32 + tx, rows strided over y, four loads in
+// flight.  Each thread's running sum is a compensated fp32 pair (two-sum: 48 bits), joined in
+// fp64 at the end: GB300 adds fp64 at 1/64 of the fp32 rate, and with fp64 running sums the
+// 200,000 x 128 columns took 98 us against less than 30 (the read alone: 15).
 __global__ void k_col_sum(const float* __restrict__ X, int64_t n, int d, int ld,
                           double* __restrict__ sum) {
   __shared__ double part[8][33];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int c = blockIdx.x * 32 + tx;
-  double s = 0.0;
-  if (c < d)
-    for (int64_t r = (int64_t)blockIdx.y * 8 + ty; r < n; r += (int64_t)gridDim.y * 8)
-      s += (double)X[r * ld + c];
-  part[ty][tx] = s;
+  float s = 0.f, e = 0.f;
+  if (c < d) {
+    const int64_t step = (int64_t)gridDim.y * 8;
+    for (int64_t r = (int64_t)blockIdx.y * 8 + ty; r < n; r += 4 * step) {
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = r + u * step < n ? __ldg(X + (r + u * step) * ld + c) : 0.f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) two_sum_acc(s, e, v[u]);
+    }
+  }
+  part[ty][tx] = (double)s + (double)e;
   __syncthreads();
   if (ty == 0 && c < d) {
     double t = 0.0;
@@ -54,24 +64,40 @@ __global__ void k_col_mean(const double* __restrict__ sum, int d, int64_t n, flo
 }
 
 // Squared norms of the rows centred on mu (mu null: of the rows as given), with the same
-// fp32 subtraction as the bf16 conversion; *max_bits receives the largest (as float bits).
-__global__ void k_centred_norms(const float* __restrict__ X, int64_t n, int d, int ld,
-                                const float* __restrict__ mu, float* __restrict__ norm,
-                                unsigned* __restrict__ max_bits) {
-  const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= n) return;
+// fp32 subtraction as the bf16 conversion; *max_bits receives the largest (as float bits),
+// with one atomic per block.
+__global__ void __launch_bounds__(256) k_centred_norms(const float* __restrict__ X, int64_t n, int d,
+                                                       int ld, const float* __restrict__ mu,
+                                                       float* __restrict__ norm,
+                                                       unsigned* __restrict__ max_bits) {
+  __shared__ unsigned smax;
+  if (threadIdx.x == 0) smax = 0u;
+  __syncthreads();
   const int lane = lane_id();
-  const float* x = X + row * ld;
-  float s = 0.f;
-  for (int t = lane; t < d; t += 32) {
-    const float v = mu ? __fsub_rn(x[t], mu[t]) : x[t];
-    s = fmaf(v, v, s);
+  unsigned mx = 0u;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < n;
+       row += nwarps) {
+    const float* x = X + row * ld;
+    float s = 0.f;
+#pragma unroll 4
+    for (int t = lane; t < d; t += 32) {
+      const float v = mu ? __fsub_rn(x[t], mu[t]) : x[t];
+      s = fmaf(v, v, s);
+    }
+    s = warp_sum(s);
+    if (lane == 0) norm[row] = s;
+    mx = max(mx, __float_as_uint(s));
   }
-  s = warp_sum(s);
-  if (lane == 0) {
-    norm[row] = s;
-    if (max_bits) atomicMax(max_bits, __float_as_uint(s));
-  }
+  if (!max_bits) return;
+  if (lane == 0) atomicMax(&smax, mx);
+  __syncthreads();
+  if (threadIdx.x == 0) atomicMax(max_bits, smax);
+}
+
+// Launch shape of k_centred_norms.
+static unsigned norms_grid(int64_t n) {
+  return (unsigned)std::min<int64_t>(ceil_div(n, 8), 16 * num_sms());
 }
 
 __global__ void k_gather_rows(const float* __restrict__ X, int ld, const int32_t* __restrict__ ids,
@@ -397,18 +423,18 @@ CertResult knn_bf16_certified(const float* A, int64_t na, int ld, const float* a
   // centre on the base's column mean; centred squared norms and their maximum
   Scratch<double> csum((size_t)d, st);
   SSG_CUDA(cudaMemsetAsync(csum.p, 0, sizeof(double) * d, st));
-  const unsigned gy = (unsigned)std::min<int64_t>(ceil_div(nb, 8), 4 * num_sms());
+  const unsigned gy = (unsigned)std::min<int64_t>(ceil_div(nb, 32), 4 * num_sms());
   SSG_LAUNCH(k_col_sum, dim3((unsigned)ceil_div(d, 32), gy), dim3(32, 8), 0, st, B, nb, d, ld, csum.p);
   Scratch<float> mu((size_t)d, st);
   SSG_LAUNCH(k_col_mean, (unsigned)ceil_div(d, 128), 128, 0, st, csum.p, d, nb, mu.p);
   Scratch<float> nbc((size_t)nb, st), nac_own;
   Scratch<unsigned> mx(1, st);
   SSG_CUDA(cudaMemsetAsync(mx.p, 0, sizeof(unsigned), st));
-  SSG_LAUNCH(k_centred_norms, (unsigned)ceil_div(nb, 8), 256, 0, st, B, nb, d, ld, mu.p, nbc.p, mx.p);
+  SSG_LAUNCH(k_centred_norms, norms_grid(nb), 256, 0, st, B, nb, d, ld, mu.p, nbc.p, mx.p);
   const float* nac = nbc.p;
   if (!self) {
     nac_own.alloc((size_t)na, st);
-    SSG_LAUNCH(k_centred_norms, (unsigned)ceil_div(na, 8), 256, 0, st, A, na, d, ld, mu.p,
+    SSG_LAUNCH(k_centred_norms, norms_grid(na), 256, 0, st, A, na, d, ld, mu.p,
                nac_own.p, (unsigned*)nullptr);
     nac = nac_own.p;
   }
@@ -434,7 +460,7 @@ CertResult knn_bf16_certified(const float* A, int64_t na, int ld, const float* a
     SSG_CUDA(cudaMemcpyAsync(sid.p, sid_h.data(), sizeof(int32_t) * s, cudaMemcpyHostToDevice, st));
     Scratch<float> As((size_t)s * ld, st), asn((size_t)s, st), asc((size_t)s, st);
     SSG_LAUNCH(k_gather_rows, grid, 256, 0, st, A, ld, sid.p, (int64_t)s, As.p);
-    SSG_LAUNCH(k_centred_norms, (unsigned)ceil_div(s, 8), 256, 0, st, As.p, (int64_t)s, d, ld,
+    SSG_LAUNCH(k_centred_norms, norms_grid(s), 256, 0, st, As.p, (int64_t)s, d, ld,
                (const float*)nullptr, asn.p, (unsigned*)nullptr);
     SSG_LAUNCH(k_gather_vals, (unsigned)ceil_div(s, 256), 256, 0, st, nac, sid.p, (int64_t)s, asc.p);
     // the sample's exact K-th distance (itself included as a column when self: K + 1),
@@ -552,7 +578,7 @@ CertResult knn_bf16_certified(const float* A, int64_t na, int ld, const float* a
       const int K1 = K + self;
       Scratch<float> Ag((size_t)nlast * ld, st), agn((size_t)nlast, st);
       SSG_LAUNCH(k_gather_rows, grid, 256, 0, st, A, ld, last, (int64_t)nlast, Ag.p);
-      SSG_LAUNCH(k_centred_norms, (unsigned)ceil_div(nlast, 8), 256, 0, st, Ag.p, (int64_t)nlast, d,
+      SSG_LAUNCH(k_centred_norms, norms_grid(nlast), 256, 0, st, Ag.p, (int64_t)nlast, d,
                  ld, (const float*)nullptr, agn.p, (unsigned*)nullptr);
       Scratch<int32_t> ids((size_t)nlast * K1, st);
       Scratch<float> dd((size_t)nlast * K1, st);

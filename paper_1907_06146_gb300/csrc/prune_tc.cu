@@ -460,18 +460,6 @@ k_prune_tc(PtArgs p) {
   }
 }
 
-// bf16 rows padded to dp (exact for the integer data this path takes).
-__global__ void k_rows_bf16(const float* __restrict__ X, int64_t n, int d, int ld,
-                            __nv_bfloat16* __restrict__ Y, int dp) {
-  const int64_t total = n * (int64_t)dp;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / dp;
-    const int c = (int)(i - r * dp);
-    Y[i] = __float2bfloat16_rn(c < d ? X[r * ld + c] : 0.f);
-  }
-}
-
 // Floats of one slot: the packed lower triangle of the longest pool's 1 + L rows.
 int prune_tc_slot_floats(int L) {
   const int rows = std::min(L, PT_ROWS - 1) + 1;
@@ -587,7 +575,7 @@ void prune_run_tc(const float* X, int ld, int d, int64_t n, const int32_t* pool_
   const int dp = (d + 63) & ~63;
   const int kchunks = dp / 64;
   Scratch<__nv_bfloat16> xb((size_t)n * dp, st);
-  SSG_LAUNCH(k_rows_bf16, 8 * num_sms(), 256, 0, st, X, n, d, ld, xb.p, dp);
+  rows_to_bf16(X, n, d, ld, xb.p, dp, nullptr, nullptr, nullptr, nullptr, 0, st);
   Scratch<int> err(3, st);
   SSG_CUDA(cudaMemsetAsync(err.p, 0, 3 * sizeof(int), st));
   constexpr int SHORT = 63;   // pools of up to 63 candidates: slots a third the size

@@ -543,18 +543,22 @@ __global__ void __launch_bounds__(256, 3)
   }
 }
 
-__global__ void k_rows_u8(const float* __restrict__ X, int ld, int d, int64_t n,
-                          uint8_t* __restrict__ out) {
-  const int64_t total = n * (int64_t)ld;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+// Four values (one 16-byte load, one 4-byte store) per thread and step; rows are zero from d
+// to ld.  1M x 128: 0.09 ms, 0.26 ms with one value per thread.
+__global__ void k_rows_u8(const float4* __restrict__ X, int64_t n4, uchar4* __restrict__ out) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n4;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int t = (int)(e % ld);
-    out[e] = t < d ? (uint8_t)__float2uint_rn(X[e]) : (uint8_t)0;
+    const float4 v = __ldg(X + e);
+    out[e] = make_uchar4((uint8_t)__float2uint_rn(v.x), (uint8_t)__float2uint_rn(v.y),
+                         (uint8_t)__float2uint_rn(v.z), (uint8_t)__float2uint_rn(v.w));
   }
 }
 
 void rows_to_u8(const float* X, int ld, int d, int64_t n, uint8_t* out, cudaStream_t st) {
-  SSG_LAUNCH(k_rows_u8, 8 * num_sms(), 256, 0, st, X, ld, d, n, out);
+  (void)d;
+  const int64_t n4 = n * ld / 4;
+  SSG_LAUNCH(k_rows_u8, (unsigned)std::min<int64_t>(ceil_div(n4, 256), 16 * num_sms()), 256, 0, st,
+             (const float4*)X, n4, (uchar4*)out);
 }
 
 template <typename T>
