@@ -16,7 +16,7 @@
 // Pass 2 (k_knn_rerank) recomputes the KS candidates in double precision, sorts them by
 // (d2, id) and certifies the K-th against the pass-1 threshold minus a rigorous error
 // bound of the single-precision GEMM form.  Rows that fail certification are recomputed
-// exhaustively (k_knn_fallback).
+// exhaustively (k_fallback_scan).
 #include "common.cuh"
 #include "knn.cuh"
 #include "knn_select.cuh"
@@ -377,49 +377,104 @@ __global__ void k_knn_rerank(const float* __restrict__ A, int lda, const float* 
 // Exhaustive double-precision recomputation of flagged rows: every column whose
 // single-precision direct distance could be <= the K-th re-ranked value is recomputed in
 // double and collected; the collected set is sorted by (d2, id).
-__global__ void k_knn_fallback(const float* __restrict__ A, int lda, const float* __restrict__ B,
-                               int ldb, int d, int64_t nb, int self_exclude,
-                               const int32_t* __restrict__ fb_rows,
-                               const double* __restrict__ fb_kth, int K, int cap,
-                               int32_t* __restrict__ out_id, float* __restrict__ out_d2,
-                               int* __restrict__ overflow) {
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  double* dv = (double*)sm_raw;
-  int32_t* iv = (int32_t*)(dv + cap);
-  __shared__ int count;
-  const int64_t row = fb_rows[blockIdx.x];
-  const double bound = fb_kth[blockIdx.x];
-  const float* a = A + row * lda;
-  const double rel = (d + 4) * U32 * 1.01;
-  if (threadIdx.x == 0) count = 0;
-  __syncthreads();
-  for (int64_t j = threadIdx.x; j < nb; j += blockDim.x) {
-    if (self_exclude && j == row) continue;
-    const float* b = B + j * ldb;
-    float s = 0.f;
-    for (int t = 0; t < d; ++t) {
-      float u = a[t] - b[t];
-      s = fmaf(u, u, s);
+// k_fallback_scan: blockIdx.y picks FB_ROWS flagged rows, held in shared memory; the blocks of
+// blockIdx.x share the columns, two per team of 8 lanes at a time, so every column is read
+// once per FB_ROWS rows with 16-byte loads by the whole chip.  Bound by that read.  (One block
+// per flagged row with a thread per column read 4 bytes of 32 rows per load and left most SMs
+// idle: for the rows two passes had left of a 100,000 x 960 graph 133 ms, now 6.6; of a
+// 200,000 x 128 one 16 ms, now below 0.1.)
+// SHARED = false: rows too long for that (above 12,800 values) are read from memory.
+constexpr int FB_ROWS = 4, FB_CAP = 4096;
+template <bool SHARED>
+__global__ void __launch_bounds__(256)
+k_fallback_scan(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, int d,
+                int64_t nb, int self_exclude, const int32_t* __restrict__ fb_rows,
+                const double* __restrict__ fb_kth, int count, double rel, double* __restrict__ dv,
+                int32_t* __restrict__ iv, int* __restrict__ found) {
+  extern __shared__ __align__(16) float xs[];  // [FB_ROWS][ldb]
+  const int r0 = blockIdx.y * FB_ROWS;
+  const float4* xr[FB_ROWS];
+#pragma unroll
+  for (int r = 0; r < FB_ROWS; ++r)
+    xr[r] = (const float4*)(A + (int64_t)fb_rows[min(r0 + r, count - 1)] * lda);
+  if (SHARED) {
+    const int q = ldb >> 2;
+#pragma unroll
+    for (int r = 0; r < FB_ROWS; ++r) {
+      for (int i = threadIdx.x; i < q; i += blockDim.x) ((float4*)xs)[r * q + i] = __ldg(xr[r] + i);
+      xr[r] = (const float4*)xs + r * q;
     }
-    if ((double)s <= bound * (1.0 + rel) + 1e-30) {
-      double e = dist2_f64(a, b, d);
+    __syncthreads();
+  }
+  const int lane = lane_id(), team = lane >> 3, tl = lane & 7, ld4 = ldb >> 2;
+  // lane tl of a team settles row tl % 4 against column tl / 4 of its pair
+  const int mr = r0 + (tl & 3);
+  const int64_t row = mr < count ? (int64_t)fb_rows[mr] : -1;
+  const double bound = mr < count ? fb_kth[mr] : -1.0;
+  const double lim = bound * (1.0 + rel) + 1e-30;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t j0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 8; j0 < nb;
+       j0 += nwarps * 8) {
+    const int64_t ja = j0 + team, jb = ja + 4;
+    const float4* pa = (const float4*)(B + (ja < nb ? ja : 0) * ldb);
+    const float4* pb = (const float4*)(B + (jb < nb ? jb : 0) * ldb);
+    float s[2 * FB_ROWS];
+#pragma unroll
+    for (int k = 0; k < 2 * FB_ROWS; ++k) s[k] = 0.f;
+#pragma unroll 4
+    for (int f = tl; f < ld4; f += 8) {
+      const float4 a = __ldg(pa + f), b = __ldg(pb + f);
+#pragma unroll
+      for (int r = 0; r < FB_ROWS; ++r) {
+        const float4 x = xr[r][f];
+        float u;
+        u = x.x - a.x; s[r] = fmaf(u, u, s[r]);
+        u = x.y - a.y; s[r] = fmaf(u, u, s[r]);
+        u = x.z - a.z; s[r] = fmaf(u, u, s[r]);
+        u = x.w - a.w; s[r] = fmaf(u, u, s[r]);
+        u = x.x - b.x; s[4 + r] = fmaf(u, u, s[4 + r]);
+        u = x.y - b.y; s[4 + r] = fmaf(u, u, s[4 + r]);
+        u = x.z - b.z; s[4 + r] = fmaf(u, u, s[4 + r]);
+        u = x.w - b.w; s[4 + r] = fmaf(u, u, s[4 + r]);
+      }
+    }
+    float mine = 0.f;
+#pragma unroll
+    for (int k = 0; k < 2 * FB_ROWS; ++k) {
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+      if (k == tl) mine = s[k];
+    }
+    const int64_t j = tl < 4 ? ja : jb;
+    if (row >= 0 && j < nb && !(self_exclude && j == row) && (double)mine <= lim) {
+      const double e = dist2_f64(A + row * lda, B + j * ldb, d);
       if (e <= bound) {
-        int p = atomicAdd(&count, 1);
-        if (p < cap) {
-          dv[p] = e;
-          iv[p] = (int32_t)j;
+        const int p = atomicAdd(found + mr, 1);
+        if (p < FB_CAP) {
+          dv[(int64_t)mr * FB_CAP + p] = e;
+          iv[(int64_t)mr * FB_CAP + p] = (int32_t)j;
         }
       }
     }
   }
-  __syncthreads();
-  const int m = count < cap ? count : cap;
-  if (count > cap && threadIdx.x == 0) atomicOr(overflow, 1);
+}
+
+// The collected columns of flagged row blockIdx.x sorted by (d2, id); the K nearest go out.
+__global__ void k_fallback_finish(const int32_t* __restrict__ fb_rows, const double* __restrict__ dg,
+                                  const int32_t* __restrict__ ig, const int* __restrict__ found,
+                                  int K, int32_t* __restrict__ out_id, float* __restrict__ out_d2,
+                                  int* __restrict__ overflow) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  double* dv = (double*)sm_raw;
+  int32_t* iv = (int32_t*)(dv + FB_CAP);
+  const int64_t row = fb_rows[blockIdx.x];
+  const int all = found[blockIdx.x], m = min(all, FB_CAP);
+  if (all > FB_CAP && threadIdx.x == 0) atomicOr(overflow, 1);
   int mp = 1;
   while (mp < m) mp <<= 1;
-  for (int i = m + threadIdx.x; i < mp; i += blockDim.x) {
-    dv[i] = __longlong_as_double(0x7ff0000000000000ll);
-    iv[i] = -1;
+  for (int i = threadIdx.x; i < mp; i += blockDim.x) {
+    dv[i] = i < m ? dg[(int64_t)blockIdx.x * FB_CAP + i] : __longlong_as_double(0x7ff0000000000000ll);
+    iv[i] = i < m ? ig[(int64_t)blockIdx.x * FB_CAP + i] : -1;
   }
   __syncthreads();
   for (int k = 2; k <= mp; k <<= 1) {
@@ -452,19 +507,40 @@ void knn_fallback_rows(const float* A, int lda, const float* B, int ldb, int d, 
                        int self, const int32_t* rows, const double* kth, int count, int K,
                        int32_t* out_id, float* out_d2, cudaStream_t st) {
   if (count <= 0) return;
-  const int cap = 4096;
-  const size_t smem_fb = (size_t)cap * (sizeof(double) + sizeof(int32_t));
-  ensure_smem((const void*)k_knn_fallback, smem_fb);
-  Scratch<int> ovf(1, st);
-  SSG_CUDA(cudaMemsetAsync(ovf.p, 0, sizeof(int), st));
-  SSG_LAUNCH(k_knn_fallback, count, 256, smem_fb, st, A, lda, B, ldb, d, nb, self, rows, kth, K, cap,
-             out_id, out_d2, ovf.p);
+  const size_t smem_scan = (size_t)FB_ROWS * ldb * sizeof(float);
+  const size_t smem_fin = (size_t)FB_CAP * (sizeof(double) + sizeof(int32_t));
+  const bool shared = smem_scan <= 200 * 1024;
+  if (shared) ensure_smem((const void*)k_fallback_scan<true>, smem_scan);
+  ensure_smem((const void*)k_fallback_finish, smem_fin);
+  const int batch = std::min(count, 512);  // flagged rows per launch: bounds the lists' memory
+  Scratch<double> dv((size_t)batch * FB_CAP, st);
+  Scratch<int32_t> iv((size_t)batch * FB_CAP, st);
+  Scratch<int> found((size_t)batch + 1, st);
+  int* ovf = found.p + batch;
+  SSG_CUDA(cudaMemsetAsync(ovf, 0, sizeof(int), st));
+  for (int s = 0; s < count; s += batch) {
+    const int m = std::min(batch, count - s);
+    SSG_CUDA(cudaMemsetAsync(found.p, 0, sizeof(int) * m, st));
+    const unsigned gy = (unsigned)ceil_div(m, FB_ROWS);
+    const unsigned gx = (unsigned)std::max<int64_t>(
+        1, std::min<int64_t>(ceil_div(nb, 64), 8 * num_sms() / (int64_t)gy));
+    auto scan = [&](auto kernel, size_t smem) {
+      SSG_LAUNCH(kernel, dim3(gx, gy), 256, smem, st, A, lda, B, ldb, d, nb, self, rows + s, kth + s,
+                 m, (double)dist_rel_team8(ldb), dv.p, iv.p, found.p);
+    };
+    if (shared)
+      scan(k_fallback_scan<true>, smem_scan);
+    else
+      scan(k_fallback_scan<false>, 0);
+    SSG_LAUNCH(k_fallback_finish, (unsigned)m, 256, smem_fin, st, rows + s, dv.p, iv.p, found.p, K,
+               out_id, out_d2, ovf);
+  }
   int h = 0;
-  SSG_CUDA(cudaMemcpyAsync(&h, ovf.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+  SSG_CUDA(cudaMemcpyAsync(&h, ovf, sizeof(int), cudaMemcpyDeviceToHost, st));
   SSG_CUDA(cudaStreamSynchronize(st));
   if (h) note_device_status(SSG_EINTERNAL);
   SSG_REQUIRE(h == 0, SSG_EINTERNAL,
-              "kNN fallback: more than %d columns tie with a row's K-th distance", cap);
+              "kNN fallback: more than %d columns tie with a row's K-th distance", FB_CAP);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -569,8 +645,8 @@ KnnResult knn_exact(const float* A, int64_t na, int lda, const float* a_norm, co
   if (gemm_timer) gemm_timer->stop();
   Scratch<int32_t> fb_rows((size_t)na, st);
   Scratch<double> fb_kth((size_t)na, st);
-  Scratch<int> fb_count(2, st);
-  SSG_CUDA(cudaMemsetAsync(fb_count.p, 0, 2 * sizeof(int), st));
+  Scratch<int> fb_count(1, st);
+  SSG_CUDA(cudaMemsetAsync(fb_count.p, 0, sizeof(int), st));
   const int KSP = next_pow2(KS);
   const int wpb = 4;
   const size_t smem = (size_t)wpb * KSP * (sizeof(double) + sizeof(int32_t));
@@ -582,17 +658,7 @@ KnnResult knn_exact(const float* A, int64_t na, int lda, const float* a_norm, co
   SSG_CUDA(cudaStreamSynchronize(st));
   res.fallback_rows = nfb;
   if (nfb > 0) {
-    const int cap = 4096;
-    const size_t smem_fb = (size_t)cap * (sizeof(double) + sizeof(int32_t));
-    ensure_smem((const void*)k_knn_fallback, smem_fb);
-    SSG_LAUNCH(k_knn_fallback, nfb, 256, smem_fb, st, A, lda, B, ldb, d, nb, self, fb_rows.p,
-               fb_kth.p, K, cap, out_id, out_d2, fb_count.p + 1);
-    int ovf = 0;
-    SSG_CUDA(cudaMemcpyAsync(&ovf, fb_count.p + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
-    SSG_CUDA(cudaStreamSynchronize(st));
-    if (ovf) note_device_status(SSG_EINTERNAL);
-    SSG_REQUIRE(ovf == 0, SSG_EINTERNAL,
-                "kNN fallback: more than %d columns tie with a row's K-th distance", cap);
+    knn_fallback_rows(A, lda, B, ldb, d, nb, self, fb_rows.p, fb_kth.p, nfb, K, out_id, out_d2, st);
   }
   return res;
 }

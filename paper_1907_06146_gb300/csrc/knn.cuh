@@ -124,7 +124,7 @@ struct Counters {
   unsigned long long angle_border;  // fp64 cosines within the reporting band of cos(alpha)
 };
 
-// Exhaustive exact rows (k_knn_fallback): row rows[t] of A gets the K nearest of B by
+// Exhaustive exact rows (k_fallback_scan): row rows[t] of A gets the K nearest of B by
 // (fp64 d2, id) among the columns whose fp64 d2 is at most kth[t] (an upper bound of the
 // row's K-th distance); EINTERNAL if more than 4,096 columns lie within it.
 void knn_fallback_rows(const float* A, int lda, const float* B, int ldb, int d, int64_t nb,

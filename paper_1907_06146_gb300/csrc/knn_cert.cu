@@ -244,99 +244,194 @@ __global__ void k_band_limit(const float* __restrict__ d2, int ld, int col, int 
     lim[t] = (double)d2[(int64_t)t * ld + col] + widen * bf16_dist_bound(nac[t], ymax2, d, pairs);
 }
 
-// Exact order of each row's candidates and its certificate.  One warp per row r (rows:
-// compact index -> row id, null = identity).  Of the candidates cand[r][0, KS) (-1
-// padded) only those whose tensor-core distance cd2 lies within 2 E (plus the rounding of
-// that value) of the K-th smallest one can be among the K nearest: K candidates lie at
-// most at that K-th value plus E, any other candidate at least 2 E further minus E.  Those
-// get fp32 distances from the original rows, are sorted by (d2, id), and runs of
-// near-equal values up to position K are re-sorted in fp64; the first K go to row rows[r]
-// of the output (d2 in fp64 rounded to float when exact_d2, else the fp32 value).  The row
-// is certified when the K-th exact distance (bounded above through the fp32 value) lies
-// below thr[r] - slop - E; otherwise it is listed in fb (with that bound) for another pass.
-__global__ void k_knn_cert(const float* __restrict__ A, const float* __restrict__ B, int ld, int d,
-                           const int32_t* __restrict__ rows, int64_t count,
-                           const int32_t* __restrict__ cand, const float* __restrict__ cd2, int KS,
-                           const float* __restrict__ thr,
-                           const float* __restrict__ nac, double ymax2, int pairs, int K, int cap,
-                           float rel, int exact_d2, int32_t* __restrict__ out_id,
-                           float* __restrict__ out_d2,
-                           int32_t* __restrict__ fb, double* __restrict__ fb_kth,
-                           int* __restrict__ fb_count, unsigned long long* __restrict__ n_order) {
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = lane_id();
-  uint64_t* keys = (uint64_t*)(sm_raw + (size_t)warp * cap * 16);
-  double* d64 = (double*)(keys + cap);
-  const int64_t r = (int64_t)blockIdx.x * wpb + warp;
-  if (r >= count) return;
-  const int64_t row = rows ? (int64_t)rows[r] : r;
-  const float* xi = A + r * ld;
-  int m = 0;
-  for (int c = 0; c < KS; c += 32) {
-    const int t = c + lane;
-    const int32_t id = t < KS ? cand[r * KS + t] : -1;
-    const bool v = id >= 0;
-    const unsigned bal = __ballot_sync(0xffffffffu, v);
-    if (v) keys[m + __popc(bal & lanemask_lt())] = make_key(cd2[r * KS + t], id);
-    m += __popc(bal);
-  }
-  __syncwarp();
-  int mp = 1;
-  while (mp < m) mp <<= 1;
-  for (int t = m + lane; t < mp; t += 32) keys[t] = KEY_NONE;
-  __syncwarp();
-  if (m > K) {
-    // keep the candidates that can be among the K nearest (by their tensor-core distance)
-    warp_sort_keys(keys, mp);
-    const double nx = (double)nac[row];
-    const double aK = (double)key_dist(keys[K - 1]);
-    const double lim = aK + 2.0 * bf16_dist_bound(nx, ymax2, d, pairs) + stream_slop(nx, aK);
-    int keep = K;
-    for (int c = K; c < m; c += 32) {
-      const int t = c + lane;
-      const unsigned bal = __ballot_sync(0xffffffffu, t < m && (double)key_dist(keys[t]) <= lim);
-      keep += __popc(bal);
-      if (bal != 0xffffffffu) break;
-    }
-    m = keep;
-  }
-  for (int t = lane; t < m; t += 32) keys[t] = (uint64_t)(uint32_t)key_id(keys[t]);
-  __syncwarp();
-  warp_fill_dist_keys(keys, m, B, ld, xi);
-  mp = 1;
-  while (mp < m) mp <<= 1;
-  for (int t = m + lane; t < mp; t += 32) keys[t] = KEY_NONE;
-  __syncwarp();
-  warp_sort_keys(keys, mp);
-  if (m > 1) {
-    int f = warp_fix_runs(keys, m, K, d64, B, ld, d, xi, rel);
-    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-    if (lane == 0 && f) atomicAdd(n_order, (unsigned long long)f);
-  }
-  const float INF = __int_as_float(0x7f800000);
-  for (int t = lane; t < K; t += 32) {
-    const bool v = t < m;
-    const int32_t id = v ? key_id(keys[t]) : -1;
-    float dd = v ? key_dist(keys[t]) : INF;
-    if (v && exact_d2) dd = (float)dist2_f64(xi, B + (int64_t)id * ld, d);
-    out_id[row * K + t] = id;
-    out_d2[row * K + t] = dd;
-  }
-  if (lane == 0) {
-    const float t = thr[r];
-    bool ok = m >= K && isinf(t) && t > 0.f;  // every column was a candidate
-    double kth = INF;
-    if (m >= K) {
-      kth = (double)key_dist(keys[K - 1]) * (1.0 + 1.01 * (double)rel) + 1e-30;
-      if (!ok) {
-        const double nx = (double)nac[row];
-        ok = kth < (double)t - stream_slop(nx, t) - bf16_dist_bound(nx, ymax2, d, pairs);
+// keys[t] holds a candidate id in its low 32 bits; replaces keys [0, m) by (plain fp32 d2, id):
+// each lane of a team of 8 adds its terms in one sequence (dist_rel_team8), two candidates per
+// team at a time, eight row loads per lane in flight.  ONE: rows of at most 128 values, whose
+// query side stays in registers.
+template <bool ONE>
+__device__ __forceinline__ void warp_fill_plain_keys(uint64_t* keys, int m,
+                                                     const float* __restrict__ X, int ld,
+                                                     const float* __restrict__ xi) {
+  const int lane = lane_id(), team = lane >> 3, tl = lane & 7, ld4 = ld >> 2;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 x[4];
+  auto load_x = [&](int f0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = f0 + 8 * i < ld4 ? __ldg((const float4*)xi + f0 + 8 * i) : zero;
+  };
+  if (ONE) load_x(tl);
+  for (int t0 = 0; t0 < m; t0 += 8) {
+    const int ta = t0 + team, tb = ta + 4;
+    const int32_t ia = ta < m ? key_id(keys[ta]) : key_id(keys[0]);
+    const int32_t ib = tb < m ? key_id(keys[tb]) : ia;
+    const float4* pa = (const float4*)(X + (int64_t)ia * ld);
+    const float4* pb = (const float4*)(X + (int64_t)ib * ld);
+    float s0 = 0.f, s1 = 0.f;
+    for (int f0 = tl; f0 < (ONE ? tl + 1 : ld4); f0 += 32) {
+      if (!ONE) load_x(f0);
+      float4 a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const bool in = f0 + 8 * i < ld4;
+        a[i] = in ? __ldg(pa + f0 + 8 * i) : zero;
+        b[i] = in ? __ldg(pb + f0 + 8 * i) : zero;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float u;
+        u = x[i].x - a[i].x; s0 = fmaf(u, u, s0);
+        u = x[i].y - a[i].y; s0 = fmaf(u, u, s0);
+        u = x[i].z - a[i].z; s0 = fmaf(u, u, s0);
+        u = x[i].w - a[i].w; s0 = fmaf(u, u, s0);
+        u = x[i].x - b[i].x; s1 = fmaf(u, u, s1);
+        u = x[i].y - b[i].y; s1 = fmaf(u, u, s1);
+        u = x[i].z - b[i].z; s1 = fmaf(u, u, s1);
+        u = x[i].w - b[i].w; s1 = fmaf(u, u, s1);
       }
     }
-    if (!ok) {
-      const int p = atomicAdd(fb_count, 1);
-      fb[p] = (int32_t)row;
-      fb_kth[p] = kth;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    }
+    __syncwarp();
+    if (tl == 0) {
+      if (ta < m) keys[ta] = make_key(s0, ia);
+      if (tb < m) keys[tb] = make_key(s1, ib);
+    }
+  }
+  __syncwarp();
+}
+
+// Exact order of each row's candidates and its certificate.  One warp per row r (rows:
+// compact index -> row id, null = identity).  The candidates cand[r][0, KS) come sorted by
+// their tensor-core distance cd2 (-1 padded), and only those whose cd2 lies within 2 E (plus
+// the rounding of that value) of the K-th smallest one can be among the K nearest: K
+// candidates lie at most at that K-th value plus E, any other candidate at least 2 E further
+// minus E.  Those get plain fp32 distances p, whose relative error is at most rel_plain: a
+// candidate among the K nearest has p <= v (1 + rel_plain) / (1 - rel_plain) for v the K-th
+// smallest p, and the rest are dropped.  The survivors, about K of them, get compensated
+// fp32 distances, are sorted by (d2, id), and runs of near-equal values up to position K are
+// re-sorted in fp64; the first K go to row rows[r] of the output (d2 in fp64 rounded to
+// float when exact_d2, else the fp32 value).  The row is certified when the K-th exact
+// distance (bounded above through the fp32 value) lies below thr[r] - slop - E; otherwise it
+// is listed in fb (with that bound) for another pass.
+// Bound by the candidate rows' reads (200,000 x 128, KS = 532: 51 GB, from L2).  Only the K
+// survivors are sorted (the K-th value comes from a bisection), and a warp keeps one 8-byte
+// slot per candidate, so 24 warps share an SM: 6.1 ms; sorting all candidates twice, with
+// compensated sums for each and 16 bytes a slot, took 41 ms (100,000 x 960, KS = 740: 106 ms,
+// now 36, 284 GB of reads).
+// slots: 8-byte slots per warp, a power of two; spill: slots doubles per warp, for rows where
+// the survivors' fp64 scratch does not fit behind their keys (many ties).
+constexpr int CERT_WARPS = 8;
+template <bool ONE>
+__global__ void __launch_bounds__(CERT_WARPS * 32, 3)
+k_knn_cert(const float* __restrict__ A, const float* __restrict__ B, int ld, int d,
+           const int32_t* __restrict__ rows, int64_t count, const int32_t* __restrict__ cand,
+           const float* __restrict__ cd2, int KS, const float* __restrict__ thr,
+           const float* __restrict__ nac, double ymax2, int pairs, int K, int slots, float rel,
+           float rel_plain, int exact_d2, double* __restrict__ spill, int32_t* __restrict__ out_id,
+           float* __restrict__ out_d2, int32_t* __restrict__ fb, double* __restrict__ fb_kth,
+           int* __restrict__ fb_count, unsigned long long* __restrict__ n_order) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  const int warp = threadIdx.x >> 5, lane = lane_id();
+  uint64_t* keys = (uint64_t*)sm_raw + (size_t)warp * slots;
+  const int64_t gw = (int64_t)blockIdx.x * CERT_WARPS + warp;
+  const float INF = __int_as_float(0x7f800000);
+  for (int64_t r = gw; r < count; r += (int64_t)gridDim.x * CERT_WARPS) {
+    __syncwarp();
+    const int64_t row = rows ? (int64_t)rows[r] : r;
+    const float* xi = A + r * ld;
+    const int32_t* cr = cand + r * KS;
+    const float* dr = cd2 + r * KS;
+    const double nx = (double)nac[row];
+    const double E = bf16_dist_bound(nx, ymax2, d, pairs);
+    double lim = __longlong_as_double(0x7ff0000000000000ll);
+    if (K <= KS && cr[K - 1] >= 0) {
+      const double aK = (double)dr[K - 1];
+      lim = aK + 2.0 * E + stream_slop(nx, aK);
+    }
+    int m = 0;
+    for (int c = 0; c < KS; c += 32) {
+      const int t = c + lane;
+      const int32_t id = t < KS ? cr[t] : -1;
+      const bool v = id >= 0 && (t < K || (double)dr[t] <= lim);
+      const unsigned bal = __ballot_sync(0xffffffffu, v);
+      if (v) keys[t] = (uint64_t)(uint32_t)id;
+      m += __popc(bal);
+      if (bal != 0xffffffffu) break;  // a prefix: sorted, padding last
+    }
+    __syncwarp();
+    if (m > K + 8) {
+      warp_fill_plain_keys<ONE>(keys, m, B, ld, xi);
+      // a value between the K-th and the (K + 8)-th smallest, by bisection over the order bits
+      uint32_t lo = 0xffffffffu, hi = 0u;
+      for (int t = lane; t < m; t += 32) {
+        const uint32_t k = (uint32_t)(keys[t] >> 32);
+        lo = min(lo, k);
+        hi = max(hi, k);
+      }
+      lo = __reduce_min_sync(0xffffffffu, lo);
+      hi = __reduce_max_sync(0xffffffffu, hi);
+      while (lo < hi) {
+        const uint32_t mid = lo + ((hi - lo) >> 1);
+        int c = 0;
+        for (int t = lane; t < m; t += 32) c += (uint32_t)(keys[t] >> 32) <= mid;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (c >= K) {
+          hi = mid;
+          if (c <= K + 8) break;
+        } else {
+          lo = mid + 1;
+        }
+      }
+      const double keep = (double)order_bits_float(hi) * (1.0 + 2.1 * (double)rel_plain) + 1e-30;
+      int kept = 0;
+      for (int c = 0; c < m; c += 32) {
+        const int t = c + lane;
+        const uint64_t key = t < m ? keys[t] : 0ull;
+        const bool v = t < m && !((double)key_dist(key) > keep);
+        const unsigned bal = __ballot_sync(0xffffffffu, v);
+        __syncwarp();
+        if (v) keys[kept + __popc(bal & lanemask_lt())] = key;
+        kept += __popc(bal);
+      }
+      __syncwarp();
+      m = kept;
+    }
+    warp_fill_dist_keys(keys, m, B, ld, xi);
+    int mp = 1;
+    while (mp < m) mp <<= 1;
+    for (int t = m + lane; t < mp; t += 32) keys[t] = KEY_NONE;
+    __syncwarp();
+    warp_sort_keys(keys, mp);
+    if (m > 1) {
+      double* d64 = 2 * mp <= slots ? (double*)(keys + mp) : spill + (size_t)gw * slots;
+      int f = warp_fix_runs(keys, m, K, d64, B, ld, d, xi, rel);
+      for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+      if (lane == 0 && f) atomicAdd(n_order, (unsigned long long)f);
+    }
+    for (int t = lane; t < K; t += 32) {
+      const bool v = t < m;
+      const int32_t id = v ? key_id(keys[t]) : -1;
+      float dd = v ? key_dist(keys[t]) : INF;
+      if (v && exact_d2) dd = (float)dist2_f64(xi, B + (int64_t)id * ld, d);
+      out_id[row * K + t] = id;
+      out_d2[row * K + t] = dd;
+    }
+    if (lane == 0) {
+      const float t = thr[r];
+      bool ok = m >= K && isinf(t) && t > 0.f;  // every column was a candidate
+      double kth = INF;
+      if (m >= K) {
+        kth = (double)key_dist(keys[K - 1]) * (1.0 + 1.01 * (double)rel) + 1e-30;
+        if (!ok) ok = kth < (double)t - stream_slop(nx, t) - E;
+      }
+      if (!ok) {
+        const int p = atomicAdd(fb_count, 1);
+        fb[p] = (int32_t)row;
+        fb_kth[p] = kth;
+      }
     }
   }
 }
@@ -400,14 +495,21 @@ static int certify(const float* A, const float* B, int ld, int d, const int32_t*
                    int* fbc, unsigned long long* n_order, cudaStream_t st) {
   SSG_CUDA(cudaMemsetAsync(fbc, 0, sizeof(int), st));
   if (count == 0) return 0;
-  const int cap = next_pow2(std::max(KS, 32));
-  const int wpb = 4;
-  const size_t smem = (size_t)cap * 16 * wpb;
-  ensure_smem((const void*)k_knn_cert, smem);
-  SSG_LAUNCH(k_knn_cert, (unsigned)ceil_div(count, wpb), wpb * 32, smem, st, A, B, ld, d, rows, count,
-             cand, cd2, KS, thr, nac, ymax2, pairs, K, cap, dist_rel_team8c(ld), exact_d2 ? 1 : 0, out_id,
-             out_d2, fb,
-             fbk, fbc, n_order);
+  // room for every candidate, and where the survivors are about K for their fp64 scratch too
+  const int slots = std::max(next_pow2(std::max(KS, 32)), 2 * next_pow2(K + 32));
+  const size_t smem = (size_t)slots * 8 * CERT_WARPS;
+  const int64_t grid = std::min<int64_t>(ceil_div(count, CERT_WARPS), 3 * num_sms());
+  Scratch<double> spill((size_t)grid * CERT_WARPS * slots, st);
+  auto launch = [&](auto kernel) {
+    ensure_smem((const void*)kernel, smem);
+    SSG_LAUNCH(kernel, (unsigned)grid, CERT_WARPS * 32, smem, st, A, B, ld, d, rows, count, cand, cd2,
+               KS, thr, nac, ymax2, pairs, K, slots, dist_rel_team8c(ld), dist_rel_team8(ld),
+               exact_d2 ? 1 : 0, spill.p, out_id, out_d2, fb, fbk, fbc, n_order);
+  };
+  if (ld <= 128)
+    launch(k_knn_cert<true>);
+  else
+    launch(k_knn_cert<false>);
   return read_count(fbc, st);
 }
 
