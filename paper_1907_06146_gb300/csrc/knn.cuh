@@ -32,14 +32,15 @@ KnnResult knn_exact(const float* A, int64_t na, int lda, const float* a_norm, co
                     StageTimer* gemm_timer);
 
 // Near-first column order: rows clustered and stored cluster by cluster (perm maps a
-// stored position to the original row, inv the other way); for each cluster the ntiles BN-column tiles of the
+// stored position to the original row); for each cluster the ntiles BN-column tiles of the
 // stored order, nearest cluster first (tile_order, ncl x ntiles); rb_cluster gives the
 // cluster of each block of BM stored rows.
 struct KnnOrder {
   int ncl = 0;
   int64_t ntiles = 0;
   int64_t tstride = 0;  // length of each cluster's tile list (ntiles, or the walk limit)
-  Scratch<int32_t> perm, inv, tile_order, rb_cluster;
+  Scratch<int32_t> perm, tile_order, rb_cluster;
+  Scratch<int32_t> pair_tiles, pair_len;  // knn_pair_tiles
 };
 bool knn_order_fits(int64_t n, int BN);
 // walk > 0: every block of rows visits only its first walk tiles (Alg. 4), so each
@@ -48,6 +49,10 @@ bool knn_order_fits(int64_t n, int BN);
 // cores.
 void knn_cluster_order(const float* X, int ld, int d, int64_t n, int BM, int BN, cudaStream_t st,
                        KnnOrder& o, int64_t walk = 0, const float* x_norm = nullptr);
+
+// Of an order for a limited walk: the list of each pair of row blocks, in tiles twice as wide
+// (pair_tiles, 2 tstride entries apart; pair_len of them).
+void knn_pair_tiles(int64_t n, int BM, cudaStream_t st, KnnOrder& o);
 
 // bf16 tensor-core variant of the exact top-K (only for info.bf16_exact data).
 // True on sm_103 for rows of up to 4,096 values: the resident pipeline holds d <= 128, wider

@@ -171,12 +171,11 @@ __global__ void k_count_labels(int32_t* __restrict__ label, int64_t n, int ncl,
 }
 
 __global__ void k_scatter_perm(const int32_t* __restrict__ label, int64_t n, int* __restrict__ cursor,
-                               int32_t* __restrict__ perm, int32_t* __restrict__ inv) {
+                               int32_t* __restrict__ perm) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int pos = atomicAdd(cursor + label[i], 1);
     perm[pos] = (int32_t)i;
-    inv[i] = pos;
   }
 }
 
@@ -240,6 +239,45 @@ __global__ void k_tile_order(const int32_t* __restrict__ order, const int32_t* _
     }
   }
   if (k != cap) atomicOr(err, 1);
+}
+
+// The tile list of each pair of row blocks (2 rb, 2 rb + 1) of a limited walk, in tiles twice
+// as wide: the tiles that hold those of either block's list (list entries taken in turn, so
+// nearest first for both), each once.  One thread per pair walks the lists with a bitmap of
+// the tiles already listed.
+__global__ void k_pair_tiles(const int32_t* __restrict__ tile_order, const int32_t* __restrict__ rbc,
+                             int64_t nrb, int64_t tstride, int64_t words,
+                             int32_t* __restrict__ out, int32_t* __restrict__ len) {
+  extern __shared__ uint32_t seen[];
+  const int64_t pr = blockIdx.x;
+  for (int64_t w = threadIdx.x; w < words; w += blockDim.x) seen[w] = 0u;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const int32_t* l0 = tile_order + (int64_t)rbc[2 * pr] * tstride;
+  const int32_t* l1 =
+      2 * pr + 1 < nrb ? tile_order + (int64_t)rbc[2 * pr + 1] * tstride : l0;
+  int32_t* o = out + pr * 2 * tstride;
+  int k = 0;
+  for (int64_t i = 0; i < tstride; ++i) {
+    for (int b = 0; b < 2; ++b) {
+      if (b == 1 && l1 == l0) break;
+      const int32_t t = (b ? l1[i] : l0[i]) >> 1;
+      const uint32_t bit = 1u << (t & 31);
+      if (seen[t >> 5] & bit) continue;
+      seen[t >> 5] |= bit;
+      o[k++] = t;
+    }
+  }
+  len[pr] = k;
+}
+
+void knn_pair_tiles(int64_t n, int BM, cudaStream_t st, KnnOrder& o) {
+  const int64_t nrb = ceil_div(n, BM), npr = ceil_div(nrb, 2);
+  const int64_t words = (ceil_div(o.ntiles, 2) + 31) >> 5;
+  o.pair_tiles.alloc((size_t)npr * 2 * o.tstride, st);
+  o.pair_len.alloc((size_t)npr, st);
+  SSG_LAUNCH(k_pair_tiles, (unsigned)npr, 32, (size_t)words * 4, st, o.tile_order.p, o.rb_cluster.p,
+             nrb, o.tstride, words, o.pair_tiles.p, o.pair_len.p);
 }
 
 bool knn_order_fits(int64_t n, int BN) {
@@ -309,7 +347,6 @@ void knn_cluster_order(const float* X, int ld, int d, int64_t n, int BM, int BN,
   Scratch<int32_t> cl_start((size_t)ncl, st), cl_end((size_t)ncl, st), order((size_t)ncl * ncl, st);
   Scratch<int> cursor((size_t)ncl, st), err(1, st);
   o.perm.alloc((size_t)n, st);
-  o.inv.alloc((size_t)n, st);
   o.tile_order.alloc((size_t)ncl * o.tstride, st);
   const int64_t nrb = ceil_div(n, BM);
   o.rb_cluster.alloc((size_t)nrb, st);
@@ -317,7 +354,7 @@ void knn_cluster_order(const float* X, int ld, int d, int64_t n, int BM, int BN,
   SSG_CUDA(cudaMemcpyAsync(cl_end.p, end.data(), sizeof(int32_t) * ncl, cudaMemcpyHostToDevice, st));
   SSG_CUDA(cudaMemcpyAsync(cursor.p, start.data(), sizeof(int32_t) * ncl, cudaMemcpyHostToDevice, st));
   SSG_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
-  SSG_LAUNCH(k_scatter_perm, grid, 256, 0, st, label.p, n, cursor.p, o.perm.p, o.inv.p);
+  SSG_LAUNCH(k_scatter_perm, grid, 256, 0, st, label.p, n, cursor.p, o.perm.p);
   const int p2 = next_pow2(ncl);
   ensure_smem((const void*)k_cluster_order, p2 * sizeof(uint64_t));
   SSG_LAUNCH(k_cluster_order, ncl, 256, p2 * sizeof(uint64_t), st, C.p, ncl, dc, p2, order.p);

@@ -1,35 +1,49 @@
-// Exact kNN graph on the 5th-generation tensor cores (tcgen05, sm_103a) for integer data
-// that bf16 holds exactly (|x| <= 256, and the bounds of DataInfo::exact).
+// kNN graph selection on the 5th-generation tensor cores (tcgen05, sm_103a): every row's KS
+// nearest columns by the distance of bf16 operands.  Exact for integer data that bf16 holds
+// exactly (|x| <= 256, and the bounds of DataInfo::exact); on other data the caller certifies
+// the result (knn_cert.cu).
 //
 // The GEMM is augmented so that the accumulator already holds what the threshold test
 // needs: A = [x | 1 1 1 1 0..], B = [y | -p1 -p2 -p3 -p4 0..] with p1 + .. + p4 = |y|^2 / 2
 // (bf16 parts of an integer or half-integer below 2^23), so acc = x.y - |y|^2 / 2 and
-// d2 = |x|^2 - 2 acc.  Every product and partial sum is a multiple of 1/2 below 2^23 in
-// magnitude (2 d max|x|^2 <= 2^24 for non-negative data, 4 d max|x|^2 <= 2^24 otherwise),
-// so the accumulation is exact in fp32 whatever its order, and so is d2.
+// d2 = |x|^2 - 2 acc.  On exact data every product and partial sum is a multiple of 1/2 below
+// 2^23 in magnitude (2 d max|x|^2 <= 2^24 for non-negative data, 4 d max|x|^2 <= 2^24
+// otherwise), so the accumulation is exact in fp32 whatever its order, and so is d2.
 //
-// Persistent kernel, one CTA per SM, 10 warps:
-//   warp 0      TMA producer: the CTA's 256 query rows (A, resident per row block) and a
-//               pipeline of 128-column base tiles (B), bf16 with 128-byte swizzle, plus the
-//               16-element augmentation rows with 32-byte swizzle;
-//   warp 1      allocates 512 TMEM columns and issues tcgen05.mma: for every B tile two
-//               128x128 accumulators (the two 128-row halves of A) into one of NBUF = 2
-//               TMEM buffers, so the epilogue drains one buffer while the MMAs fill the
-//               other;
-//   warps 2..9  epilogue, one thread per query row (TMEM lane): tcgen05.ld 64 columns at
-//               a time, their largest accumulator against the row's threshold (a tree of
-//               three-input maxes), and only where some lane passes, the passing values go
-//               to the row's buffer in global scratch (L2); a warp compacts a full buffer
-//               with a bisection or a register bitonic sort (top-KS, new threshold).  The
-//               row's own column (self) takes one extra slot and is dropped at output.
-// The last block's padding rows start from a bound of -inf: they append and compact
-// nothing.  (As rows of distance 0 they kept every column: a second pass over 11 rows, 245
-// of its 256 rows padding, took 3.44 ms for 79 tiles at KS = 640.)
-// Columns are visited in BN-wide tiles, in id order or (large self-joins) nearest cluster
-// first; in id order "d2 < threshold" also settles equal distances by id, otherwise ties
-// are admitted and settled by the compaction.  (64-column tiles with four TMEM buffers and
-// twice the TMA stages were measured 1.65x slower: the MMAs then take about as long per
-// instruction while doing half the work.)
+// k_knn_pair: persistent clusters of two CTAs (one CTA per SM), 10 warps each.  A work item is
+// a block of 512 query rows, 256 per CTA, and one of `nseg` interleaved shares of the column
+// tiles it visits (256 columns, 128 rows of B in each CTA).
+//   warp 0      TMA producer: the CTA's query rows (A; resident for rows of up to 128 values,
+//               else streamed with B in 64-value chunks) and its half of the column tiles,
+//               bf16 with 128-byte swizzle, plus the 16-element augmentation rows with 32-byte
+//               swizzle.  All of them complete on the leader CTA's barriers;
+//   warp 1      allocates 512 TMEM columns; the leader's issues tcgen05.mma of the pair: M =
+//               256 (128 rows of each CTA), N = 256, one accumulator of 256 columns for each
+//               of the two 128-row halves of a CTA's rows, so the epilogue drains one half
+//               while the MMAs fill the other;
+//   warps 2..9  epilogue, one thread per query row (TMEM lane): tcgen05.ld 64 columns at a
+//               time, their largest accumulator against the row's threshold (a tree of
+//               three-input maxes), and only where some lane passes, the passing (id,
+//               accumulator) pairs go straight from registers to the row's buffer in global
+//               scratch; a warp cuts a full buffer back to its KS largest with a bisection.
+// k_knn_finish then takes each row's KS largest from the buffers of its shares, sorts them by
+// (distance, original id) and writes the K neighbours, with many rows per SM in flight.
+//
+// Why this shape.  128 x 128 x 16 MMAs of one CTA take 98 cycles each instead of 64: both
+// operands come from shared memory.  A pair reads half of B per CTA for an MMA of four times
+// the work, and each column tile is read from L2 once for 512 rows instead of 256 (773 GB of
+// DRAM reads for a graph of 1M x 128 before).  A tile's two halves wait for their own
+// epilogue warps only.  Appending from registers costs four instructions per column of an
+// eight-column group that some lane passes; parking the chunk in shared memory and scanning it
+// back cost about 250 cycles per chunk.  Few row blocks (10,000 queries, a sample of 256 rows)
+// used to leave most SMs idle: their columns are shared out over `nseg` items per block, and
+// the shares exchange thresholds through global memory.
+// Measured, whole kNN stage, against the kernel of one CTA and 128 x 128 MMAs: 1M x 128,
+// K = 200, 341 -> 233 ms; 10,000 queries over 1M rows, K = 100, 15.0 -> 6.8 ms.
+//
+// Columns are visited in 256-wide tiles, in id order or (large self-joins) nearest cluster
+// first; in id order and one share "acc > threshold" also settles equal distances by id,
+// otherwise ties are admitted and settled at the end.
 // Every wait on an mbarrier is bounded (about 2 s); a wait that runs out sets an error
 // word, tells the other roles to stop, and the CTA releases its TMEM and exits.
 #include <cuda.h>
@@ -46,46 +60,46 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 256;               // query rows per CTA (two UMMA_M = 128 halves)
-constexpr int BN = 128;               // base columns per pipeline stage (UMMA_N)
+constexpr int BM = 512;               // query rows per work item (256 per CTA of the pair)
+constexpr int CM = 256;               // query rows per CTA: two halves of 128 TMEM lanes
+constexpr int BN = 256;               // base columns per tile (UMMA_N), 128 rows of B per CTA
 constexpr int API_TILE = 128;         // tile limits are given in 128-point tiles
-constexpr int NBUF = 2;               // TMEM accumulator buffers
-constexpr uint32_t IDESC_N = idesc_bf16(BN);
+constexpr uint32_t IDESC = idesc_bf16_pair(BN);
 constexpr int EPI_WARPS = 8;
 constexpr int THREADS = 64 + EPI_WARPS * 32;
-constexpr int TMEM_COLS = 512;        // 2 buffers x 2 halves x 128 fp32 columns
+constexpr int TMEM_COLS = 512;        // 2 halves x 256 fp32 columns
 constexpr int MAX_STAGES = 6;
+constexpr int MAX_D_RESIDENT = 128;   // rows of up to this many values stay resident
+constexpr int MAX_D_STREAM = 4096;    // longer ones, up to this, are streamed
 constexpr int AUG = 16;               // augmentation K-step (bf16 elements)
 constexpr int AUG_BYTES = AUG * 2;    // one augmentation row: 32 bytes
+constexpr float LOWEST = -3.402823466e38f;  // the threshold that every finite value meets
+constexpr uint32_t A_CHUNK = CM * 128;        // 64 values of the CTA's query rows: 32 KB
+constexpr uint32_t B_CHUNK = (BN / 2) * 128;  // 64 values of its half of a tile: 16 KB
+constexpr uint32_t A_AUG = 128 * AUG_BYTES;   // one half's rows (all halves' rows are alike)
+constexpr uint32_t B_AUG = (BN / 2) * AUG_BYTES;
+
 struct TcArgs {
-  const float* a_norm;  // |x|^2 of the stored query rows (exact integers)
   int64_t na;           // query rows
   int64_t nb;           // base rows: stored column positions >= nb are padding
-  int64_t ntiles;       // BN-column tiles of the base
+  int64_t rb0, nrb;     // row blocks of this launch: rb0 .. rb0 + nrb - 1
   int64_t tstride;      // length of each cluster's tile list
-  int64_t nwalk;        // tiles each block of rows visits (ntiles, or fewer for Alg. 4)
-  int kchunks;          // padded d / 64
+  int64_t nwalk;        // tiles each block of rows visits (all, or fewer for Alg. 4)
+  int nseg;             // shares of a block's tiles
+  int kchunks;          // row width / 64
+  int dp_chunks, d;     // chunks of one part of a row (bf16 pairs: three parts), its values
   int stages;
-  int self;
-  int KS, K;
-  int trig;             // a row buffer holding more than trig keys is compacted (<= C - BN)
-  uint64_t* rowbuf;
-  int32_t* out_id;
-  float* out_d2;
+  int strict;           // 1: columns equal to the threshold are not admitted
+  int KS;
+  uint2* rowbuf;        // [rows of this launch][nseg][C] (id, accumulator bits)
+  int* cnt;             // [rows of this launch][nseg]
+  uint32_t* ts_g;       // nullable, per query row: order bits of a lower bound of its KS-th
+                        // largest accumulator (read first; with shares, raised by all)
   int* err;
   const int32_t* perm;        // stored position -> original id (null: the identity)
-  const int32_t* inv;         // original id -> stored position
-  const int32_t* tile_order;  // per cluster, its first tstride tile indices (null: in order)
-  const int32_t* rb_cluster;  // cluster of each block of BM stored query rows
-  float* out_thresh;          // nullable: per output row, the KS-th smallest distance kept
-                              // (or, with fewer kept, the final admission bound)
-  const int32_t* qid;         // nullable: query row r is base row qid[r] (the self column);
-                              // outputs then go to row r
-  const float* tau_in;        // nullable: per stored row, an upper bound of its KS-th
-                              // distance to start the streaming threshold from
-  float tau_relax;            // tau_in is widened by (|tau_in| + |x|^2) tau_relax (0: exact)
-  float* tau_out;             // thresh_only: per stored row, the KS-th distance of its walk
-  int thresh_only;            // 1: no output rows, only tau_out
+  const int32_t* tile_order;  // tile lists, tstride entries apart (null: in order)
+  const int32_t* rb_cluster;  // list of each block of BM stored query rows (null: its own)
+  const int32_t* walk_len;    // nullable: tiles that each block visits (else nwalk)
 };
 
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
@@ -94,298 +108,361 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return d;
 }
 
-// Largest of 32 accumulators: a depth-4 tree of three-input maxes.
-__device__ __forceinline__ float max32(const uint32_t (&v)[32]) {
-  float a[11];
-#pragma unroll
-  for (int i = 0; i < 10; ++i)
-    a[i] = fmax3(__uint_as_float(v[3 * i]), __uint_as_float(v[3 * i + 1]),
-                 __uint_as_float(v[3 * i + 2]));
-  a[10] = fmaxf(__uint_as_float(v[30]), __uint_as_float(v[31]));
-  const float b0 = fmax3(a[0], a[1], a[2]), b1 = fmax3(a[3], a[4], a[5]);
-  const float b2 = fmax3(a[6], a[7], a[8]), b3 = fmaxf(a[9], a[10]);
-  return fmaxf(fmax3(b0, b1, b2), b3);
+// Largest of eight values.
+__device__ __forceinline__ float max8(const uint32_t* v) {
+  const float a = fmax3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
+  const float b = fmax3(__uint_as_float(v[3]), __uint_as_float(v[4]), __uint_as_float(v[5]));
+  return fmax3(a, b, fmaxf(__uint_as_float(v[6]), __uint_as_float(v[7])));
 }
 
-// Parks 32 accumulators in a thread's stash: float4 slots XOR-swizzled by sw = lane & 7,
-// so 8 lanes store to 8 different bank groups.
-__device__ __forceinline__ void stash32(float* st, int sw, const uint32_t (&v)[32]) {
-#pragma unroll
-  for (int k = 0; k < 8; ++k)
-    *(float4*)(st + ((k ^ sw) << 2)) =
-        make_float4(__uint_as_float(v[4 * k]), __uint_as_float(v[4 * k + 1]),
-                    __uint_as_float(v[4 * k + 2]), __uint_as_float(v[4 * k + 3]));
-}
-
-// Appends the parked accumulators above ts to a row's buffer as (|x|^2 - 2 acc, stored
-// position) keys; column e of the chunk is stored position jc + e (padding from nb on).
-// Out of line: once the threshold has settled it runs for few chunks, and one copy keeps
-// the scan loop small in the instruction cache.
-__device__ __noinline__ int append_stash(const float* st, int sw, float ts, float nx, int32_t jc,
-                                         int64_t nb, uint64_t* buf, int cnt) {
-  uint32_t m = 0;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const float4 q = *(const float4*)(st + ((k ^ sw) << 2));
-    m |= ((q.x > ts ? 1u : 0u) | (q.y > ts ? 2u : 0u) | (q.z > ts ? 4u : 0u) |
-          (q.w > ts ? 8u : 0u))
-         << (4 * k);
-  }
-  while (m) {
-    const int e = __ffs(m) - 1;
-    m &= m - 1;
-    const int32_t j = jc + e;
-    if (j >= nb) break;  // padding columns come last within a chunk
-    const float acc = st[(((e >> 2) ^ sw) << 2) | (e & 3)];
-    buf[cnt++] = make_key(fmaf(-2.f, acc, nx), j);
-  }
-  return cnt;
-}
-
-// Maps the ids of a row's first cnt keys through map (stored position -> original id, or
-// back), warp-wide; a sort then settles equal distances by original id.  Without a map
-// nothing changes.
-__device__ __forceinline__ void map_key_ids(uint64_t* buf, int cnt, const int32_t* __restrict__ map) {
-  if (!map) return;
-  __syncwarp();
-  for (int i = lane_id(); i < cnt; i += 32) {
-    const uint64_t k = buf[i];
-    buf[i] = (k & 0xFFFFFFFF00000000ull) | (uint32_t)map[(uint32_t)k];
-  }
-  __syncwarp();
-}
-
-// Cuts back the row buffers of a warp's 32 rows that the next tile could overflow (count
-// above trig) to the entries at or below their KS-th smallest distance (a full sort only if
-// ties would keep too many).  wbuf: the buffer of lane 0's row; lane l's is wbuf + l C.
+// Cuts one row's buffer of cnt >= KS (id, accumulator) pairs back to the entries at or above a
+// threshold with between KS and `good` of them (in no particular order), found by bisection
+// over the order bits; if ties at the KS-th largest would keep more than `cap`,
+// exactly KS stay, the ties with the smallest original ids.  Returns the new count; *ts gets
+// the threshold (at least KS entries are not below it).  Warp-wide, out of line: it runs
+// rarely, and one copy keeps the scan small in the instruction cache.
 template <int C>
-__device__ __forceinline__ void compact_needed(const TcArgs& p, uint64_t* wbuf, int& cnt,
-                                               float& tau) {
-  unsigned need = __ballot_sync(0xffffffffu, cnt > p.trig);
-  while (need) {
-    const int l = __ffs(need) - 1;
-    need &= need - 1;
-    uint64_t* lb = wbuf + (size_t)l * C;
-    const int cl = __shfl_sync(0xffffffffu, cnt, l);
-    float t2;
-    int c2 = select_row<C>(lb, cl, p.KS, (p.KS + p.trig) / 2, p.trig, &t2);
-    if (c2 < 0) {
-      // too many ties at the threshold: a sort settles them by original id, and the
-      // kept keys go back to stored positions like the ones still to come
-      map_key_ids(lb, cl, p.perm);
-      c2 = compact_row<C>(lb, cl, p.KS, &t2);
-      map_key_ids(lb, c2, p.inv);
-    }
-    if (lane_id() == l) {
-      cnt = c2;
-      tau = t2;
-    }
-  }
-}
-
-// Final compaction of a warp's 32 rows (stored rows r0 .. r0 + 31, buffers as for
-// compact_needed), then their output: the first K keys after dropping the row itself (or,
-// thresh_only, the KS-th distance), and the threshold when asked.
-template <int C>
-__device__ __forceinline__ void finish_rows(const TcArgs& p, uint64_t* wbuf, int64_t r0, int cnt,
-                                            float tau) {
+__device__ __noinline__ int cut_row(uint2* __restrict__ buf, int cnt, int KS, int good, int cap,
+                                    const int32_t* __restrict__ perm, float* ts) {
+  constexpr int E = C / 32;
   const int lane = lane_id();
-  const float INF = __int_as_float(0x7f800000);
-  for (int l = 0; l < 32; ++l) {
-    const int64_t r = r0 + l;
-    uint64_t* lb = wbuf + (size_t)l * C;
-    float t2;
-    int cl = __shfl_sync(0xffffffffu, cnt, l);
-    if (cl > 256 && cl > p.KS) {
-      const int c1 = select_row<C>(lb, cl, p.KS, 256, 256, &t2);
-      if (c1 >= 0) cl = c1;
-    }
-    if (p.thresh_only) {
-      // the KS-th distance of this walk (the order of equal distances is irrelevant)
-      if (cl <= 256)
-        compact_row<256>(lb, cl, p.KS, &t2);
-      else
-        compact_row<C>(lb, cl, p.KS, &t2);
-      if (r < p.na && lane == 0) p.tau_out[r] = t2;
-      __syncwarp();
-      continue;
-    }
-    map_key_ids(lb, cl, p.perm);
-    const int c2 = cl <= 256 ? compact_row<256>(lb, cl, p.KS, &t2)
-                             : compact_row<C>(lb, cl, p.KS, &t2);
-    // the row's last admission bound: with fewer than KS kept (a bound from tau_in that
-    // few columns meet) every column not kept lies above it
-    const float taul = __shfl_sync(0xffffffffu, tau, l);
-    if (r >= p.na) continue;
-    // the output row, and the base id of the row itself (the self column)
-    const int64_t ro = p.qid ? r : (p.perm ? (int64_t)p.perm[r] : r);
-    const int32_t sid = p.qid ? p.qid[r] : (int32_t)ro;
-    if (p.out_thresh && lane == 0) p.out_thresh[ro] = fminf(t2, taul);
-    int selfpos = c2;
-    if (p.self) {
-      for (int e0 = 0; e0 < c2; e0 += 32) {
-        const int e = e0 + lane;
-        const unsigned m = __ballot_sync(0xffffffffu, e < c2 && key_id(lb[e]) == sid);
-        if (m) {
-          selfpos = e0 + __ffs(m) - 1;
-          break;
-        }
-      }
-    }
-    for (int t = lane; t < p.K; t += 32) {
-      const int src = t < selfpos ? t : t + 1;
-      const uint64_t key = src < c2 ? lb[src] : KEY_NONE;
-      p.out_id[ro * p.K + t] = key == KEY_NONE ? -1 : key_id(key);
-      p.out_d2[ro * p.K + t] = key == KEY_NONE ? INF : key_dist(key);
-    }
-    __syncwarp();
+  uint2 v[E];
+  uint32_t k[E];  // ascending: larger accumulators first
+  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = (e << 5) | lane;
+    v[e] = i < cnt ? buf[i] : make_uint2(0u, 0u);
   }
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = (e << 5) | lane;
+    k[e] = i < cnt ? ~float_order_bits(__uint_as_float(v[e].y)) : 0xFFFFFFFFu;
+    if (i < cnt) {
+      lo = min(lo, k[e]);
+      hi = max(hi, k[e]);
+    }
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  int n = cnt;  // entries <= hi
+  while (lo < hi) {
+    const uint32_t mid = lo + ((hi - lo) >> 1);
+    int part[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int e = 0; e < E; ++e) part[e & 3] += k[e] <= mid ? 1 : 0;
+    const int c = __reduce_add_sync(0xffffffffu, (part[0] + part[1]) + (part[2] + part[3]));
+    if (c >= KS) {
+      hi = mid;
+      n = c;
+      if (c <= good) break;
+    } else {
+      lo = mid + 1;
+    }
+  }
+  uint32_t idmax = 0xFFFFFFFFu;  // of the entries equal to hi, those with an id up to this stay
+  if (n > cap) {
+    int below = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) below += k[e] < hi ? 1 : 0;
+    const int need = KS - __reduce_add_sync(0xffffffffu, below);
+    uint32_t l2 = 0u, h2 = 0x7FFFFFFFu;
+    while (l2 < h2) {
+      const uint32_t mid = l2 + ((h2 - l2) >> 1);
+      int c = 0;
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (k[e] == hi) c += (perm ? (uint32_t)perm[v[e].x] : v[e].x) <= mid ? 1 : 0;
+      c = __reduce_add_sync(0xffffffffu, c);
+      if (c >= need)
+        h2 = mid;
+      else
+        l2 = mid + 1;
+    }
+    idmax = h2;
+  }
+  // each lane's kept entries go out one after another behind those of the lanes before it
+  uint32_t keep = 0u;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    bool in = ((e << 5) | lane) < cnt && k[e] <= hi;
+    if (idmax != 0xFFFFFFFFu && in && k[e] == hi)
+      in = (perm ? (uint32_t)perm[v[e].x] : v[e].x) <= idmax;
+    keep |= in ? 1u << e : 0u;
+  }
+  int incl = __popc(keep);
+  const int own = incl;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  const int total = __shfl_sync(0xffffffffu, incl, 31);
+  uint2* out = buf + (incl - own);
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    if ((keep >> e) & 1u) *out++ = v[e];
+  __syncwarp();
+  *ts = order_bits_float(~hi);
+  return total;
 }
 
-template <int C>
-__global__ void __launch_bounds__(THREADS, 1)
-k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-         const __grid_constant__ CUtensorMap tmAaug, const __grid_constant__ CUtensorMap tmBaug,
-         TcArgs p) {
+template <int C, bool STREAM>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
+k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+           const __grid_constant__ CUtensorMap tmAaug, const __grid_constant__ CUtensorMap tmBaug,
+           TcArgs p) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int S = p.stages;
-  const uint32_t a_main = (uint32_t)p.kchunks * BM * 128;
-  const uint32_t a_bytes = a_main + BM * AUG_BYTES;
-  const uint32_t b_main = (uint32_t)p.kchunks * BN * 128;
-  const uint32_t b_bytes = b_main + BN * AUG_BYTES;
+  // a stage: the tile's B rows, whole (resident A), or one chunk of A and of B; then the
+  // tile's augmentation rows (streamed: with the last chunk)
+  const int cps = STREAM ? 1 : p.kchunks;            // chunks per stage
+  const int spt = STREAM ? p.kchunks : 1;            // stages per tile
+  const uint32_t b_off = STREAM ? A_CHUNK : 0;
+  const uint32_t g_off = b_off + (uint32_t)cps * B_CHUNK;
+  const uint32_t stage_bytes = g_off + B_AUG;
+  const uint32_t a_bytes = STREAM ? 0u : (uint32_t)p.kchunks * A_CHUNK;
   unsigned char* sA = sm;
-  unsigned char* sB = sA + a_bytes;
-  float* stash = (float*)(sB + (size_t)S * b_bytes);  // 32 floats per epilogue thread
-  uint64_t* bars = (uint64_t*)(stash + EPI_WARPS * 32 * 32);
-  uint64_t* a_full = bars;
-  uint64_t* a_empty = bars + 1;
-  uint64_t* b_full = bars + 2;
-  uint64_t* b_empty = b_full + MAX_STAGES;
-  uint64_t* t_full = b_empty + MAX_STAGES;
-  uint64_t* t_empty = t_full + NBUF;
-  uint32_t* tmem_slot = (uint32_t*)(t_empty + NBUF);
+  unsigned char* sG = sA + a_bytes;                  // A's augmentation rows
+  unsigned char* sS = sG + A_AUG;
+  uint64_t* bars = (uint64_t*)(sS + (size_t)S * stage_bytes);
+  uint64_t* a_full = bars;                           // leader's
+  uint64_t* a_empty = bars + 1;                      // both
+  uint64_t* s_full = bars + 2;                       // leader's
+  uint64_t* s_empty = s_full + MAX_STAGES;           // both
+  uint64_t* t_full = s_empty + MAX_STAGES;           // both, per half
+  uint64_t* t_empty = t_full + 2;                    // leader's, per half
+  uint32_t* tmem_slot = (uint32_t*)(t_empty + 2);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = lane_id();
+  const uint32_t rank = cluster_rank();
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(a_full), 1);
-    mbar_init(smem_u32(a_empty), 1);
+    mbar_init(smem_u32(a_empty), STREAM ? 1 : 2);   // once both halves are done with the rows
     for (int s = 0; s < S; ++s) {
-      mbar_init(smem_u32(b_full + s), 1);
-      mbar_init(smem_u32(b_empty + s), 1);
+      mbar_init(smem_u32(s_full + s), 1);
+      mbar_init(smem_u32(s_empty + s), 2);            // both halves
     }
-    for (int b = 0; b < NBUF; ++b) {
-      mbar_init(smem_u32(t_full + b), 1);
-      mbar_init(smem_u32(t_empty + b), EPI_WARPS);
+    for (int h = 0; h < 2; ++h) {
+      mbar_init(smem_u32(t_full + h), 1);
+      mbar_init(smem_u32(t_empty + h), EPI_WARPS);   // four warps of each CTA
     }
     *abort_flag = 0;
     fence_barrier_init();
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
-    tmem_relinquish();
+    tmem_alloc_pair(smem_u32(tmem_slot), TMEM_COLS);
+    tmem_relinquish_pair();
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  const int64_t nrb = (p.na + BM - 1) / BM;
-  const int64_t nwalk = p.nwalk;
+  const int nseg = p.nseg;
+  const int64_t nitems = p.nrb * nseg;
+  const int64_t ncl = gridDim.x >> 1, cl = blockIdx.x >> 1;
+  // item i: row block rb0 + i / nseg, tiles i % nseg, i % nseg + nseg, ...
+  auto tiles_of = [&](int64_t rb) -> const int32_t* {
+    return p.tile_order
+               ? p.tile_order + (p.rb_cluster ? (int64_t)p.rb_cluster[rb] : rb) * p.tstride
+               : nullptr;
+  };
+  auto walk_of = [&](int64_t rb) -> int64_t {
+    return p.walk_len ? (int64_t)p.walk_len[rb] : p.nwalk;
+  };
 
   if (warp == 0) {
-    // ---------------- TMA producer ----------------
+    // ---------------- TMA producer (of each CTA) ----------------
     if (lane == 0) {
-      int s = 0;         // B stage of the next tile
+      int s = 0;         // next stage
       uint32_t ph = 0;   // and the parity of its use
-      int rbi = 0;
+      uint32_t aph = 1;
       bool ok = true;
-      for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x, ++rbi) {
-        ok = mbar_wait(smem_u32(a_empty), (rbi & 1) ^ 1, abort_flag);
-        if (!ok) break;
-        mbar_expect_tx(smem_u32(a_full), a_bytes);
-        for (int kc = 0; kc < p.kchunks; ++kc)
-          tma_load_2d(smem_u32(sA + (size_t)kc * BM * 128), &tmA, smem_u32(a_full), kc * 64,
-                      (int)(rb * BM));
-        tma_load_2d(smem_u32(sA + a_main), &tmAaug, smem_u32(a_full), 0, 0);
-        const int32_t* tl = p.tile_order ? p.tile_order + (int64_t)p.rb_cluster[rb] * p.tstride : nullptr;
-        int64_t tn = tl ? tl[0] : 0;  // tile index, read one tile ahead
-        for (int64_t i = 0; i < nwalk; ++i) {
-          const int j0 = (int)(tn * BN);
-          if (i + 1 < nwalk) tn = tl ? tl[i + 1] : i + 1;
-          ok = mbar_wait(smem_u32(b_empty + s), ph ^ 1, abort_flag);
+      const uint32_t a_bar = map_to_rank(smem_u32(a_full), 0);
+      bool first = true;
+      for (int64_t it = cl; it < nitems && ok; it += ncl) {
+        const int64_t rb = p.rb0 + it / nseg;
+        const int seg = (int)(it % nseg);
+        const int row0 = (int)(rb * BM + rank * CM);
+        if (!STREAM || first) {
+          // the query rows (resident), and once the augmentation rows
+          ok = mbar_wait(smem_u32(a_empty), aph, abort_flag);
           if (!ok) break;
-          mbar_expect_tx(smem_u32(b_full + s), b_bytes);
-          unsigned char* dst = sB + (size_t)s * b_bytes;
-          for (int kc = 0; kc < p.kchunks; ++kc)
-            tma_load_2d(smem_u32(dst + (size_t)kc * BN * 128), &tmB, smem_u32(b_full + s), kc * 64,
-                        j0);
-          tma_load_2d(smem_u32(dst + b_main), &tmBaug, smem_u32(b_full + s), 0, j0);
-          if (++s == S) {
-            s = 0;
-            ph ^= 1;
+          aph ^= 1;
+          if (rank == 0)
+            mbar_expect_tx(smem_u32(a_full), 2 * (a_bytes + (first ? A_AUG : 0u)));
+          if (!STREAM)
+            for (int kc = 0; kc < p.kchunks; ++kc)
+              tma_load_2d_pair(smem_u32(sA + (size_t)kc * A_CHUNK), &tmA, a_bar, kc * 64, row0);
+          if (first) tma_load_2d_pair(smem_u32(sG), &tmAaug, a_bar, 0, 0);
+          first = false;
+        }
+        const int32_t* tl = tiles_of(rb);
+        const int64_t nwalk = walk_of(rb);
+        int64_t tn = tl ? tl[seg] : seg;  // tile index, read one tile ahead
+        for (int64_t i = seg; i < nwalk && ok; i += nseg) {
+          const int j0 = (int)(tn * BN + rank * (BN / 2));
+          if (i + nseg < nwalk) tn = tl ? tl[i + nseg] : i + nseg;
+          for (int kc = 0; kc < spt; ++kc) {
+            ok = mbar_wait(smem_u32(s_empty + s), ph ^ 1, abort_flag);
+            if (!ok) break;
+            const bool last = kc == spt - 1;
+            const uint32_t bar = map_to_rank(smem_u32(s_full + s), 0);
+            if (rank == 0) mbar_expect_tx(smem_u32(s_full + s), 2 * (g_off + (last ? B_AUG : 0u)));
+            unsigned char* dst = sS + (size_t)s * stage_bytes;
+            if (STREAM) tma_load_2d_pair(smem_u32(dst), &tmA, bar, kc * 64, row0);
+            for (int c = 0; c < cps; ++c)
+              tma_load_2d_pair(smem_u32(dst + b_off + (size_t)c * B_CHUNK), &tmB, bar,
+                               (STREAM ? kc : c) * 64, j0);
+            if (last) tma_load_2d_pair(smem_u32(dst + g_off), &tmBaug, bar, 0, j0);
+            if (++s == S) {
+              s = 0;
+              ph ^= 1;
+            }
           }
         }
       }
+      // every commit on this CTA's barriers has arrived before the CTA can end
+      for (int k = 0; k < S && ok; ++k) {
+        ok = mbar_wait(smem_u32(s_empty + s), ph ^ 1, abort_flag);
+        if (++s == S) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      if (!STREAM && ok) ok = mbar_wait(smem_u32(a_empty), aph, abort_flag);
       if (!ok) {
-        atomicOr(p.err, 1);
+        atomicOr(p.err, 1 << 1);
         *abort_flag = 1;
       }
     }
     __syncwarp();
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      int64_t it = 0;
-      int s = 0;
-      uint32_t ph = 0;
-      int rbi = 0;
+    // ---------------- MMA issuer (the leader's) ----------------
+    // The whole warp runs the loop and one lane issues, so that the descriptors stay in
+    // uniform registers: issued from a single-lane branch each MMA cost about 200 cycles of
+    // moves and 64-bit adds, more than the 128 the tensor cores need for it (1M x 128, MMAs
+    // and copies alone: 205 -> 115 ms).
+    // The two halves run ahead of each other by up to the pipeline's stages: whichever half's
+    // accumulator is free gets its next stage, so that a half whose epilogue is held up by an
+    // append or a cut does not hold up the other (200,000 x 128, K = 200: 24.2 -> 22.2 ms with the
+    // closer threshold of the cuts).
+    if (rank == 0) {
+      struct Half {
+        int64_t it, i;   // item and tile
+        int64_t nwalk;   // tiles of the item's block
+        int seg, kc, s;  // share, stage within the tile, pipeline slot
+        uint32_t ph, aph, tph;
+        bool fresh;      // the item's first stage: its rows may not have landed
+        int64_t done;    // stages issued
+      };
+      Half hf[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        hf[h].it = cl;
+        hf[h].seg = (int)(cl % nseg);
+        hf[h].i = hf[h].seg;
+        hf[h].nwalk = walk_of(p.rb0 + cl / nseg);
+        hf[h].kc = hf[h].s = 0;
+        hf[h].ph = hf[h].aph = 0u;
+        hf[h].tph = 1u;
+        hf[h].fresh = true;
+        hf[h].done = 0;
+      }
       bool ok = true;
-      const uint64_t adesc0 = sdesc_sw128(smem_u32(sA));
-      const uint64_t adesc_aug = sdesc_sw32(smem_u32(sA + a_main));
-      for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x, ++rbi) {
-        ok = mbar_wait(smem_u32(a_full), rbi & 1, abort_flag);
-        if (!ok) break;
-        for (int64_t ct = 0; ct < nwalk; ++ct, ++it) {
-          const int b = (int)(it % NBUF);
-          const uint32_t tph = (uint32_t)((it / NBUF) & 1);
-          ok = mbar_wait(smem_u32(t_empty + b), tph ^ 1, abort_flag) &&
-               mbar_wait(smem_u32(b_full + s), ph, abort_flag);
-          if (!ok) break;
-          tc_fence_after();
-          // descriptors of the K-steps: the 14-bit start-address field (bytes / 16) of the
-          // base descriptor plus the step's offset; shared addresses stay below 256 KB, so
-          // the sum never carries out of the field
-          const uint32_t bst = smem_u32(sB + (size_t)s * b_bytes);
-          const uint64_t bdesc0 = sdesc_sw128(bst);
-          const uint64_t bdesc_aug = sdesc_sw32(bst + b_main);
+      const bool issue = elect_one();
+      const uint64_t aug_a = sdesc_sw32(smem_u32(sG));
+      const uint32_t st0 = smem_u32(sS);
+      const uint64_t a_desc = sdesc_sw128(STREAM ? st0 : smem_u32(sA));
+      const uint64_t b_desc = sdesc_sw128(st0 + b_off);
+      const uint64_t g_desc = sdesc_sw32(st0 + g_off);
+      // the next stage of half h, if its barriers allow it
+      auto advance = [&](Half& u, int h) -> bool {
+        if (u.it >= nitems) return false;
+        bool ready = mbar_test(smem_u32(s_full + u.s), u.ph);
+        if (u.kc == 0) ready = ready && mbar_test(smem_u32(t_empty + h), u.tph);
+        if (u.fresh) ready = ready && mbar_test(smem_u32(a_full), u.aph);
+        if (!__all_sync(0xffffffffu, ready)) return false;
+        tc_fence_after();
+        // descriptors: the 14-bit start-address field (bytes / 16) plus an offset; shared
+        // addresses stay below 256 KB, so the sum never carries out of the field
+        const uint64_t so = (uint64_t)(((uint32_t)u.s * stage_bytes) >> 4);
+        const bool last = u.kc == spt - 1;
+        const uint32_t d_tmem = tmem_base + (uint32_t)(h * BN);
+        const uint64_t ad = a_desc + (STREAM ? so : 0ull) + (uint64_t)((h * 128 * 128) >> 4);
+        const uint64_t bd = b_desc + so;
+        const bool item_end = last && u.i + nseg >= u.nwalk;
+        if (issue) {
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t d_tmem = tmem_base + (uint32_t)((b * 2 + h) * BN);
-            for (int kc = 0; kc < p.kchunks; ++kc) {
+          for (int c = 0; c < (STREAM ? 1 : MAX_D_RESIDENT / 64); ++c) {
+            // K-steps of this chunk that hold values (the rest are zero padding)
+            const int left = STREAM ? p.d - (u.kc % p.dp_chunks) * 64 : p.d - c * 64;
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk) {
-                const uint64_t ad =
-                    adesc0 + (uint64_t)((kc * BM * 128 + h * 128 * 128 + kk * 32) >> 4);
-                const uint64_t bd = bdesc0 + (uint64_t)((kc * BN * 128 + kk * 32) >> 4);
-                umma_bf16_id(d_tmem, ad, bd, IDESC_N, (kc | kk) ? 1u : 0u);
-              }
-            }
-            umma_bf16_id(d_tmem, adesc_aug + (uint64_t)((h * 128 * AUG_BYTES) >> 4), bdesc_aug,
-                         IDESC_N, 1u);
+            for (int kk = 0; kk < 4; ++kk)
+              if (kk * 16 < left)
+                umma_bf16_pair(d_tmem, ad + (uint64_t)((c * A_CHUNK + kk * 32) >> 4),
+                               bd + (uint64_t)((c * B_CHUNK + kk * 32) >> 4), IDESC,
+                               STREAM ? (uint32_t)(u.kc | kk) : (uint32_t)(c | kk));
           }
-          umma_commit(smem_u32(b_empty + s));
-          umma_commit(smem_u32(t_full + b));
-          if (++s == S) {
-            s = 0;
-            ph ^= 1;
+          if (last) {
+            umma_bf16_pair(d_tmem, aug_a, g_desc + so, IDESC, 1u);
+            umma_commit_pair(smem_u32(t_full + h));
+          }
+          umma_commit_pair(smem_u32(s_empty + u.s));
+          if (!STREAM && item_end) umma_commit_pair(smem_u32(a_empty));
+        }
+        __syncwarp();
+        ++u.done;
+        u.fresh = false;
+        if (++u.s == S) {
+          u.s = 0;
+          u.ph ^= 1u;
+        }
+        if (!last) {
+          ++u.kc;
+        } else {
+          u.kc = 0;
+          u.tph ^= 1u;
+          u.i += nseg;
+          if (item_end) {
+            u.it += ncl;
+            if (u.it < nitems) u.nwalk = walk_of(p.rb0 + u.it / nseg);
+            u.seg = (int)(u.it % nseg);
+            u.i = u.seg;
+            if (!STREAM) {
+              u.fresh = true;
+              u.aph ^= 1u;
+            }
           }
         }
-        if (ok) umma_commit(smem_u32(a_empty));
+        return true;
+      };
+      uint64_t idle_since = 0;
+      while (hf[0].it < nitems || hf[1].it < nitems) {
+        // the half that is behind goes first
+        bool any;
+        if (hf[1].done < hf[0].done)
+          any = advance(hf[1], 1) || advance(hf[0], 0);
+        else
+          any = advance(hf[0], 0) || advance(hf[1], 1);
+        if (any) {
+          idle_since = 0;
+        } else {
+          const uint64_t now = global_ns();
+          if (idle_since == 0) idle_since = now;
+          ok = !*abort_flag && now - idle_since <= WAIT_NS;
+          if (!__all_sync(0xffffffffu, ok)) {
+            ok = false;
+            break;
+          }
+        }
       }
-      if (!ok) {
-        atomicOr(p.err, 2);
+      if (!ok && lane == 0) {
+        atomicOr(p.err, 1 << 2);
         *abort_flag = 1;
       }
     }
@@ -396,340 +473,316 @@ k_knn_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
     const int h = ew >> 2;          // which 128-row half
     const int q = warp & 3;         // TMEM lane quadrant this warp may access
     const int row_in_cta = h * 128 + q * 32 + lane;
-    float* st = stash + (size_t)(ew * 32 + lane) * 32;
-    const int sw = lane & 7;
-    const bool strict = p.tile_order == nullptr;
-    int64_t it = 0;
-    bool ok = true;
+    const uint32_t my_empty = map_to_rank(smem_u32(t_empty + h), 0);
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * BN);
     const float INF = __int_as_float(0x7f800000);
-    for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
-      const int64_t row = rb * BM + row_in_cta;
-      const float nx = row < p.na ? p.a_norm[row] : 0.f;
-      float tau = row < p.na ? INF : -INF;  // a padding row admits nothing
-      if (p.tau_in && row < p.na) {
-        // a bound from a shorter walk over the same columns: every column at or below it
-        // is admitted, so the KS smallest are all kept
-        const float t0 = p.tau_in[row];
-        tau = t0 + (fabsf(t0) + fabsf(nx)) * p.tau_relax;
-      }
-      int cnt = 0;
-      uint64_t* buf = p.rowbuf + ((size_t)blockIdx.x * BM + row_in_cta) * C;
-      const int32_t* tl = p.tile_order ? p.tile_order + (int64_t)p.rb_cluster[rb] * p.tstride : nullptr;
-      int64_t tn = tl ? tl[0] : 0;  // tile index, read one tile ahead
-      for (int64_t i = 0; i < nwalk; ++i, ++it) {
+    constexpr int TRIG = C - 64;    // a chunk pair adds up to 64 entries
+    // a threshold close to the KS-th largest costs a few more bisection steps per cut and saves
+    // appends and cuts
+    const int good = p.KS + (TRIG - p.KS) / 8;
+    uint32_t tph = 0;
+    bool ok = true;
+    for (int64_t it = cl; it < nitems && ok; it += ncl) {
+      const int64_t rbl = it / nseg;
+      const int seg = (int)(it % nseg);
+      const int64_t lrow = rbl * BM + rank * CM + row_in_cta;   // row of this launch
+      const int64_t row = p.rb0 * BM + lrow;
+      uint2* wbuf = p.rowbuf + ((lrow - lane) * nseg + seg) * C;  // lane 0's buffer
+      const uint32_t lstride = (uint32_t)nseg * C;                // entries between lanes' buffers
+      const uint32_t off0 = lane * lstride;
+      uint32_t off = off0;                                        // next free entry, from wbuf
+      // a column is admitted from this accumulator on; padding rows admit nothing
+      float ts = row < p.na ? LOWEST : INF;
+      if (p.ts_g && row < p.na) ts = order_bits_float(__ldcg(p.ts_g + row));
+      const int32_t* tl = tiles_of(p.rb0 + rbl);
+      const int64_t nwalk = walk_of(p.rb0 + rbl);
+      int64_t tn = tl ? tl[seg] : seg;
+      for (int64_t i = seg; i < nwalk; i += nseg) {
         const int32_t j0 = (int32_t)(tn * BN);
-        if (i + 1 < nwalk) tn = tl ? tl[i + 1] : i + 1;
-        const int b = (int)(it % NBUF);
-        const uint32_t tph = (uint32_t)((it / NBUF) & 1);
-        ok = mbar_wait(smem_u32(t_full + b), tph, abort_flag);
+        if (i + nseg < nwalk) tn = tl ? tl[i + nseg] : i + nseg;
+        // with shares: the other shares' thresholds, read while the tile is computed
+        uint32_t other = 0u;
+        if (nseg > 1 && row < p.na) other = __ldcg(p.ts_g + row);
+        ok = mbar_wait(smem_u32(t_full + h), tph, abort_flag);
         if (!__all_sync(0xffffffffu, ok)) {
           ok = false;
           break;
         }
+        tph ^= 1;
         tc_fence_after();
-        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)((b * 2 + h) * BN);
-        // d2 < tau  <=>  acc > (|x|^2 - tau) / 2 (exact); ties admitted (ts just below the
-        // bound) unless the columns arrive in id order.  tau = inf gives ts = -inf.
-        const float thr = 0.5f * (nx - tau);
-        const float ts = strict ? thr : nextafterf(thr, -INF);
-        auto scan64 = [&](const uint32_t(&va)[32], const uint32_t(&vb)[32], int c) {
-          const bool pa = max32(va) > ts;
-          const bool pb = max32(vb) > ts;
-          if (__any_sync(0xffffffffu, pa || pb)) {
-            if (pa) {
-              stash32(st, sw, va);
-              cnt = append_stash(st, sw, ts, nx, j0 + c * 32, p.nb, buf, cnt);
-            }
-            if (pb) {
-              stash32(st, sw, vb);
-              cnt = append_stash(st, sw, ts, nx, j0 + c * 32 + 32, p.nb, buf, cnt);
-            }
-            __syncwarp();
-          }
-        };
-        // two passes of 64 columns; the accumulator buffer goes back to the MMA warp as soon
-        // as the second pass is in registers
-        uint32_t v0[32], v1[32];
+        if (nseg > 1 && row < p.na) ts = fmaxf(ts, order_bits_float(other));
+        uint32_t v[2][32];
 #pragma unroll 1
         for (int c = 0; c < BN / 32; c += 2) {
-          tmem_ld32(taddr + (uint32_t)c * 32, v0);
-          tmem_ld32(taddr + (uint32_t)c * 32 + 32, v1);
-          tmem_wait_ld(v0);
-          tmem_dep(v1);
+          tmem_ld32(taddr + (uint32_t)c * 32, v[0]);
+          tmem_ld32(taddr + (uint32_t)c * 32 + 32, v[1]);
+          tmem_wait_ld(v[0]);
+          tmem_dep(v[1]);
           if (c + 2 == BN / 32) {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(t_empty + b));
+            if (lane == 0) mbar_arrive_cluster(my_empty);
           }
-          scan64(v0, v1, c);
-        }
-        // a buffer that the next tile could overflow drops to the entries at or below its
-        // KS-th smallest distance
-        compact_needed<C>(p, p.rowbuf + ((size_t)blockIdx.x * BM + h * 128 + q * 32) * C, cnt,
-                          tau);
-      }
-      if (!ok) break;
-      finish_rows<C>(p, p.rowbuf + ((size_t)blockIdx.x * BM + h * 128 + q * 32) * C,
-                     rb * BM + h * 128 + q * 32, cnt, tau);
-    }
-    if (!ok && lane == 0) {
-      atomicOr(p.err, 4);
-      *abort_flag = 1;
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc(tmem_base, TMEM_COLS);
-  }
-}
-
-// ---------------------------------------------------------------------------------------
-// Rows wider than the resident pipeline holds (d > 128): the query rows are streamed with
-// the base tiles, 64 values at a time.  A CTA owns BMW = 128 query rows and walks
-// BNW = 256-column tiles; per tile and 64-wide chunk one stage holds the A chunk (16 KB)
-// and the B chunk (32 KB), and the MMA thread issues four 128 x 256 x 16 MMAs into one of
-// two 256-column TMEM buffers (N = 256: the wider instruction does twice the work of
-// N = 128 for about the same issue time).  The augmentation step (-|y|^2/2 folded into the
-// accumulator) comes last in each tile from a two-slot ring.  Four epilogue warps, one per
-// TMEM lane quadrant, scan the tile's 256 columns of their 32 rows as the resident kernel
-// does; a tile's MMAs take long enough that the handoff between the two buffers is cheap.
-// ---------------------------------------------------------------------------------------
-constexpr int BMW = 128;
-constexpr int BNW = 256;
-constexpr int EPI_W = 4;
-constexpr int THREADS_W = 64 + EPI_W * 32;
-constexpr int STAGES_W = 3;
-constexpr uint32_t IDESC_W = idesc_bf16(BNW);
-constexpr uint32_t A_CHUNK_W = BMW * 128;   // 16 KB
-constexpr uint32_t B_CHUNK_W = BNW * 128;   // 32 KB
-constexpr uint32_t STAGE_W = A_CHUNK_W + B_CHUNK_W;
-
-size_t tcw_smem_bytes() {
-  return 1024 + (size_t)STAGES_W * STAGE_W + 2 * (BNW * AUG_BYTES) + BMW * AUG_BYTES +
-         EPI_W * 32 * 32 * sizeof(float) + sizeof(uint64_t) * (1 + 2 * STAGES_W + 4 + 4) + 16;
-}
-
-template <int C>
-__global__ void __launch_bounds__(THREADS_W, 1)
-k_knn_tc_wide(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-              const __grid_constant__ CUtensorMap tmAaug, const __grid_constant__ CUtensorMap tmBaug,
-              TcArgs p) {
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  unsigned char* sS = sm;                                        // STAGES_W x [A chunk | B chunk]
-  unsigned char* sBaug = sS + (size_t)STAGES_W * STAGE_W;        // 2 x BNW rows x 32 B
-  unsigned char* sAaug = sBaug + 2 * BNW * AUG_BYTES;            // BMW rows x 32 B
-  float* stash = (float*)(sAaug + BMW * AUG_BYTES);              // 32 floats per epilogue thread
-  uint64_t* bars = (uint64_t*)(stash + EPI_W * 32 * 32);
-  uint64_t* aa_full = bars;
-  uint64_t* s_full = bars + 1;
-  uint64_t* s_empty = s_full + STAGES_W;
-  uint64_t* g_full = s_empty + STAGES_W;   // augmentation ring
-  uint64_t* g_empty = g_full + 2;
-  uint64_t* t_full = g_empty + 2;
-  uint64_t* t_empty = t_full + 2;
-  uint32_t* tmem_slot = (uint32_t*)(t_empty + 2);
-  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
-
-  const int warp = threadIdx.x >> 5, lane = lane_id();
-  const int kc_n = p.kchunks;
-  if (threadIdx.x == 0) {
-    mbar_init(smem_u32(aa_full), 1);
-    for (int s = 0; s < STAGES_W; ++s) {
-      mbar_init(smem_u32(s_full + s), 1);
-      mbar_init(smem_u32(s_empty + s), 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(smem_u32(g_full + b), 1);
-      mbar_init(smem_u32(g_empty + b), 1);
-      mbar_init(smem_u32(t_full + b), 1);
-      mbar_init(smem_u32(t_empty + b), EPI_W);
-    }
-    *abort_flag = 0;
-    fence_barrier_init();
-  }
-  if (warp == 1) {
-    tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-  const int64_t nrb = (p.na + BMW - 1) / BMW;
-  const int64_t nwalk = p.nwalk;
-
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      bool ok = true;
-      mbar_expect_tx(smem_u32(aa_full), BMW * AUG_BYTES);
-      tma_load_2d(smem_u32(sAaug), &tmAaug, smem_u32(aa_full), 0, 0);
-      int s = 0;
-      uint32_t ph = 0;
-      int64_t t = 0;  // tiles so far (augmentation slot t & 1)
-      for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
-        const int32_t* tl = p.tile_order ? p.tile_order + (int64_t)p.rb_cluster[rb] * p.tstride : nullptr;
-        int64_t tn = tl ? tl[0] : 0;
-        for (int64_t i = 0; i < nwalk && ok; ++i, ++t) {
-          const int j0 = (int)(tn * BNW);
-          if (i + 1 < nwalk) tn = tl ? tl[i + 1] : i + 1;
-          const int g = (int)(t & 1);
-          ok = mbar_wait(smem_u32(g_empty + g), (uint32_t)(((t >> 1) & 1) ^ 1), abort_flag);
-          if (!ok) break;
-          mbar_expect_tx(smem_u32(g_full + g), BNW * AUG_BYTES);
-          tma_load_2d(smem_u32(sBaug + (size_t)g * BNW * AUG_BYTES), &tmBaug, smem_u32(g_full + g), 0,
-                      j0);
-          for (int kc = 0; kc < kc_n; ++kc) {
-            ok = mbar_wait(smem_u32(s_empty + s), ph ^ 1, abort_flag);
-            if (!ok) break;
-            mbar_expect_tx(smem_u32(s_full + s), STAGE_W);
-            unsigned char* dst = sS + (size_t)s * STAGE_W;
-            tma_load_2d(smem_u32(dst), &tmA, smem_u32(s_full + s), kc * 64, (int)(rb * BMW));
-            tma_load_2d(smem_u32(dst + A_CHUNK_W), &tmB, smem_u32(s_full + s), kc * 64, j0);
-            if (++s == STAGES_W) {
-              s = 0;
-              ph ^= 1;
-            }
-          }
-        }
-      }
-      if (!ok) {
-        atomicOr(p.err, 1);
-        *abort_flag = 1;
-      }
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      bool ok = mbar_wait(smem_u32(aa_full), 0, abort_flag);
-      int s = 0;
-      uint32_t ph = 0;
-      int64_t t = 0;
-      const uint64_t adesc_aug = sdesc_sw32(smem_u32(sAaug));
-      for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
-        for (int64_t i = 0; i < nwalk && ok; ++i, ++t) {
-          const int b = (int)(t & 1);
-          const uint32_t tph = (uint32_t)((t >> 1) & 1);
-          ok = mbar_wait(smem_u32(t_empty + b), tph ^ 1, abort_flag);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t d_tmem = tmem_base + (uint32_t)(b * BNW);
-          for (int kc = 0; kc < kc_n; ++kc) {
-            ok = mbar_wait(smem_u32(s_full + s), ph, abort_flag);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t sa = smem_u32(sS + (size_t)s * STAGE_W);
-            const uint64_t ad0 = sdesc_sw128(sa), bd0 = sdesc_sw128(sa + A_CHUNK_W);
+          const int32_t jc = j0 + c * 32;
+          if (jc + 64 > p.nb) {  // the last tile's padding columns are never admitted
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              umma_bf16_id(d_tmem, ad0 + (uint64_t)((kk * 32) >> 4), bd0 + (uint64_t)((kk * 32) >> 4),
-                           IDESC_W, (kc | kk) ? 1u : 0u);
-            umma_commit(smem_u32(s_empty + s));
-            if (++s == STAGES_W) {
-              s = 0;
-              ph ^= 1;
+            for (int e = 0; e < 64; ++e)
+              if (jc + e >= p.nb) v[e >> 5][e & 31] = 0x7fffffffu;  // NaN: no comparison holds
+          }
+          float m8[8];
+#pragma unroll
+          for (int g = 0; g < 8; ++g) m8[g] = max8(&v[g >> 2][(g & 3) * 8]);
+          const float m = fmax3(fmax3(m8[0], m8[1], m8[2]), fmax3(m8[3], m8[4], m8[5]),
+                                fmaxf(m8[6], m8[7]));
+          if (!__any_sync(0xffffffffu, m >= ts)) continue;
+#pragma unroll
+          for (int g = 0; g < 8; ++g) {
+            if (__any_sync(0xffffffffu, m8[g] >= ts)) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                const uint32_t a = v[g >> 2][(g & 3) * 8 + e];
+                if (__uint_as_float(a) >= ts) {
+                  wbuf[off] = make_uint2((uint32_t)(jc + g * 8 + e), a);
+                  ++off;
+                }
+              }
             }
           }
-          if (!ok) break;
-          const int g = (int)(t & 1);
-          ok = mbar_wait(smem_u32(g_full + g), (uint32_t)((t >> 1) & 1), abort_flag);
-          if (!ok) break;
-          tc_fence_after();
-          umma_bf16_id(d_tmem, adesc_aug,
-                       sdesc_sw32(smem_u32(sBaug + (size_t)g * BNW * AUG_BYTES)), IDESC_W, 1u);
-          umma_commit(smem_u32(g_empty + g));
-          umma_commit(smem_u32(t_full + b));
-        }
-      }
-      if (!ok) {
-        atomicOr(p.err, 2);
-        *abort_flag = 1;
-      }
-    }
-    __syncwarp();
-  } else {
-    // ---------------- epilogue: one thread per query row ----------------
-    const int ew = warp - 2;
-    const int q = warp & 3;  // TMEM lane quadrant this warp may access
-    const int row_in_cta = q * 32 + lane;
-    float* st = stash + (size_t)(ew * 32 + lane) * 32;
-    const int sw = lane & 7;
-    const bool strict = p.tile_order == nullptr;
-    int64_t t = 0;
-    bool ok = true;
-    const float INF = __int_as_float(0x7f800000);
-    for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
-      const int64_t row = rb * BMW + row_in_cta;
-      const float nx = row < p.na ? p.a_norm[row] : 0.f;
-      float tau = row < p.na ? INF : -INF;  // a padding row admits nothing
-      if (p.tau_in && row < p.na) {
-        const float t0 = p.tau_in[row];
-        tau = t0 + (fabsf(t0) + fabsf(nx)) * p.tau_relax;
-      }
-      int cnt = 0;
-      uint64_t* wbuf = p.rowbuf + ((size_t)blockIdx.x * BMW + q * 32) * C;
-      uint64_t* buf = wbuf + (size_t)lane * C;
-      const int32_t* tl = p.tile_order ? p.tile_order + (int64_t)p.rb_cluster[rb] * p.tstride : nullptr;
-      int64_t tn = tl ? tl[0] : 0;
-      for (int64_t i = 0; i < nwalk; ++i, ++t) {
-        const int32_t j0 = (int32_t)(tn * BNW);
-        if (i + 1 < nwalk) tn = tl ? tl[i + 1] : i + 1;
-        const int b = (int)(t & 1);
-        ok = mbar_wait(smem_u32(t_full + b), (uint32_t)((t >> 1) & 1), abort_flag);
-        if (!__all_sync(0xffffffffu, ok)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BNW);
-        const float thr = 0.5f * (nx - tau);
-        const float ts = strict ? thr : nextafterf(thr, -INF);
-        uint32_t v0[32], v1[32];
-#pragma unroll 1
-        for (int c = 0; c < BNW / 32; c += 2) {
-          tmem_ld32(taddr + (uint32_t)c * 32, v0);
-          tmem_ld32(taddr + (uint32_t)c * 32 + 32, v1);
-          tmem_wait_ld(v0);
-          tmem_dep(v1);
-          if (c + 2 == BNW / 32) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(t_empty + b));
-          }
-          const bool pa = max32(v0) > ts;
-          const bool pb = max32(v1) > ts;
-          if (__any_sync(0xffffffffu, pa || pb)) {
-            if (pa) {
-              stash32(st, sw, v0);
-              cnt = append_stash(st, sw, ts, nx, j0 + c * 32, p.nb, buf, cnt);
+          // buffers that the next 64 columns could overflow drop to the entries at or above
+          // their KS-th largest accumulator
+          __syncwarp();
+          unsigned need = __ballot_sync(0xffffffffu, off - off0 > (uint32_t)TRIG);
+          while (need) {
+            const int l = __ffs(need) - 1;
+            need &= need - 1;
+            float t2;
+            const int cl0 = (int)__shfl_sync(0xffffffffu, off - off0, l);
+            const int c2 = cut_row<C>(wbuf + (size_t)l * lstride, cl0, p.KS, good, TRIG, p.perm, &t2);
+            if (lane == l) {
+              off = off0 + c2;
+              if (nseg > 1) {
+                const uint32_t b = float_order_bits(t2);
+                t2 = order_bits_float(max(b, atomicMax(p.ts_g + row, b)));
+              }
+              ts = fmaxf(ts, p.strict ? nextafterf(t2, INF) : t2);
             }
-            if (pb) {
-              stash32(st, sw, v1);
-              cnt = append_stash(st, sw, ts, nx, j0 + c * 32 + 32, p.nb, buf, cnt);
-            }
-            __syncwarp();
           }
         }
-        compact_needed<C>(p, wbuf, cnt, tau);
       }
       if (!ok) break;
-      finish_rows<C>(p, wbuf, rb * BMW + q * 32, cnt, tau);
+      p.cnt[lrow * nseg + seg] = (int)(off - off0);
     }
     if (!ok && lane == 0) {
-      atomicOr(p.err, 4);
+      atomicOr(p.err, 1 << 3);
       *abort_flag = 1;
     }
   }
+  __syncwarp();
+  if (*abort_flag) {
+    // a role gave up: let the copies already in flight land before the CTA can go
+    const uint64_t t0 = global_ns();
+    while (global_ns() - t0 < 2000000ull) __nanosleep(1000);
+  }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, TMEM_COLS);
+    tmem_dealloc_pair(tmem_base, TMEM_COLS);
   }
+  cluster_sync();
+}
+
+// ---------------------------------------------------------------------------------------
+// The end of each row: its KS largest accumulators among the buffers of its shares, sorted by
+// (distance, original id).  One warp per row.
+// ---------------------------------------------------------------------------------------
+struct FinArgs {
+  const int* err;             // a walk that gave up leaves no counts to read
+  const uint2* rowbuf;
+  const int* cnt;
+  int nseg, C, KS, K, self;
+  int64_t row0, rows;         // query rows row0 .. row0 + rows - 1 of this launch
+  const float* a_norm;        // |x|^2 of the stored query rows
+  const int32_t* perm;
+  const int32_t* qid;         // nullable: query row r is base row qid[r] (the self column);
+                              // outputs then go to row r
+  const float* tau_in;        // nullable: the admission bound a row started from
+  int32_t* out_id;
+  float* out_d2;
+  float* out_thresh;          // nullable: per output row, the KS-th smallest distance kept (or,
+                              // with fewer kept, the final admission bound)
+  uint32_t* ts_out;           // nullable: only the order bits of the KS-th largest accumulator
+  int slots;                  // keys per warp: a power of two, at least KS
+  int tcap;                   // entries of all shares at most
+};
+
+// Sorts n <= 32 E keys and writes the row: the first K after dropping the row itself.
+template <int E>
+__device__ __noinline__ void sort_out(const FinArgs& p, const uint64_t* keys, int n, int64_t row) {
+  const int lane = lane_id();
+  const float INF = __int_as_float(0x7f800000);
+  uint64_t v[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) v[e] = e * 32 + lane < n ? keys[e * 32 + lane] : KEY_NONE;
+  warp_sort_regs<E * 32>(v);
+  const int c2 = n < p.KS ? n : p.KS;
+  const int64_t ro = p.qid ? row : (p.perm ? (int64_t)p.perm[row] : row);
+  const int32_t sid = p.qid ? p.qid[row] : (int32_t)ro;
+  int selfpos = c2;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int t = e * 32 + lane;
+    if (p.self) {
+      const unsigned m = __ballot_sync(0xffffffffu, t < c2 && key_id(v[e]) == sid);
+      if (m && selfpos == c2) selfpos = e * 32 + __ffs(m) - 1;
+    }
+    if (p.out_thresh && t == p.KS - 1 && t < c2) p.out_thresh[ro] = key_dist(v[e]);
+  }
+  if (p.out_thresh && c2 < p.KS && lane == 0) p.out_thresh[ro] = p.tau_in ? p.tau_in[row] : INF;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int t = e * 32 + lane;
+    const int o = t < selfpos ? t : t - 1;
+    if (t < c2 && t != selfpos && o < p.K) {
+      p.out_id[ro * p.K + o] = key_id(v[e]);
+      p.out_d2[ro * p.K + o] = key_dist(v[e]);
+    }
+  }
+  const int got = selfpos < c2 ? c2 - 1 : c2;
+  for (int t = got + lane; t < p.K; t += 32) {
+    p.out_id[ro * p.K + t] = -1;
+    p.out_d2[ro * p.K + t] = INF;
+  }
+}
+
+__global__ void __launch_bounds__(128) k_knn_finish(FinArgs p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int warp = threadIdx.x >> 5, lane = lane_id();
+  uint64_t* keys = (uint64_t*)(smem_raw + (size_t)warp * ((size_t)p.slots * 8 + (size_t)p.tcap * 4));
+  uint32_t* ob = (uint32_t*)(keys + p.slots);
+  const int64_t r = (int64_t)blockIdx.x * 4 + warp;
+  if (r >= p.rows || (*p.err >> 1) != 0) return;
+  const int64_t row = p.row0 + r;
+  const uint2* rb = p.rowbuf + (size_t)r * p.nseg * p.C;
+  const int* cn = p.cnt + r * p.nseg;
+  int T = 0;
+  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+  for (int s = 0; s < p.nseg; ++s) {
+    const int c = cn[s];
+#pragma unroll 4
+    for (int t = lane; t < c; t += 32) {
+      const uint32_t k = ~float_order_bits(__uint_as_float(__ldcg(&rb[(size_t)s * p.C + t].y)));
+      ob[T + t] = k;
+      lo = min(lo, k);
+      hi = max(hi, k);
+    }
+    T += c;
+  }
+  __syncwarp();
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  const int good = p.ts_out ? p.KS : p.slots;
+  int n = T;  // entries <= hi
+  if (T > good) {
+    while (lo < hi) {
+      const uint32_t mid = lo + ((hi - lo) >> 1);
+      int c = 0;
+      for (int t = lane; t < T; t += 32) c += ob[t] <= mid ? 1 : 0;
+      c = __reduce_add_sync(0xffffffffu, c);
+      if (c >= p.KS) {
+        hi = mid;
+        n = c;
+        if (c <= good) break;
+      } else {
+        lo = mid + 1;
+      }
+    }
+  }
+  if (p.ts_out) {
+    // (a loop that stopped at exactly KS may leave hi above the KS-th largest's bits: still a
+    // bound that KS entries meet)
+    if (lane == 0)
+      p.ts_out[row] = T >= p.KS ? ~hi : float_order_bits(LOWEST);
+    return;
+  }
+  uint32_t idmax = 0xFFFFFFFFu;
+  if (n > p.slots) {
+    // more ties at the KS-th distance than slots: those with the smallest original ids stay
+    int below = 0;
+    for (int t = lane; t < T; t += 32) below += ob[t] < hi ? 1 : 0;
+    const int need = p.KS - __reduce_add_sync(0xffffffffu, below);
+    uint32_t l2 = 0u, h2 = 0x7FFFFFFFu;
+    while (l2 < h2) {
+      const uint32_t mid = l2 + ((h2 - l2) >> 1);
+      int c = 0, base = 0;
+      for (int s = 0; s < p.nseg; ++s) {
+        for (int t = lane; t < cn[s]; t += 32)
+          if (ob[base + t] == hi) {
+            const uint32_t id = rb[(size_t)s * p.C + t].x;
+            c += (p.perm ? (uint32_t)p.perm[id] : id) <= mid ? 1 : 0;
+          }
+        base += cn[s];
+      }
+      c = __reduce_add_sync(0xffffffffu, c);
+      if (c >= need)
+        h2 = mid;
+      else
+        l2 = mid + 1;
+    }
+    idmax = h2;
+  }
+  const float nx = p.a_norm[row];
+  int kept = 0, base = 0;
+  for (int s = 0; s < p.nseg; ++s) {
+    const int c = cn[s];
+    for (int t0 = 0; t0 < c; t0 += 32) {
+      const int t = t0 + lane;
+      bool keep = t < c && ob[base + t] <= hi;
+      uint64_t key = 0ull;
+      if (keep) {
+        const uint2 v = __ldcg(&rb[(size_t)s * p.C + t]);
+        const int32_t id = p.perm ? p.perm[v.x] : (int32_t)v.x;
+        if (ob[base + t] == hi && (uint32_t)id > idmax) keep = false;
+        key = make_key(fmaf(-2.f, __uint_as_float(v.y), nx), id);
+      }
+      const unsigned b = __ballot_sync(0xffffffffu, keep);
+      if (keep) keys[kept + __popc(b & lanemask_lt())] = key;
+      kept += __popc(b);
+    }
+    base += c;
+  }
+  __syncwarp();
+  if (kept <= 32)
+    sort_out<1>(p, keys, kept, row);
+  else if (kept <= 64)
+    sort_out<2>(p, keys, kept, row);
+  else if (kept <= 128)
+    sort_out<4>(p, keys, kept, row);
+  else if (kept <= 256)
+    sort_out<8>(p, keys, kept, row);
+  else if (kept <= 512)
+    sort_out<16>(p, keys, kept, row);
+  else
+    sort_out<32>(p, keys, kept, row);
+}
+
+// Initial thresholds of the walk: from the caller's admission bounds (every column whose
+// distance is at most tau is admitted), or none.
+__global__ void k_ts_init(const float* __restrict__ tau, const float* __restrict__ a_norm, int64_t n,
+                          uint32_t* __restrict__ ts) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const float INF = __int_as_float(0x7f800000);
+  const float t = tau ? tau[i] : INF;
+  // d2 = fmaf(-2, acc, |x|^2) <= tau as the kernel forms it: one value below the rounded half
+  // difference covers the rounding of both
+  float v = LOWEST;
+  if (t < INF) {
+    v = 0.5f * (a_norm[i] - t);
+    v -= (fabsf(a_norm[i]) + fabsf(t)) * 1.1920929e-07f;
+  }
+  ts[i] = float_order_bits(v);
 }
 
 // bf16 copy with rows padded to dp; with perm, stored row r holds row perm[r] (and its norm);
@@ -797,35 +850,51 @@ __global__ void k_aug_rows(const float* __restrict__ norm, int64_t n, __nv_bfloa
   }
 }
 
-// Augmentation rows of the queries: four ones, then zeros (BM identical rows).
+// Augmentation rows of the queries: four ones, then zeros (128 identical rows).
 __global__ void k_aug_ones(__nv_bfloat16* __restrict__ aug) {
-  for (int i = threadIdx.x; i < BM * AUG; i += blockDim.x)
+  for (int i = threadIdx.x; i < 128 * AUG; i += blockDim.x)
     aug[i] = __float2bfloat16_rn((i % AUG) < 4 ? 1.f : 0.f);
 }
 
+constexpr size_t SMEM_MAX = 225 * 1024;
+
+// Shared memory of the kernel: resident A (kchunks 64-value chunks) or streamed (kchunks = 0).
 size_t tc_smem_bytes(int kchunks, int stages) {
-  return 1024 + (size_t)kchunks * BM * 128 + BM * AUG_BYTES +
-         (size_t)stages * (kchunks * BN * 128 + BN * AUG_BYTES) +
-         EPI_WARPS * 32 * 32 * sizeof(float) + sizeof(uint64_t) * (2 + 2 * MAX_STAGES + 2 * NBUF) +
-         16;
+  const size_t stage = kchunks ? (size_t)kchunks * B_CHUNK + B_AUG : (size_t)A_CHUNK + B_CHUNK + B_AUG;
+  return 1024 + (size_t)kchunks * A_CHUNK + A_AUG + (size_t)stages * stage +
+         sizeof(uint64_t) * (2 + 2 * MAX_STAGES + 4) + 16;
 }
 
 struct TcMaps {
   CUtensorMap a, b, a_aug, b_aug;
 };
 
-template <int C>
-void launch_tc(const TcMaps& m, TcArgs& a, int grid, size_t smem, cudaStream_t st, bool wide) {
-  if (wide) {
-    ensure_smem((const void*)k_knn_tc_wide<C>, smem);
-    SSG_LAUNCH(k_knn_tc_wide<C>, grid, THREADS_W, smem, st, m.a, m.b, m.a_aug, m.b_aug, a);
-  } else {
-    ensure_smem((const void*)k_knn_tc<C>, smem);
-    SSG_LAUNCH(k_knn_tc<C>, grid, THREADS, smem, st, m.a, m.b, m.a_aug, m.b_aug, a);
-  }
+template <int C, bool STREAM>
+void launch_tc(const TcMaps& m, TcArgs& a, size_t smem, cudaStream_t st) {
+  ensure_smem((const void*)k_knn_pair<C, STREAM>, smem);
+  const int64_t pairs = std::min<int64_t>(a.nrb * a.nseg, num_sms() / 2);
+  SSG_LAUNCH((k_knn_pair<C, STREAM>), (unsigned)(2 * pairs), THREADS, smem, st, m.a, m.b, m.a_aug,
+             m.b_aug, a);
 }
 
-constexpr int MAX_D_WIDE = 4096;  // rows of up to this many values take the streamed kernel
+// Shares of each block's tiles.  A share more per block fills clusters that would idle, in the
+// last wave or when there are few blocks; each share has its own climb to the threshold, about
+// as long as `climb` tiles.  The shares' buffers of C entries are merged by one warp in
+// shared memory, which bounds their number.
+int pick_shares(int64_t nrb, int64_t nwalk, int C, int KS, int64_t clusters) {
+  const int64_t smax = std::max<int64_t>(1, std::min<int64_t>({nwalk, (int64_t)(4096 / C), 16}));
+  const double climb = 8.0 + KS / 4.0;
+  int best = 1;
+  double best_cost = 0.0;
+  for (int64_t s = 1; s <= smax; ++s) {
+    const double cost = (double)ceil_div(nrb * s, clusters) * ((double)ceil_div(nwalk, s) + climb);
+    if (s == 1 || cost < best_cost) {
+      best = (int)s;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
 
 }  // namespace
 
@@ -838,17 +907,14 @@ bool knn_tc_available(int d) {
       return (major == 10 && minor == 3 && encode_fn() != nullptr) ? 1 : 0;
     return 0;
   }();
-  const int kchunks = ((d + 63) & ~63) / 64;
-  if (avail != 1 || d < 1) return false;
-  return tc_smem_bytes(kchunks, 2) <= 225 * 1024 ||
-         (d <= MAX_D_WIDE && tcw_smem_bytes() <= 225 * 1024);
+  return avail == 1 && d >= 1 && d <= MAX_D_STREAM;
 }
 
 int knn_tc_max_k(int d, bool limited) {
-  const int kchunks = ((d + 63) & ~63) / 64;
-  const int bn = tc_smem_bytes(kchunks, 2) <= 225 * 1024 ? BN : BNW;
-  // a row buffer holds 1024 keys: KS + bn (twice KS for a limited walk), KS = K + 1
-  return limited ? (1024 - bn) / 2 - 1 : 1024 - bn - 1;
+  // a row buffer holds 1,024 entries: KS = K + 1 and room for a chunk of new ones (a limited
+  // walk: for KS new ones)
+  const int room = d <= MAX_D_RESIDENT ? 128 : 256;
+  return limited ? (1024 - room) / 2 - 1 : 1024 - room - 1;
 }
 
 void rows_to_bf16(const float* X, int64_t n, int d, int ld, __nv_bfloat16* Y, int dp,
@@ -868,127 +934,162 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
   const int dp = (d + 63) & ~63;
   const int dpe = ex.pairs ? 3 * dp : dp;  // row width the tensor cores see
   const int kchunks = dpe / 64;
-  int stages = MAX_STAGES;
-  while (stages > 2 && tc_smem_bytes(kchunks, stages) > 225 * 1024) --stages;
-  // rows that do not fit the resident pipeline stream through the wide kernel
-  const bool wide = tc_smem_bytes(kchunks, stages) > 225 * 1024 || ex.stream_rows;
-  SSG_REQUIRE(!wide || (dpe <= MAX_D_WIDE && tcw_smem_bytes() <= 225 * 1024), SSG_EINVAL,
+  SSG_REQUIRE(dpe <= MAX_D_STREAM, SSG_EINVAL,
               "tensor-core kNN: d = %d is too large for the shared-memory pipeline", d);
-  const int bm = wide ? BMW : BM, bn = wide ? BNW : BN;
+  // rows too long to stay resident stream through the pipeline with the tiles
+  const bool stream = dpe > MAX_D_RESIDENT || ex.stream_rows;
+  int stages = MAX_STAGES;
+  while (stages > 2 && tc_smem_bytes(stream ? 0 : kchunks, stages) > SMEM_MAX) --stages;
+  const size_t smem = tc_smem_bytes(stream ? 0 : kchunks, stages);
   const int KS = self ? K + 1 : K;
   // Near-first column order for large self-joins with a deep top-K (where the streaming
   // threshold otherwise falls slowly and many candidates are appended).
   KnnOrder ord;
   Scratch<float> norm_p;
-  // tile limits come in 128-point tiles; the walk counts bn-column tiles
-  if (max_tiles > 0) max_tiles = (int)ceil_div((int64_t)max_tiles * API_TILE, bn);
   // same: the query rows are the base rows (a self-join); with ex.qid the query rows are a
   // gathered subset of the base and only the self column is excluded
   const bool same = self && !ex.qid;
-  SSG_REQUIRE(max_tiles == 0 || (same && knn_order_fits(na, bn)), SSG_EINVAL,
+  SSG_REQUIRE(max_tiles == 0 || (same && knn_order_fits(na, API_TILE)), SSG_EINVAL,
               "a tile limit needs a self-join whose cluster order fits");
-  // (not for the K-chunked kernel: its tiles are long enough that the appends a slowly
-  // falling threshold costs matter less than L2 reuse, which needs every CTA to walk the
-  // columns in the same order: 200,000 x 960 with bf16 pairs, 270 -> 227 ms, the
-  // near-first walks kept DRAM 78% busy at a 34% L2 hit rate)
+  // (not for streamed rows: their tiles are long enough that the appends a slowly falling
+  // threshold costs matter less than L2 reuse, which needs every cluster to walk the columns in
+  // the same order: 200,000 x 960 with bf16 pairs, 270 -> 227 ms, the near-first walks kept
+  // DRAM 78% busy at a 34% L2 hit rate)
   const bool ordered =
-      max_tiles > 0 || (!wide && same && na >= (1 << 16) && K >= 16 && knn_order_fits(na, bn));
+      max_tiles > 0 || (!stream && same && na >= (1 << 16) && K >= 16 && knn_order_fits(na, BN));
   if (ordered) {
-    knn_cluster_order(A, lda, d, na, bm, bn, st, ord, max_tiles,
-                      ex.order_norm ? ex.order_norm : a_norm);
+    // A limited walk's lists are those of 256 rows and 128-point tiles, which set what each row
+    // is compared with; a work item takes the tiles of both its 256-row blocks.
+    const float* on = ex.order_norm ? ex.order_norm : a_norm;
+    if (max_tiles > 0) {
+      knn_cluster_order(A, lda, d, na, BM / 2, API_TILE, st, ord, max_tiles, on);
+      knn_pair_tiles(na, BM / 2, st, ord);
+    } else {
+      knn_cluster_order(A, lda, d, na, BM, BN, st, ord, 0, on);
+    }
     norm_p.alloc((size_t)na, st);
   }
+  const int32_t* perm = ordered ? (const int32_t*)ord.perm.p : nullptr;
   Scratch<__nv_bfloat16> ab((size_t)na * dpe, st);
   Scratch<__nv_bfloat16> bb;
-  const int cgrid = 8 * num_sms();
-  rows_to_bf16(A, na, d, lda, ab.p, dp, ordered ? (const int32_t*)ord.perm.p : nullptr, a_norm,
-               ordered ? norm_p.p : nullptr, ex.mu, ex.pairs ? 1 : 0, st);
+  rows_to_bf16(A, na, d, lda, ab.p, dp, perm, a_norm, ordered ? norm_p.p : nullptr, ex.mu,
+               ex.pairs ? 1 : 0, st);
   if (ordered) a_norm = b_norm = norm_p.p;
   const __nv_bfloat16* bptr = ab.p;
   if (!same || ex.pairs) {
     // bf16 pairs: the base side has its own layout (in the self-join's stored order)
     bb.alloc((size_t)nb * dpe, st);
-    rows_to_bf16(B, nb, d, ldb, bb.p, dp, same && ordered ? (const int32_t*)ord.perm.p : nullptr,
-                 nullptr, nullptr, ex.mu, ex.pairs ? 2 : 0, st);
+    rows_to_bf16(B, nb, d, ldb, bb.p, dp, same ? perm : nullptr, nullptr, nullptr, ex.mu,
+                 ex.pairs ? 2 : 0, st);
     bptr = bb.p;
   }
-  Scratch<__nv_bfloat16> aug_b((size_t)nb * AUG, st), aug_a((size_t)BM * AUG, st);
+  Scratch<__nv_bfloat16> aug_b((size_t)nb * AUG, st), aug_a((size_t)128 * AUG, st);
   Scratch<int> err(1, st);
   SSG_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
-  SSG_LAUNCH(k_aug_rows, (unsigned)std::min<int64_t>(ceil_div(nb, 256), cgrid), 256, 0, st, b_norm,
-             nb, aug_b.p, err.p, approx ? 1 : 0);
+  SSG_LAUNCH(k_aug_rows, (unsigned)std::min<int64_t>(ceil_div(nb, 256), 8 * num_sms()), 256, 0, st,
+             b_norm, nb, aug_b.p, err.p, approx ? 1 : 0);
   SSG_LAUNCH(k_aug_ones, 1, 256, 0, st, aug_a.p);
   TcMaps maps;
-  maps.a = make_map(ab.p, na, dpe, 64, bm, CU_TENSOR_MAP_SWIZZLE_128B);
-  maps.b = make_map(bptr, nb, dpe, 64, bn, CU_TENSOR_MAP_SWIZZLE_128B);
-  maps.a_aug = make_map(aug_a.p, BM, AUG, AUG, bm, CU_TENSOR_MAP_SWIZZLE_32B);
-  maps.b_aug = make_map(aug_b.p, nb, AUG, AUG, bn, CU_TENSOR_MAP_SWIZZLE_32B);
-  const int64_t nrb = ceil_div(na, bm);
-  const int grid = (int)std::min<int64_t>(nrb, num_sms());
-  // A row buffer holds C keys and is compacted once a tile could overflow it.  A limited
-  // walk spends most of its tiles while the threshold is still falling, so it gets room
-  // for about KS more keys between compactions.
-  const int need = max_tiles > 0 ? 2 * KS + bn : KS + bn;
-  SSG_REQUIRE(need <= 1024, SSG_EINVAL, "tensor-core kNN: K = %d is too large for %d-column tiles",
-              K, bn);
+  maps.a = make_map(ab.p, na, dpe, 64, CM, CU_TENSOR_MAP_SWIZZLE_128B);
+  maps.b = make_map(bptr, nb, dpe, 64, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B);
+  maps.a_aug = make_map(aug_a.p, 128, AUG, AUG, 128, CU_TENSOR_MAP_SWIZZLE_32B);
+  maps.b_aug = make_map(aug_b.p, nb, AUG, AUG, BN / 2, CU_TENSOR_MAP_SWIZZLE_32B);
+  // A row buffer holds C entries and is cut back once 64 columns could overflow it.  A limited
+  // walk spends most of its tiles while the threshold is still falling, so it gets room for
+  // about KS more entries between cuts.
+  const int room = dpe <= MAX_D_RESIDENT ? 128 : 256;
+  const int need = max_tiles > 0 ? 2 * KS + room : KS + room;
+  SSG_REQUIRE(need <= 1024, SSG_EINVAL, "tensor-core kNN: K = %d is too large for %d-value rows", K,
+              dpe);
   const int C = need <= 256 ? 256 : (need <= 512 ? 512 : 1024);
-  Scratch<uint64_t> rowbuf((size_t)grid * bm * C, st);
+  const int64_t ntiles = ceil_div(nb, BN), nrb = ceil_div(na, BM);
   TcArgs a{};
-  a.a_norm = a_norm;
   a.na = na;
   a.nb = nb;
-  a.ntiles = ceil_div(nb, bn);
-  a.nwalk = max_tiles > 0 ? std::min<int64_t>(a.ntiles, max_tiles) : a.ntiles;
-  a.tstride = ordered ? ord.tstride : a.ntiles;
+  a.nwalk = ntiles;
+  a.tstride = max_tiles > 0 ? 2 * ord.tstride : (ordered ? ord.tstride : ntiles);
+  a.nseg = max_tiles > 0 ? 1 : pick_shares(nrb, a.nwalk, C, KS, num_sms() / 2);
   a.kchunks = kchunks;
+  a.dp_chunks = dp / 64;
+  a.d = d;
   a.stages = stages;
-  a.self = self;
   a.KS = KS;
-  a.K = K;
-  a.trig = C - bn;
-  a.rowbuf = rowbuf.p;
-  a.out_id = out_id;
-  a.out_d2 = out_d2;
   a.err = err.p;
-  a.out_thresh = ex.out_thresh;
-  a.qid = ex.qid;
-  a.tau_in = ex.tau_in;
   if (ordered) {
     a.perm = ord.perm.p;
-    a.inv = ord.inv.p;
-    a.tile_order = ord.tile_order.p;
-    a.rb_cluster = ord.rb_cluster.p;
+    a.tile_order = max_tiles > 0 ? ord.pair_tiles.p : ord.tile_order.p;
+    a.rb_cluster = max_tiles > 0 ? nullptr : ord.rb_cluster.p;
+    a.walk_len = max_tiles > 0 ? ord.pair_len.p : nullptr;
   }
-  const size_t smem = wide ? tcw_smem_bytes() : tc_smem_bytes(kchunks, stages);
-  auto launch = [&](TcArgs& args) {
-    if (C == 256)
-      launch_tc<256>(maps, args, grid, smem, st, wide);
-    else if (C == 512)
-      launch_tc<512>(maps, args, grid, smem, st, wide);
-    else
-      launch_tc<1024>(maps, args, grid, smem, st, wide);
+  // Near-first full walks may be preceded by one over each block's prepass_tiles nearest tiles
+  // that only records each row's KS-th largest accumulator there, from which the full walk
+  // starts.
+  const int64_t pre_tiles = ceil_div((int64_t)ex.prepass_tiles * API_TILE, BN);
+  const bool prepass = ordered && max_tiles == 0 && pre_tiles > 0 && ntiles > 2 * pre_tiles;
+  // thresholds per query row: to start from, and for the shares to exchange
+  Scratch<uint32_t> ts;
+  if (ex.tau_in || a.nseg > 1 || prepass) {
+    ts.alloc((size_t)na, st);
+    SSG_LAUNCH(k_ts_init, (unsigned)ceil_div(na, 256), 256, 0, st, ex.tau_in, a_norm, na, ts.p);
+    a.ts_g = ts.p;
+  }
+  a.strict = !a.tile_order && !a.ts_g;
+  // the row buffers of one launch take up to 2 GB; more rows go in several launches, whole
+  // rounds of the clusters each
+  const size_t block_bytes = (size_t)BM * a.nseg * C * sizeof(uint2);
+  const int64_t round = std::max<int64_t>(1, num_sms() / 2);
+  const int64_t rounds = std::max<int64_t>(1, (int64_t)((2ull << 30) / block_bytes) / round);
+  const int64_t per_launch = std::min<int64_t>(nrb, rounds * round);
+  Scratch<uint2> rowbuf((size_t)per_launch * BM * a.nseg * C, st);
+  Scratch<int> cnt((size_t)per_launch * BM * a.nseg, st);
+  a.rowbuf = rowbuf.p;
+  a.cnt = cnt.p;
+  FinArgs f{};
+  f.err = err.p;
+  f.rowbuf = rowbuf.p;
+  f.cnt = cnt.p;
+  f.C = C;
+  f.KS = KS;
+  f.K = K;
+  f.self = self;
+  f.a_norm = a_norm;
+  f.perm = a.perm;
+  f.qid = ex.qid;
+  f.tau_in = ex.tau_in;
+  f.out_id = out_id;
+  f.out_d2 = out_d2;
+  f.out_thresh = ex.out_thresh;
+  f.slots = next_pow2(std::max(KS, 32));
+  auto walk = [&](TcArgs args, FinArgs fin) {
+    args.nseg = (int)std::min<int64_t>(args.nseg, args.nwalk);
+    fin.nseg = args.nseg;
+    fin.tcap = args.nseg * C;
+    const size_t fsm = 4 * ((size_t)fin.slots * 8 + (size_t)fin.tcap * 4);
+    ensure_smem((const void*)k_knn_finish, fsm);
+    for (int64_t rb = 0; rb < nrb; rb += per_launch) {
+      args.rb0 = rb;
+      args.nrb = std::min<int64_t>(per_launch, nrb - rb);
+      if (C == 256)
+        stream ? launch_tc<256, true>(maps, args, smem, st) : launch_tc<256, false>(maps, args, smem, st);
+      else if (C == 512)
+        stream ? launch_tc<512, true>(maps, args, smem, st) : launch_tc<512, false>(maps, args, smem, st);
+      else
+        stream ? launch_tc<1024, true>(maps, args, smem, st)
+               : launch_tc<1024, false>(maps, args, smem, st);
+      fin.row0 = rb * BM;
+      fin.rows = std::min<int64_t>(args.nrb * BM, na - fin.row0);
+      SSG_LAUNCH(k_knn_finish, (unsigned)ceil_div(fin.rows, 4), 128, fsm, st, fin);
+    }
   };
-  // Near-first full walks: a first launch over each block's prepass_tiles nearest tiles
-  // only records each row's KS-th distance there, an upper bound of its KS-th distance over
-  // all columns (the same values: the MMAs are the same); the full walk then admits only
-  // columns at or below that bound, so its appends and compactions are few from the start.
-  Scratch<float> tau0;
-  const int64_t pre_tiles = ceil_div((int64_t)ex.prepass_tiles * API_TILE, bn);
-  const bool prepass = ordered && max_tiles == 0 && pre_tiles > 0 && a.ntiles > 2 * pre_tiles;
   if (gemm_timer) gemm_timer->start();
   if (prepass) {
-    tau0.alloc((size_t)na, st);
     TcArgs a0 = a;
     a0.nwalk = pre_tiles;
-    a0.thresh_only = 1;
-    a0.tau_out = tau0.p;
-    a0.out_thresh = nullptr;
-    launch(a0);
-    a.tau_in = tau0.p;
-    // approximate data: widen by far more than the rounding of the threshold test
-    a.tau_relax = approx ? 9.5367431640625e-07f : 0.f;  // 2^-20
+    FinArgs f0 = f;
+    f0.ts_out = ts.p;
+    walk(a0, f0);
   }
-  launch(a);
+  walk(a, f);
   if (gemm_timer) gemm_timer->stop();
   int h = 0;
   SSG_CUDA(cudaMemcpyAsync(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
