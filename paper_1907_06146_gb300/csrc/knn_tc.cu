@@ -18,9 +18,9 @@
 //               bf16 with 128-byte swizzle, plus the 16-element augmentation rows with 32-byte
 //               swizzle.  All of them complete on the leader CTA's barriers;
 //   warp 1      allocates 512 TMEM columns; the leader's issues tcgen05.mma of the pair: M =
-//               256 (128 rows of each CTA), N = 256, one accumulator of 256 columns for each
-//               of the two 128-row halves of a CTA's rows, so the epilogue drains one half
-//               while the MMAs fill the other;
+//               256 (128 rows of each CTA), N = 128 (streamed: 256), into four accumulators of
+//               128 columns: two column halves for each of the two 128-row halves of a CTA's
+//               rows, so the epilogue drains some while the MMAs fill others;
 //   warps 2..9  epilogue, one thread per query row (TMEM lane): tcgen05.ld 64 columns at a
 //               time, their largest accumulator against the row's threshold (a tree of
 //               three-input maxes), and only where some lane passes, the passing (id,
@@ -29,21 +29,22 @@
 // k_knn_finish then takes each row's KS largest from the buffers of its shares, sorts them by
 // (distance, original id) and writes the K neighbours, with many rows per SM in flight.
 //
-// Why this shape.  128 x 128 x 16 MMAs of one CTA take 98 cycles each instead of 64: both
-// operands come from shared memory.  A pair reads half of B per CTA for an MMA of four times
-// the work, and each column tile is read from L2 once for 512 rows instead of 256 (773 GB of
-// DRAM reads for a graph of 1M x 128 before).  A tile's two halves wait for their own
-// epilogue warps only.  Appending from registers costs four instructions per column of an
-// eight-column group that some lane passes; parking the chunk in shared memory and scanning it
-// back cost about 250 cycles per chunk.  Few row blocks (10,000 queries, a sample of 256 rows)
-// used to leave most SMs idle: their columns are shared out over `nseg` items per block, and
-// the shares exchange thresholds through global memory.
+// Why this shape.  A pair reads half of B per CTA for an MMA of four times the work of one
+// CTA's 128 x 128, and each column tile is read from L2 once for 512 rows instead of 256 (773
+// GB of DRAM reads for a graph of 1M x 128 before).  The epilogue holds an accumulator for two
+// TMEM loads of 64 columns, about 900 cycles with the handoff, against the 2,300 the four take
+// to fill at d = 128 (two accumulators of 256 columns, held for four loads, were the bound:
+// 1M x 128, K = 200, 249 -> 223 ms).  Appending from registers needs no stash in shared memory
+// (its scan cost about 250 cycles per chunk).  Few row blocks (10,000 queries, a sample of 256
+// rows) used to leave most SMs idle: their columns are shared out over `nseg` items per block,
+// and the shares exchange thresholds through global memory.  What bounds it now: the epilogue
+// of the tiles in which rows still append (a warp's chunk with appends takes 500-1,800 cycles,
+// a cut of a row's buffer 3,000-5,000), then the MMAs.
 // Measured, whole kNN stage, against the kernel of one CTA and 128 x 128 MMAs: 1M x 128,
-// K = 200, 341 -> 233 ms; 10,000 queries over 1M rows, K = 100, 15.0 -> 6.8 ms.
+// K = 200, 341 -> 223 ms; 10,000 queries over 1M rows, K = 100, 15.0 -> 6.0 ms.
 //
 // Columns are visited in 256-wide tiles, in id order or (large self-joins) nearest cluster
-// first; in id order and one share "acc > threshold" also settles equal distances by id,
-// otherwise ties are admitted and settled at the end.
+// first; ties at the threshold are admitted and settled by original id at the end.
 // Every wait on an mbarrier is bounded (about 2 s); a wait that runs out sets an error
 // word, tells the other roles to stop, and the CTA releases its TMEM and exits.
 #include <cuda.h>
@@ -64,10 +65,11 @@ constexpr int BM = 512;               // query rows per work item (256 per CTA o
 constexpr int CM = 256;               // query rows per CTA: two halves of 128 TMEM lanes
 constexpr int BN = 256;               // base columns per tile (UMMA_N), 128 rows of B per CTA
 constexpr int API_TILE = 128;         // tile limits are given in 128-point tiles
-constexpr uint32_t IDESC = idesc_bf16_pair(BN);
+constexpr uint32_t IDESC = idesc_bf16_pair(BN), IDESC_HALF = idesc_bf16_pair(BN / 2);
+constexpr int NBUF = 4;               // TMEM accumulators of 128 columns: two per half of the rows
 constexpr int EPI_WARPS = 8;
 constexpr int THREADS = 64 + EPI_WARPS * 32;
-constexpr int TMEM_COLS = 512;        // 2 halves x 256 fp32 columns
+constexpr int TMEM_COLS = 512;        // NBUF x 128 fp32 columns
 constexpr int MAX_STAGES = 6;
 constexpr int MAX_D_RESIDENT = 128;   // rows of up to this many values stay resident
 constexpr int MAX_D_STREAM = 4096;    // longer ones, up to this, are streamed
@@ -89,7 +91,6 @@ struct TcArgs {
   int kchunks;          // row width / 64
   int dp_chunks, d;     // chunks of one part of a row (bf16 pairs: three parts), its values
   int stages;
-  int strict;           // 1: columns equal to the threshold are not admitted
   int KS;
   uint2* rowbuf;        // [rows of this launch][nseg][C] (id, accumulator bits)
   int* cnt;             // [rows of this launch][nseg]
@@ -115,96 +116,125 @@ __device__ __forceinline__ float max8(const uint32_t* v) {
   return fmax3(a, b, fmaxf(__uint_as_float(v[6]), __uint_as_float(v[7])));
 }
 
-// Cuts one row's buffer of cnt >= KS (id, accumulator) pairs back to the entries at or above a
-// threshold with between KS and `good` of them (in no particular order), found by bisection
-// over the order bits; if ties at the KS-th largest would keep more than `cap`,
-// exactly KS stay, the ties with the smallest original ids.  Returns the new count; *ts gets
-// the threshold (at least KS entries are not below it).  Warp-wide, out of line: it runs
-// rarely, and one copy keeps the scan small in the instruction cache.
+// The order keys of one row's values (ascending: larger accumulators first; absent ones
+// 0xFFFFFFFF) are spread over the warp, E per lane.  Finds hi such that between KS and `good`
+// keys are at most hi (more only where ties at the KS-th force it) by a search over the bits,
+// three pivots a step; lo .. hi: the present keys' range, n: their number, at least KS.
+// Returns the number of keys at most hi.
+template <int E>
+__device__ __forceinline__ int search_keys(const uint32_t (&k)[E], int KS, int good, uint32_t lo,
+                                           uint32_t& hi, int n) {
+  while (lo < hi) {
+    const uint32_t q = (hi - lo) >> 2;
+    const uint32_t m1 = lo + q, m2 = lo + ((hi - lo) >> 1), m3 = m2 + q;
+    uint32_t c12[4] = {0u, 0u, 0u, 0u}, c3[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      c12[e & 3] += (k[e] <= m1 ? 1u : 0u) + (k[e] <= m2 ? 0x10000u : 0u);
+      c3[e & 3] += k[e] <= m3 ? 1u : 0u;
+    }
+    const uint32_t a12 = __reduce_add_sync(0xffffffffu, (c12[0] + c12[1]) + (c12[2] + c12[3]));
+    const int a3 = (int)__reduce_add_sync(0xffffffffu, (c3[0] + c3[1]) + (c3[2] + c3[3]));
+    const int a1 = (int)(a12 & 0xffffu), a2 = (int)(a12 >> 16);
+    if (a1 >= KS) {
+      hi = m1;
+      n = a1;
+    } else if (a2 >= KS) {
+      lo = m1 + 1;
+      hi = m2;
+      n = a2;
+    } else if (a3 >= KS) {
+      lo = m2 + 1;
+      hi = m3;
+      n = a3;
+    } else {
+      lo = m3 + 1;
+      continue;
+    }
+    if (n <= good) break;
+  }
+  return n;
+}
+
+// Of the keys equal to hi, the largest original id such that `want` of them have an id up to
+// it; id(e): the original id of key e.
+template <int E, class Id>
+__device__ __forceinline__ uint32_t tie_bound(const uint32_t (&k)[E], uint32_t hi, int KS, Id id) {
+  int below = 0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) below += k[e] < hi ? 1 : 0;
+  const int want = KS - __reduce_add_sync(0xffffffffu, below);
+  uint32_t l2 = 0u, h2 = 0x7FFFFFFFu;
+  while (l2 < h2) {
+    const uint32_t mid = l2 + ((h2 - l2) >> 1);
+    int c = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (k[e] == hi) c += id(e) <= mid ? 1 : 0;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (c >= want)
+      h2 = mid;
+    else
+      l2 = mid + 1;
+  }
+  return h2;
+}
+
+// Cuts the buffers of the warp's rows named by `need` (lane l's has mycnt of lane l, more than
+// KS, (id, accumulator) pairs) back to the entries at or above a threshold with between KS and
+// `good` of them; if ties at the KS-th largest would keep more than `cap`, exactly KS stay, the
+// ties with the smallest original ids.  Returns (new count, threshold bits) of this lane's
+// row: at least KS entries are not below the threshold.  Out of line: it runs rarely, and one
+// copy keeps the scan small in the instruction cache.
 template <int C>
-__device__ __noinline__ int cut_row(uint2* __restrict__ buf, int cnt, int KS, int good, int cap,
-                                    const int32_t* __restrict__ perm, float* ts) {
+__device__ __noinline__ uint2 cut_rows(uint2* __restrict__ wbuf, uint32_t lstride, unsigned need,
+                                       int mycnt, int KS, int good, int cap,
+                                       const int32_t* __restrict__ perm) {
   constexpr int E = C / 32;
   const int lane = lane_id();
-  uint2 v[E];
-  uint32_t k[E];  // ascending: larger accumulators first
-  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+  const unsigned lt = lanemask_lt();
+  uint2 mine = make_uint2((uint32_t)mycnt, 0u);
+  while (need) {
+    const int l = __ffs(need) - 1;
+    need &= need - 1;
+    const int cnt = __shfl_sync(0xffffffffu, mycnt, l);
+    uint2* buf = wbuf + (size_t)l * lstride;
+    uint2 v[E];
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int i = (e << 5) | lane;
-    v[e] = i < cnt ? buf[i] : make_uint2(0u, 0u);
-  }
+    for (int e = 0; e < E; ++e)
+      v[e] = ((e << 5) | lane) < cnt ? buf[(e << 5) | lane] : make_uint2(0u, 0u);
+    uint32_t k[E];
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int i = (e << 5) | lane;
-    k[e] = i < cnt ? ~float_order_bits(__uint_as_float(v[e].y)) : 0xFFFFFFFFu;
-    if (i < cnt) {
+    for (int e = 0; e < E; ++e) {
+      const bool in = ((e << 5) | lane) < cnt;
+      k[e] = in ? ~float_order_bits(__uint_as_float(v[e].y)) : 0xFFFFFFFFu;
       lo = min(lo, k[e]);
-      hi = max(hi, k[e]);
+      hi = max(hi, in ? k[e] : 0u);
     }
-  }
-  lo = __reduce_min_sync(0xffffffffu, lo);
-  hi = __reduce_max_sync(0xffffffffu, hi);
-  int n = cnt;  // entries <= hi
-  while (lo < hi) {
-    const uint32_t mid = lo + ((hi - lo) >> 1);
-    int part[4] = {0, 0, 0, 0};
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    const int n = search_keys<E>(k, KS, good, lo, hi, cnt);
+    auto orig = [&](int e) { return perm ? (uint32_t)perm[v[e].x] : v[e].x; };
+    uint32_t idmax = 0xFFFFFFFFu;  // of the entries equal to hi, those with an id up to this stay
+    if (n > cap) idmax = tie_bound<E>(k, hi, KS, orig);
+    unsigned b[E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) part[e & 3] += k[e] <= mid ? 1 : 0;
-    const int c = __reduce_add_sync(0xffffffffu, (part[0] + part[1]) + (part[2] + part[3]));
-    if (c >= KS) {
-      hi = mid;
-      n = c;
-      if (c <= good) break;
-    } else {
-      lo = mid + 1;
+    for (int e = 0; e < E; ++e) {
+      bool in = k[e] <= hi;
+      if (idmax != 0xFFFFFFFFu && in && k[e] == hi) in = orig(e) <= idmax;
+      b[e] = __ballot_sync(0xffffffffu, in);
     }
-  }
-  uint32_t idmax = 0xFFFFFFFFu;  // of the entries equal to hi, those with an id up to this stay
-  if (n > cap) {
-    int below = 0;
+    int base = 0;
 #pragma unroll
-    for (int e = 0; e < E; ++e) below += k[e] < hi ? 1 : 0;
-    const int need = KS - __reduce_add_sync(0xffffffffu, below);
-    uint32_t l2 = 0u, h2 = 0x7FFFFFFFu;
-    while (l2 < h2) {
-      const uint32_t mid = l2 + ((h2 - l2) >> 1);
-      int c = 0;
-#pragma unroll
-      for (int e = 0; e < E; ++e)
-        if (k[e] == hi) c += (perm ? (uint32_t)perm[v[e].x] : v[e].x) <= mid ? 1 : 0;
-      c = __reduce_add_sync(0xffffffffu, c);
-      if (c >= need)
-        h2 = mid;
-      else
-        l2 = mid + 1;
+    for (int e = 0; e < E; ++e) {
+      if ((b[e] >> lane) & 1u) buf[base + __popc(b[e] & lt)] = v[e];
+      base += __popc(b[e]);
     }
-    idmax = h2;
+    if (lane == l) mine = make_uint2((uint32_t)base, __float_as_uint(order_bits_float(~hi)));
   }
-  // each lane's kept entries go out one after another behind those of the lanes before it
-  uint32_t keep = 0u;
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    bool in = ((e << 5) | lane) < cnt && k[e] <= hi;
-    if (idmax != 0xFFFFFFFFu && in && k[e] == hi)
-      in = (perm ? (uint32_t)perm[v[e].x] : v[e].x) <= idmax;
-    keep |= in ? 1u << e : 0u;
-  }
-  int incl = __popc(keep);
-  const int own = incl;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  const int total = __shfl_sync(0xffffffffu, incl, 31);
-  uint2* out = buf + (incl - own);
-#pragma unroll
-  for (int e = 0; e < E; ++e)
-    if ((keep >> e) & 1u) *out++ = v[e];
   __syncwarp();
-  *ts = order_bits_float(~hi);
-  return total;
+  return mine;
 }
 
 template <int C, bool STREAM>
@@ -231,9 +261,9 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
   uint64_t* a_empty = bars + 1;                      // both
   uint64_t* s_full = bars + 2;                       // leader's
   uint64_t* s_empty = s_full + MAX_STAGES;           // both
-  uint64_t* t_full = s_empty + MAX_STAGES;           // both, per half
-  uint64_t* t_empty = t_full + 2;                    // leader's, per half
-  uint32_t* tmem_slot = (uint32_t*)(t_empty + 2);
+  uint64_t* t_full = s_empty + MAX_STAGES;           // both, per accumulator (2 half + column half)
+  uint64_t* t_empty = t_full + NBUF;                 // leader's, per accumulator
+  uint32_t* tmem_slot = (uint32_t*)(t_empty + NBUF);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = lane_id();
@@ -245,9 +275,9 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
       mbar_init(smem_u32(s_full + s), 1);
       mbar_init(smem_u32(s_empty + s), 2);            // both halves
     }
-    for (int h = 0; h < 2; ++h) {
-      mbar_init(smem_u32(t_full + h), 1);
-      mbar_init(smem_u32(t_empty + h), EPI_WARPS);   // four warps of each CTA
+    for (int b = 0; b < NBUF; ++b) {
+      mbar_init(smem_u32(t_full + b), 1);
+      mbar_init(smem_u32(t_empty + b), EPI_WARPS);   // four warps of each CTA
     }
     *abort_flag = 0;
     fence_barrier_init();
@@ -349,16 +379,16 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
     // and copies alone: 205 -> 115 ms).
     // The two halves run ahead of each other by up to the pipeline's stages: whichever half's
     // accumulator is free gets its next stage, so that a half whose epilogue is held up by an
-    // append or a cut does not hold up the other (200,000 x 128, K = 200: 24.2 -> 22.2 ms with the
-    // closer threshold of the cuts).
+    // append or a cut does not hold up the other (200,000 x 128, K = 200: 24.2 -> 22.2 ms with
+    // closer thresholds from the cuts).
     if (rank == 0) {
       struct Half {
         int64_t it, i;   // item and tile
         int64_t nwalk;   // tiles of the item's block
-        int seg, kc, s;  // share, stage within the tile, pipeline slot
+        int seg, sub, s; // share, step within the tile, pipeline slot
         uint32_t ph, aph, tph;
-        bool fresh;      // the item's first stage: its rows may not have landed
-        int64_t done;    // stages issued
+        bool fresh;      // the item's first step: its rows may not have landed
+        int64_t done;    // steps issued
       };
       Half hf[2];
 #pragma unroll
@@ -367,7 +397,7 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
         hf[h].seg = (int)(cl % nseg);
         hf[h].i = hf[h].seg;
         hf[h].nwalk = walk_of(p.rb0 + cl / nseg);
-        hf[h].kc = hf[h].s = 0;
+        hf[h].sub = hf[h].s = 0;
         hf[h].ph = hf[h].aph = 0u;
         hf[h].tph = 1u;
         hf[h].fresh = true;
@@ -380,52 +410,64 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
       const uint64_t a_desc = sdesc_sw128(STREAM ? st0 : smem_u32(sA));
       const uint64_t b_desc = sdesc_sw128(st0 + b_off);
       const uint64_t g_desc = sdesc_sw32(st0 + g_off);
-      // the next stage of half h, if its barriers allow it
+      // The next step of half h, if its barriers allow it.  Resident rows: a step is one column
+      // half of a tile (all its K-steps, an N = 128 MMA each); streamed rows: one 64-value chunk
+      // of both column halves (N = 256).
+      const int nsub = STREAM ? spt : 2;
       auto advance = [&](Half& u, int h) -> bool {
         if (u.it >= nitems) return false;
         bool ready = mbar_test(smem_u32(s_full + u.s), u.ph);
-        if (u.kc == 0) ready = ready && mbar_test(smem_u32(t_empty + h), u.tph);
+        if (!STREAM) ready = ready && mbar_test(smem_u32(t_empty + 2 * h + u.sub), u.tph);
+        if (STREAM && u.sub == 0)
+          ready = ready && mbar_test(smem_u32(t_empty + 2 * h), u.tph) &&
+                  mbar_test(smem_u32(t_empty + 2 * h + 1), u.tph);
         if (u.fresh) ready = ready && mbar_test(smem_u32(a_full), u.aph);
         if (!__all_sync(0xffffffffu, ready)) return false;
         tc_fence_after();
         // descriptors: the 14-bit start-address field (bytes / 16) plus an offset; shared
         // addresses stay below 256 KB, so the sum never carries out of the field
         const uint64_t so = (uint64_t)(((uint32_t)u.s * stage_bytes) >> 4);
-        const bool last = u.kc == spt - 1;
-        const uint32_t d_tmem = tmem_base + (uint32_t)(h * BN);
+        const bool last = u.sub == nsub - 1;
+        const uint32_t d_tmem = tmem_base + (uint32_t)(h * BN + (STREAM ? 0 : u.sub * (BN / 2)));
         const uint64_t ad = a_desc + (STREAM ? so : 0ull) + (uint64_t)((h * 128 * 128) >> 4);
-        const uint64_t bd = b_desc + so;
+        // column half u.sub: B's rows 64 u.sub .. + 63 of each CTA
+        const uint64_t bd = b_desc + so + (STREAM ? 0ull : (uint64_t)(u.sub * ((64 * 128) >> 4)));
+        const uint64_t gd = g_desc + so + (STREAM ? 0ull : (uint64_t)(u.sub * ((64 * AUG_BYTES) >> 4)));
         const bool item_end = last && u.i + nseg >= u.nwalk;
         if (issue) {
 #pragma unroll
           for (int c = 0; c < (STREAM ? 1 : MAX_D_RESIDENT / 64); ++c) {
             // K-steps of this chunk that hold values (the rest are zero padding)
-            const int left = STREAM ? p.d - (u.kc % p.dp_chunks) * 64 : p.d - c * 64;
+            const int left = STREAM ? p.d - (u.sub % p.dp_chunks) * 64 : p.d - c * 64;
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
               if (kk * 16 < left)
                 umma_bf16_pair(d_tmem, ad + (uint64_t)((c * A_CHUNK + kk * 32) >> 4),
-                               bd + (uint64_t)((c * B_CHUNK + kk * 32) >> 4), IDESC,
-                               STREAM ? (uint32_t)(u.kc | kk) : (uint32_t)(c | kk));
+                               bd + (uint64_t)((c * B_CHUNK + kk * 32) >> 4),
+                               STREAM ? IDESC : IDESC_HALF,
+                               STREAM ? (uint32_t)(u.sub | kk) : (uint32_t)(c | kk));
           }
-          if (last) {
-            umma_bf16_pair(d_tmem, aug_a, g_desc + so, IDESC, 1u);
-            umma_commit_pair(smem_u32(t_full + h));
+          if (!STREAM || last) {
+            umma_bf16_pair(d_tmem, aug_a, gd, STREAM ? IDESC : IDESC_HALF, 1u);
+            umma_commit_pair(smem_u32(t_full + 2 * h + (STREAM ? 0 : u.sub)));
+            if (STREAM) umma_commit_pair(smem_u32(t_full + 2 * h + 1));
           }
-          umma_commit_pair(smem_u32(s_empty + u.s));
+          if (STREAM || last) umma_commit_pair(smem_u32(s_empty + u.s));
           if (!STREAM && item_end) umma_commit_pair(smem_u32(a_empty));
         }
         __syncwarp();
         ++u.done;
         u.fresh = false;
-        if (++u.s == S) {
-          u.s = 0;
-          u.ph ^= 1u;
+        if (STREAM || last) {
+          if (++u.s == S) {
+            u.s = 0;
+            u.ph ^= 1u;
+          }
         }
         if (!last) {
-          ++u.kc;
+          ++u.sub;
         } else {
-          u.kc = 0;
+          u.sub = 0;
           u.tph ^= 1u;
           u.i += nseg;
           if (item_end) {
@@ -473,13 +515,14 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
     const int h = ew >> 2;          // which 128-row half
     const int q = warp & 3;         // TMEM lane quadrant this warp may access
     const int row_in_cta = h * 128 + q * 32 + lane;
-    const uint32_t my_empty = map_to_rank(smem_u32(t_empty + h), 0);
+    const uint32_t my_empty = map_to_rank(smem_u32(t_empty + 2 * h), 0);
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * BN);
     const float INF = __int_as_float(0x7f800000);
-    constexpr int TRIG = C - 64;    // a chunk pair adds up to 64 entries
-    // a threshold close to the KS-th largest costs a few more bisection steps per cut and saves
-    // appends and cuts
-    const int good = p.KS + (TRIG - p.KS) / 8;
+    // a row is cut once it holds more than trig entries (a chunk pair adds up to 64), back to
+    // `good` at most: a threshold close to the KS-th largest costs a few more search steps per
+    // cut and saves appends and cuts
+    const int trig = min(C - 64, max(3 * p.KS, p.KS + 64));
+    const int good = p.KS + (trig - p.KS) / 8;
     uint32_t tph = 0;
     bool ok = true;
     for (int64_t it = cl; it < nitems && ok; it += ncl) {
@@ -497,33 +540,47 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
       const int32_t* tl = tiles_of(p.rb0 + rbl);
       const int64_t nwalk = walk_of(p.rb0 + rbl);
       int64_t tn = tl ? tl[seg] : seg;
+      // the row's new count and threshold
+      auto settle = [&](uint2 r) {
+        off = off0 + r.x;
+        float t2 = __uint_as_float(r.y);
+        if (nseg > 1) {
+          const uint32_t b = float_order_bits(t2);
+          t2 = order_bits_float(max(b, atomicMax(p.ts_g + row, b)));
+        }
+        ts = fmaxf(ts, t2);
+      };
       for (int64_t i = seg; i < nwalk; i += nseg) {
         const int32_t j0 = (int32_t)(tn * BN);
         if (i + nseg < nwalk) tn = tl ? tl[i + nseg] : i + nseg;
         // with shares: the other shares' thresholds, read while the tile is computed
         uint32_t other = 0u;
         if (nseg > 1 && row < p.na) other = __ldcg(p.ts_g + row);
-        ok = mbar_wait(smem_u32(t_full + h), tph, abort_flag);
-        if (!__all_sync(0xffffffffu, ok)) {
-          ok = false;
-          break;
-        }
-        tph ^= 1;
-        tc_fence_after();
-        if (nseg > 1 && row < p.na) ts = fmaxf(ts, order_bits_float(other));
+        // the tile's two column halves, an accumulator each, in 64-column chunks: chunk c & 1 of
+        // half c >> 1
         uint32_t v[2][32];
 #pragma unroll 1
-        for (int c = 0; c < BN / 32; c += 2) {
-          tmem_ld32(taddr + (uint32_t)c * 32, v[0]);
-          tmem_ld32(taddr + (uint32_t)c * 32 + 32, v[1]);
+        for (int c = 0; c < BN / 64; ++c) {
+          if (!(c & 1)) {
+            ok = mbar_wait(smem_u32(t_full + 2 * h + (c >> 1)), tph, abort_flag);
+            if (!__all_sync(0xffffffffu, ok)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            if (c == 0 && nseg > 1 && row < p.na) ts = fmaxf(ts, order_bits_float(other));
+          }
+          tmem_ld32(taddr + (uint32_t)c * 64, v[0]);
+          tmem_ld32(taddr + (uint32_t)c * 64 + 32, v[1]);
           tmem_wait_ld(v[0]);
           tmem_dep(v[1]);
-          if (c + 2 == BN / 32) {
+          if (c & 1) {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(my_empty);
+            if (lane == 0) mbar_arrive_cluster(my_empty + (c >> 1) * (uint32_t)sizeof(uint64_t));
           }
-          const int32_t jc = j0 + c * 32;
+          // resident rows: a column half is 64 columns of each CTA's 128
+          const int32_t jc = j0 + (STREAM ? c * 64 : (c >> 1) * 64 + (c & 1) * (BN / 2));
           if (jc + 64 > p.nb) {  // the last tile's padding columns are never admitted
 #pragma unroll
             for (int e = 0; e < 64; ++e)
@@ -535,15 +592,46 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
           const float m = fmax3(fmax3(m8[0], m8[1], m8[2]), fmax3(m8[3], m8[4], m8[5]),
                                 fmaxf(m8[6], m8[7]));
           if (!__any_sync(0xffffffffu, m >= ts)) continue;
+          uint32_t pm = 0u;  // this lane's groups of eight columns with one to append
 #pragma unroll
-          for (int g = 0; g < 8; ++g) {
-            if (__any_sync(0xffffffffu, m8[g] >= ts)) {
+          for (int g = 0; g < 8; ++g) pm |= m8[g] >= ts ? 1u << g : 0u;
+          if (__reduce_max_sync(0xffffffffu, (unsigned)__popc(pm)) <= 3u) {
+            // Few per lane (the usual case once the threshold has settled): each lane takes its
+            // own groups one by one, their values picked by selects on the group's bits.  Walking
+            // every group that some lane passes (below) costs a vote, a branch and eight
+            // dependent appends for each.
 #pragma unroll
-              for (int e = 0; e < 8; ++e) {
-                const uint32_t a = v[g >> 2][(g & 3) * 8 + e];
-                if (__uint_as_float(a) >= ts) {
-                  wbuf[off] = make_uint2((uint32_t)(jc + g * 8 + e), a);
-                  ++off;
+            for (int hh = 0; hh < 2; ++hh) {
+              uint32_t pq = (pm >> (4 * hh)) & 15u;
+              while (__any_sync(0xffffffffu, pq != 0u)) {
+                const int g = pq ? __ffs(pq) - 1 : 0;
+                const bool g1 = g & 2, g0 = g & 1;
+                const float lim = pq != 0u ? ts : __int_as_float(0x7fffffff);  // NaN: through
+                const int32_t jg = jc + hh * 32 + g * 8;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                  const uint32_t a = g1 ? v[hh][16 + e] : v[hh][e];
+                  const uint32_t b = g1 ? v[hh][24 + e] : v[hh][8 + e];
+                  const uint32_t x = g0 ? b : a;
+                  if (__uint_as_float(x) >= lim) {
+                    wbuf[off] = make_uint2((uint32_t)(jg + e), x);
+                    ++off;
+                  }
+                }
+                pq &= pq - 1u;
+              }
+            }
+          } else {
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+              if (__any_sync(0xffffffffu, m8[g] >= ts)) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                  const uint32_t a = v[g >> 2][(g & 3) * 8 + e];
+                  if (__uint_as_float(a) >= ts) {
+                    wbuf[off] = make_uint2((uint32_t)(jc + g * 8 + e), a);
+                    ++off;
+                  }
                 }
               }
             }
@@ -551,23 +639,14 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
           // buffers that the next 64 columns could overflow drop to the entries at or above
           // their KS-th largest accumulator
           __syncwarp();
-          unsigned need = __ballot_sync(0xffffffffu, off - off0 > (uint32_t)TRIG);
-          while (need) {
-            const int l = __ffs(need) - 1;
-            need &= need - 1;
-            float t2;
-            const int cl0 = (int)__shfl_sync(0xffffffffu, off - off0, l);
-            const int c2 = cut_row<C>(wbuf + (size_t)l * lstride, cl0, p.KS, good, TRIG, p.perm, &t2);
-            if (lane == l) {
-              off = off0 + c2;
-              if (nseg > 1) {
-                const uint32_t b = float_order_bits(t2);
-                t2 = order_bits_float(max(b, atomicMax(p.ts_g + row, b)));
-              }
-              ts = fmaxf(ts, p.strict ? nextafterf(t2, INF) : t2);
-            }
+          const unsigned need = __ballot_sync(0xffffffffu, off - off0 > (uint32_t)trig);
+          if (need) {
+            const uint2 r = cut_rows<C>(wbuf, lstride, need, (int)(off - off0), p.KS, good, trig, p.perm);
+            if ((need >> lane) & 1u) settle(r);
           }
         }
+        if (!ok) break;
+        tph ^= 1;
       }
       if (!ok) break;
       p.cnt[lrow * nseg + seg] = (int)(off - off0);
@@ -862,7 +941,7 @@ constexpr size_t SMEM_MAX = 225 * 1024;
 size_t tc_smem_bytes(int kchunks, int stages) {
   const size_t stage = kchunks ? (size_t)kchunks * B_CHUNK + B_AUG : (size_t)A_CHUNK + B_CHUNK + B_AUG;
   return 1024 + (size_t)kchunks * A_CHUNK + A_AUG + (size_t)stages * stage +
-         sizeof(uint64_t) * (2 + 2 * MAX_STAGES + 4) + 16;
+         sizeof(uint64_t) * (2 + 2 * MAX_STAGES + 2 * NBUF) + 16;
 }
 
 struct TcMaps {
@@ -1033,7 +1112,6 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
     SSG_LAUNCH(k_ts_init, (unsigned)ceil_div(na, 256), 256, 0, st, ex.tau_in, a_norm, na, ts.p);
     a.ts_g = ts.p;
   }
-  a.strict = !a.tile_order && !a.ts_g;
   // the row buffers of one launch take up to 2 GB; more rows go in several launches, whole
   // rounds of the clusters each
   const size_t block_bytes = (size_t)BM * a.nseg * C * sizeof(uint2);
