@@ -7,7 +7,10 @@
 // a free slot (deg(v) < R) that minimises (d2(v, u), id), and mark everything reachable
 // from u.  The reached set does not depend on the traversal order, so the GPU uses a
 // level-synchronous frontier traversal (a visited bitmap with atomicOr) in place of a
-// depth-first one and gets the same graph.  The argmin is taken in fp64 with the
+// depth-first one and gets the same graph.  Once the first root reaches every node, a later
+// root that reaches the first one reaches every node too and changes nothing: a beam search
+// from it that meets the first root proves that, and only roots for which it does not are
+// traversed (1M nodes, 10 roots: connectivity 6.8 -> 1.3 ms; 60,000 nodes 3.2 -> 0.4).  The argmin is taken in fp64 with the
 // coordinate-order sum, so its ties resolve exactly as a sequential double loop would.
 #include <climits>
 #include <mutex>
@@ -19,66 +22,6 @@
 #include "knn.cuh"
 
 namespace ssg {
-
-__global__ void k_mark(uint32_t* __restrict__ bm, int32_t* __restrict__ frontier,
-                       int* __restrict__ fcount, int32_t root) {
-  atomicOr(bm + (root >> 5), 1u << (root & 31));
-  frontier[0] = root;
-  *fcount = 1;
-}
-
-// Level l of the grid-wide traversal launched in batches (no host round trip per level):
-// the frontier size is lvl[l % 3], the next one is counted in lvl[(l + 1) % 3], and
-// lvl[(l + 2) % 3] (level l - 1's input, level l + 1's output) is cleared for the next
-// launch.  A level whose frontier is empty does nothing.
-__global__ void k_bfs_level_ring(const int32_t* __restrict__ adj, const int32_t* __restrict__ deg,
-                                 int R, uint32_t* __restrict__ bm,
-                                 const int32_t* __restrict__ frontier, int32_t* __restrict__ next,
-                                 int* __restrict__ lvl, int l) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) lvl[(l + 2) % 3] = 0;
-  const int lane = lane_id();
-  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  const int fc = lvl[l % 3];
-  int* ncount = lvl + (l + 1) % 3;
-  for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < fc;
-       w += nwarps) {
-    const int32_t node = frontier[w];
-    const int dg = deg[node];
-    for (int c = 0; c < dg; c += 32) {
-      const int t = c + lane;
-      bool fresh = false;
-      int32_t v = 0;
-      if (t < dg) {
-        v = adj[(int64_t)node * R + t];
-        const uint32_t bit = 1u << (v & 31);
-        fresh = !(atomicOr(bm + (v >> 5), bit) & bit);
-      }
-      const unsigned bal = __ballot_sync(0xffffffffu, fresh);
-      int basep = 0;
-      if (lane == 0 && bal) basep = atomicAdd(ncount, __popc(bal));
-      basep = __shfl_sync(0xffffffffu, basep, 0);
-      if (fresh) next[basep + __popc(bal & lanemask_lt())] = v;
-    }
-  }
-}
-
-__global__ void k_ring_init(int* __restrict__ lvl, const int* __restrict__ fcount) {
-  lvl[0] = *fcount;
-  lvl[1] = 0;
-}
-
-__global__ void k_first_unreached(const uint32_t* __restrict__ bm, int64_t nw, int64_t n,
-                                  int64_t start_word, unsigned long long* __restrict__ out) {
-  for (int64_t w = start_word + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nw;
-       w += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t word = bm[w];
-    if (w == nw - 1 && (n & 31)) word |= ~((1u << (n & 31)) - 1u);
-    if (word != 0xffffffffu) {
-      const unsigned long long u = (unsigned long long)(w * 32 + __ffs(~word) - 1);
-      atomicMin(out, u);
-    }
-  }
-}
 
 // Exhaustive fp64 argmin (used only when the fp32 band below overflows its list).
 __global__ void k_repair_dist(const float* __restrict__ X, int ld, int d, int64_t n,
@@ -109,82 +52,316 @@ __global__ void k_repair_pick_all(const double* __restrict__ dv, int64_t n,
   }
 }
 
-// Device-side state of one repair step.
+// Device-side state of the connectivity of one root.
 struct RepairState {
   unsigned long long u;  // smallest unreached id (n if none)
   unsigned hi_bits;      // smallest fp32 upper bound of d2(v, u) over the candidates
   int band;              // candidates whose fp32 lower bound reaches that upper bound
-  int best;              // chosen v (INT_MAX: none; -2: band overflow)
-  int fcnt[2];           // frontier sizes
-  int bfs_state;         // -1 traversal finished, else index of the frontier still to expand
-  int lvl[3];            // frontier sizes of the batched traversal, by level mod 3
+  int best;              // chosen v; one of the STOP codes when a kernel ends before u = n
+  int cur;               // frontier buffer still to expand (0 or 1)
+  int lvl[3];            // frontier sizes, by level mod 3; lvl[0] the next one to expand
+  unsigned bar;          // grid barrier: arrivals since the launch
+  int abort;             // a barrier timed out
+  unsigned long long rep_full, rep_knn;  // repairs made, by the full scan and by kNN rows
+};
+constexpr int STOP_NONE = INT_MAX;  // no reached node has a free slot
+constexpr int STOP_BAND = -2;       // the band list overflowed
+constexpr int STOP_ROW = -3;        // u's kNN row settles nothing: the full scan takes u
+constexpr int STOP_BFS = -4;        // u is linked, its traversal outgrew the block
+constexpr int STOP_KNN = -5;        // unreached nodes remain, k_repair_knn is next
+
+__global__ void k_mark(uint32_t* __restrict__ bm, int32_t* __restrict__ frontier,
+                       RepairState* __restrict__ s, int32_t root) {
+  atomicOr(bm + (root >> 5), 1u << (root & 31));
+  frontier[0] = root;
+  s->cur = 0;
+  s->lvl[0] = 1;
+  s->lvl[1] = s->lvl[2] = 0;
+}
+
+struct ConnArgs {
+  const float* X;
+  int ld, d;
+  int64_t n, nw;
+  int32_t *adj, *deg;
+  int R;
+  uint32_t* bm;
+  int32_t *f0, *f1;
+  const int32_t* knn;     // nullable: exact kNN rows
+  int K;
+  float* d32;
+  int32_t* band_ids;
+  double* band_d;
+  int cap;                // band entries
+  float rel;
+  RepairState* s;
+  int64_t start;          // no unreached node lies in a bitmap word before this one
+  int stop_at_knn;        // 1: after the first traversal leave the repairs to k_repair_knn
 };
 
-__global__ void k_repair_init(RepairState* __restrict__ s, int64_t n) {
-  s->u = (unsigned long long)n;
-  s->hi_bits = 0x7f800000u;
-  s->band = 0;
-  s->best = INT_MAX;
-  s->fcnt[0] = 0;
-}
+__device__ __forceinline__ uint32_t peek(const uint32_t* p) { return *(const volatile uint32_t*)p; }
 
-// Pass 1: fp32 distance of every reached node with a free slot to u, by teams of 8 lanes;
-// the smallest upper bound d32 (1 + 2 rel) over them.
-__global__ void k_repair_fp32(const float* __restrict__ X, int ld, int64_t n,
-                              const uint32_t* __restrict__ bm, const int32_t* __restrict__ deg,
-                              int R, float rel, float* __restrict__ d32,
-                              RepairState* __restrict__ s) {
-  const int64_t u = (int64_t)s->u;
-  if (u >= n) return;
-  const int lane = lane_id(), team = lane >> 3, tl = lane & 7;
-  const float* xu = X + u * ld;
-  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  float best = __int_as_float(0x7f800000);
-  for (int64_t v0 = gw * 4; v0 < n; v0 += nwarp * 4) {
-    const int64_t v = v0 + team;
-    const bool cand = v < n && ((bm[v >> 5] >> (v & 31)) & 1u) && deg[v] < R;
-    const float e = team8_dist(X + (cand ? v : 0) * ld, xu, ld >> 2, tl, cand);
-    if (tl == 0 && v < n) d32[v] = cand ? e : -1.f;
-    if (cand) best = fminf(best, e);
-  }
-  for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-  if (lane == 0 && best < __int_as_float(0x7f800000))
-    atomicMin(&s->hi_bits, __float_as_uint(best * (1.f + 2.f * rel) + 1e-30f));
-}
-
-// Pass 2: every candidate whose fp32 lower bound does not exceed that upper bound goes
-// into a short list ...
-__global__ void k_repair_band(const float* __restrict__ X, int ld, int d, int64_t n,
-                              const float* __restrict__ d32, float rel, int cap,
-                              int32_t* __restrict__ ids, double* __restrict__ dv,
-                              RepairState* __restrict__ s) {
-  const int64_t u = (int64_t)s->u;
-  if (u >= n) return;
-  const float hi = __uint_as_float(s->hi_bits);
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
-       v += (int64_t)gridDim.x * blockDim.x) {
-    const float e = d32[v];
-    if (e >= 0.f && e * (1.f - 2.f * rel) <= hi) {
-      const int p = atomicAdd(&s->band, 1);
-      if (p < cap) ids[p] = (int32_t)v;
+// Smallest unreached id from bitmap word w0 on (n if none), by one warp.
+__device__ __forceinline__ int64_t warp_first_unreached(const uint32_t* bits, int64_t nw, int64_t n,
+                                                        int64_t w0) {
+  const int lane = lane_id();
+  for (int64_t b = w0; b < nw; b += 128) {
+    uint32_t word[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int64_t w = b + j * 32 + lane;
+      word[j] = w < nw ? peek(bits + w) : 0xffffffffu;
+      if (w == nw - 1 && (n & 31)) word[j] |= ~((1u << (n & 31)) - 1u);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const unsigned bal = __ballot_sync(0xffffffffu, word[j] != 0xffffffffu);
+      if (bal) {
+        const int l = __ffs(bal) - 1;
+        const uint32_t w = __shfl_sync(0xffffffffu, word[j], l);
+        return (b + j * 32 + l) * 32 + __ffs(~w) - 1;
+      }
     }
   }
+  return n;
 }
 
-// ... whose fp64 distances to u are then summed, one list entry per warp
-// (warp_dist2_f64; k_repair_pick re-takes near-equal ones in coordinate order).
-__global__ void k_repair_band64(const float* __restrict__ X, int ld, int d, int64_t n,
-                                int cap, const int32_t* __restrict__ ids, double* __restrict__ dv,
-                                const RepairState* __restrict__ s) {
-  const int64_t u = (int64_t)s->u;
-  if (u >= n) return;
-  const int m = min(s->band, cap);
-  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t p = gw; p < m; p += nwarp) {
-    const double x = warp_dist2_f64(X + (int64_t)ids[p] * ld, X + u * ld, d);
-    if (lane_id() == 0) dv[p] = x;
+// Expands one node by a warp: its unreached neighbours are marked and appended to next.
+__device__ __forceinline__ void warp_expand(const ConnArgs& a, uint32_t* bits, int32_t node,
+                                            int32_t* next, int* ncount) {
+  const int lane = lane_id();
+  const int dg = __ldcg(a.deg + node);
+  for (int c = 0; c < dg; c += 32) {
+    const int t = c + lane;
+    bool fresh = false;
+    int32_t v = 0;
+    if (t < dg) {
+      v = __ldcg(a.adj + (int64_t)node * a.R + t);
+      const uint32_t bit = 1u << (v & 31);
+      // most neighbours are reached already: a read first spares their atomics
+      if (!(peek(bits + (v >> 5)) & bit)) fresh = !(atomicOr(bits + (v >> 5), bit) & bit);
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, fresh);
+    int basep = 0;
+    if (lane == 0 && bal) basep = atomicAdd(ncount, __popc(bal));
+    basep = __shfl_sync(0xffffffffu, basep, 0);
+    if (fresh) next[basep + __popc(bal & lanemask_lt())] = v;
+  }
+}
+
+// Repairs that kNN rows settle, back to back by one warp.  A row lists u's K nearest nodes in
+// exact (d2, id) order, so when some of them is reached and has a free slot the first such one
+// is the (d2, id)-smallest of all reached nodes with a free slot: the same choice as the
+// argmin over all n nodes, without a pass over them.  Each round: the smallest unreached u,
+// the link from the first qualifying row entry, and the traversal from u while its frontier
+// stays small.  bits: the bitmap of reached nodes (in shared or global memory).  Returns
+// (in every lane) n when every node is reached, else the node it stopped at, with
+// *why = STOP_ROW, STOP_KNN after `most` repairs, or STOP_BFS and the frontier in the state.  A repair is a chain of
+// latencies, so the next unreached node's row, out-edges and degree (which no repair before
+// its own changes) load while the current one is settled.
+struct RepairRow {
+  static constexpr int PIECES = 4;  // of 32 entries, kept in registers
+  int32_t row[PIECES], adj[PIECES];
+  int dg;
+  __device__ __forceinline__ void fetch(const ConnArgs& a, int64_t u) {
+    const int lane = lane_id();
+    const bool in = u < a.n;
+    dg = in ? __ldcg(a.deg + u) : 0;
+#pragma unroll
+    for (int j = 0; j < PIECES; ++j) {
+      const int t = j * 32 + lane;
+      row[j] = in && t < a.K ? __ldg(a.knn + u * a.K + t) : -1;
+      adj[j] = in && t < a.R ? __ldcg(a.adj + u * a.R + t) : -1;
+    }
+  }
+};
+__device__ __noinline__ int64_t warp_knn_repairs(const ConnArgs& a, uint32_t* bits, int64_t start,
+                                                 int most, int* why) {
+  constexpr int LIMIT = 256;  // frontier nodes one warp expands itself
+  constexpr int P = RepairRow::PIECES;
+  const int lane = lane_id();
+  RepairState* s = a.s;
+  unsigned long long made = 0;
+  RepairRow now, next;
+  int64_t u = warp_first_unreached(bits, a.nw, a.n, start);
+  now.fetch(a, u);
+  *why = 0;
+  // marks v and appends it to the list, if it is unreached (v < 0: nothing)
+  auto reach = [&](int32_t v, int32_t* list, int& count) {
+    const uint32_t bit = 1u << (v & 31);
+    bool fresh = v >= 0 && !(peek(bits + (v >> 5)) & bit);
+    if (!__any_sync(0xffffffffu, fresh)) return;
+    if (fresh) fresh = !(atomicOr(bits + (v >> 5), bit) & bit);
+    const unsigned bal = __ballot_sync(0xffffffffu, fresh);
+    if (fresh) list[count + __popc(bal & lanemask_lt())] = v;
+    count += __popc(bal);
+  };
+  while (u < a.n) {
+    if (made >= (unsigned long long)most) {
+      *why = STOP_KNN;
+      break;
+    }
+    // (u's own bit is still clear, so look behind it)
+    int64_t guess = warp_first_unreached(bits, a.nw, a.n, u >> 5);
+    if (guess == u) {
+      const uint32_t w = peek(bits + (u >> 5)) | ((2u << (u & 31)) - 1u);
+      guess = w != 0xffffffffu ? (u >> 5) * 32 + __ffs(~w) - 1
+                               : warp_first_unreached(bits, a.nw, a.n, (u >> 5) + 1);
+      if (guess > a.n) guess = a.n;
+    }
+    next.fetch(a, guess);
+    // the row's first reached node with a free slot
+    int32_t found = -1;
+    int slot = 0;
+    for (int c = 0, j = 0; c < a.K && found < 0; c += 32, ++j) {
+      int32_t v = -1;
+      if (j < P) {
+#pragma unroll
+        for (int k = 0; k < P; ++k)
+          if (k == j) v = now.row[k];
+      } else if (c + lane < a.K) {
+        v = __ldg(a.knn + u * a.K + c + lane);
+      }
+      const bool reached = v >= 0 && ((peek(bits + (v >> 5)) >> (v & 31)) & 1u);
+      if (!__any_sync(0xffffffffu, reached)) continue;
+      const int dv = reached ? __ldcg(a.deg + v) : a.R;
+      const unsigned bal = __ballot_sync(0xffffffffu, dv < a.R);
+      if (bal) {
+        found = __shfl_sync(0xffffffffu, v, __ffs(bal) - 1);
+        slot = __shfl_sync(0xffffffffu, dv, __ffs(bal) - 1);
+      }
+    }
+    if (found < 0) {
+      *why = STOP_ROW;
+      break;
+    }
+    if (lane == 0) {
+      a.adj[(int64_t)found * a.R + slot] = (int32_t)u;
+      a.deg[found] = slot + 1;
+      atomicOr(bits + (u >> 5), 1u << (u & 31));
+    }
+    ++made;
+    __syncwarp();
+    int32_t *fr = a.f1, *nx = a.f0;
+    int fc = 0;
+#pragma unroll
+    for (int j = 0; j < P; ++j) reach(j * 32 + lane < now.dg ? now.adj[j] : -1, fr, fc);
+    for (int c = P * 32; c < now.dg; c += 32)
+      reach(c + lane < now.dg ? __ldcg(a.adj + u * a.R + c + lane) : -1, fr, fc);
+    __syncwarp();
+    while (fc > 0 && fc <= LIMIT) {
+      int nc = 0;
+      for (int w = 0; w < fc; ++w) {
+        const int32_t node = __ldcg(fr + w);
+        const int dg = __ldcg(a.deg + node);
+        for (int c = 0; c < dg; c += 32)
+          reach(c + lane < dg ? __ldcg(a.adj + (int64_t)node * a.R + c + lane) : -1, nx, nc);
+      }
+      __syncwarp();
+      int32_t* t = fr;
+      fr = nx;
+      nx = t;
+      fc = nc;
+    }
+    if (fc > 0) {
+      if (lane == 0) {
+        s->cur = fr == a.f1 ? 1 : 0;
+        s->lvl[0] = fc;
+        s->lvl[1] = s->lvl[2] = 0;
+      }
+      *why = STOP_BFS;
+      break;
+    }
+    // (u is its own guess's predecessor: the guess stands unless the traversal reached it)
+    const int64_t from = u;
+    u = guess < a.n && !((peek(bits + (guess >> 5)) >> (guess & 31)) & 1u)
+            ? guess
+            : warp_first_unreached(bits, a.nw, a.n, from >> 5);
+    if (u == guess)
+      now = next;
+    else
+      now.fetch(a, u);
+  }
+  if (lane == 0) s->rep_knn += made;
+  __threadfence();
+  __syncwarp();
+  return u;
+}
+
+// warp_knn_repairs with the bitmap in shared memory where it fits (up to 1.6M nodes): a chain
+// of dependent reads, each a shared-memory or an L2 latency.  200,000 nodes, 4,500 repairs:
+// 10.5 ms; one block that met at about ten barriers per repair took 15.5 ms.
+__global__ void __launch_bounds__(256) k_repair_knn(ConnArgs a, int shared_bits) {
+  extern __shared__ uint32_t sbits[];
+  uint32_t* bits = a.bm;
+  if (shared_bits) {
+    for (int64_t w = threadIdx.x; w < a.nw; w += blockDim.x) sbits[w] = a.bm[w];
+    bits = sbits;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    int why;
+    const int64_t u = warp_knn_repairs(a, bits, a.start, INT_MAX, &why);
+    if (threadIdx.x == 0) {
+      a.s->u = (unsigned long long)u;
+      a.s->best = u < a.n ? why : STOP_NONE;
+    }
+  }
+  __syncthreads();
+  if (shared_bits)
+    for (int64_t w = threadIdx.x; w < a.nw; w += blockDim.x) a.bm[w] = sbits[w];
+}
+
+// Barrier of the whole (cooperative) grid, bounded: false, in every thread, once a block has
+// waited about 20 s or another one gave up.  phase: barriers so far (the same in every block).
+__device__ __forceinline__ bool grid_barrier(RepairState* s, unsigned& phase) {
+  __shared__ int ok;
+  __syncthreads();
+  ++phase;
+  if (threadIdx.x == 0) {
+    const unsigned target = phase * gridDim.x;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&s->bar) : "memory");
+    unsigned long long t0 = 0;
+    ok = 1;
+    for (unsigned spins = 0;; ++spins) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&s->bar) : "memory");
+      if ((int)(v - target) >= 0) break;
+      if (spins < 64) continue;
+      unsigned long long t;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      if (t0 == 0) t0 = t;
+      if (*(volatile int*)&s->abort || t - t0 > 20000000000ull) {
+        *(volatile int*)&s->abort = 1;
+        ok = 0;
+        break;
+      }
+      __nanosleep(64);
+    }
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+// Level-synchronous traversal by the whole grid from frontier buffer s->cur (lvl[0] nodes), a
+// warp per node: frontier sizes go round lvl[0..2], level l clearing the counter that level
+// l + 1 fills, and a barrier at the end, after which the state may change.  False if a barrier
+// gave up.
+__device__ __forceinline__ bool grid_bfs(const ConnArgs& a, unsigned& phase) {
+  RepairState* s = a.s;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  int cur = *(volatile int*)&s->cur;
+  for (int l = 0;; ++l) {
+    const int fc = *(volatile int*)&s->lvl[l % 3];
+    if (fc == 0) return grid_barrier(s, phase);
+    if (blockIdx.x == 0 && threadIdx.x == 0) s->lvl[(l + 2) % 3] = 0;
+    const int32_t* fr = cur ? a.f1 : a.f0;
+    int32_t* nx = cur ? a.f0 : a.f1;
+    for (int64_t w = gw; w < fc; w += nwarps)
+      warp_expand(a, a.bm, __ldcg(fr + w), nx, &s->lvl[(l + 1) % 3]);
+    if (!grid_barrier(s, phase)) return false;
+    cur ^= 1;
   }
 }
 
@@ -212,71 +389,162 @@ __device__ __forceinline__ void block_argmin(double& best, int& bid, double* bd,
     }
 }
 
-// Pass 3 (one block): the (d2, id)-smallest entry of the list; link it to u and make u the
-// frontier of the next traversal.  Where other entries lie within fp64_order_rel of the
-// smallest warp-summed value, those entries are re-taken in coordinate order, so the
-// choice is the one the coordinate-order fp64 values give.
-__global__ void k_repair_pick(const float* __restrict__ X, int ld, int d,
-                              const int32_t* __restrict__ ids, const double* __restrict__ dv,
-                              int cap, int32_t* __restrict__ adj, int32_t* __restrict__ deg, int R,
-                              uint32_t* __restrict__ bm, int32_t* __restrict__ frontier,
-                              int64_t n, RepairState* __restrict__ s) {
+// The connectivity of one root by one cooperative grid: the traversal from the frontier in the
+// state, then (unless stop_at_knn) repairs until every node is reached.  A repair: the smallest
+// unreached u; where kNN rows are given, first those that they settle (one warp of block 0, a
+// few of them: the bitmap is not in its shared memory, so it leaves many to k_repair_knn);
+// else the full scan: fp32 distances of every reached node with a free slot by teams of 8
+// lanes; the fp64 distances of those whose lower bound reaches the smallest upper bound seen by
+// then (its block's at most, so a superset of the band that can hold the minimum; a warp each);
+// then, in block 0, the (d2, id)-smallest of them, re-taken in coordinate order among those
+// within fp64_order_rel of the smallest.  Two grid barriers per repair; a host round trip and
+// seven launches took 60 us (30,011 x 100, 172 repairs: 12.7 -> 5.0 ms).
+__global__ void __launch_bounds__(512) k_connect(ConnArgs a) {
   __shared__ double bd[32];
   __shared__ int bi[32];
   __shared__ int nties;
-  const int64_t u = (int64_t)s->u;
-  if (u >= n) return;
-  const int m = s->band;
-  if (m > cap) {
-    if (threadIdx.x == 0) s->best = -2;
-    return;
-  }
+  __shared__ unsigned bmin;
+  RepairState* s = a.s;
+  unsigned phase = 0;
+  const int lane = lane_id(), team = lane >> 3, tl = lane & 7, warp = threadIdx.x >> 5;
+  const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
   const double INF = __longlong_as_double(0x7ff0000000000000ll);
-  double best = INF;
-  int bid = INT_MAX;
-  for (int t = threadIdx.x; t < m; t += blockDim.x) {
-    const double x = dv[t];
-    const int v = ids[t];
-    if (x < best || (x == best && v < bid)) {
-      best = x;
-      bid = v;
+  int64_t start = a.start;
+  // block 0, warp 0: the next node that needs the full scan (or what ends this kernel)
+  auto next_node = [&]() {
+    int why = STOP_ROW;
+    int64_t u;
+    if (a.knn && !a.stop_at_knn)
+      u = warp_knn_repairs(a, a.bm, start, 16, &why);
+    else
+      u = warp_first_unreached(a.bm, a.nw, a.n, start);
+    start = u >> 5;
+    if (lane == 0) {
+      s->hi_bits = 0x7f800000u;
+      s->band = 0;
+      s->best = a.stop_at_knn ? STOP_KNN : why;
+      s->u = (unsigned long long)u;
     }
-  }
-  if (threadIdx.x == 0) nties = 0;
-  block_argmin(best, bid, bd, bi);
-  const double lim = best + fp64_order_rel(d) * best;
-  int mine = 0;
-  for (int t = threadIdx.x; t < m; t += blockDim.x) mine += dv[t] <= lim;
-  if (mine) atomicAdd(&nties, mine);
-  __syncthreads();
-  if (nties > 1) {
-    double b2 = INF;
-    int i2 = INT_MAX;
-    for (int t = threadIdx.x; t < m; t += blockDim.x) {
-      if (dv[t] > lim) continue;
-      const int v = ids[t];
-      const double x = dist2_f64(X + (int64_t)v * ld, X + u * ld, d);
-      if (x < b2 || (x == b2 && v < i2)) {
-        b2 = x;
-        i2 = v;
+  };
+  if (!grid_bfs(a, phase)) return;
+  if (blockIdx.x == 0 && warp == 0) next_node();
+  for (;;) {
+    if (!grid_barrier(s, phase)) return;
+    const int64_t u = (int64_t)*(volatile unsigned long long*)&s->u;
+    const int what = *(volatile int*)&s->best;
+    if (u >= a.n || (what != STOP_BFS && what != STOP_ROW)) return;
+    if (what == STOP_BFS) {
+      if (!grid_bfs(a, phase)) return;
+      if (blockIdx.x == 0 && warp == 0) next_node();
+      continue;
+    }
+    const float* xu = a.X + u * a.ld;
+    if (threadIdx.x == 0) bmin = 0x7f800000u;
+    __syncthreads();
+    float best = __int_as_float(0x7f800000);
+    for (int64_t v0 = gw * 4; v0 < a.n; v0 += nwarps * 4) {
+      const int64_t v = v0 + team;
+      const bool cand =
+          v < a.n && ((__ldcg(a.bm + (v >> 5)) >> (v & 31)) & 1u) && __ldcg(a.deg + v) < a.R;
+      const float e = team8_dist(a.X + (cand ? v : 0) * a.ld, xu, a.ld >> 2, tl, cand);
+      if (tl == 0 && v < a.n) a.d32[v] = cand ? e : -1.f;
+      if (cand) best = fminf(best, e);
+    }
+    for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+    if (lane == 0 && best < __int_as_float(0x7f800000))
+      atomicMin(&bmin, __float_as_uint(best * (1.f + 2.f * a.rel) + 1e-30f));
+    __syncthreads();
+    if (threadIdx.x == 0 && bmin != 0x7f800000u) bmin = min(bmin, atomicMin(&s->hi_bits, bmin));
+    __syncthreads();
+    const float hi = __uint_as_float(bmin);
+    for (int64_t v0 = gw * 4; v0 < a.n; v0 += nwarps * 32) {
+      // this warp's own distances: four nodes of each of eight rounds
+      const int64_t v1 = v0 + (int64_t)(lane >> 2) * nwarps * 4 + (lane & 3);
+      const float e = v1 < a.n ? __ldcg(a.d32 + v1) : -1.f;
+      unsigned bal = __ballot_sync(0xffffffffu, e >= 0.f && e * (1.f - 2.f * a.rel) <= hi);
+      while (bal) {
+        const int l = __ffs(bal) - 1;
+        bal &= bal - 1;
+        const int64_t v = __shfl_sync(0xffffffffu, v1, l);
+        int p = 0;
+        if (lane == 0) p = atomicAdd(&s->band, 1);
+        p = __shfl_sync(0xffffffffu, p, 0);
+        if (p >= a.cap) break;
+        const double x = warp_dist2_f64(a.X + v * a.ld, xu, a.d);
+        if (lane == 0) {
+          a.band_ids[p] = (int32_t)v;
+          a.band_d[p] = x;
+        }
       }
     }
-    block_argmin(b2, i2, bd, bi);
-    bid = i2;
-  }
-  if (threadIdx.x == 0) {
-    s->best = bid;
-    if (bid != INT_MAX) {
-      adj[(int64_t)bid * R + deg[bid]] = (int32_t)u;
-      deg[bid] += 1;
-      atomicOr(bm + (u >> 5), 1u << (u & 31));
-      frontier[0] = (int32_t)u;
-      s->fcnt[0] = 1;
+    if (!grid_barrier(s, phase)) return;
+    if (blockIdx.x != 0) continue;
+    // block 0 links the smallest, expands u, and finds the next node
+    const int m = *(volatile int*)&s->band;
+    if (m == 0 || m > a.cap) {
+      if (threadIdx.x == 0) s->best = m == 0 ? STOP_NONE : STOP_BAND;
+      continue;
     }
+    double b1 = INF;
+    int bid = INT_MAX;
+    for (int t = threadIdx.x; t < m; t += blockDim.x) {
+      const double x = __ldcg(a.band_d + t);
+      const int v = __ldcg(a.band_ids + t);
+      if (x < b1 || (x == b1 && v < bid)) {
+        b1 = x;
+        bid = v;
+      }
+    }
+    if (threadIdx.x == 0) nties = 0;
+    block_argmin(b1, bid, bd, bi);
+    const double lim = b1 + fp64_order_rel(a.d) * b1;
+    int mine = 0;
+    for (int t = threadIdx.x; t < m; t += blockDim.x) mine += __ldcg(a.band_d + t) <= lim;
+    if (mine) atomicAdd(&nties, mine);
+    __syncthreads();
+    if (nties > 1) {
+      double b2 = INF;
+      int i2 = INT_MAX;
+      for (int t = threadIdx.x; t < m; t += blockDim.x) {
+        if (__ldcg(a.band_d + t) > lim) continue;
+        const int v = __ldcg(a.band_ids + t);
+        const double x = dist2_f64(a.X + (int64_t)v * a.ld, xu, a.d);
+        if (x < b2 || (x == b2 && v < i2)) {
+          b2 = x;
+          i2 = v;
+        }
+      }
+      block_argmin(b2, i2, bd, bi);
+      bid = i2;
+    }
+    if (warp == 0) {
+      if (lane == 0) {
+        const int dv = __ldcg(a.deg + bid);
+        a.adj[(int64_t)bid * a.R + dv] = (int32_t)u;
+        a.deg[bid] = dv + 1;
+        atomicOr(a.bm + (u >> 5), 1u << (u & 31));
+        s->rep_full += 1;
+        s->cur = 1;
+        s->lvl[0] = s->lvl[1] = s->lvl[2] = 0;
+      }
+      __threadfence();
+      __syncwarp();
+      warp_expand(a, a.bm, (int32_t)u, a.f1, &s->lvl[0]);
+      __threadfence();
+      __syncwarp();
+      start = u >> 5;
+      if (*(volatile int*)&s->lvl[0] > 0) {
+        if (lane == 0) s->best = STOP_BFS;
+      } else {
+        next_node();
+      }
+    }
+    __syncthreads();
   }
 }
 
-// Link v = *best (exhaustive path) and make u the next frontier.
+// Link v = *best_id (after the exhaustive argmin) and make u the next frontier.
 __global__ void k_add_edge(int32_t* __restrict__ adj, int32_t* __restrict__ deg, int R,
                            const int* __restrict__ best_id, uint32_t* __restrict__ bm,
                            int32_t* __restrict__ frontier, RepairState* __restrict__ s) {
@@ -288,213 +556,99 @@ __global__ void k_add_edge(int32_t* __restrict__ adj, int32_t* __restrict__ deg,
   deg[v] += 1;
   atomicOr(bm + (u >> 5), 1u << (u & 31));
   frontier[0] = (int32_t)u;
-  s->fcnt[0] = 1;
+  s->cur = 0;
+  s->lvl[0] = 1;
+  s->lvl[1] = s->lvl[2] = 0;
+  s->rep_full += 1;
 }
 
-// Traversal by one block while the frontier stays small (no host round trip per level);
-// leaves bfs_state = -1 when done, or the index of the frontier buffer still to expand.
-__global__ void k_bfs_small(const int32_t* __restrict__ adj, const int32_t* __restrict__ deg, int R,
-                            uint32_t* __restrict__ bm, int32_t* __restrict__ f0,
-                            int32_t* __restrict__ f1, int limit, RepairState* __restrict__ s) {
-  const int lane = lane_id();
-  const int nwarps = blockDim.x >> 5;
-  int cur = 0;
-  for (;;) {
-    __syncthreads();
-    const int fc = s->fcnt[cur];
-    if (fc == 0 || fc > limit) {
-      if (threadIdx.x == 0) s->bfs_state = fc == 0 ? -1 : cur;
-      return;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) s->fcnt[cur ^ 1] = 0;
-    __syncthreads();
-    const int32_t* fr = cur ? f1 : f0;
-    int32_t* nx = cur ? f0 : f1;
-    for (int w = threadIdx.x >> 5; w < fc; w += nwarps) {
-      const int32_t node = fr[w];
-      const int dg = deg[node];
-      for (int c = 0; c < dg; c += 32) {
-        const int t = c + lane;
-        bool fresh = false;
-        int32_t v = 0;
-        if (t < dg) {
-          v = adj[(int64_t)node * R + t];
-          const uint32_t bit = 1u << (v & 31);
-          fresh = !(atomicOr(bm + (v >> 5), bit) & bit);
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, fresh);
-        int basep = 0;
-        if (lane == 0 && bal) basep = atomicAdd(&s->fcnt[cur ^ 1], __popc(bal));
-        basep = __shfl_sync(0xffffffffu, basep, 0);
-        if (fresh) nx[basep + __popc(bal & lanemask_lt())] = v;
+// Launches k_connect and reads the state back.
+static RepairState run_connect(ConnArgs a, cudaStream_t st) {
+  SSG_CUDA(cudaMemsetAsync(&a.s->bar, 0, sizeof(unsigned), st));
+  static const int per_sm = [] {
+    int b = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_connect, 512, 0);
+    return b;
+  }();
+  SSG_REQUIRE(per_sm >= 1, SSG_ECUDA, "connectivity: no room for the grid kernel");
+  // one block per SM for large graphs; few nodes need few blocks (a barrier's cost grows
+  // with them)
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(num_sms(), ceil_div(a.n, 128)));
+  void* args[] = {&a};
+  SSG_CUDA(cudaLaunchCooperativeKernel((const void*)k_connect, dim3(grid), dim3(512), args, 0, st));
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  ++t_launches;
+  RepairState h;
+  SSG_CUDA(cudaMemcpyAsync(&h, a.s, sizeof(h), cudaMemcpyDeviceToHost, st));
+  SSG_CUDA(cudaStreamSynchronize(st));
+  if (h.abort) note_device_status(SSG_ETIMEOUT);
+  SSG_REQUIRE(!h.abort, SSG_ETIMEOUT, "connectivity: a grid barrier timed out");
+  return h;
+}
+
+// One root: its traversal and the repairs until it reaches every node.  on_band(u): the
+// caller's way out when the fp64 band of one repair overflows (it links u).
+template <class F>
+static void connect_root(ConnArgs a, int32_t root, cudaStream_t st, F on_band) {
+  SSG_CUDA(cudaMemsetAsync(a.bm, 0, sizeof(uint32_t) * a.nw, st));
+  SSG_LAUNCH(k_mark, 1, 1, 0, st, a.bm, a.f0, a.s, root);
+  a.start = 0;
+  a.stop_at_knn = a.knn != nullptr;
+  RepairState h = run_connect(a, st);
+  a.stop_at_knn = 0;
+  while ((int64_t)h.u < a.n) {
+    a.start = (int64_t)h.u >> 5;
+    if (h.best == STOP_KNN && a.knn) {
+      const size_t smem = (size_t)a.nw * sizeof(uint32_t);
+      const bool shared = smem <= 200 * 1024;
+      if (shared) ensure_smem((const void*)k_repair_knn, smem);
+      SSG_LAUNCH(k_repair_knn, 1, 256, shared ? smem : 0, st, a, shared ? 1 : 0);
+      SSG_CUDA(cudaMemcpyAsync(&h, a.s, sizeof(h), cudaMemcpyDeviceToHost, st));
+      SSG_CUDA(cudaStreamSynchronize(st));
+      if ((int64_t)h.u >= a.n) break;
+      a.start = (int64_t)h.u >> 5;
+      if (h.best == STOP_ROW) {  // no frontier is left
+        const int none[3] = {0, 0, 0};
+        SSG_CUDA(cudaMemcpyAsync(a.s->lvl, none, sizeof(none), cudaMemcpyHostToDevice, st));
       }
+    } else if (h.best == STOP_BAND) {
+      on_band(h);
     }
-    cur ^= 1;
+    SSG_REQUIRE(h.best != STOP_NONE, SSG_EINTERNAL,
+                "connectivity: node %lld is unreached and no reached node has a free slot",
+                (long long)h.u);
+    h = run_connect(a, st);
   }
 }
 
-// Repairs that u's own kNN row settles, back to back in one block.  The row lists u's K
-// nearest nodes in exact (d2, id) order, so when some of them is reached and has a free
-// slot the first such one is the (d2, id)-smallest of all reached nodes with a free slot:
-// the same choice as the exhaustive argmin, without a pass over all n nodes.  Each round:
-// the smallest unreached u (from bitmap word `start` on), the link from the first
-// qualifying row entry, and the traversal from u while its frontier stays within `limit`.
-// Stops with s->u = n when every node is reached, with s->best = -3 when u's row has no
-// qualifying node (the exhaustive path takes u), or with s->bfs_state set when a frontier
-// outgrows the block (the grid-wide traversal finishes it).  *nrep += the repairs made.
-__global__ void __launch_bounds__(1024)
-    k_repair_knn(const int32_t* __restrict__ knn, int K, int32_t* __restrict__ adj,
-                 int32_t* __restrict__ deg, int R, uint32_t* __restrict__ bm, int64_t nw,
-                 int64_t n, int64_t start, int32_t* __restrict__ f0, int32_t* __restrict__ f1,
-                 int limit, RepairState* __restrict__ s, unsigned long long* __restrict__ nrep) {
-  __shared__ unsigned long long su;
-  __shared__ int sv, sfc[2];
-  const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5, nwarps = blockDim.x >> 5;
-  unsigned long long made = 0;
-  for (;;) {
-    // the smallest unreached id from word `start` on
-    for (;;) {
-      if (tid == 0) su = (unsigned long long)n;
-      __syncthreads();
-      const int64_t w = start + tid;
-      if (w < nw) {
-        uint32_t word = bm[w];
-        if (w == nw - 1 && (n & 31)) word |= ~((1u << (n & 31)) - 1u);
-        if (word != 0xffffffffu) atomicMin(&su, (unsigned long long)(w * 32 + __ffs(~word) - 1));
-      }
-      __syncthreads();
-      const bool stop = su < (unsigned long long)n || start + blockDim.x >= nw;
-      __syncthreads();
-      if (stop) break;
-      start += blockDim.x;
-    }
-    const int64_t u = (int64_t)su;
-    if (u >= n) {
-      if (tid == 0) {
-        s->u = (unsigned long long)n;
-        s->best = INT_MAX;
-        s->bfs_state = -1;
-      }
-      break;
-    }
-    if (warp == 0) {
-      int found = -1;
-      for (int c = 0; c < K; c += 32) {
-        const int t = c + lane;
-        int32_t v = -1;
-        bool ok = false;
-        if (t < K) {
-          v = knn[u * K + t];
-          ok = v >= 0 && ((bm[v >> 5] >> (v & 31)) & 1u) && deg[v] < R;
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, ok);
-        if (bal) {
-          found = __shfl_sync(0xffffffffu, v, __ffs(bal) - 1);
-          break;
-        }
-      }
-      if (lane == 0) sv = found;
-    }
-    __syncthreads();
-    const int v = sv;
-    if (v < 0) {
-      if (tid == 0) {
-        s->u = (unsigned long long)u;
-        s->best = -3;
-        s->bfs_state = -1;
-      }
-      break;
-    }
-    if (tid == 0) {
-      adj[(int64_t)v * R + deg[v]] = (int32_t)u;
-      deg[v] += 1;
-      atomicOr(bm + (u >> 5), 1u << (u & 31));
-      f0[0] = (int32_t)u;
-      sfc[0] = 1;
-      ++made;
-    }
-    __syncthreads();
-    int cur = 0;
-    bool big = false;
-    for (;;) {
-      const int fc = sfc[cur];
-      if (fc == 0) break;
-      if (fc > limit) {
-        big = true;
-        break;
-      }
-      __syncthreads();
-      if (tid == 0) sfc[cur ^ 1] = 0;
-      __syncthreads();
-      const int32_t* fr = cur ? f1 : f0;
-      int32_t* nx = cur ? f0 : f1;
-      for (int w = warp; w < fc; w += nwarps) {
-        const int32_t node = fr[w];
-        const int dg = deg[node];
-        for (int c = 0; c < dg; c += 32) {
-          const int t = c + lane;
-          bool fresh = false;
-          int32_t x = 0;
-          if (t < dg) {
-            x = adj[(int64_t)node * R + t];
-            const uint32_t bit = 1u << (x & 31);
-            fresh = !(atomicOr(bm + (x >> 5), bit) & bit);
-          }
-          const unsigned bal = __ballot_sync(0xffffffffu, fresh);
-          int basep = 0;
-          if (lane == 0 && bal) basep = atomicAdd(&sfc[cur ^ 1], __popc(bal));
-          basep = __shfl_sync(0xffffffffu, basep, 0);
-          if (fresh) nx[basep + __popc(bal & lanemask_lt())] = x;
-        }
-      }
-      __syncthreads();
-      cur ^= 1;
-    }
-    if (big) {
-      if (tid == 0) {
-        s->u = (unsigned long long)u;
-        s->best = v;
-        s->fcnt[cur] = sfc[cur];
-        s->bfs_state = cur;
-      }
-      break;
-    }
-    start = u >> 5;
-    __syncthreads();
-  }
-  if (tid == 0 && made) atomicAdd(nrep, made);
+__global__ void k_repeat_row(const float* __restrict__ x, int ld, float* __restrict__ out) {
+  for (int t = threadIdx.x; t < ld; t += blockDim.x) out[(size_t)blockIdx.x * ld + t] = x[t];
 }
 
-// Level-synchronous traversal by the whole grid, starting from frontier buffer `cur`: the
-// levels are launched in batches (4, 8, 16, then 32 at a time) and the host reads the
-// next frontier's size once per batch.
-static void bfs_levels(const int32_t* adj, const int32_t* deg, int R, uint32_t* bm, int32_t* f[2],
-                       RepairState* s, int cur, cudaStream_t st) {
-  const int grid = 4 * num_sms();
-  SSG_LAUNCH(k_ring_init, 1, 1, 0, st, s->lvl, &s->fcnt[cur]);
-  int l = 0, batch = 4;
-  for (;;) {
-    for (int b = 0; b < batch; ++b, ++l)
-      SSG_LAUNCH(k_bfs_level_ring, grid, 256, 0, st, adj, deg, R, bm, f[(cur + l) & 1],
-                 f[(cur + l + 1) & 1], s->lvl, l);
-    int h = 0;
-    SSG_CUDA(cudaMemcpyAsync(&h, &s->lvl[l % 3], sizeof(int), cudaMemcpyDeviceToHost, st));
-    SSG_CUDA(cudaStreamSynchronize(st));
-    if (h == 0) break;
-    batch = std::min(2 * batch, 32);
-  }
+// Whether each later root provably reaches the first one (which reaches every node): a beam
+// search from it towards the first root's vector meets that node.
+static std::vector<char> roots_reach_first(const ConnArgs& a, const int32_t* nav_host, int n_nav,
+                                           cudaStream_t st) {
+  std::vector<char> ok((size_t)n_nav, 0);
+  const int m = n_nav - 1;
+  if (m < 1 || a.R > 128) return ok;
+  const int ls = 32;
+  Scratch<float> q((size_t)m * a.ld, st);
+  Scratch<int32_t> from((size_t)m, st), ids((size_t)m, st);
+  SSG_LAUNCH(k_repeat_row, (unsigned)m, 128, 0, st, a.X + (int64_t)nav_host[0] * a.ld, a.ld, q.p);
+  SSG_CUDA(cudaMemcpyAsync(from.p, nav_host + 1, sizeof(int32_t) * m, cudaMemcpyHostToDevice, st));
+  if (!search_from(a.X, a.ld, a.d, a.adj, a.deg, a.R, from.p, q.p, a.ld, m, ls, ids.p, st)) return ok;
+  std::vector<int32_t> h((size_t)m);
+  SSG_CUDA(cudaMemcpyAsync(h.data(), ids.p, sizeof(int32_t) * m, cudaMemcpyDeviceToHost, st));
+  SSG_CUDA(cudaStreamSynchronize(st));
+  for (int t = 0; t < m; ++t) ok[(size_t)t + 1] = h[(size_t)t] == nav_host[0];
+  return ok;
 }
 
 int64_t connect_run(const float* X, int ld, int d, int64_t n, int32_t* adj, int32_t* deg,
                     int R, const int32_t* nav_dev, const int32_t* nav_host, int n_nav,
                     cudaStream_t st, const int32_t* knn, int K, int64_t* knn_repairs) {
   (void)nav_dev;
-  Scratch<unsigned long long> knn_rep;
-  if (knn) {
-    knn_rep.alloc(1, st);
-    SSG_CUDA(cudaMemsetAsync(knn_rep.p, 0, sizeof(unsigned long long), st));
-  }
   const int64_t nw = ceil_div(n, 32);
   const int cap = 1 << 16;
   Scratch<uint32_t> bm((size_t)nw, st);
@@ -502,85 +656,38 @@ int64_t connect_run(const float* X, int ld, int d, int64_t n, int32_t* adj, int3
   Scratch<double> band_d((size_t)cap, st);
   Scratch<float> d32((size_t)n, st);
   Scratch<RepairState> state(1, st);
+  SSG_CUDA(cudaMemsetAsync(state.p, 0, sizeof(RepairState), st));
   Scratch<unsigned long long> ull(1, st);
   Scratch<double> dv;
-  int32_t* f[2] = {f0.p, f1.p};
-  RepairState* S = state.p;
+  ConnArgs a{X, ld, d, n, nw, adj, deg, R, bm.p, f0.p, f1.p, knn, K, d32.p, band_ids.p, band_d.p,
+             cap, dist_rel_team8(ld), state.p, 0, 0};
   const int grid = 8 * num_sms();
-  const float rel = dist_rel_team8(ld);
-  const int small_limit = 4096;
-  int64_t repairs = 0;
-  for (int r = 0; r < n_nav; ++r) {
-    SSG_CUDA(cudaMemsetAsync(bm.p, 0, sizeof(uint32_t) * nw, st));
-    SSG_LAUNCH(k_mark, 1, 1, 0, st, bm.p, f[0], &S->fcnt[0], nav_host[r]);
-    int64_t start = 0;
-    bool first = true;
-    for (;;) {
-      if (!first && knn) {
-        // the repairs the kNN rows settle, in one launch; the rest below
-        SSG_LAUNCH(k_repair_knn, 1, 1024, 0, st, knn, K, adj, deg, R, bm.p, nw, n, start, f[0], f[1],
-                   small_limit, S, knn_rep.p);
-        RepairState h;
-        SSG_CUDA(cudaMemcpyAsync(&h, S, sizeof(h), cudaMemcpyDeviceToHost, st));
-        SSG_CUDA(cudaStreamSynchronize(st));
-        if ((int64_t)h.u >= n) break;
-        start = (int64_t)h.u >> 5;
-        if (h.best != -3) {
-          // u is linked and its traversal outgrew the block: the grid finishes it
-          if (h.bfs_state >= 0) bfs_levels(adj, deg, R, bm.p, f, S, h.bfs_state, st);
-          continue;
-        }
-      }
-      if (!first) {
-        SSG_LAUNCH(k_repair_init, 1, 1, 0, st, S, n);
-        SSG_LAUNCH(k_first_unreached, grid, 256, 0, st, bm.p, nw, n, start, &S->u);
-        SSG_LAUNCH(k_repair_fp32, grid, 256, 0, st, X, ld, n, bm.p, deg, R, rel, d32.p, S);
-        SSG_LAUNCH(k_repair_band, grid, 256, 0, st, X, ld, d, n, d32.p, rel, cap, band_ids.p,
-                   band_d.p, S);
-        SSG_LAUNCH(k_repair_band64, 2 * num_sms(), 256, 0, st, X, ld, d, n, cap, band_ids.p,
-                   band_d.p, S);
-        SSG_LAUNCH(k_repair_pick, 1, 256, 0, st, X, ld, d, band_ids.p, band_d.p, cap, adj, deg, R,
-                   bm.p, f[0], n, S);
-      }
-      SSG_LAUNCH(k_bfs_small, 1, 1024, 0, st, adj, deg, R, bm.p, f[0], f[1], small_limit, S);
-      RepairState h;
-      SSG_CUDA(cudaMemcpyAsync(&h, S, sizeof(h), cudaMemcpyDeviceToHost, st));
-      SSG_CUDA(cudaStreamSynchronize(st));
-      if (!first) {
-        if ((int64_t)h.u >= n) break;
-        if (h.best == -2) {
-          // the band list overflowed (many exact ties): exhaustive fp64 argmin instead
-          if (!dv.p) dv.alloc((size_t)n, st);
-          const unsigned long long init = ~0ull;
-          const int imax = INT_MAX;
-          SSG_CUDA(cudaMemcpyAsync(ull.p, &init, sizeof(init), cudaMemcpyHostToDevice, st));
-          SSG_CUDA(cudaMemcpyAsync(&S->best, &imax, sizeof(int), cudaMemcpyHostToDevice, st));
-          SSG_LAUNCH(k_repair_dist, grid, 256, 0, st, X, ld, d, n, bm.p, deg, R, (int64_t)h.u,
-                     dv.p, ull.p);
-          SSG_LAUNCH(k_repair_pick_all, grid, 256, 0, st, dv.p, n, ull.p, &S->best);
-          SSG_LAUNCH(k_add_edge, 1, 1, 0, st, adj, deg, R, &S->best, bm.p, f[0], S);
-          SSG_LAUNCH(k_bfs_small, 1, 1024, 0, st, adj, deg, R, bm.p, f[0], f[1], small_limit, S);
-          SSG_CUDA(cudaMemcpyAsync(&h, S, sizeof(h), cudaMemcpyDeviceToHost, st));
-          SSG_CUDA(cudaStreamSynchronize(st));
-        }
-        SSG_REQUIRE(h.best != INT_MAX, SSG_EINTERNAL,
-                    "connectivity: node %lld is unreached and no reached node has a free slot",
-                    (long long)h.u);
-        start = (int64_t)h.u >> 5;
-        ++repairs;
-      }
-      if (h.bfs_state >= 0) bfs_levels(adj, deg, R, bm.p, f, S, h.bfs_state, st);
-      first = false;
-    }
-  }
-  if (knn) {
-    unsigned long long kr = 0;
-    SSG_CUDA(cudaMemcpyAsync(&kr, knn_rep.p, sizeof(kr), cudaMemcpyDeviceToHost, st));
+  auto on_band = [&](RepairState& h) {
+    // the band list overflowed (many exact ties): exhaustive fp64 argmin instead
+    if (!dv.p) dv.alloc((size_t)n, st);
+    const unsigned long long init = ~0ull;
+    const int imax = INT_MAX;
+    SSG_CUDA(cudaMemcpyAsync(ull.p, &init, sizeof(init), cudaMemcpyHostToDevice, st));
+    SSG_CUDA(cudaMemcpyAsync(&state.p->best, &imax, sizeof(int), cudaMemcpyHostToDevice, st));
+    SSG_LAUNCH(k_repair_dist, grid, 256, 0, st, X, ld, d, n, bm.p, deg, R, (int64_t)h.u, dv.p, ull.p);
+    SSG_LAUNCH(k_repair_pick_all, grid, 256, 0, st, dv.p, n, ull.p, &state.p->best);
+    SSG_LAUNCH(k_add_edge, 1, 1, 0, st, adj, deg, R, &state.p->best, bm.p, f0.p, state.p);
+    int best = 0;
+    SSG_CUDA(cudaMemcpyAsync(&best, &state.p->best, sizeof(int), cudaMemcpyDeviceToHost, st));
     SSG_CUDA(cudaStreamSynchronize(st));
-    repairs += (int64_t)kr;
-    if (knn_repairs) *knn_repairs = (int64_t)kr;
+    if (best == INT_MAX) h.best = STOP_NONE;
+  };
+  std::vector<char> skip;
+  for (int r = 0; r < n_nav; ++r) {
+    if (r == 1) skip = roots_reach_first(a, nav_host, n_nav, st);
+    if (r >= 1 && skip[(size_t)r]) continue;
+    connect_root(a, nav_host[r], st, on_band);
   }
-  return repairs;
+  RepairState h;
+  SSG_CUDA(cudaMemcpyAsync(&h, state.p, sizeof(h), cudaMemcpyDeviceToHost, st));
+  SSG_CUDA(cudaStreamSynchronize(st));
+  if (knn_repairs) *knn_repairs = (int64_t)h.rep_knn;
+  return (int64_t)(h.rep_full + h.rep_knn);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -634,56 +741,23 @@ static int64_t connect_run_noalloc(const float* X, int ld, int d, int64_t n, int
                                    const int32_t* nav_host, int n_nav, cudaStream_t st) {
   (void)nav_dev;
   unsigned char* base = noalloc_scratch();
-  uint32_t* bm = (uint32_t*)(base + OFF_BM);
-  int32_t* f[2] = {(int32_t*)(base + OFF_F0), (int32_t*)(base + OFF_F1)};
-  float* d32 = (float*)(base + OFF_D32);
-  int32_t* band_ids = (int32_t*)(base + OFF_BAND_ID);
-  double* band_d = (double*)(base + OFF_BAND_D);
   RepairState* S = (RepairState*)(base + OFF_STATE);
-  const int64_t nw = ceil_div(n, 32);
-  const int grid = 8 * num_sms();
-  const float rel = dist_rel_team8(ld);
-  const int small_limit = 4096;
-  int64_t repairs = 0;
-  for (int r = 0; r < n_nav; ++r) {
-    const int32_t root = nav_host[r];
-    SSG_CUDA(cudaMemsetAsync(bm, 0, sizeof(uint32_t) * nw, st));
-    SSG_LAUNCH(k_mark, 1, 1, 0, st, bm, f[0], &S->fcnt[0], root);
-    int64_t start = 0;
-    bool first = true;
-    for (;;) {
-      if (!first) {
-        SSG_LAUNCH(k_repair_init, 1, 1, 0, st, S, n);
-        SSG_LAUNCH(k_first_unreached, grid, 256, 0, st, bm, nw, n, start, &S->u);
-        SSG_LAUNCH(k_repair_fp32, grid, 256, 0, st, X, ld, n, bm, deg, R, rel, d32, S);
-        SSG_LAUNCH(k_repair_band, grid, 256, 0, st, X, ld, d, n, d32, rel, NOALLOC_BAND, band_ids,
-                   band_d, S);
-        SSG_LAUNCH(k_repair_band64, 2 * num_sms(), 256, 0, st, X, ld, d, n, NOALLOC_BAND, band_ids,
-                   band_d, S);
-        SSG_LAUNCH(k_repair_pick, 1, 256, 0, st, X, ld, d, band_ids, band_d, NOALLOC_BAND, adj, deg,
-                   R, bm, f[0], n, S);
-      }
-      SSG_LAUNCH(k_bfs_small, 1, 1024, 0, st, adj, deg, R, bm, f[0], f[1], small_limit, S);
-      RepairState h;
-      SSG_CUDA(cudaMemcpyAsync(&h, S, sizeof(h), cudaMemcpyDeviceToHost, st));
-      SSG_CUDA(cudaStreamSynchronize(st));
-      if (!first) {
-        if ((int64_t)h.u >= n) break;
-        SSG_REQUIRE(h.best != -2, SSG_EINTERNAL,
-                    "connectivity without allocation: more than %d nodes tie for the nearest "
-                    "reached node of node %lld; use ssg_connect",
-                    NOALLOC_BAND, (long long)h.u);
-        SSG_REQUIRE(h.best != INT_MAX, SSG_EINTERNAL,
-                    "connectivity: node %lld is unreached and no reached node has a free slot",
-                    (long long)h.u);
-        start = (int64_t)h.u >> 5;
-        ++repairs;
-      }
-      if (h.bfs_state >= 0) bfs_levels(adj, deg, R, bm, f, S, h.bfs_state, st);
-      first = false;
-    }
-  }
-  return repairs;
+  SSG_CUDA(cudaMemsetAsync(S, 0, sizeof(RepairState), st));
+  ConnArgs a{X, ld, d, n, ceil_div(n, 32), adj, deg, R, (uint32_t*)(base + OFF_BM),
+             (int32_t*)(base + OFF_F0), (int32_t*)(base + OFF_F1), nullptr, 0,
+             (float*)(base + OFF_D32), (int32_t*)(base + OFF_BAND_ID),
+             (double*)(base + OFF_BAND_D), NOALLOC_BAND, dist_rel_team8(ld), S, 0, 0};
+  auto on_band = [&](RepairState& h) {
+    SSG_REQUIRE(false, SSG_EINTERNAL,
+                "connectivity without allocation: more than %d nodes tie for the nearest "
+                "reached node of node %lld; use ssg_connect",
+                NOALLOC_BAND, (long long)h.u);
+  };
+  for (int r = 0; r < n_nav; ++r) connect_root(a, nav_host[r], st, on_band);
+  RepairState h;
+  SSG_CUDA(cudaMemcpyAsync(&h, S, sizeof(h), cudaMemcpyDeviceToHost, st));
+  SSG_CUDA(cudaStreamSynchronize(st));
+  return (int64_t)(h.rep_full + h.rep_knn);
 }
 
 }  // namespace ssg

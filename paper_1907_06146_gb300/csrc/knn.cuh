@@ -259,6 +259,12 @@ void search_run_mixed(const float* X, const uint8_t* X8, int ld, int d, const in
                       int ldq, int64_t nq, const int32_t* qk, const int32_t* qls, int ls_max,
                       int ldo, int32_t* out_ids, float* out_d2, cudaStream_t st);
 
+// The nearest node that Alg. 1 finds for each query from a start node of its own (from[q]), pool
+// size Ls; false (nothing launched) where a row is too long for the kernel's shared memory.
+bool search_from(const float* X, int ld, int d, const int32_t* adj, const int32_t* deg, int R,
+                 const int32_t* from, const float* Q, int ldq, int64_t nq, int Ls, int32_t* out_ids,
+                 cudaStream_t st);
+
 // Byte copy [n][ld] of rows that hold integers 0..255 (ld: the float rows' stride, a
 // multiple of 4; padding bytes 0).
 void rows_to_u8(const float* X, int ld, int d, int64_t n, uint8_t* out, cudaStream_t st);

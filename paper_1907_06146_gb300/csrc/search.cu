@@ -284,8 +284,8 @@ __global__ void __launch_bounds__(256, 3)
     k_search(const T* __restrict__ X, int ld, int d, const int32_t* __restrict__ adj,
                          const int32_t* __restrict__ deg, int R, const int32_t* __restrict__ nav,
                          int n_nav, const float* __restrict__ Q, int ldq, int64_t nq, int k,
-                         const int32_t* __restrict__ qk, const int32_t* __restrict__ qls, int ldo,
-                         SearchLayout lay, int32_t* __restrict__ out_ids,
+                         const int32_t* __restrict__ qk, const int32_t* __restrict__ qls,
+                         const int32_t* __restrict__ from, int ldo, SearchLayout lay, int32_t* __restrict__ out_ids,
                          float* __restrict__ out_d2, unsigned long long* __restrict__ work) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = lane_id();
@@ -340,12 +340,13 @@ __global__ void __launch_bounds__(256, 3)
       }
     }
 
-    // entry: the nearest navigating node by (d2, id)
+    // entry: the nearest navigating node by (d2, id), or the query's own start node
     uint64_t best = KEY_NONE;
+    const int32_t* starts = from ? from + qi : nav;
     for (int s0 = 0; s0 < n_nav; s0 += 4) {
       const int s = s0 + team;
       const bool valid = s < n_nav;
-      const int32_t id = valid ? nav[s] : 0;
+      const int32_t id = valid ? starts[s] : 0;
       const float dd = team8_dist_q(qs, X + (int64_t)id * ld, ld4, tl, valid);
       const uint64_t key = valid ? make_key(dd, id) : KEY_NONE;
       best = key < best ? key : best;
@@ -564,7 +565,8 @@ void rows_to_u8(const float* X, int ld, int d, int64_t n, uint8_t* out, cudaStre
 template <typename T>
 static void launch_search(const T* X, int ld, int d, const int32_t* adj, const int32_t* deg, int R,
                           const int32_t* nav, int n_nav, const float* Q, int ldq, int64_t nq, int k,
-                          const int32_t* qk, const int32_t* qls, int ldo, SearchLayout lay, int wpb,
+                          const int32_t* qk, const int32_t* qls, const int32_t* from, int ldo,
+                          SearchLayout lay, int wpb,
                           int32_t* out_ids, float* out_d2, unsigned long long* work,
                           cudaStream_t st) {
   while (lay.per_warp() * wpb > 200 * 1024 && lay.log2h > 8) --lay.log2h;
@@ -576,7 +578,7 @@ static void launch_search(const T* X, int ld, int d, const int32_t* adj, const i
   const int64_t want = ceil_div(nq, wpb);
   const int grid = (int)std::min<int64_t>(want, (int64_t)std::max(1, blocks_per_sm) * num_sms());
   SSG_LAUNCH(k_search<T>, grid, wpb * 32, smem, st, X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq,
-             k, qk, qls, ldo, lay, out_ids, out_d2, work);
+             k, qk, qls, from, ldo, lay, out_ids, out_d2, work);
 }
 
 void search_run_mixed(const float* X, const uint8_t* X8, int ld, int d, const int32_t* adj,
@@ -592,10 +594,10 @@ void search_run_mixed(const float* X, const uint8_t* X8, int ld, int d, const in
   // limit) keep more row gathers in flight than a larger cache would save
   lay.log2h = 10;
   if (X8)
-    launch_search(X8, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, 0, qk, qls, ldo, lay, 8,
+    launch_search(X8, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, 0, qk, qls, nullptr, ldo, lay, 8,
                   out_ids, out_d2, (unsigned long long*)nullptr, st);
   else
-    launch_search(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, 0, qk, qls, ldo, lay, 8, out_ids,
+    launch_search(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, 0, qk, qls, nullptr, ldo, lay, 8, out_ids,
                   out_d2, (unsigned long long*)nullptr, st);
 }
 
@@ -617,10 +619,26 @@ void search_run(const float* X, const uint8_t* X8, int ld, int d, int64_t n, con
   const int wpb = work ? 2 : 8;
   if (X8)
     launch_search(X8, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, (const int32_t*)nullptr,
-                  (const int32_t*)nullptr, k, lay, wpb, out_ids, out_d2, work, st);
+                  (const int32_t*)nullptr, nullptr, k, lay, wpb, out_ids, out_d2, work, st);
   else
     launch_search(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, (const int32_t*)nullptr,
-                  (const int32_t*)nullptr, k, lay, wpb, out_ids, out_d2, work, st);
+                  (const int32_t*)nullptr, nullptr, k, lay, wpb, out_ids, out_d2, work, st);
+}
+
+bool search_from(const float* X, int ld, int d, const int32_t* adj, const int32_t* deg, int R,
+                 const int32_t* from, const float* Q, int ldq, int64_t nq, int Ls, int32_t* out_ids,
+                 cudaStream_t st) {
+  SearchLayout lay;
+  lay.Ls = Ls;
+  lay.RP = std::max(32, next_pow2(R));
+  lay.ld = ld;
+  lay.log2h = 10;
+  const int wpb = 1;  // few queries: a block, and an SM, each
+  if (lay.per_warp() > 200 * 1024) return false;
+  launch_search(X, ld, d, adj, deg, R, from, 1, Q, ldq, nq, 1, (const int32_t*)nullptr,
+                (const int32_t*)nullptr, from, 1, lay, wpb, out_ids, (float*)nullptr,
+                (unsigned long long*)nullptr, st);
+  return true;
 }
 
 }  // namespace ssg
