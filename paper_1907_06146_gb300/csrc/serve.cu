@@ -134,9 +134,11 @@ void finish_slot(ssg_server* s, Slot& sl) {
         std::chrono::duration<double, std::milli>(now - s->t_busy_start).count();
 }
 
-// Pack waiting requests into a free slot and launch it (mutex held).  Returns false if
-// nothing could be admitted.
-bool launch_batch(ssg_server* s, Slot& sl) {
+// Pack waiting requests into a free slot (mutex held) and launch it.  Returns false if
+// nothing could be admitted.  The mutex is released around the CUDA calls: a first launch of a
+// kernel may wait for the work in flight (lazy loading), and that work ends in callbacks that
+// take the mutex.
+bool launch_batch(ssg_server* s, Slot& sl, std::unique_lock<std::mutex>& lk) {
   int64_t nq = 0;
   int kmax = 1, lsmax = 1;
   size_t bytes = 0;
@@ -175,6 +177,8 @@ bool launch_batch(ssg_server* s, Slot& sl) {
   for (auto& o : s->slots)
     if (o->busy) inflight_q += o->nq;
   s->stats.max_queries_in_flight = std::max<int64_t>(s->stats.max_queries_in_flight, inflight_q);
+  lk.unlock();
+  ssg_status failed = SSG_OK;
   try {
     const ssg_graph* g = s->g;
     SSG_CUDA(cudaMemcpyAsync(sl.d_q, sl.h_q, sizeof(float) * nq * s->ld, cudaMemcpyHostToDevice, sl.st));
@@ -189,7 +193,11 @@ bool launch_batch(ssg_server* s, Slot& sl) {
     SSG_CUDA(cudaMemcpyAsync(sl.h_d2, sl.d_d2, sizeof(float) * nq * kmax, cudaMemcpyDeviceToHost, sl.st));
     SSG_CUDA(cudaLaunchHostFunc(sl.st, on_slot_done, &sl));
   } catch (const ssg::Fail& e) {
-    sl.launch_status = e.st;
+    failed = e.st;
+  }
+  lk.lock();
+  if (failed != SSG_OK) {
+    sl.launch_status = failed;
     sl.ready = true;  // finish it with the error status on the next pass
   }
   return true;
@@ -204,7 +212,7 @@ void scheduler(ssg_server* s) {
     bool launched = false;
     for (auto& sl : s->slots) {
       if (s->pending.empty()) break;
-      if (!sl->busy && launch_batch(s, *sl)) launched = true;
+      if (!sl->busy && launch_batch(s, *sl, lk)) launched = true;
     }
     if (launched) continue;
     if (s->stop && s->pending.empty() && s->busy_slots == 0) break;
