@@ -1,12 +1,11 @@
 // Search-on-Graph (Alg. 1) from the navigating node nearest the query (Sec. 4.1).
 //
-// One warp per query.  The candidate pool S (at most L_search entries, sorted by
-// (d2, id), with a checked flag each) lives in shared memory; each round expands the
-// first unchecked entry, gathers its adjacency row (coalesced), computes the distances
-// of the neighbours not seen before with teams of 8 lanes, two rows per team at a time
-// (all of both rows' float4 loads issued before the first multiply-add, so a warp keeps
-// 8 row gathers in flight), sorts them with a warp bitonic sort and merges them into S
-// with a rank-based parallel merge, cut at L_search.
+// One warp per query.  The candidate pool S (at most L_search entries, sorted by (d2, id),
+// with a checked flag in each key's last bit) lives in shared memory; each round expands the
+// first unchecked entry, gathers its adjacency row, computes the distances of the neighbours
+// not seen before, and merges those below the pool's last key into it: a sort in registers, one
+// binary search for each new key's place and duplicate test, and a move of the entries behind
+// the first new one.
 //
 // Rows: float32, or -- for data that are integers 0..255 -- a byte copy of the same
 // values.  A byte row of 128 dimensions is one 128-byte line instead of four; every lane
@@ -57,93 +56,54 @@ struct RawOf<uint8_t> {
   static __device__ __forceinline__ uint32_t zero() { return 0u; }
 };
 
-// x: a row of ld values (ld4 = ld / 4 groups of four)
-template <typename T>
-__device__ __forceinline__ float team8_dist_q(const float* __restrict__ qs,
-                                              const T* __restrict__ x, int ld4, int tl,
-                                              bool valid) {
-  using Raw = typename RawOf<T>::type;
-  float s = 0.f;
-  if (valid) {
-    const float4* q4 = (const float4*)qs;
-    // the row's loads (up to four per lane per 128 values) are all issued before the first
-    // multiply-add
-    for (int f0 = tl; f0 < ld4; f0 += 32) {
-      Raw b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int f = f0 + 8 * i;
-        b[i] = f < ld4 ? row_raw(x, f) : RawOf<T>::zero();
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int f = f0 + 8 * i;
-        if (f < ld4) {
-          const float4 a = q4[f];
-          const float4 v = raw_f4(b[i]);
-          float u;
-          u = a.x - v.x;
-          s = fmaf(u, u, s);
-          u = a.y - v.y;
-          s = fmaf(u, u, s);
-          u = a.z - v.z;
-          s = fmaf(u, u, s);
-          u = a.w - v.w;
-          s = fmaf(u, u, s);
-        }
-      }
-    }
-  }
-  s += __shfl_xor_sync(0xffffffffu, s, 1);
-  s += __shfl_xor_sync(0xffffffffu, s, 2);
-  s += __shfl_xor_sync(0xffffffffu, s, 4);
-  return s;
-}
-
-// NR rows per team at once (4 NR rows in flight per warp): the loads of all NR rows are
-// issued before the first multiply-add.  Each row's sum runs in the same order as in
-// team8_dist_q.  Rows are X + ids[r] * ld; rows with valid[r] false give 0.
+// Squared distances of the query to NR rows per team of four lanes (8 NR rows per warp): row r is
+// X + ids[r] * ld (rows with valid[r] false give 0).  Lane tl of a team sums float4 groups 2 tl
+// and 2 tl + 1 modulo 8, each modulus in one sequence; the eight sums of a row are then added
+// pairwise.  (The order of teams of eight lanes with one modulus each, kept so that results
+// stay the same to the bit; four lanes need two shuffles per row set instead of three.)
 template <typename T, int NR>
-__device__ __forceinline__ void team8_distN_q(const float* __restrict__ qs,
-                                              const T* __restrict__ X, int ld,
-                                              const int32_t (&ids)[NR], const bool (&valid)[NR],
-                                              int ld4, int tl, float (&out)[NR]) {
+__device__ __forceinline__ void team4_dist_q(const float* __restrict__ qs, const T* __restrict__ X,
+                                             int ld, const int32_t (&ids)[NR],
+                                             const bool (&valid)[NR], int tl, float (&out)[NR]) {
   using Raw = typename RawOf<T>::type;
   const float4* q4 = (const float4*)qs;
+  const int ld4 = ld >> 2;
+  float s[NR][2];
 #pragma unroll
-  for (int r = 0; r < NR; ++r) out[r] = 0.f;
-  for (int f0 = tl; f0 < ld4; f0 += 32) {
-    Raw raw[NR][4];
+  for (int r = 0; r < NR; ++r) s[r][0] = s[r][1] = 0.f;
+  for (int f0 = 2 * tl; f0 < ld4; f0 += 32) {
+    Raw raw[NR][8];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       const T* x = X + (int64_t)ids[r] * ld;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int f = f0 + 8 * i;
+      for (int i = 0; i < 8; ++i) {
+        const int f = f0 + 8 * (i >> 1) + (i & 1);
         raw[r][i] = (valid[r] && f < ld4) ? row_raw(x, f) : RawOf<T>::zero();
       }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int f = f0 + 8 * i;
+    for (int i = 0; i < 8; ++i) {
+      const int f = f0 + 8 * (i >> 1) + (i & 1);
       if (f < ld4) {
         const float4 q = q4[f];
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
           const float4 v = raw_f4(raw[r][i]);
           float u;
-          u = q.x - v.x; out[r] = fmaf(u, u, out[r]);
-          u = q.y - v.y; out[r] = fmaf(u, u, out[r]);
-          u = q.z - v.z; out[r] = fmaf(u, u, out[r]);
-          u = q.w - v.w; out[r] = fmaf(u, u, out[r]);
+          u = q.x - v.x; s[r][i & 1] = fmaf(u, u, s[r][i & 1]);
+          u = q.y - v.y; s[r][i & 1] = fmaf(u, u, s[r][i & 1]);
+          u = q.z - v.z; s[r][i & 1] = fmaf(u, u, s[r][i & 1]);
+          u = q.w - v.w; s[r][i & 1] = fmaf(u, u, s[r][i & 1]);
         }
       }
     }
   }
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
-#pragma unroll
-    for (int r = 0; r < NR; ++r) out[r] += __shfl_xor_sync(0xffffffffu, out[r], o);
+  for (int r = 0; r < NR; ++r) {
+    out[r] = valid[r] ? s[r][0] + s[r][1] : 0.f;
+    out[r] += __shfl_xor_sync(0xffffffffu, out[r], 1);
+    out[r] += __shfl_xor_sync(0xffffffffu, out[r], 2);
   }
 }
 
@@ -151,96 +111,90 @@ __device__ __forceinline__ void team8_distN_q(const float* __restrict__ qs,
 // packed four to a word (qw) and q2 = |q|^2, d2 = q2 + |x|^2 - 2 q.x from byte dot products
 // (dp4a), all in exact integer arithmetic.  Every value and partial sum of the float path
 // is an integer below 2^24 in that case, so the float path's sums are exact too and the two
-// give the same distances.
+// give the same distances.  Rows of a multiple of 16 bytes load in 16-byte pieces.
+__device__ __forceinline__ int sum_dp4a(uint32_t q, uint32_t x, int s) {
+  return s + (int)__dp4a(x, x, 0u) - 2 * (int)__dp4a(q, x, 0u);
+}
 template <int NR>
-__device__ __forceinline__ void team8_distN_qi(const uint32_t* __restrict__ qw,
-                                               const uint8_t* __restrict__ X, int ld,
-                                               const int32_t (&ids)[NR],
-                                               const bool (&valid)[NR], int ld4, int tl, int q2,
-                                               float (&out)[NR]) {
-  unsigned dot[NR], xx[NR];
+__device__ __forceinline__ void team4_dist_qi(const uint32_t* __restrict__ qw,
+                                              const uint8_t* __restrict__ X, int ld,
+                                              const int32_t (&ids)[NR], const bool (&valid)[NR],
+                                              int tl, int q2, float (&out)[NR]) {
+  int s[NR];
 #pragma unroll
-  for (int r = 0; r < NR; ++r) dot[r] = xx[r] = 0u;
-  for (int f0 = tl; f0 < ld4; f0 += 32) {
-    uint32_t raw[NR][4];
+  for (int r = 0; r < NR; ++r) s[r] = 0;
+  if ((ld & 15) == 0) {
+    const int np = ld >> 4;
+    for (int c0 = tl; c0 < np; c0 += 8) {
+      uint4 raw[NR][2];
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const uint8_t* x = X + (int64_t)ids[r] * ld;
+      for (int r = 0; r < NR; ++r) {
+        const uint4* x = (const uint4*)(X + (int64_t)ids[r] * ld);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int f = f0 + 8 * i;
-        raw[r][i] = (valid[r] && f < ld4) ? row_raw(x, f) : 0u;
+        for (int i = 0; i < 2; ++i) {
+          const int c = c0 + 4 * i;
+          raw[r][i] = (valid[r] && c < np) ? __ldg(x + c) : make_uint4(0u, 0u, 0u, 0u);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int c = c0 + 4 * i;
+        if (c < np) {
+          const uint4 q = ((const uint4*)qw)[c];
+#pragma unroll
+          for (int r = 0; r < NR; ++r) {
+            s[r] = sum_dp4a(q.x, raw[r][i].x, s[r]);
+            s[r] = sum_dp4a(q.y, raw[r][i].y, s[r]);
+            s[r] = sum_dp4a(q.z, raw[r][i].z, s[r]);
+            s[r] = sum_dp4a(q.w, raw[r][i].w, s[r]);
+          }
+        }
       }
     }
+  } else {
+    const int nw = ld >> 2;
+    for (int w0 = tl; w0 < nw; w0 += 16) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int f = f0 + 8 * i;
-      if (f < ld4) {
-        const uint32_t q = qw[f];
+      for (int i = 0; i < 4; ++i) {
+        const int w = w0 + 4 * i;
+        if (w < nw) {
+          const uint32_t q = qw[w];
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          dot[r] = __dp4a(q, raw[r][i], dot[r]);
-          xx[r] = __dp4a(raw[r][i], raw[r][i], xx[r]);
+          for (int r = 0; r < NR; ++r)
+            if (valid[r]) s[r] = sum_dp4a(q, row_raw(X + (int64_t)ids[r] * ld, w), s[r]);
         }
       }
     }
   }
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      dot[r] += __shfl_xor_sync(0xffffffffu, dot[r], o);
-      xx[r] += __shfl_xor_sync(0xffffffffu, xx[r], o);
-    }
+  for (int r = 0; r < NR; ++r) {
+    s[r] += __shfl_xor_sync(0xffffffffu, s[r], 1);
+    s[r] += __shfl_xor_sync(0xffffffffu, s[r], 2);
+    out[r] = (float)(q2 + s[r]);
   }
-#pragma unroll
-  for (int r = 0; r < NR; ++r) out[r] = (float)((int)q2 + (int)xx[r] - 2 * (int)dot[r]);
 }
 
-// Ascending bitonic sort of one key per lane across the warp (in registers).
-__device__ __forceinline__ uint64_t warp_bitonic32(uint64_t b, int lane) {
+// Pool keys: (distance bits, id, checked flag) packed so that they sort by (distance, id).
+__device__ __forceinline__ uint64_t pool_key(float d, int32_t id) {
+  return ((uint64_t)float_order_bits(d) << 32) | ((uint32_t)id << 1);
+}
+__device__ __forceinline__ int32_t pool_id_of(uint64_t k) { return (int32_t)((uint32_t)k >> 1); }
+
+// One compare-exchange step of a bitonic network over the warp (one key per lane).
+__device__ __forceinline__ uint64_t exchange(uint64_t b, int j, bool take_min) {
+  const uint64_t o = __shfl_xor_sync(0xffffffffu, b, j);
+  return take_min == (o < b) ? o : b;
+}
+// Ascending sort of one key per lane within groups of N lanes (a power of two).
+template <int N>
+__device__ __forceinline__ uint64_t warp_bitonic(uint64_t b, int lane) {
 #pragma unroll
-  for (int k = 2; k <= 32; k <<= 1) {
+  for (int k = 2; k <= N; k <<= 1) {
 #pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      const uint64_t o = __shfl_xor_sync(0xffffffffu, b, j);
-      const bool take_min = ((lane & j) == 0) == ((lane & k) == 0);
-      b = take_min ? (o < b ? o : b) : (o > b ? o : b);
-    }
+    for (int j = k >> 1; j > 0; j >>= 1)
+      b = exchange(b, j, ((lane & j) == 0) == (k == N || (lane & k) == 0));
   }
   return b;
-}
-
-// Same for two keys per lane (element e * 32 + lane in v[e]), 64 in all.
-__device__ __forceinline__ void warp_bitonic64(uint64_t (&v)[2], int lane) {
-#pragma unroll
-  for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const uint64_t o = __shfl_xor_sync(0xffffffffu, v[e], j);
-        const bool up = (((e << 5) | lane) & k) == 0;
-        const bool take_min = ((lane & j) == 0) == up;
-        v[e] = take_min ? (o < v[e] ? o : v[e]) : (o > v[e] ? o : v[e]);
-      }
-    }
-  }
-  // k = 64: the pair within a lane, then the halves
-  if (v[1] < v[0]) {
-    const uint64_t t = v[0];
-    v[0] = v[1];
-    v[1] = t;
-  }
-#pragma unroll
-  for (int j = 16; j > 0; j >>= 1) {
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const uint64_t o = __shfl_xor_sync(0xffffffffu, v[e], j);
-      const bool take_min = (lane & j) == 0;
-      v[e] = take_min ? (o < v[e] ? o : v[e]) : (o > v[e] ? o : v[e]);
-    }
-  }
 }
 
 // number of entries of a[0, len) that are < x (a sorted ascending)
@@ -256,70 +210,152 @@ __device__ __forceinline__ int count_less(const uint64_t* a, int len, uint64_t x
   return lo;
 }
 
-struct SearchLayout {
-  int Ls, RP, ld, log2h;
-  __host__ __device__ size_t pool_bytes() const { return (size_t)Ls * 8; }
-  __host__ __device__ size_t per_warp() const {
-    size_t b = 2 * pool_bytes() + (((size_t)2 * Ls + 15) & ~(size_t)15) + (size_t)RP * 8 +
-               (size_t)ld * 4 + ((size_t)4 << log2h) + (((size_t)ld + 15) & ~(size_t)15);
-    return (b + 15) & ~(size_t)15;
+// The candidate pool S of one warp, sorted, in shared memory.
+struct Pool {
+  uint64_t* p;
+  uint64_t worst;  // the Ls-th key, above every key with its node (KEY_NONE until S is full)
+  int s, Ls;       // entries, and their largest number
+  int lo;          // every entry before this one is checked
+
+  __device__ __forceinline__ void init(uint64_t* buf, uint64_t first, int size) {
+    p = buf;
+    Ls = size;
+    if (lane_id() == 0) p[0] = first;
+    s = 1;
+    lo = 0;
+    worst = Ls == 1 ? first | 1ull : KEY_NONE;
+    __syncwarp();
+  }
+  // The first unchecked entry's id (marked checked), or -1; second: the id of the one after it.
+  __device__ __forceinline__ int32_t take(int32_t& second) {
+    const int lane = lane_id();
+    int32_t first = -1;
+    second = -1;
+    for (int c = lo & ~31; c < s; c += 32) {
+      const uint32_t w = c + lane < s ? (uint32_t)p[c + lane] : 1u;
+      unsigned bal = __ballot_sync(0xffffffffu, !(w & 1u));
+      if (!bal) continue;
+      const int l = __ffs(bal) - 1;
+      if (first < 0) {
+        first = (int32_t)(__shfl_sync(0xffffffffu, w, l) >> 1);
+        if (lane == l) p[c + l] |= 1ull;
+        lo = c + l + 1;
+        bal &= bal - 1u;
+      }
+      if (bal) {
+        second = (int32_t)(__shfl_sync(0xffffffffu, w, __ffs(bal) - 1) >> 1);
+        break;
+      }
+    }
+    __syncwarp();
+    return first;
+  }
+  // Merges up to 32 keys (mine: one per lane, KEY_NONE for none; flags clear) into S: those
+  // below the pool's last key, without the nodes it holds.  Most expansions late in a search
+  // leave few of them, so the sort is as small as they allow, and only the entries behind the
+  // first new one move.  tmp: room for 32 keys.
+  __device__ __forceinline__ void merge(uint64_t mine, uint64_t* tmp) {
+    const int lane = lane_id();
+    const unsigned lt = lanemask_lt();
+    unsigned bal = __ballot_sync(0xffffffffu, mine < worst);
+    if (!bal) return;
+    const int m = __popc(bal);
+    uint64_t x = mine < worst ? mine : KEY_NONE;
+    if (m <= 16) {
+      __syncwarp();
+      if (mine < worst) tmp[__popc(bal & lt)] = mine;
+      __syncwarp();
+      x = lane < m ? tmp[lane] : KEY_NONE;
+      x = m <= 8 ? warp_bitonic<8>(x, lane) : warp_bitonic<16>(x, lane);
+    } else {
+      x = warp_bitonic<32>(x, lane);
+    }
+    int r = 0;
+    bool keep = false;
+    if (lane < m) {
+      r = count_less(p, s, x);
+      keep = r >= s || (p[r] ^ x) >= 2ull;
+    }
+    bal = __ballot_sync(0xffffffffu, keep);
+    if (!bal) return;
+    const int kept = __popc(bal), j = __popc(bal & lt);
+    __syncwarp();
+    if (keep) tmp[j] = x;
+    const int r0 = __shfl_sync(0xffffffffu, r, __ffs(bal) - 1);
+    __syncwarp();
+    // entries move up, so the last 32 go first
+    for (int c = (s - 1) & ~31; c + 31 >= r0 && c >= 0; c -= 32) {
+      const int i = c + lane;
+      const bool moves = i >= r0 && i < s;
+      const uint64_t a = moves ? p[i] : 0ull;
+      const int pos = moves ? i + count_less(tmp, kept, a) : Ls;
+      __syncwarp();
+      if (pos < Ls) p[pos] = a;
+    }
+    __syncwarp();
+    if (keep && r + j < Ls) p[r + j] = x;
+    s = s + kept < Ls ? s + kept : Ls;
+    lo = r0 < lo ? r0 : lo;
+    __syncwarp();
+    if (s == Ls) worst = p[Ls - 1] | 1ull;
   }
 };
 
-// Rows per team in the distance loop: a float row takes 16 registers per lane at d = 128,
-// a byte row 4, so byte rows keep twice as many rows in flight at the same 24 warps per SM
-// (measured on 1M x 128, L_search 40: 1.30 ms with 4 rows per team at 24 warps, 1.35 ms
-// with 2 at 32 warps, 1.76 ms with 8 at 16 warps; float rows 1.45 ms).
-template <typename T>
-struct RowsPerTeam {
-  static constexpr int value = 2;
-};
-template <>
-struct RowsPerTeam<uint8_t> {
-  static constexpr int value = 4;
+struct SearchLayout {
+  int Ls, RP, ld, log2h;  // Ls: the largest pool, even; RP: a multiple of 32, at least R
+  __host__ __device__ size_t per_warp() const {
+    return (size_t)Ls * 8 + (size_t)(RP + 32) * 8 + (size_t)ld * 4 + (((size_t)ld + 15) & ~(size_t)15) + ((size_t)4 << log2h);
+  }
 };
 
+// One warp per query.  Per expansion: the node's neighbours not in the visited cache (its row
+// and degree load together, and the row of the next unchecked entry is fetched ahead, so that
+// the next expansion often starts with it), their distances by teams of four lanes with all
+// loads of 8 NR rows issued at once, and a merge of those below the pool's last key.  Bound by
+// that chain of latencies and by its instructions, not by memory.  Against teams of eight lanes,
+// a dependent degree and row load, and a sort of all new neighbours merged into a second copy
+// of the pool: 10,000 queries over 1M x 128 byte rows, L_search 40, 0.74 -> 0.54 ms; 4,096 over
+// 300,000 x 96 float rows, L_search 256, 2.68 -> 1.36 ms; one query 128 -> 90 us.  Byte rows
+// take 24 warps per SM with 16 rows in flight (32 warps, 0.56 ms, spill; 32 rows 0.63), float
+// rows 32 warps with 8 (24 warps 1.76 ms; 16 warps with 16 rows 1.70).  A pool in registers
+// with an insertion per accepted neighbour was slower (0.93 and 3.5 ms): on the way to the
+// query about half the neighbours are accepted.
 template <typename T>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(256, std::is_same<T, uint8_t>::value ? 3 : 4)
     k_search(const T* __restrict__ X, int ld, int d, const int32_t* __restrict__ adj,
-                         const int32_t* __restrict__ deg, int R, const int32_t* __restrict__ nav,
-                         int n_nav, const float* __restrict__ Q, int ldq, int64_t nq, int k,
-                         const int32_t* __restrict__ qk, const int32_t* __restrict__ qls,
-                         const int32_t* __restrict__ from, int ldo, SearchLayout lay, int32_t* __restrict__ out_ids,
-                         float* __restrict__ out_d2, unsigned long long* __restrict__ work) {
+             const int32_t* __restrict__ deg, int R, const int32_t* __restrict__ nav, int n_nav,
+             const float* __restrict__ Q, int ldq, int64_t nq, int k, int ls,
+             const int32_t* __restrict__ qk, const int32_t* __restrict__ qls,
+             const int32_t* __restrict__ from, int ldo, SearchLayout lay,
+             int32_t* __restrict__ out_ids, float* __restrict__ out_d2,
+             unsigned long long* __restrict__ work) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
+  constexpr bool BYTES = std::is_same<T, uint8_t>::value;
+  constexpr int NR = BYTES ? 2 : 1;  // rows per team at once: 16 or 8 rows per warp
+  constexpr int PIECES = 4;          // of 32 neighbours (R <= 128)
   const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = lane_id();
-  const int team = lane >> 3, tl = lane & 7;
-  const int LsCap = lay.Ls;
+  const int team = lane >> 2, tl = lane & 3;
   unsigned char* base = sm_raw + (size_t)warp * lay.per_warp();
-  uint64_t* pA0 = (uint64_t*)base;
-  uint64_t* pB0 = pA0 + LsCap;
-  unsigned char* fA0 = (unsigned char*)(pB0 + LsCap);
-  unsigned char* fB0 = fA0 + LsCap;
-  uint64_t* newk = (uint64_t*)(base + 2 * lay.pool_bytes() + (((size_t)2 * LsCap + 15) & ~(size_t)15));
-  float* qs = (float*)(newk + lay.RP);
-  int32_t* cache = (int32_t*)(qs + ld);
+  uint64_t* pool = (uint64_t*)base;
+  uint64_t* newk = pool + lay.Ls;                        // [RP] ids, then keys
+  uint64_t* tmp = newk + lay.RP;                         // [32]
+  float* qs = (float*)(tmp + 32);                        // [ld]
+  uint32_t* qw = (uint32_t*)(qs + ld);                   // the query's bytes, if integer 0..255
+  int32_t* cache = (int32_t*)((unsigned char*)qw + (((size_t)ld + 15) & ~(size_t)15));
   const int hcap = 1 << lay.log2h;
-  uint32_t* qw = (uint32_t*)(cache + hcap);  // the query's bytes, when it is integer 0..255
-  const int ld4 = ld >> 2;
-  (void)d;
 
   for (int64_t qi = (int64_t)blockIdx.x * wpb + warp; qi < nq; qi += (int64_t)gridDim.x * wpb) {
-    // per-query pool size and result count (a batch may mix them; the layout is sized for
-    // the largest pool)
-    const int Ls = qls ? qls[qi] : LsCap;
+    // per-query pool size and result count (a batch may mix them; the layout holds the
+    // largest pool)
+    const int Ls = qls ? qls[qi] : ls;
     const int kq = qk ? qk[qi] : k;
-    uint64_t* pA = pA0;
-    uint64_t* pB = pB0;
-    unsigned char* fA = fA0;
-    unsigned char* fB = fB0;
     const float* qg = Q + qi * ldq;
     for (int t = lane; t < ld; t += 32) qs[t] = t < d ? qg[t] : 0.f;
-    for (int t = lane; t < hcap; t += 32) cache[t] = -1;
+    for (int t = lane * 4; t < hcap; t += 128) *(int4*)(cache + t) = make_int4(-1, -1, -1, -1);
     __syncwarp();
     bool qint = false;
     int q2 = 0;
-    if constexpr (std::is_same<T, uint8_t>::value) {
+    if constexpr (BYTES) {
       bool ok = true;
       int sq = 0;
       for (int t = lane; t < ld; t += 32) {
@@ -333,7 +369,7 @@ __global__ void __launch_bounds__(256, 3)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
         q2 = sq;
-        for (int w = lane; w < ld4; w += 32)
+        for (int w = lane; w < ld >> 2; w += 32)
           qw[w] = (uint32_t)qs[4 * w] | ((uint32_t)qs[4 * w + 1] << 8) |
                   ((uint32_t)qs[4 * w + 2] << 16) | ((uint32_t)qs[4 * w + 3] << 24);
         __syncwarp();
@@ -343,197 +379,102 @@ __global__ void __launch_bounds__(256, 3)
     // entry: the nearest navigating node by (d2, id), or the query's own start node
     uint64_t best = KEY_NONE;
     const int32_t* starts = from ? from + qi : nav;
-    for (int s0 = 0; s0 < n_nav; s0 += 4) {
-      const int s = s0 + team;
-      const bool valid = s < n_nav;
-      const int32_t id = valid ? starts[s] : 0;
-      const float dd = team8_dist_q(qs, X + (int64_t)id * ld, ld4, tl, valid);
-      const uint64_t key = valid ? make_key(dd, id) : KEY_NONE;
+    for (int s0 = 0; s0 < n_nav; s0 += 8) {
+      const bool valid[1] = {s0 + team < n_nav};
+      const int32_t id[1] = {valid[0] ? starts[s0 + team] : 0};
+      float dd[1];
+      team4_dist_q<T, 1>(qs, X, ld, id, valid, tl, dd);
+      const uint64_t key = valid[0] ? pool_key(dd[0], id[0]) : KEY_NONE;
       best = key < best ? key : best;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      uint64_t other = __shfl_xor_sync(0xffffffffu, best, o);
+      const uint64_t other = __shfl_xor_sync(0xffffffffu, best, o);
       best = other < best ? other : best;
     }
+    Pool S;
+    S.init(pool, best, Ls);
     if (lane == 0) {
-      pA[0] = best;
-      fA[0] = 0;
-      const int32_t e = key_id(best);
+      const int32_t e = pool_id_of(best);
       cache[((uint32_t)e * 2654435761u) >> (32 - lay.log2h)] = e;
     }
-    int s = 1;
     unsigned long long w_exp = 0, w_dist = (unsigned long long)n_nav, w_adj = 0;
     __syncwarp();
 
+    // a node's row and degree (entries past the degree are dropped when it is expanded)
+    int32_t row[PIECES];
+    int dg = 0;
+    auto fetch = [&](int32_t node) {
+      dg = deg[node];
+#pragma unroll
+      for (int c = 0; c < PIECES; ++c)
+        row[c] = c * 32 + lane < R ? adj[(int64_t)node * R + c * 32 + lane] : -1;
+    };
+    int32_t have = -1;  // the node whose row is in the registers
     for (;;) {
-      int p = -1;
-      for (int c = 0; c < s; c += 32) {
-        const int idx = c + lane;
-        const unsigned bal = __ballot_sync(0xffffffffu, idx < s && !fA[idx]);
-        if (bal) {
-          p = c + __ffs(bal) - 1;
-          break;
-        }
-      }
-      if (p < 0) break;
-      const int32_t node = key_id(pA[p]);
-      __syncwarp();
-      if (lane == 0) fA[p] = 1;
-      const int dg = deg[node];
+      int32_t ahead;
+      const int32_t node = S.take(ahead);
+      if (node < 0) break;
+      if (node != have) fetch(node);
       int cnt = 0;
-      for (int c = 0; c < dg; c += 32) {
-        const int t = c + lane;
-        bool fresh = false;
-        int32_t id = -1;
-        if (t < dg) {
-          id = adj[(int64_t)node * R + t];
-          const uint32_t slot = ((uint32_t)id * 2654435761u) >> (32 - lay.log2h);
-          if (cache[slot] != id) {
-            cache[slot] = id;
-            fresh = true;
+      const int dgn = dg;
+#pragma unroll
+      for (int c = 0; c < PIECES; ++c) {
+        if (c * 32 < dgn) {
+          bool fresh = false;
+          const int32_t id = row[c];
+          if (c * 32 + lane < dgn) {
+            const uint32_t slot = ((uint32_t)id * 2654435761u) >> (32 - lay.log2h);
+            if (cache[slot] != id) {
+              cache[slot] = id;
+              fresh = true;
+            }
           }
+          const unsigned bal = __ballot_sync(0xffffffffu, fresh);
+          if (fresh) newk[cnt + __popc(bal & lanemask_lt())] = (uint64_t)(uint32_t)id;
+          cnt += __popc(bal);
         }
-        const unsigned bal = __ballot_sync(0xffffffffu, fresh);
-        if (fresh) newk[cnt + __popc(bal & lanemask_lt())] = (uint64_t)(uint32_t)id;
-        cnt += __popc(bal);
       }
+      have = ahead;
+      if (ahead >= 0) fetch(ahead);
       ++w_exp;
-      w_adj += (unsigned long long)dg;
+      w_adj += (unsigned long long)dgn;
       w_dist += (unsigned long long)cnt;
       __syncwarp();
-      constexpr int NR = RowsPerTeam<T>::value;
-      for (int t0 = 0; t0 < cnt; t0 += 4 * NR) {
+      for (int t0 = 0; t0 < cnt; t0 += 8 * NR) {
         int32_t ir[NR];
         bool vr[NR];
         float dd[NR];
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-          const int t = t0 + 4 * r + team;
+          const int t = t0 + 8 * r + team;
           vr[r] = t < cnt;
-          ir[r] = vr[r] ? key_id(newk[t]) : 0;
+          ir[r] = vr[r] ? (int32_t)(uint32_t)newk[t] : 0;
         }
-        if constexpr (std::is_same<T, uint8_t>::value) {
+        if constexpr (BYTES) {
           if (qint)
-            team8_distN_qi<NR>(qw, X, ld, ir, vr, ld4, tl, q2, dd);
+            team4_dist_qi<NR>(qw, X, ld, ir, vr, tl, q2, dd);
           else
-            team8_distN_q<T, NR>(qs, X, ld, ir, vr, ld4, tl, dd);
+            team4_dist_q<T, NR>(qs, X, ld, ir, vr, tl, dd);
         } else {
-          team8_distN_q<T, NR>(qs, X, ld, ir, vr, ld4, tl, dd);
+          team4_dist_q<T, NR>(qs, X, ld, ir, vr, tl, dd);
         }
         __syncwarp();
         if (tl == 0) {
 #pragma unroll
           for (int r = 0; r < NR; ++r)
-            if (vr[r]) newk[t0 + 4 * r + team] = make_key(dd[r], ir[r]);
+            if (vr[r]) newk[t0 + 8 * r + team] = pool_key(dd[r], ir[r]);
         }
       }
       __syncwarp();
-      if (cnt <= 64) {
-        // one or two new keys per lane (element e * 32 + lane), sorted in registers; one
-        // binary search in S gives both the duplicate test and the key's place in the merge
-        uint64_t b[2];
-        b[0] = lane < cnt ? newk[lane] : KEY_NONE;
-        b[1] = lane + 32 < cnt ? newk[lane + 32] : KEY_NONE;
-        if (cnt <= 32)
-          b[0] = warp_bitonic32(b[0], lane);
-        else
-          warp_bitonic64(b, lane);
-        int r[2] = {0, 0}, j[2];
-        bool keep[2] = {false, false};
-        int kept = 0;
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          if (e * 32 + lane < cnt) {
-            r[e] = count_less(pA, s, b[e]);
-            keep[e] = !(r[e] < s && pA[r[e]] == b[e]);
-          }
-          const unsigned bal = __ballot_sync(0xffffffffu, keep[e]);
-          j[e] = kept + __popc(bal & lanemask_lt());
-          kept += __popc(bal);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-          if (keep[e]) newk[j[e]] = b[e];
-        __syncwarp();
-        for (int i = lane; i < s; i += 32) {
-          const uint64_t a = pA[i];
-          const int pos = i + count_less(newk, kept, a);
-          if (pos < Ls) {
-            pB[pos] = a;
-            fB[pos] = fA[i];
-          }
-        }
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          if (keep[e] && j[e] + r[e] < Ls) {
-            pB[j[e] + r[e]] = b[e];
-            fB[j[e] + r[e]] = 0;
-          }
-        }
-        s = s + kept < Ls ? s + kept : Ls;
-        __syncwarp();
-        uint64_t* tp = pA;
-        pA = pB;
-        pB = tp;
-        unsigned char* tf = fA;
-        fA = fB;
-        fB = tf;
-        continue;
-      }
-      int cp = 1;
-      while (cp < cnt) cp <<= 1;
-      for (int t = cnt + lane; t < cp; t += 32) newk[t] = KEY_NONE;
+      for (int c = 0; c < cnt; c += 32)
+        S.merge(c + lane < cnt ? newk[c + lane] : KEY_NONE, tmp);
       __syncwarp();
-      warp_sort_keys(newk, cp);
-      // drop keys already in S (same id => same key), compacting in place
-      int kept = 0;
-      for (int c = 0; c < cnt; c += 32) {
-        const int j = c + lane;
-        uint64_t b = KEY_NONE;
-        bool keep = false;
-        if (j < cnt) {
-          b = newk[j];
-          const int r = count_less(pA, s, b);
-          keep = !(r < s && pA[r] == b);
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, keep);
-        __syncwarp();
-        if (keep) newk[kept + __popc(bal & lanemask_lt())] = b;
-        kept += __popc(bal);
-        __syncwarp();
-      }
-      // merge S and the new keys into the other buffer, cut at Ls
-      for (int i = lane; i < s; i += 32) {
-        const uint64_t a = pA[i];
-        const int pos = i + count_less(newk, kept, a);
-        if (pos < Ls) {
-          pB[pos] = a;
-          fB[pos] = fA[i];
-        }
-      }
-      for (int j = lane; j < kept; j += 32) {
-        const uint64_t b = newk[j];
-        const int pos = j + count_less(pA, s, b);
-        if (pos < Ls) {
-          pB[pos] = b;
-          fB[pos] = 0;
-        }
-      }
-      s = s + kept < Ls ? s + kept : Ls;
-      __syncwarp();
-      uint64_t* tp = pA;
-      pA = pB;
-      pB = tp;
-      unsigned char* tf = fA;
-      fA = fB;
-      fB = tf;
     }
     for (int t = lane; t < ldo; t += 32) {
-      const bool v = t < s && t < kq;
-      out_ids[qi * ldo + t] = v ? key_id(pA[t]) : -1;
-      if (out_d2) out_d2[qi * ldo + t] = v ? key_dist(pA[t]) : __int_as_float(0x7f800000);
+      const bool v = t < S.s && t < kq;
+      out_ids[qi * ldo + t] = v ? pool_id_of(pool[t]) : -1;
+      if (out_d2) out_d2[qi * ldo + t] = v ? key_dist(pool[t]) : __int_as_float(0x7f800000);
     }
     if (work && lane == 0) {
       atomicAdd(work, w_exp);
@@ -562,14 +503,24 @@ void rows_to_u8(const float* X, int ld, int d, int64_t n, uint8_t* out, cudaStre
              (const float4*)X, n4, (uchar4*)out);
 }
 
+// ls: the pool size, or the largest one of qls.  Warps per block: eight, fewer where there are
+// too few queries to give every SM a block of eight (a query alone on an SM runs without the
+// others' instructions in its way).
 template <typename T>
 static void launch_search(const T* X, int ld, int d, const int32_t* adj, const int32_t* deg, int R,
                           const int32_t* nav, int n_nav, const float* Q, int ldq, int64_t nq, int k,
-                          const int32_t* qk, const int32_t* qls, const int32_t* from, int ldo,
-                          SearchLayout lay, int wpb,
-                          int32_t* out_ids, float* out_d2, unsigned long long* work,
-                          cudaStream_t st) {
+                          int ls, const int32_t* qk, const int32_t* qls, const int32_t* from,
+                          int ldo, int log2h, int32_t* out_ids, float* out_d2,
+                          unsigned long long* work, cudaStream_t st) {
+  SearchLayout lay;
+  lay.Ls = (ls + 1) & ~1;
+  lay.RP = (R + 31) & ~31;
+  lay.ld = ld;
+  lay.log2h = log2h;
+  int wpb = work ? 2 : 8;
+  wpb = (int)std::min<int64_t>(wpb, std::max<int64_t>(1, ceil_div(nq, num_sms())));
   while (lay.per_warp() * wpb > 200 * 1024 && lay.log2h > 8) --lay.log2h;
+  while (lay.per_warp() * wpb > 200 * 1024 && wpb > 1) wpb >>= 1;
   const size_t smem = lay.per_warp() * wpb;
   SSG_REQUIRE(smem <= 220 * 1024, SSG_EINVAL, "search: L_search and d too large for shared memory");
   ensure_smem((const void*)k_search<T>, smem);
@@ -577,28 +528,25 @@ static void launch_search(const T* X, int ld, int d, const int32_t* adj, const i
   SSG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_search<T>, wpb * 32, smem));
   const int64_t want = ceil_div(nq, wpb);
   const int grid = (int)std::min<int64_t>(want, (int64_t)std::max(1, blocks_per_sm) * num_sms());
-  SSG_LAUNCH(k_search<T>, grid, wpb * 32, smem, st, X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq,
-             k, qk, qls, from, ldo, lay, out_ids, out_d2, work);
+  SSG_LAUNCH(k_search<T>, grid, wpb * 32, smem, st, X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k,
+             ls, qk, qls, from, ldo, lay, out_ids, out_d2, work);
 }
+
+// A 1,024-entry visited cache: its size only sets how often a distance is taken again, and a
+// larger one costs warps per SM.
+constexpr int CACHE_LOG2 = 10;
 
 void search_run_mixed(const float* X, const uint8_t* X8, int ld, int d, const int32_t* adj,
                       const int32_t* deg, int R, const int32_t* nav, int n_nav, const float* Q,
                       int ldq, int64_t nq, const int32_t* qk, const int32_t* qls, int ls_max,
                       int ldo, int32_t* out_ids, float* out_d2, cudaStream_t st) {
   if (nq == 0) return;
-  SearchLayout lay;
-  lay.Ls = ls_max;
-  lay.RP = std::max(32, next_pow2(R));
-  lay.ld = ld;
-  // 8 warps per block and a 1,024-entry visited cache: 24 warps per SM (the register
-  // limit) keep more row gathers in flight than a larger cache would save
-  lay.log2h = 10;
   if (X8)
-    launch_search(X8, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, 0, qk, qls, nullptr, ldo, lay, 8,
-                  out_ids, out_d2, (unsigned long long*)nullptr, st);
+    launch_search(X8, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, 0, ls_max, qk, qls, nullptr, ldo,
+                  CACHE_LOG2, out_ids, out_d2, (unsigned long long*)nullptr, st);
   else
-    launch_search(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, 0, qk, qls, nullptr, ldo, lay, 8, out_ids,
-                  out_d2, (unsigned long long*)nullptr, st);
+    launch_search(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, 0, ls_max, qk, qls, nullptr, ldo,
+                  CACHE_LOG2, out_ids, out_d2, (unsigned long long*)nullptr, st);
 }
 
 void search_run(const float* X, const uint8_t* X8, int ld, int d, int64_t n, const int32_t* adj,
@@ -607,36 +555,28 @@ void search_run(const float* X, const uint8_t* X8, int ld, int d, int64_t n, con
                 cudaStream_t st, unsigned long long* work) {
   (void)n;
   if (nq == 0) return;
-  SearchLayout lay;
-  lay.Ls = Ls;
-  lay.RP = std::max(32, next_pow2(R));
-  lay.ld = ld;
-  // 8 warps per block and a 1,024-entry visited cache: 24 warps per SM (the register
-  // limit) keep more row gathers in flight than a larger cache would save.  A call that
-  // counts the work takes a 16,384-entry cache instead, so that its distance count is
-  // Alg. 1's (each node once) and not inflated by recomputations after cache evictions.
-  lay.log2h = work ? 14 : 10;
-  const int wpb = work ? 2 : 8;
+  // a call that counts the work takes a 16,384-entry cache, so that its distance count is
+  // Alg. 1's (each node once) and not inflated by recomputations after cache evictions
+  const int log2h = work ? 14 : CACHE_LOG2;
   if (X8)
-    launch_search(X8, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, (const int32_t*)nullptr,
-                  (const int32_t*)nullptr, nullptr, k, lay, wpb, out_ids, out_d2, work, st);
+    launch_search(X8, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, Ls, (const int32_t*)nullptr,
+                  (const int32_t*)nullptr, nullptr, k, log2h, out_ids, out_d2, work, st);
   else
-    launch_search(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, (const int32_t*)nullptr,
-                  (const int32_t*)nullptr, nullptr, k, lay, wpb, out_ids, out_d2, work, st);
+    launch_search(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, Ls, (const int32_t*)nullptr,
+                  (const int32_t*)nullptr, nullptr, k, log2h, out_ids, out_d2, work, st);
 }
 
 bool search_from(const float* X, int ld, int d, const int32_t* adj, const int32_t* deg, int R,
                  const int32_t* from, const float* Q, int ldq, int64_t nq, int Ls, int32_t* out_ids,
                  cudaStream_t st) {
   SearchLayout lay;
-  lay.Ls = Ls;
-  lay.RP = std::max(32, next_pow2(R));
+  lay.Ls = Ls + 1;
+  lay.RP = (R + 31) & ~31;
   lay.ld = ld;
-  lay.log2h = 10;
-  const int wpb = 1;  // few queries: a block, and an SM, each
+  lay.log2h = 8;
   if (lay.per_warp() > 200 * 1024) return false;
-  launch_search(X, ld, d, adj, deg, R, from, 1, Q, ldq, nq, 1, (const int32_t*)nullptr,
-                (const int32_t*)nullptr, from, 1, lay, wpb, out_ids, (float*)nullptr,
+  launch_search(X, ld, d, adj, deg, R, from, 1, Q, ldq, nq, 1, Ls, (const int32_t*)nullptr,
+                (const int32_t*)nullptr, from, 1, CACHE_LOG2, out_ids, (float*)nullptr,
                 (unsigned long long*)nullptr, st);
   return true;
 }
