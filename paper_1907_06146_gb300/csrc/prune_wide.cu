@@ -10,13 +10,20 @@
 //      it would take if every candidate before it in the window were kept, and tests it
 //      against the node's kept vectors as they stood when the window began (four dot
 //      products at a time, stopping at the first definite conflict);
-//   2. after one barrier, warp 0 settles the window in candidate order: a candidate that
-//      passed step 1 is also tested against the candidates of this window kept before it,
-//      then kept (its vector moved down to the next kept slot) or dropped, until R are
-//      kept.
+//   2. after one barrier (and only if some candidate of the window survived), every survivor is
+//      tested against the window's earlier survivors in their slots, all warps at once;
+//   3. after another, warp 0 settles the window in candidate order from those verdicts: a
+//      candidate that conflicts with none kept is kept (its vector moved down to the next kept
+//      slot), until R are kept.
 // The kept vectors sit in the block's shared memory (the first `cap` of them; the rest in
-// a device slot of the block, which stays in L2).  So the eight warps run eight
-// independent chains of dot products and meet twice per window, not once per candidate.
+// a device slot of the block, which stays in L2).  So the eight warps run eight independent
+// chains of dot products and meet once per window without a survivor, else four times.  Bound
+// by the latencies of those chains (a window's load, a round of four dot products, a barrier):
+// rows of up to 256 values take four blocks per SM and load a window ahead, the lengths' square
+// roots are taken once per vector, and the cosine's quotient is a product.  200,000 x 128, L =
+// 200, R = 32: 26.9 -> 19.2 ms; 100,000 x 960, L = 500, R = 70: 102 -> 90 ms, and the reverse
+// merge's short lists, most of which survive, 31 -> 21 ms (warp 0 used to take the survivors'
+// dot products alone, one after another).
 // The decisions are those of the warp prune: the fp32 cosine decides outside a margin that
 // bounds its rounding error for any summation order; the rest, and zero-length edges, are
 // re-taken in fp64 from the original vectors.  Those fp64 dot products are summed by the
@@ -24,6 +31,8 @@
 // more than the two summation orders can move it for any d up to 4,096 -- the three dot
 // products are re-taken in coordinate order, so every decision is the one the
 // coordinate-order fp64 rule takes.
+#include <type_traits>
+
 #include "common.cuh"
 #include "graph_dev.cuh"
 #include "knn.cuh"
@@ -64,11 +73,12 @@ __host__ __device__ inline WideLayout wide_layout(int d, int R, int cap) {
   WideLayout L;
   L.xs = 0;
   L.V = L.xs + row;                          // cap kept vectors
-  L.gkk = L.V + (size_t)cap * row;           // [R1a] fp32 |c_k - x|^2
+  L.gkk = L.V + (size_t)cap * row;           // [R1a] fp32 |c_k - x|
   L.g64 = L.gkk + R1a * 4;                   // [R1a] fp64 |c_k - x|^2 (< 0: not computed)
   L.kid = L.g64 + R1a * 8;                   // [R1a] kept ids
-  L.wmeta = L.kid + R1a * 4;                 // per window slot: |v|^2, id, verdict, near count
-  L.nlist = L.wmeta + 4 * PW_WARPS * 4;      // [PW_WARPS][R1a] kept vectors to re-test in fp64
+  L.wmeta = L.kid + R1a * 4;                 // per window slot: |v|, id, verdict, near count,
+                                             // conflicts and near ones within the window
+  L.nlist = L.wmeta + 6 * PW_WARPS * 4;      // [PW_WARPS][R1a] kept vectors to re-test in fp64
   L.total = L.nlist + PW_WARPS * R1a * 4;
   return L;
 }
@@ -96,14 +106,15 @@ __device__ __forceinline__ float dot4(float4 a, float4 b, float s) {
   return fmaf(a.w, b.w, s);
 }
 
-// fp32 angle test of one pair from its centred dot product g and squared lengths:
-// 2 = definite conflict, 1 = to be re-taken in fp64, 0 = no conflict.
-__device__ __forceinline__ int angle_test32(float g, float gjj, float gk, float cosA32,
-                                            float margin) {
-  if (gjj == 0.f || gk == 0.f) return 1;
-  const float c = g / (sqrtf(gjj) * sqrtf(gk));
-  if (c > cosA32 + margin) return 2;
-  return c >= cosA32 - margin ? 1 : 0;
+// fp32 angle test of one pair from its centred dot product g and the two lengths (square roots
+// of the squared sums): 2 = definite conflict, 1 = to be re-taken in fp64, 0 = no conflict.
+// hi, lo = cos(alpha) + and - the margin; the comparison with the product of the lengths in
+// place of a quotient costs two roundings of the margin's twenty to spare.
+__device__ __forceinline__ int angle_test32(float g, float sj, float sk, float hi, float lo) {
+  const float p = sj * sk;
+  if (p == 0.f) return 1;
+  if (g > hi * p) return 2;
+  return g >= lo * p ? 1 : 0;
 }
 
 // One node i of a (a.len, a.cand, ...) by the whole block.  NVR: float4 columns of the
@@ -121,10 +132,12 @@ __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, u
   float* gkk = (float*)(smw + Ly.gkk);
   double* g64 = (double*)(smw + Ly.g64);
   int32_t* kid = (int32_t*)(smw + Ly.kid);
-  float* wg = (float*)(smw + Ly.wmeta);                  // [8] |v|^2 of the window's vectors
+  float* wg = (float*)(smw + Ly.wmeta);                  // [8] |v| of the window's vectors
   int32_t* wid = (int32_t*)(wg + PW_WARPS);              // [8] their ids
   int* wdead = (int*)(wid + PW_WARPS);                   // [8] definite conflict in step 1
   int* wnn = wdead + PW_WARPS;                           // [8] fp64 re-tests listed
+  uint32_t* wconf = (uint32_t*)(wnn + PW_WARPS);         // [8] bit q: definite conflict with
+  uint32_t* wnear = wconf + PW_WARPS;                    // window slot q; or too near to say
   int* nlist = (int*)(smw + Ly.nlist);                   // [8][R1a]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   auto kept_row = [&](int k) -> float* {
@@ -139,19 +152,65 @@ __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, u
     for (int f = tid; f < nq4; f += PW_THREADS) ((float4*)xs)[f] = __ldg((const float4*)xg + f);
     __syncthreads();
     int kept = 0;  // the same in every thread
+    const float hi = a.cosA32 + a.margin, lo = a.cosA32 - a.margin;
+    // short rows: the warp's next candidate's row loads while the current window is tested, its
+    // id a window before that (rows of more than 256 values have no registers to spare for it)
+    constexpr bool AHEAD = NVR <= 2;
+    float4 ahead[AHEAD ? NVR : 1];
+    auto fetch = [&](int32_t j, float4* o) {
+      const float4* c4 = (const float4*)(a.X + (int64_t)j * a.ld);
+#pragma unroll
+      for (int r = 0; r < NVR; ++r) {
+        const int f = lane + 32 * r;
+        o[r] = f < nq4 ? __ldg(c4 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    };
+    int32_t j1 = warp < len ? cand[warp] : -1;
+    int32_t j2 = warp + PW_WARPS < len ? cand[warp + PW_WARPS] : -1;
+    if (AHEAD && j1 >= 0) fetch(j1, ahead);
     for (int t0 = 0; t0 < len && kept < a.R; t0 += PW_WARPS) {
       // ---- step 1: warp w takes candidate t0 + w against the kept vectors 0 .. kept-1
       const int t = t0 + warp;
-      if (t < len) {
-        const int32_t j = cand[t];
-        const float4* c4 = (const float4*)(a.X + (int64_t)j * a.ld);
-        const float4* xs4 = (const float4*)xs;
-        float4 v[NVR];
+      bool alive = false;
+      float4 v[NVR];
+      float sj = 0.f;
+      // four dot products of v with the rows w0 .. w3, reduced together: lanes 8u .. 8u+7 end
+      // up holding dot product u
+      auto dots = [&](const float4* w0, const float4* w1, const float4* w2, const float4* w3) -> float {
+        float g0 = 0.f, g1 = 0.f, g2 = 0.f, g3 = 0.f;
 #pragma unroll
         for (int r = 0; r < NVR; ++r) {
           const int f = lane + 32 * r;
-          v[r] = f < nq4 ? __ldg(c4 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+          if (f < nq4) {
+            g0 = dot4(v[r], w0[f], g0);
+            g1 = dot4(v[r], w1[f], g1);
+            g2 = dot4(v[r], w2[f], g2);
+            g3 = dot4(v[r], w3[f], g3);
+          }
         }
+        const bool hi16 = (lane & 16) != 0, hi8 = (lane & 8) != 0;
+        const float r0 = __shfl_xor_sync(0xffffffffu, hi16 ? g0 : g2, 16);
+        const float r1 = __shfl_xor_sync(0xffffffffu, hi16 ? g1 : g3, 16);
+        const float h0 = (hi16 ? g2 : g0) + r0, h1 = (hi16 ? g3 : g1) + r1;
+        float g = (hi8 ? h1 : h0) + __shfl_xor_sync(0xffffffffu, hi8 ? h0 : h1, 8);
+        g += __shfl_xor_sync(0xffffffffu, g, 4);
+        g += __shfl_xor_sync(0xffffffffu, g, 2);
+        g += __shfl_xor_sync(0xffffffffu, g, 1);
+        return g;
+      };
+      const int mine = lane >> 3;
+      if (t < len) {
+        const int32_t j = j1;
+        const float4* xs4 = (const float4*)xs;
+        if (AHEAD) {
+#pragma unroll
+          for (int r = 0; r < NVR; ++r) v[r] = ahead[AHEAD ? r : 0];
+          if (j2 >= 0) fetch(j2, ahead);
+        } else {
+          fetch(j, v);
+        }
+        j1 = j2;
+        j2 = t + 2 * PW_WARPS < len ? cand[t + 2 * PW_WARPS] : -1;
         float part = 0.f;
         float4* slot = (float4*)kept_row(kept + warp);
 #pragma unroll
@@ -164,37 +223,15 @@ __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, u
           }
           part = dot4(v[r], v[r], part);
         }
-        const float gjj = warp_sum(part);
+        sj = sqrtf(warp_sum(part));
         int dead = 0, nn = 0;
-        // four kept vectors per round; the four sums are reduced together (lanes 8u .. 8u+7
-        // end up holding dot product u)
-        const int mine = ((lane >> 4) & 1) * 2 + ((lane >> 3) & 1);
         for (int k0 = 0; k0 < kept && !dead; k0 += 4) {
           const int kn = min(4, kept - k0);
           const float4* w0 = (const float4*)kept_row(k0);
-          const float4* w1 = kn > 1 ? (const float4*)kept_row(k0 + 1) : w0;
-          const float4* w2 = kn > 2 ? (const float4*)kept_row(k0 + 2) : w0;
-          const float4* w3 = kn > 3 ? (const float4*)kept_row(k0 + 3) : w0;
-          float g0 = 0.f, g1 = 0.f, g2 = 0.f, g3 = 0.f;
-#pragma unroll
-          for (int r = 0; r < NVR; ++r) {
-            const int f = lane + 32 * r;
-            if (f < nq4) {
-              g0 = dot4(v[r], w0[f], g0);
-              g1 = dot4(v[r], w1[f], g1);
-              g2 = dot4(v[r], w2[f], g2);
-              g3 = dot4(v[r], w3[f], g3);
-            }
-          }
-          const bool hi16 = (lane & 16) != 0, hi8 = (lane & 8) != 0;
-          const float r0 = __shfl_xor_sync(0xffffffffu, hi16 ? g0 : g2, 16);
-          const float r1 = __shfl_xor_sync(0xffffffffu, hi16 ? g1 : g3, 16);
-          const float h0 = (hi16 ? g2 : g0) + r0, h1 = (hi16 ? g3 : g1) + r1;
-          float g = (hi8 ? h1 : h0) + __shfl_xor_sync(0xffffffffu, hi8 ? h0 : h1, 8);
-          g += __shfl_xor_sync(0xffffffffu, g, 4);
-          g += __shfl_xor_sync(0xffffffffu, g, 2);
-          g += __shfl_xor_sync(0xffffffffu, g, 1);
-          const int res = mine < kn ? angle_test32(g, gjj, gkk[k0 + mine], a.cosA32, a.margin) : 0;
+          const float g = dots(w0, kn > 1 ? (const float4*)kept_row(k0 + 1) : w0,
+                               kn > 2 ? (const float4*)kept_row(k0 + 2) : w0,
+                               kn > 3 ? (const float4*)kept_row(k0 + 3) : w0);
+          const int res = mine < kn ? angle_test32(g, sj, gkk[k0 + mine], hi, lo) : 0;
           if (__any_sync(0xffffffffu, res == 2)) {
             dead = 1;
           } else {
@@ -207,35 +244,62 @@ __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, u
           }
         }
         if (lane == 0) {
-          wg[warp] = gjj;
+          wg[warp] = sj;
           wid[warp] = j;
           wdead[warp] = dead;
           wnn[warp] = nn;
         }
+        alive = !dead;
+      }
+      // most windows behind the first ones have no survivor: nothing to settle
+      if (!__syncthreads_or(alive)) continue;
+      // ---- step 2: every survivor against the window's earlier survivors (their slots)
+      if (alive) {
+        uint32_t conf = 0u, near = 0u;
+        for (int q0 = 0; q0 < warp; q0 += 4) {
+          bool on[4];
+          bool some = false;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            on[u] = q0 + u < warp && !wdead[q0 + u];
+            some |= on[u];
+          }
+          if (!some) continue;
+          const float4* own = (const float4*)kept_row(kept + warp);
+          const float g = dots(on[0] ? (const float4*)kept_row(kept + q0) : own,
+                               on[1] ? (const float4*)kept_row(kept + q0 + 1) : own,
+                               on[2] ? (const float4*)kept_row(kept + q0 + 2) : own,
+                               on[3] ? (const float4*)kept_row(kept + q0 + 3) : own);
+          const bool use = mine == 0 ? on[0] : mine == 1 ? on[1] : mine == 2 ? on[2] : on[3];
+          const int res = use ? angle_test32(g, sj, wg[q0 + mine], hi, lo) : 0;
+          const unsigned b2 = __ballot_sync(0xffffffffu, res == 2);
+          const unsigned b1 = __ballot_sync(0xffffffffu, res == 1);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            conf |= ((b2 >> (8 * u)) & 1u) << (q0 + u);
+            near |= ((b1 >> (8 * u)) & 1u) << (q0 + u);
+          }
+        }
+        if (lane == 0) {
+          wconf[warp] = conf;
+          wnear[warp] = near;
+        }
       }
       __syncthreads();
-      // ---- step 2: warp 0 settles the window in candidate order
+      // ---- step 3: warp 0 settles the window in candidate order
       if (warp == 0) {
         const int kept0 = kept;
         const int wend = min(PW_WARPS, len - t0);
+        uint32_t in = 0u;  // the window's kept ones (the n-th of them in kept slot kept0 + n)
+#pragma unroll 1
         for (int w = 0; w < wend && kept < a.R; ++w) {
           if (wdead[w]) continue;
-          const float gjj = wg[w];
+          const float sw = wg[w];
           const int32_t j = wid[w];
           const float4* vw = (const float4*)kept_row(kept0 + w);
-          // against the vectors kept earlier in this window (their window slots)
-          bool conflict = false;
-          int wnear = 0;  // bit q: kept vector kept0 + q to re-take in fp64
-          for (int q = 0; q < kept - kept0 && !conflict; ++q) {
-            const float4* vu = (const float4*)kept_row(kept0 + q);
-            float g = 0.f;
-            for (int f = lane; f < nq4; f += 32) g = dot4(vw[f], vu[f], g);
-            g = warp_sum(g);
-            const int r = angle_test32(g, gjj, gkk[kept0 + q], a.cosA32, a.margin);
-            if (r == 2) conflict = true;
-            else if (r == 1) wnear |= 1 << q;
-          }
-          if (!conflict && (wnn[w] > 0 || wnear)) {
+          bool conflict = (wconf[w] & in) != 0u;
+          const uint32_t wn = wnear[w] & in;    // window ones to re-take in fp64
+          if (!conflict && (wnn[w] > 0 || wn)) {
             // fp64 re-tests, kept order: first those listed in step 1, then this window's
             const float* cj = a.X + (int64_t)j * a.ld;
             const double gj = warp_cdot_f64(cj, cj, xg, a.d);
@@ -245,8 +309,8 @@ __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, u
               if (u < nl) {
                 k = nlist[w * R1a + u];
               } else {
-                if (!((wnear >> (u - nl)) & 1)) continue;
-                k = kept0 + (u - nl);
+                if (!((wn >> (u - nl)) & 1u)) continue;
+                k = kept0 + __popc(in & ((1u << (u - nl)) - 1u));
               }
               const float* ck = a.X + (int64_t)kid[k] * a.ld;
               double gk = g64[k];
@@ -274,10 +338,11 @@ __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, u
               for (int f = lane; f < nq4; f += 32) dst[f] = vw[f];
             }
             if (lane == 0) {
-              gkk[kept] = gjj;
+              gkk[kept] = sw;
               kid[kept] = j;
               out[kept] = j;
             }
+            in |= 1u << w;
             ++kept;
           }
           __syncwarp();
@@ -294,7 +359,7 @@ __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, u
 }
 
 template <int NVR>
-__global__ void __launch_bounds__(PW_THREADS) k_prune_wide(WideArgs a) {
+__global__ void __launch_bounds__(PW_THREADS, NVR <= 2 ? 4 : 2) k_prune_wide(WideArgs a) {
   extern __shared__ __align__(16) unsigned char smw[];
   const int d4 = (a.d + 3) & ~3;
   float* spill = a.Vg ? a.Vg + (size_t)blockIdx.x * (a.R + PW_WARPS - a.cap) * d4 : nullptr;
@@ -308,7 +373,7 @@ __global__ void __launch_bounds__(PW_THREADS) k_prune_wide(WideArgs a) {
 // The same over the (index, node) work items of a batch, handed out from one counter in
 // the order of items (longest pools first); each block's spill slot holds vg_stride floats.
 template <int NVR>
-__global__ void __launch_bounds__(PW_THREADS)
+__global__ void __launch_bounds__(PW_THREADS, NVR <= 2 ? 4 : 2)
     k_prune_wide_batched(const WideArgs* __restrict__ jobs, const int2* __restrict__ items,
                          int64_t nitems, unsigned long long* __restrict__ next,
                          float* __restrict__ Vg, size_t vg_stride) {
@@ -331,6 +396,21 @@ __global__ void __launch_bounds__(PW_THREADS)
 }
 
 }  // namespace
+
+// float4 columns of a vector that each lane holds, for rows of d4 values (each is a template of
+// its own: a lane's loops over columns that the rows do not have still issue).
+static int wide_nvr(int d4) { return d4 <= 128 ? 1 : d4 <= 256 ? 2 : d4 <= 512 ? 4 : 8; }
+template <class F>
+static void wide_switch(int nvr, F f) {
+  if (nvr == 1)
+    f(std::integral_constant<int, 1>());
+  else if (nvr == 2)
+    f(std::integral_constant<int, 2>());
+  else if (nvr == 4)
+    f(std::integral_constant<int, 4>());
+  else
+    f(std::integral_constant<int, 8>());
+}
 
 bool prune_wide_available(int d) { return ((d + 3) & ~3) <= 1024; }
 
@@ -364,9 +444,9 @@ void prune_wide_batched_prepare(const std::vector<PruneJob>& js, WideBatchPlan& 
     plan.vg_stride = std::max(plan.vg_stride, (size_t)(p.R + PW_WARPS - cap) * d4);
     d4max = std::max(d4max, d4);
   }
-  plan.nvr = d4max <= 512 ? 4 : 8;
-  const void* fn = plan.nvr == 4 ? (const void*)k_prune_wide_batched<4>
-                                 : (const void*)k_prune_wide_batched<8>;
+  plan.nvr = wide_nvr(d4max);
+  const void* fn = nullptr;
+  wide_switch(plan.nvr, [&](auto nvr) { fn = (const void*)k_prune_wide_batched<decltype(nvr)::value>; });
   ensure_smem(fn, plan.smem);
   int per_sm = 0;
   SSG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, PW_THREADS, plan.smem));
@@ -381,12 +461,10 @@ void prune_wide_batched_prepare(const std::vector<PruneJob>& js, WideBatchPlan& 
 void prune_wide_batched_launch(const WideBatchPlan& plan, const int2* items, int64_t nitems,
                                unsigned long long* next, cudaStream_t st) {
   const WideArgs* jobs = (const WideArgs*)plan.jobs.p;
-  if (plan.nvr == 4)
-    SSG_LAUNCH(k_prune_wide_batched<4>, plan.grid, PW_THREADS, plan.smem, st, jobs, items, nitems,
-               next, plan.Vg.p, plan.vg_stride);
-  else
-    SSG_LAUNCH(k_prune_wide_batched<8>, plan.grid, PW_THREADS, plan.smem, st, jobs, items, nitems,
-               next, plan.Vg.p, plan.vg_stride);
+  wide_switch(plan.nvr, [&](auto nvr) {
+    SSG_LAUNCH(k_prune_wide_batched<decltype(nvr)::value>, plan.grid, PW_THREADS, plan.smem, st, jobs,
+               items, nitems, next, plan.Vg.p, plan.vg_stride);
+  });
 }
 
 void prune_run_wide(const float* X, int ld, int d, int64_t n, const int32_t* cand,
@@ -400,7 +478,9 @@ void prune_run_wide(const float* X, int ld, int d, int64_t n, const int32_t* can
   SSG_REQUIRE(fixed + row <= budget, SSG_EINTERNAL, "wide prune: rows of %d values do not fit", d);
   const int cap = (int)std::min<size_t>((size_t)R + PW_WARPS, (budget - fixed) / row);
   const size_t smem = wide_layout(d, R, cap).total;
-  const void* fn = d4 <= 512 ? (const void*)k_prune_wide<4> : (const void*)k_prune_wide<8>;
+  const int nv = wide_nvr(d4);
+  const void* fn = nullptr;
+  wide_switch(nv, [&](auto nvr) { fn = (const void*)k_prune_wide<decltype(nvr)::value>; });
   ensure_smem(fn, smem);
   int per_sm = 0;
   SSG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, PW_THREADS, smem));
@@ -411,10 +491,9 @@ void prune_run_wide(const float* X, int ld, int d, int64_t n, const int32_t* can
   WideArgs a{X, ld, d, n, cand, len, stride, R, (float)cos_a,
              angle_margin_fp32(d) + (float)border, cos_a, border, adj, deg, Vg.p, cap,
              &dctr->angle_fp64, &dctr->angle_border};
-  if (d4 <= 512)
-    SSG_LAUNCH(k_prune_wide<4>, (unsigned)grid, PW_THREADS, smem, st, a);
-  else
-    SSG_LAUNCH(k_prune_wide<8>, (unsigned)grid, PW_THREADS, smem, st, a);
+  wide_switch(nv, [&](auto nvr) {
+    SSG_LAUNCH(k_prune_wide<decltype(nvr)::value>, (unsigned)grid, PW_THREADS, smem, st, a);
+  });
 }
 
 }  // namespace ssg
