@@ -59,7 +59,7 @@ typedef enum {
  *         certified against the GEMM's error bound (uncertified rows recomputed exhaustively).
  *   BF16  bf16 tcgen05 GEMM with fp32 accumulation (sm_103, d <= 4096: rows of up to 128
  *         values stay resident in shared memory, wider rows stream in 64-value chunks
- *         through 128 x 256 tiles).  On integer data
+ *         with the 256-column tiles).  On integer data
  *         that bf16 holds exactly the GEMM itself is exact.  On other data the rows are
  *         centred on the column mean before rounding, each row keeps the KS nearest by bf16
  *         distance (KS sized from a seeded sample of rows so that about 99% of rows
@@ -67,8 +67,9 @@ typedef enum {
  *         K-th exact distance lies below the KS-th bf16 distance minus the rigorous bound
  *         |d2_bf16 - d2| <= (2^-7 + ..) |x - mu| max_y |y - mu| + ..; every other row is
  *         recomputed exhaustively (counted in ssg_build_stats.n_knn_fallback_rows).  Where
- *         that band would need more than 768 candidates (high intrinsic dimension, as in
- *         the GIST-shaped data), every value goes in as a bf16 pair hi + lo (three products
+ *         that band holds more candidates than the kernel keeps (high intrinsic dimension, as
+ *         in the GIST-shaped data), or so many that the pairs are estimated to take less time
+ *         (fewer rows, shorter rows), every value goes in as a bf16 pair hi + lo (three products
  *         per coordinate, K three times as long, error about 3 * 2^-16 |x| |y| plus the
  *         fp32 accumulation), for rows of up to 1,344 values
  *         (ssg_build_stats.knn_bf16_pairs).
@@ -138,7 +139,7 @@ typedef struct {
                                prune's longest-first order, 1..1024), knn_bf16_pairs (the
                                certified bf16 kNN's operands as bf16 pairs: 1 always, 0
                                never, -1 = automatic: where the sized single-bf16 band
-                               needs more than 768 candidates), prune_wide_blocks
+                               does not fit or is estimated dearer), prune_wide_blocks
                                (blocks per SM of the block prune of rows of 330 to 1,024
                                values, 0 = automatic (2), up to 4; fewer blocks hold more
                                kept vectors in shared memory) */
@@ -363,7 +364,7 @@ ssg_status ssg_build_batched(int32_t count, const float* const* bases, const int
 /* Autotuner of ssg_build_batched's launch parameters (no paper counterpart): on the four
  * largest indices of the batch (same arguments as ssg_build_batched) it times the batched
  * prune for 2, 4 and 8 warps per block and pool-length buckets 16, 64 and 1,024 wide, and
- * the resident (256 x 128 tiles) against the streamed (128 x 256 tiles) kNN kernel for
+ * the resident against the streamed kNN kernel for
  * rows of up to 128 values, then writes the fastest choice as a tune_table file at path_out
  * (prune_warps, prune_bucket_width, knn_stream_rows).  best_ms_host (nullable, 2 entries)
  * receives the best batched-prune and kNN times.  EIO if the file cannot be written. */

@@ -81,6 +81,7 @@ struct TcExtra {
                                       // [hi | lo | hi] and B rows [lo | hi | hi] (each part
                                       // padded to 64 values), so one accumulator sums
                                       // hi.lo + lo.hi, then hi.hi (K three times as long)
+  int any_order = 0;                  // 1: the K neighbours of a row come in any order
   int prepass_tiles = 0;              // near-first self-joins: a first walk over this many
                                       // tiles gives each row an upper bound of its KS-th
                                       // distance, from which the full walk starts (0: off;

@@ -304,11 +304,10 @@ __device__ __forceinline__ void warp_fill_plain_keys(uint64_t* keys, int m,
 }
 
 // Exact order of each row's candidates and its certificate.  One warp per row r (rows:
-// compact index -> row id, null = identity).  The candidates cand[r][0, KS) come sorted by
-// their tensor-core distance cd2 (-1 padded), and only those whose cd2 lies within 2 E (plus
-// the rounding of that value) of the K-th smallest one can be among the K nearest: K
-// candidates lie at most at that K-th value plus E, any other candidate at least 2 E further
-// minus E.  Those get plain fp32 distances p, whose relative error is at most rel_plain: a
+// compact index -> row id, null = identity).  Of the candidates cand[r][0, KS) (in any order,
+// -1 padded) only those whose tensor-core distance cd2 lies within 2 E (plus the rounding of
+// that value) of the K-th smallest one can be among the K nearest: K candidates lie at most at
+// that K-th value plus E, any other candidate at least 2 E further minus E.  Those get plain fp32 distances p, whose relative error is at most rel_plain: a
 // candidate among the K nearest has p <= v (1 + rel_plain) / (1 - rel_plain) for v the K-th
 // smallest p, and the rest are dropped.  The survivors, about K of them, get compensated
 // fp32 distances, are sorted by (d2, id), and runs of near-equal values up to position K are
@@ -346,25 +345,19 @@ k_knn_cert(const float* __restrict__ A, const float* __restrict__ B, int ld, int
     const float* dr = cd2 + r * KS;
     const double nx = (double)nac[row];
     const double E = bf16_dist_bound(nx, ymax2, d, pairs);
-    double lim = __longlong_as_double(0x7ff0000000000000ll);
-    if (K <= KS && cr[K - 1] >= 0) {
-      const double aK = (double)dr[K - 1];
-      lim = aK + 2.0 * E + stream_slop(nx, aK);
-    }
     int m = 0;
     for (int c = 0; c < KS; c += 32) {
       const int t = c + lane;
       const int32_t id = t < KS ? cr[t] : -1;
-      const bool v = id >= 0 && (t < K || (double)dr[t] <= lim);
-      const unsigned bal = __ballot_sync(0xffffffffu, v);
-      if (v) keys[t] = (uint64_t)(uint32_t)id;
+      const unsigned bal = __ballot_sync(0xffffffffu, id >= 0);
+      if (id >= 0) keys[t] = make_key(dr[t], id);
       m += __popc(bal);
-      if (bal != 0xffffffffu) break;  // a prefix: sorted, padding last
+      if (bal != 0xffffffffu) break;  // padding comes last
     }
     __syncwarp();
-    if (m > K + 8) {
-      warp_fill_plain_keys<ONE>(keys, m, B, ld, xi);
-      // a value between the K-th and the (K + 8)-th smallest, by bisection over the order bits
+    // a value between the K-th and the (K + 8)-th smallest distance of the keys (more only
+    // with ties), by bisection over the order bits
+    auto kth_bound = [&]() -> float {
       uint32_t lo = 0xffffffffu, hi = 0u;
       for (int t = lane; t < m; t += 32) {
         const uint32_t k = (uint32_t)(keys[t] >> 32);
@@ -385,12 +378,15 @@ k_knn_cert(const float* __restrict__ A, const float* __restrict__ B, int ld, int
           lo = mid + 1;
         }
       }
-      const double keep = (double)order_bits_float(hi) * (1.0 + 2.1 * (double)rel_plain) + 1e-30;
+      return order_bits_float(hi);
+    };
+    // drops the keys above a distance
+    auto drop_above = [&](double lim) {
       int kept = 0;
       for (int c = 0; c < m; c += 32) {
         const int t = c + lane;
         const uint64_t key = t < m ? keys[t] : 0ull;
-        const bool v = t < m && !((double)key_dist(key) > keep);
+        const bool v = t < m && !((double)key_dist(key) > lim);
         const unsigned bal = __ballot_sync(0xffffffffu, v);
         __syncwarp();
         if (v) keys[kept + __popc(bal & lanemask_lt())] = key;
@@ -398,6 +394,14 @@ k_knn_cert(const float* __restrict__ A, const float* __restrict__ B, int ld, int
       }
       __syncwarp();
       m = kept;
+    };
+    if (m > K) {
+      const double aK = (double)kth_bound();
+      drop_above(aK + 2.0 * E + stream_slop(nx, aK));
+    }
+    if (m > K + 8) {
+      warp_fill_plain_keys<ONE>(keys, m, B, ld, xi);
+      drop_above((double)kth_bound() * (1.0 + 2.1 * (double)rel_plain) + 1e-30);
     }
     warp_fill_dist_keys(keys, m, B, ld, xi);
     int mp = 1;
@@ -513,6 +517,21 @@ static int certify(const float* A, const float* B, int ld, int d, const int32_t*
   return read_count(fbc, st);
 }
 
+// Whether bf16 pairs take less time per row than single bf16 with KS candidates: their three
+// products per coordinate against the candidates that they do without (about 1.25 K are left).
+// Seconds per row and column: 1.25e-14 per K-step of 16 values for resident rows (the epilogue's
+// 1e-13 at least), 2.4e-14 and 6e-13 once for streamed ones; per candidate 2.7e-10 to append,
+// finish and order it at short rows, doubled at 1,024 values.  Fitted to the kNN stage of both
+// (ms, single / pairs): 50,000 x 64 8.4 / 6.0, x 128 9.4 / 7.1, x 256 11.9 / 10.1; 100,000 x 96
+// 13.0 / 15.3; 200,000 x 128 34 / 49; 20,000 x 960 8.1 / 8.9, 100,000 x 960 84 (KS 740) or 63
+// (KS 563) / 72.
+static bool pairs_cheaper(int64_t nb, int d, int K, int KS) {
+  const double steps = (d + 15) / 16;
+  const double s1 = d <= 128 ? std::max(1.25e-14 * (steps + 1.0), 1e-13) : 2.4e-14 * (steps + 1.0) + 6e-13;
+  const double s3 = 2.4e-14 * (3.0 * steps + 1.0) + 6e-13;
+  return (double)nb * (s3 - s1) < (KS - 1.25 * K) * 2.7e-10 * (1.0 + d / 1024.0);
+}
+
 CertResult knn_bf16_certified(const float* A, int64_t na, int ld, const float* a_norm_raw,
                               const float* B, int64_t nb, const float* b_norm_raw, int d,
                               const DataInfo& info, int self, int K, int32_t* out_id, float* out_d2,
@@ -604,11 +623,10 @@ CertResult knn_bf16_certified(const float* A, int64_t na, int ld, const float* a
       return (int)std::ceil(h[std::max(qi, 0)] * 1.05) + 8;
     };
     int need = need_for(pairs);
-    // single bf16 too coarse for these data (its band would need more candidates than
-    // PAIRS_AT, or than the kernel keeps): bf16 pairs, three products per coordinate
-    constexpr int PAIRS_AT = 768;
+    // single bf16 too coarse for these data (its band holds more candidates than the kernel
+    // keeps), or dearer: bf16 pairs, three products per coordinate
     if (!pairs && pairs_ok && tune.bf16_pairs < 0 &&
-        (need > PAIRS_AT || need > knn_tc_max_k(d, false))) {
+        (need > knn_tc_max_k(d, false) || pairs_cheaper(nb, d, K, need))) {
       pairs = 1;
       need = need_for(1);
     }
@@ -629,6 +647,7 @@ CertResult knn_bf16_certified(const float* A, int64_t na, int ld, const float* a
   ex.prepass_tiles = tune.prepass_tiles;
   ex.stream_rows = tune.stream_rows;
   ex.pairs = pairs;
+  ex.any_order = 1;
   knn_exact_tc(A, na, ld, nac, B, nb, ld, nbc.p, d, self, KS, cid.p, cd2.p, st, gemm_timer, 0, true,
                ex);
   Scratch<int32_t> fb((size_t)na, st), fb2((size_t)na, st);
@@ -660,6 +679,7 @@ CertResult knn_bf16_certified(const float* A, int64_t na, int ld, const float* a
     ex2.qid = self ? fb.p : nullptr;
     ex2.tau_in = tau2.p;
     ex2.pairs = pairs;
+    ex2.any_order = 1;
     knn_exact_tc(Ag.p, nfb, ld, nag.p, B, nb, ld, nbc.p, d, self, KS2, cid2.p, cd22.p, st, nullptr, 0,
                  true, ex2);
     nlast = certify(Ag.p, B, ld, d, fb.p, nfb, cid2.p, cd22.p, KS2, thr2.p, nac, ymax2, pairs, K, exact_d2, out_id,

@@ -692,6 +692,7 @@ struct FinArgs {
   float* out_thresh;          // nullable: per output row, the KS-th smallest distance kept (or,
                               // with fewer kept, the final admission bound)
   uint32_t* ts_out;           // nullable: only the order bits of the KS-th largest accumulator
+  int sorted;                 // 0: the K neighbours in any order (for a caller that reorders them)
   int slots;                  // keys per warp: a power of two, at least KS
   int tcap;                   // entries of all shares at most
 };
@@ -735,6 +736,47 @@ __device__ __noinline__ void sort_out(const FinArgs& p, const uint64_t* keys, in
   }
 }
 
+// The same without the sort: the n <= KS keys that stay, in any order, less the row itself (or,
+// where it is not among KS of them, the last in order).
+__device__ __forceinline__ void raw_out(const FinArgs& p, const uint64_t* keys, int n, int64_t row) {
+  const int lane = lane_id();
+  const float INF = __int_as_float(0x7f800000);
+  const int64_t ro = p.qid ? row : (p.perm ? (int64_t)p.perm[row] : row);
+  const int32_t sid = p.qid ? p.qid[row] : (int32_t)ro;
+  uint64_t last = 0ull;
+  int drop = n;
+  for (int e = 0; e < n; e += 32) {
+    const uint64_t k = e + lane < n ? keys[e + lane] : 0ull;
+    last = k > last ? k : last;
+    if (p.self && drop == n) {
+      const unsigned m = __ballot_sync(0xffffffffu, e + lane < n && key_id(k) == sid);
+      if (m) drop = e + __ffs(m) - 1;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const uint64_t k = __shfl_xor_sync(0xffffffffu, last, o);
+    last = k > last ? k : last;
+  }
+  if (p.out_thresh && lane == 0)
+    p.out_thresh[ro] = n >= p.KS ? key_dist(last) : (p.tau_in ? p.tau_in[row] : INF);
+  if (p.self && drop == n && n >= p.KS) {
+    for (int e = 0; e < n; e += 32) {
+      const unsigned m = __ballot_sync(0xffffffffu, e + lane < n && keys[e + lane] == last);
+      if (m) {
+        drop = e + __ffs(m) - 1;
+        break;
+      }
+    }
+  }
+  const int got = drop < n ? n - 1 : n;
+  for (int t = lane; t < p.K; t += 32) {
+    const uint64_t k = t < got ? keys[t < drop ? t : t + 1] : KEY_NONE;
+    p.out_id[ro * p.K + t] = k == KEY_NONE ? -1 : key_id(k);
+    p.out_d2[ro * p.K + t] = k == KEY_NONE ? INF : key_dist(k);
+  }
+}
+
 __global__ void __launch_bounds__(128) k_knn_finish(FinArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = lane_id();
@@ -761,7 +803,7 @@ __global__ void __launch_bounds__(128) k_knn_finish(FinArgs p) {
   __syncwarp();
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
-  const int good = p.ts_out ? p.KS : p.slots;
+  const int good = p.ts_out || !p.sorted ? p.KS : p.slots;
   int n = T;  // entries <= hi
   if (T > good) {
     while (lo < hi) {
@@ -786,8 +828,8 @@ __global__ void __launch_bounds__(128) k_knn_finish(FinArgs p) {
     return;
   }
   uint32_t idmax = 0xFFFFFFFFu;
-  if (n > p.slots) {
-    // more ties at the KS-th distance than slots: those with the smallest original ids stay
+  if (n > good) {
+    // more ties at the KS-th distance than that: those with the smallest original ids stay
     int below = 0;
     for (int t = lane; t < T; t += 32) below += ob[t] < hi ? 1 : 0;
     const int need = p.KS - __reduce_add_sync(0xffffffffu, below);
@@ -832,7 +874,9 @@ __global__ void __launch_bounds__(128) k_knn_finish(FinArgs p) {
     base += c;
   }
   __syncwarp();
-  if (kept <= 32)
+  if (!p.sorted)
+    raw_out(p, keys, kept, row);
+  else if (kept <= 32)
     sort_out<1>(p, keys, kept, row);
   else if (kept <= 64)
     sort_out<2>(p, keys, kept, row);
@@ -1130,6 +1174,7 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
   f.KS = KS;
   f.K = K;
   f.self = self;
+  f.sorted = !ex.any_order;
   f.a_norm = a_norm;
   f.perm = a.perm;
   f.qid = ex.qid;
