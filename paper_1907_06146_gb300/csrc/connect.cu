@@ -157,14 +157,17 @@ __device__ __forceinline__ void warp_expand(const ConnArgs& a, uint32_t* bits, i
 // stays small.  bits: the bitmap of reached nodes (in shared or global memory).  Returns
 // (in every lane) n when every node is reached, else the node it stopped at, with
 // *why = STOP_ROW, STOP_KNN after `most` repairs, or STOP_BFS and the frontier in the state.  A repair is a chain of
-// latencies, so the next unreached node's row, out-edges and degree (which no repair before
-// its own changes) load while the current one is settled.
+// latencies, so the rows, out-edges and degrees of the next two unreached nodes (which no repair
+// before their own changes) load while the current one is settled, and the degrees of the next
+// one's row entries too (a repair changes one degree, the one it links from).
 struct RepairRow {
   static constexpr int PIECES = 4;  // of 32 entries, kept in registers
-  int32_t row[PIECES], adj[PIECES];
+  int64_t u;
+  int32_t row[PIECES], adj[PIECES], rdeg[PIECES];
   int dg;
-  __device__ __forceinline__ void fetch(const ConnArgs& a, int64_t u) {
+  __device__ __forceinline__ void fetch(const ConnArgs& a, int64_t node) {
     const int lane = lane_id();
+    u = node;
     const bool in = u < a.n;
     dg = in ? __ldcg(a.deg + u) : 0;
 #pragma unroll
@@ -174,6 +177,15 @@ struct RepairRow {
       adj[j] = in && t < a.R ? __ldcg(a.adj + u * a.R + t) : -1;
     }
   }
+  __device__ __forceinline__ void fetch_degrees(const ConnArgs& a) {
+#pragma unroll
+    for (int j = 0; j < PIECES; ++j) rdeg[j] = row[j] >= 0 ? __ldcg(a.deg + row[j]) : a.R;
+  }
+  // `v` has been linked from since fetch_degrees
+  __device__ __forceinline__ void linked(int32_t v) {
+#pragma unroll
+    for (int j = 0; j < PIECES; ++j) rdeg[j] += row[j] == v ? 1 : 0;
+  }
 };
 __device__ __noinline__ int64_t warp_knn_repairs(const ConnArgs& a, uint32_t* bits, int64_t start,
                                                  int most, int* why) {
@@ -182,9 +194,6 @@ __device__ __noinline__ int64_t warp_knn_repairs(const ConnArgs& a, uint32_t* bi
   const int lane = lane_id();
   RepairState* s = a.s;
   unsigned long long made = 0;
-  RepairRow now, next;
-  int64_t u = warp_first_unreached(bits, a.nw, a.n, start);
-  now.fetch(a, u);
   *why = 0;
   // marks v and appends it to the list, if it is unreached (v < 0: nothing)
   auto reach = [&](int32_t v, int32_t* list, int& count) {
@@ -196,32 +205,46 @@ __device__ __noinline__ int64_t warp_knn_repairs(const ConnArgs& a, uint32_t* bi
     if (fresh) list[count + __popc(bal & lanemask_lt())] = v;
     count += __popc(bal);
   };
-  while (u < a.n) {
+  // the smallest unreached node after u
+  auto after = [&](int64_t u) -> int64_t {
+    if (u >= a.n) return a.n;
+    const uint32_t w = peek(bits + (u >> 5)) | ((2u << (u & 31)) - 1u);
+    const int64_t g = w != 0xffffffffu ? (u >> 5) * 32 + __ffs(~w) - 1
+                                       : warp_first_unreached(bits, a.nw, a.n, (u >> 5) + 1);
+    return g < a.n ? g : a.n;
+  };
+  auto unreached = [&](int64_t u) {
+    return u < a.n && !((peek(bits + (u >> 5)) >> (u & 31)) & 1u);
+  };
+  RepairRow now, n1, n2;
+  now.fetch(a, warp_first_unreached(bits, a.nw, a.n, start));
+  now.fetch_degrees(a);
+  n1.fetch(a, after(now.u));
+  while (now.u < a.n) {
+    const int64_t u = now.u;
     if (made >= (unsigned long long)most) {
       *why = STOP_KNN;
       break;
     }
-    // (u's own bit is still clear, so look behind it)
-    int64_t guess = warp_first_unreached(bits, a.nw, a.n, u >> 5);
-    if (guess == u) {
-      const uint32_t w = peek(bits + (u >> 5)) | ((2u << (u & 31)) - 1u);
-      guess = w != 0xffffffffu ? (u >> 5) * 32 + __ffs(~w) - 1
-                               : warp_first_unreached(bits, a.nw, a.n, (u >> 5) + 1);
-      if (guess > a.n) guess = a.n;
-    }
-    next.fetch(a, guess);
+    n2.fetch(a, after(n1.u));
+    n1.fetch_degrees(a);
     // the row's first reached node with a free slot
     int32_t found = -1;
     int slot = 0;
-    for (int c = 0, j = 0; c < a.K && found < 0; c += 32, ++j) {
-      int32_t v = -1;
-      if (j < P) {
 #pragma unroll
-        for (int k = 0; k < P; ++k)
-          if (k == j) v = now.row[k];
-      } else if (c + lane < a.K) {
-        v = __ldg(a.knn + u * a.K + c + lane);
+    for (int j = 0; j < P; ++j) {
+      if (found < 0 && j * 32 < a.K) {
+        const int32_t v = now.row[j];
+        const unsigned bal = __ballot_sync(
+            0xffffffffu, v >= 0 && now.rdeg[j] < a.R && ((peek(bits + (v >> 5)) >> (v & 31)) & 1u));
+        if (bal) {
+          found = __shfl_sync(0xffffffffu, v, __ffs(bal) - 1);
+          slot = __shfl_sync(0xffffffffu, now.rdeg[j], __ffs(bal) - 1);
+        }
       }
+    }
+    for (int c = P * 32; c < a.K && found < 0; c += 32) {
+      const int32_t v = c + lane < a.K ? __ldg(a.knn + u * a.K + c + lane) : -1;
       const bool reached = v >= 0 && ((peek(bits + (v >> 5)) >> (v & 31)) & 1u);
       if (!__any_sync(0xffffffffu, reached)) continue;
       const int dv = reached ? __ldcg(a.deg + v) : a.R;
@@ -245,7 +268,8 @@ __device__ __noinline__ int64_t warp_knn_repairs(const ConnArgs& a, uint32_t* bi
     int32_t *fr = a.f1, *nx = a.f0;
     int fc = 0;
 #pragma unroll
-    for (int j = 0; j < P; ++j) reach(j * 32 + lane < now.dg ? now.adj[j] : -1, fr, fc);
+    for (int j = 0; j < P; ++j)
+      if (j * 32 < now.dg) reach(j * 32 + lane < now.dg ? now.adj[j] : -1, fr, fc);
     for (int c = P * 32; c < now.dg; c += 32)
       reach(c + lane < now.dg ? __ldcg(a.adj + u * a.R + c + lane) : -1, fr, fc);
     __syncwarp();
@@ -272,25 +296,29 @@ __device__ __noinline__ int64_t warp_knn_repairs(const ConnArgs& a, uint32_t* bi
       *why = STOP_BFS;
       break;
     }
-    // (u is its own guess's predecessor: the guess stands unless the traversal reached it)
-    const int64_t from = u;
-    u = guess < a.n && !((peek(bits + (guess >> 5)) >> (guess & 31)) & 1u)
-            ? guess
-            : warp_first_unreached(bits, a.nw, a.n, from >> 5);
-    if (u == guess)
-      now = next;
-    else
-      now.fetch(a, u);
+    // the traversal may have reached the nodes fetched ahead
+    if (n1.u >= a.n || unreached(n1.u)) {
+      now = n1;
+      now.linked(found);
+      if (n2.u >= a.n || unreached(n2.u))
+        n1 = n2;
+      else
+        n1.fetch(a, after(now.u));
+    } else {
+      now.fetch(a, after(u));
+      now.fetch_degrees(a);
+      n1.fetch(a, after(now.u));
+    }
   }
   if (lane == 0) s->rep_knn += made;
   __threadfence();
   __syncwarp();
-  return u;
+  return now.u;
 }
 
 // warp_knn_repairs with the bitmap in shared memory where it fits (up to 1.6M nodes): a chain
 // of dependent reads, each a shared-memory or an L2 latency.  200,000 nodes, 4,500 repairs:
-// 10.5 ms; one block that met at about ten barriers per repair took 15.5 ms.
+// 7.6 ms; one block that met at about ten barriers per repair took 15.5 ms.
 __global__ void __launch_bounds__(256) k_repair_knn(ConnArgs a, int shared_bits) {
   extern __shared__ uint32_t sbits[];
   uint32_t* bits = a.bm;
@@ -632,7 +660,7 @@ static std::vector<char> roots_reach_first(const ConnArgs& a, const int32_t* nav
   std::vector<char> ok((size_t)n_nav, 0);
   const int m = n_nav - 1;
   if (m < 1 || a.R > 128) return ok;
-  const int ls = 32;
+  const int ls = 16;
   Scratch<float> q((size_t)m * a.ld, st);
   Scratch<int32_t> from((size_t)m, st), ids((size_t)m, st);
   SSG_LAUNCH(k_repeat_row, (unsigned)m, 128, 0, st, a.X + (int64_t)nav_host[0] * a.ld, a.ld, q.p);
