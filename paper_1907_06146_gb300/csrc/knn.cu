@@ -48,7 +48,10 @@ __global__ void __launch_bounds__(256) k_row_stats(
   float mx = 0.f;
   unsigned mn = 0u;
   int bad = 0, neg = 0;
-  for (int64_t r0 = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; r0 < n;
+  // the warp's first row bounds the loop: a warp's teams leave it together, as the sums' shuffles
+  // name all its lanes
+  const int in_warp = (threadIdx.x & 31) / T;
+  for (int64_t r0 = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; r0 - in_warp < n;
        r0 += teams * STATS_U) {
     float s[STATS_U];
 #pragma unroll
