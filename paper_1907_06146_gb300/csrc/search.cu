@@ -107,6 +107,71 @@ __device__ __forceinline__ void team4_dist_q(const float* __restrict__ qs, const
   }
 }
 
+// The same for float rows, by teams of eight lanes (4 NR rows per warp): a load instruction of
+// the warp then takes whole 128-byte lines of four rows, where teams of four would take half
+// lines of eight.  The eight sums of a row are added in the same pairs, each lane handing on half
+// of its rows at every step: the distance of row team8_row<NR>(tl) is returned in lane tl.
+template <int NR>
+__device__ __forceinline__ int team8_row(int tl) {
+  return NR == 4 ? 2 * (tl & 1) + ((tl >> 1) & 1) : tl & 1;
+}
+template <int NR>
+__device__ __forceinline__ float team8_dist_q(const float* __restrict__ qs,
+                                              const float* __restrict__ X, int ld,
+                                              const int32_t (&ids)[NR], const bool (&valid)[NR],
+                                              int tl) {
+  static_assert(NR == 2 || NR == 4, "two or four rows per team");
+  const float4* q4 = (const float4*)qs;
+  const int ld4 = ld >> 2;
+  float s[NR];
+#pragma unroll
+  for (int r = 0; r < NR; ++r) s[r] = 0.f;
+  for (int f0 = tl; f0 < ld4; f0 += 32) {
+    float4 raw[NR][4];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const float* x = X + (int64_t)ids[r] * ld;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int f = f0 + 8 * i;
+        raw[r][i] = (valid[r] && f < ld4) ? row_raw(x, f) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int f = f0 + 8 * i;
+      if (f < ld4) {
+        const float4 q = q4[f];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const float4 v = raw[r][i];
+          float u;
+          u = q.x - v.x; s[r] = fmaf(u, u, s[r]);
+          u = q.y - v.y; s[r] = fmaf(u, u, s[r]);
+          u = q.z - v.z; s[r] = fmaf(u, u, s[r]);
+          u = q.w - v.w; s[r] = fmaf(u, u, s[r]);
+        }
+      }
+    }
+  }
+  const bool odd = tl & 1, two = tl & 2;
+  float t;
+  if constexpr (NR == 4) {
+    const float a = odd ? s[0] : s[2], b = odd ? s[1] : s[3];
+    float k0 = odd ? s[2] : s[0], k1 = odd ? s[3] : s[1];
+    k0 += __shfl_xor_sync(0xffffffffu, a, 1);
+    k1 += __shfl_xor_sync(0xffffffffu, b, 1);
+    t = two ? k1 : k0;
+    t += __shfl_xor_sync(0xffffffffu, two ? k0 : k1, 2);
+  } else {
+    t = odd ? s[1] : s[0];
+    t += __shfl_xor_sync(0xffffffffu, odd ? s[0] : s[1], 1);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+  }
+  t += __shfl_xor_sync(0xffffffffu, t, 4);
+  return t;
+}
+
 // Integer queries (every value an integer 0..255) against byte rows: with the query's bytes
 // packed four to a word (qw) and q2 = |q|^2, d2 = q2 + |x|^2 - 2 q.x from byte dot products
 // (dp4a), all in exact integer arithmetic.  Every value and partial sum of the float path
@@ -310,18 +375,18 @@ struct SearchLayout {
 
 // One warp per query.  Per expansion: the node's neighbours not in the visited cache (its row
 // and degree load together, and the row of the next unchecked entry is fetched ahead, so that
-// the next expansion often starts with it), their distances by teams of four lanes with all
-// loads of 8 NR rows issued at once, and a merge of those below the pool's last key.  Bound by
+// the next expansion often starts with it), their distances by teams of four lanes (byte
+// rows) or eight (float rows) with all loads of 16 or 8 rows issued at once, and a merge of those below the pool's last key.  Bound by
 // that chain of latencies and by its instructions, not by memory.  Against teams of eight lanes,
 // a dependent degree and row load, and a sort of all new neighbours merged into a second copy
-// of the pool: 10,000 queries over 1M x 128 byte rows, L_search 40, 0.74 -> 0.54 ms; 4,096 over
-// 300,000 x 96 float rows, L_search 256, 2.68 -> 1.36 ms; one query 128 -> 90 us.  Byte rows
-// take 24 warps per SM with 16 rows in flight (32 warps, 0.56 ms, spill; 32 rows 0.63), float
-// rows 32 warps with 8 (24 warps 1.76 ms; 16 warps with 16 rows 1.70).  A pool in registers
-// with an insertion per accepted neighbour was slower (0.93 and 3.5 ms): on the way to the
-// query about half the neighbours are accepted.
-template <typename T>
-__global__ void __launch_bounds__(256, std::is_same<T, uint8_t>::value ? 3 : 4)
+// of the pool: 10,000 queries over 1M x 128 byte rows, L_search 40, 0.74 -> 0.54 ms; one query
+// 128 -> 90 us.  Byte rows take 24 warps per SM with 16 rows in flight (32 warps, 0.56 ms, spill;
+// 32 rows 0.63).  Float rows take teams of eight: 50,000 x 128, L_search 40, 10,000 queries 883 ->
+// 723 us, one query 172 -> 122 (teams of four: 796 and 181; 32 warps per SM with spills 738).  A
+// pool in registers with an insertion per accepted neighbour was slower (0.93 ms): on the way to
+// the query about half the neighbours are accepted.
+template <typename T, int NR, int MIN_BLOCKS>
+__global__ void __launch_bounds__(256, MIN_BLOCKS)
     k_search(const T* __restrict__ X, int ld, int d, const int32_t* __restrict__ adj,
              const int32_t* __restrict__ deg, int R, const int32_t* __restrict__ nav, int n_nav,
              const float* __restrict__ Q, int ldq, int64_t nq, int k, int ls,
@@ -331,10 +396,10 @@ __global__ void __launch_bounds__(256, std::is_same<T, uint8_t>::value ? 3 : 4)
              unsigned long long* __restrict__ work) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   constexpr bool BYTES = std::is_same<T, uint8_t>::value;
-  constexpr int NR = BYTES ? 2 : 1;  // rows per team at once: 16 or 8 rows per warp
+  constexpr int TEAMS = BYTES ? 8 : 4;  // a team takes NR rows at once
   constexpr int PIECES = 4;          // of 32 neighbours (R <= 128)
   const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = lane_id();
-  const int team = lane >> 2, tl = lane & 3;
+  const int team = lane / (32 / TEAMS), tl = lane % (32 / TEAMS);
   unsigned char* base = sm_raw + (size_t)warp * lay.per_warp();
   uint64_t* pool = (uint64_t*)base;
   uint64_t* newk = pool + lay.Ls;                        // [RP] ids, then keys
@@ -379,13 +444,30 @@ __global__ void __launch_bounds__(256, std::is_same<T, uint8_t>::value ? 3 : 4)
     // entry: the nearest navigating node by (d2, id), or the query's own start node
     uint64_t best = KEY_NONE;
     const int32_t* starts = from ? from + qi : nav;
-    for (int s0 = 0; s0 < n_nav; s0 += 8) {
-      const bool valid[1] = {s0 + team < n_nav};
-      const int32_t id[1] = {valid[0] ? starts[s0 + team] : 0};
-      float dd[1];
-      team4_dist_q<T, 1>(qs, X, ld, id, valid, tl, dd);
-      const uint64_t key = valid[0] ? pool_key(dd[0], id[0]) : KEY_NONE;
-      best = key < best ? key : best;
+    if constexpr (BYTES) {
+      for (int s0 = 0; s0 < n_nav; s0 += 8) {
+        const bool valid[1] = {s0 + team < n_nav};
+        const int32_t id[1] = {valid[0] ? starts[s0 + team] : 0};
+        float dd[1];
+        team4_dist_q<T, 1>(qs, X, ld, id, valid, tl, dd);
+        const uint64_t key = valid[0] ? pool_key(dd[0], id[0]) : KEY_NONE;
+        best = key < best ? key : best;
+      }
+    } else {
+      for (int s0 = 0; s0 < n_nav; s0 += TEAMS * NR) {
+        int32_t ir[NR];
+        bool vr[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const int t = s0 + TEAMS * r + team;
+          vr[r] = t < n_nav;
+          ir[r] = vr[r] ? starts[t] : 0;
+        }
+        const float dd = team8_dist_q<NR>(qs, X, ld, ir, vr, tl);
+        const int t = s0 + TEAMS * team8_row<NR>(tl) + team;
+        const uint64_t key = t < n_nav ? pool_key(dd, starts[t]) : KEY_NONE;
+        best = key < best ? key : best;
+      }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -441,29 +523,33 @@ __global__ void __launch_bounds__(256, std::is_same<T, uint8_t>::value ? 3 : 4)
       w_adj += (unsigned long long)dgn;
       w_dist += (unsigned long long)cnt;
       __syncwarp();
-      for (int t0 = 0; t0 < cnt; t0 += 8 * NR) {
+      for (int t0 = 0; t0 < cnt; t0 += TEAMS * NR) {
         int32_t ir[NR];
         bool vr[NR];
-        float dd[NR];
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-          const int t = t0 + 8 * r + team;
+          const int t = t0 + TEAMS * r + team;
           vr[r] = t < cnt;
           ir[r] = vr[r] ? (int32_t)(uint32_t)newk[t] : 0;
         }
         if constexpr (BYTES) {
+          float dd[NR];
           if (qint)
             team4_dist_qi<NR>(qw, X, ld, ir, vr, tl, q2, dd);
           else
             team4_dist_q<T, NR>(qs, X, ld, ir, vr, tl, dd);
-        } else {
-          team4_dist_q<T, NR>(qs, X, ld, ir, vr, tl, dd);
-        }
-        __syncwarp();
-        if (tl == 0) {
+          __syncwarp();
+          if (tl == 0) {
 #pragma unroll
-          for (int r = 0; r < NR; ++r)
-            if (vr[r]) newk[t0 + 8 * r + team] = pool_key(dd[r], ir[r]);
+            for (int r = 0; r < NR; ++r)
+              if (vr[r]) newk[t0 + TEAMS * r + team] = pool_key(dd[r], ir[r]);
+          }
+        } else {
+          const float dd = team8_dist_q<NR>(qs, X, ld, ir, vr, tl);
+          const int t = t0 + TEAMS * team8_row<NR>(tl) + team;
+          const int32_t id = t < cnt ? (int32_t)(uint32_t)newk[t] : 0;
+          __syncwarp();
+          if (tl < NR && t < cnt) newk[t] = pool_key(dd, id);
         }
       }
       __syncwarp();
@@ -506,12 +592,14 @@ void rows_to_u8(const float* X, int ld, int d, int64_t n, uint8_t* out, cudaStre
 // ls: the pool size, or the largest one of qls.  Warps per block: eight, fewer where there are
 // too few queries to give every SM a block of eight (a query alone on an SM runs without the
 // others' instructions in its way).
-template <typename T>
-static void launch_search(const T* X, int ld, int d, const int32_t* adj, const int32_t* deg, int R,
+template <typename T, int NR, int MIN_BLOCKS>
+static bool launch_rows(const T* X, int ld, int d, const int32_t* adj, const int32_t* deg, int R,
                           const int32_t* nav, int n_nav, const float* Q, int ldq, int64_t nq, int k,
                           int ls, const int32_t* qk, const int32_t* qls, const int32_t* from,
                           int ldo, int log2h, int32_t* out_ids, float* out_d2,
-                          unsigned long long* work, cudaStream_t st) {
+                          unsigned long long* work, cudaStream_t st,
+                          bool one_wave = false) {
+  auto kernel = k_search<T, NR, MIN_BLOCKS>;
   SearchLayout lay;
   lay.Ls = (ls + 1) & ~1;
   lay.RP = (R + 31) & ~31;
@@ -523,13 +611,49 @@ static void launch_search(const T* X, int ld, int d, const int32_t* adj, const i
   while (lay.per_warp() * wpb > 200 * 1024 && wpb > 1) wpb >>= 1;
   const size_t smem = lay.per_warp() * wpb;
   SSG_REQUIRE(smem <= 220 * 1024, SSG_EINVAL, "search: L_search and d too large for shared memory");
-  ensure_smem((const void*)k_search<T>, smem);
+  ensure_smem((const void*)kernel, smem);
   int blocks_per_sm = 0;
-  SSG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_search<T>, wpb * 32, smem));
+  SSG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, kernel, wpb * 32, smem));
   const int64_t want = ceil_div(nq, wpb);
+  if (one_wave && want > (int64_t)blocks_per_sm * num_sms()) return false;
   const int grid = (int)std::min<int64_t>(want, (int64_t)std::max(1, blocks_per_sm) * num_sms());
-  SSG_LAUNCH(k_search<T>, grid, wpb * 32, smem, st, X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k,
+  SSG_LAUNCH(kernel, grid, wpb * 32, smem, st, X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k,
              ls, qk, qls, from, ldo, lay, out_ids, out_d2, work);
+  return true;
+}
+
+static void launch_search(const uint8_t* X, int ld, int d, const int32_t* adj, const int32_t* deg,
+                          int R, const int32_t* nav, int n_nav, const float* Q, int ldq, int64_t nq,
+                          int k, int ls, const int32_t* qk, const int32_t* qls, const int32_t* from,
+                          int ldo, int log2h, int32_t* out_ids, float* out_d2,
+                          unsigned long long* work, cudaStream_t st) {
+  launch_rows<uint8_t, 2, 3>(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo,
+                             log2h, out_ids, out_d2, work, st);
+}
+// Float rows: while every warp of the batch fits two blocks of eight per SM, 16 rows in flight
+// per warp and 16 warps per SM; above, 8 rows and 24 warps.  50,000 x 128, us at L_search 40 and
+// 200, 16 rows / 8 rows: 600 queries 217 / 245 and 923 / 1,001; 10,000 queries 709 / 723 and
+// 3,834 / 3,080; 10,000 over 100,000 x 96: 588 / 462 and 2,446 / 1,832.  Between 24 and 32 queries
+// per SM 32 warps of 64 registers take them all at once where shared memory lets them: 4,000
+// queries, L_search 200, 50,000 x 61 and x 128 2,307 -> 1,848 and 2,111 -> 1,786, 100,000 x 96
+// 1,035 -> 977.
+static void launch_search(const float* X, int ld, int d, const int32_t* adj, const int32_t* deg,
+                          int R, const int32_t* nav, int n_nav, const float* Q, int ldq, int64_t nq,
+                          int k, int ls, const int32_t* qk, const int32_t* qls, const int32_t* from,
+                          int ldo, int log2h, int32_t* out_ids, float* out_d2,
+                          unsigned long long* work, cudaStream_t st) {
+  const int64_t sms = num_sms();
+  if (nq <= 16 * sms) {
+    launch_rows<float, 4, 2>(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo,
+                             log2h, out_ids, out_d2, work, st);
+    return;
+  }
+  if (nq > 24 * sms && nq <= 32 * sms &&
+      launch_rows<float, 2, 4>(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from,
+                               ldo, log2h, out_ids, out_d2, work, st, true))
+    return;
+  launch_rows<float, 2, 3>(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo,
+                           log2h, out_ids, out_d2, work, st);
 }
 
 // A 1,024-entry visited cache: its size only sets how often a distance is taken again, and a
