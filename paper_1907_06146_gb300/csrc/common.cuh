@@ -101,10 +101,14 @@ struct Scratch {
   Scratch() = default;
   Scratch(size_t n, cudaStream_t st) { alloc(n, st); }
   void alloc(size_t n, cudaStream_t st) {
+    if (!try_alloc(n, st)) throw Fail{SSG_ENOMEM};
+  }
+  // False, with the error's text set, where the device has no room.
+  bool try_alloc(size_t n, cudaStream_t st) {
     release();
     s = st;
     count = n;
-    if (n == 0) return;
+    if (n == 0) return true;
     if (alloc_fault_injected()) {
       set_error("scratch allocation of %zu bytes failed: injected", n * sizeof(T));
       throw Fail{SSG_ENOMEM};
@@ -114,8 +118,10 @@ struct Scratch {
     if (e != cudaSuccess) {
       p = nullptr;
       set_error("scratch allocation of %zu bytes failed: %s", n * sizeof(T), cudaGetErrorString(e));
-      throw Fail{SSG_ENOMEM};
+      if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+      return false;
     }
+    return true;
   }
   void release() {
     if (p) cudaFreeAsync(p, s);

@@ -1160,9 +1160,16 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
   // rounds of the clusters each
   const size_t block_bytes = (size_t)BM * a.nseg * C * sizeof(uint2);
   const int64_t round = std::max<int64_t>(1, num_sms() / 2);
-  const int64_t rounds = std::max<int64_t>(1, (int64_t)((2ull << 30) / block_bytes) / round);
-  const int64_t per_launch = std::min<int64_t>(nrb, rounds * round);
-  Scratch<uint2> rowbuf((size_t)per_launch * BM * a.nseg * C, st);
+  int64_t rounds = std::max<int64_t>(1, (int64_t)((2ull << 30) / block_bytes) / round);
+  rounds = std::min(rounds, ceil_div(nrb, round));
+  int64_t per_launch = std::min<int64_t>(nrb, rounds * round);
+  Scratch<uint2> rowbuf;
+  while (!rowbuf.try_alloc((size_t)per_launch * BM * a.nseg * C, st)) {
+    // where the device has less room, fewer rounds a launch, down to one (about 160 MB at C = 512)
+    if (rounds == 1) throw Fail{SSG_ENOMEM};
+    rounds = ceil_div(rounds, 2);
+    per_launch = rounds * round;
+  }
   Scratch<int> cnt((size_t)per_launch * BM * a.nseg, st);
   a.rowbuf = rowbuf.p;
   a.cnt = cnt.p;
