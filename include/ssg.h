@@ -108,7 +108,10 @@ typedef struct {
                                each node's L nearest among the points of the pool_tiles
                                128-point tiles nearest to it in the cluster order (an
                                IVF-style index over k-means clusters of the data, searched
-                               nearest cluster first); needs sm_103 and d <= 4096 (EINVAL
+                               nearest cluster first).  Blocks of 256 nodes in that order
+                               share a list of tiles; rows of more than 128 values: blocks
+                               of 128 nodes and 256-point tiles, pool_tiles / 2 rounded up;
+                               needs sm_103 and d <= 4096 (EINVAL
                                otherwise).  On data exact in bf16 the selection is exact;
                                on other data the tensor cores select L + slack candidates
                                by bf16 distance and each pool is re-ranked exactly (so a

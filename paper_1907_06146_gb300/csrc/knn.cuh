@@ -40,7 +40,6 @@ struct KnnOrder {
   int64_t ntiles = 0;
   int64_t tstride = 0;  // length of each cluster's tile list (ntiles, or the walk limit)
   Scratch<int32_t> perm, tile_order, rb_cluster;
-  Scratch<int32_t> pair_tiles, pair_len;  // knn_pair_tiles
 };
 bool knn_order_fits(int64_t n, int BN);
 // walk > 0: every block of rows visits only its first walk tiles (Alg. 4), so each
@@ -50,9 +49,12 @@ bool knn_order_fits(int64_t n, int BN);
 void knn_cluster_order(const float* X, int ld, int d, int64_t n, int BM, int BN, cudaStream_t st,
                        KnnOrder& o, int64_t walk = 0, const float* x_norm = nullptr);
 
-// Of an order for a limited walk: the list of each pair of row blocks, in tiles twice as wide
-// (pair_tiles, 2 tstride entries apart; pair_len of them).
-void knn_pair_tiles(int64_t n, int BM, cudaStream_t st, KnnOrder& o);
+// Of an order for a limited walk, over blocks of BM rows and BN-column tiles (256 and 128, or 128
+// and 256): the 256-column tiles of the work items item0 .. item0 + items - 1 of 512 rows, in out
+// (stride entries apart, enough for the item's blocks' lists or for all tiles), their number in
+// len.  An entry is tile << 8 | mask, bit 2 s + c: the item's rows 128 s .. visit columns 128 c ..
+void knn_item_tiles(const KnnOrder& o, int64_t n, int BM, int BN, int64_t item0, int64_t items,
+                    int64_t stride, int32_t* out, int32_t* len, cudaStream_t st);
 
 // bf16 tensor-core variant of the exact top-K (only for info.bf16_exact data).
 // True on sm_103 for rows of up to 4,096 values: the resident pipeline holds d <= 128, wider

@@ -241,43 +241,55 @@ __global__ void k_tile_order(const int32_t* __restrict__ order, const int32_t* _
   if (k != cap) atomicOr(err, 1);
 }
 
-// The tile list of each pair of row blocks (2 rb, 2 rb + 1) of a limited walk, in tiles twice
-// as wide: the tiles that hold those of either block's list (list entries taken in turn, so
-// nearest first for both), each once.  One thread per pair walks the lists with a bitmap of
-// the tiles already listed.
-__global__ void k_pair_tiles(const int32_t* __restrict__ tile_order, const int32_t* __restrict__ rbc,
-                             int64_t nrb, int64_t tstride, int64_t words,
-                             int32_t* __restrict__ out, int32_t* __restrict__ len) {
-  extern __shared__ uint32_t seen[];
-  const int64_t pr = blockIdx.x;
-  for (int64_t w = threadIdx.x; w < words; w += blockDim.x) seen[w] = 0u;
+// The tile list of each work item of a limited walk: the 256-column tiles that hold those of its
+// `per` row blocks' lists (list entries taken in turn, so nearest first for all), each once, with
+// the mask of who visits what (knn_item_tiles).  All threads mark the lists in a bitmap per row
+// block; then one walks the lists with a bitmap of the tiles already listed.
+__global__ void k_item_tiles(const int32_t* __restrict__ tile_order, const int32_t* __restrict__ rbc,
+                             int64_t nrb, int per, int wide, int64_t tstride, int words, int64_t item0,
+                             int64_t stride, int32_t* __restrict__ out, int32_t* __restrict__ len) {
+  extern __shared__ uint32_t marks[];  // [per][words] of the lists' tiles, then [words] of those seen
+  uint32_t* seen = marks + per * words;
+  const int64_t b0 = (item0 + blockIdx.x) * per;
+  const int blocks = (int)min((int64_t)per, nrb - b0);
+  for (int w = threadIdx.x; w < (per + 1) * words; w += blockDim.x) marks[w] = 0u;
+  __syncthreads();
+  for (int b = 0; b < blocks; ++b)
+    for (int64_t i = threadIdx.x; i < tstride; i += blockDim.x) {
+      const int32_t t = tile_order[(int64_t)rbc[b0 + b] * tstride + i];
+      atomicOr(marks + b * words + (t >> 5), 1u << (t & 31));
+    }
   __syncthreads();
   if (threadIdx.x != 0) return;
-  const int32_t* l0 = tile_order + (int64_t)rbc[2 * pr] * tstride;
-  const int32_t* l1 =
-      2 * pr + 1 < nrb ? tile_order + (int64_t)rbc[2 * pr + 1] * tstride : l0;
-  int32_t* o = out + pr * 2 * tstride;
+  int32_t* o = out + (int64_t)blockIdx.x * stride;
   int k = 0;
   for (int64_t i = 0; i < tstride; ++i) {
-    for (int b = 0; b < 2; ++b) {
-      if (b == 1 && l1 == l0) break;
-      const int32_t t = (b ? l1[i] : l0[i]) >> 1;
+    for (int b = 0; b < blocks; ++b) {
+      int32_t t = tile_order[(int64_t)rbc[b0 + b] * tstride + i];
+      if (!wide) t >>= 1;
       const uint32_t bit = 1u << (t & 31);
       if (seen[t >> 5] & bit) continue;
       seen[t >> 5] |= bit;
-      o[k++] = t;
+      uint32_t mask = 0u;
+      for (int v = 0; v < blocks; ++v) {
+        const uint32_t* m = marks + v * words;
+        const uint32_t cols = wide ? ((m[t >> 5] >> (t & 31)) & 1u) * 3u
+                                   : (m[t >> 4] >> (2 * (t & 15))) & 3u;
+        mask |= per == 2 ? (cols * 5u) << (4 * v) : cols << (2 * v);
+      }
+      o[k++] = t << 8 | (int32_t)mask;
     }
   }
-  len[pr] = k;
+  len[blockIdx.x] = k;
 }
 
-void knn_pair_tiles(int64_t n, int BM, cudaStream_t st, KnnOrder& o) {
-  const int64_t nrb = ceil_div(n, BM), npr = ceil_div(nrb, 2);
-  const int64_t words = (ceil_div(o.ntiles, 2) + 31) >> 5;
-  o.pair_tiles.alloc((size_t)npr * 2 * o.tstride, st);
-  o.pair_len.alloc((size_t)npr, st);
-  SSG_LAUNCH(k_pair_tiles, (unsigned)npr, 32, (size_t)words * 4, st, o.tile_order.p, o.rb_cluster.p,
-             nrb, o.tstride, words, o.pair_tiles.p, o.pair_len.p);
+void knn_item_tiles(const KnnOrder& o, int64_t n, int BM, int BN, int64_t item0, int64_t items,
+                    int64_t stride, int32_t* out, int32_t* len, cudaStream_t st) {
+  const int per = 512 / BM, words = (int)((o.ntiles + 31) >> 5);
+  const size_t smem = (size_t)(per + 1) * words * sizeof(uint32_t);
+  ensure_smem((const void*)k_item_tiles, smem);
+  SSG_LAUNCH(k_item_tiles, (unsigned)items, 128, smem, st, o.tile_order.p, o.rb_cluster.p,
+             ceil_div(n, BM), per, BN == 256 ? 1 : 0, o.tstride, words, item0, stride, out, len);
 }
 
 bool knn_order_fits(int64_t n, int BN) {

@@ -50,6 +50,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
+#include <type_traits>
 
 #include "common.cuh"
 #include "knn.cuh"
@@ -100,7 +101,9 @@ struct TcArgs {
   const int32_t* perm;        // stored position -> original id (null: the identity)
   const int32_t* tile_order;  // tile lists, tstride entries apart (null: in order)
   const int32_t* rb_cluster;  // list of each block of BM stored query rows (null: its own)
-  const int32_t* walk_len;    // nullable: tiles that each block visits (else nwalk)
+  // limited walks: block rb0 + i has the i-th list, of walk_len[i] entries tile << 8 | mask, bit
+  // 4 r + 2 h + c: rows 128 h .. of CTA r visit the tile's columns 128 c ..
+  const int32_t* walk_len;
 };
 
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
@@ -237,7 +240,9 @@ __device__ __noinline__ uint2 cut_rows(uint2* __restrict__ wbuf, uint32_t lstrid
   return mine;
 }
 
-template <int C, bool STREAM>
+// LIMITED: a walk over part of the tiles, with masked list entries (TcArgs::walk_len).  A kernel of
+// its own: the mask's test in the one for full walks cost 258 -> 270 ms for a build of 1M x 128.
+template <int C, bool STREAM, bool LIMITED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
            const __grid_constant__ CUtensorMap tmAaug, const __grid_constant__ CUtensorMap tmBaug,
@@ -297,13 +302,15 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
   const int64_t ncl = gridDim.x >> 1, cl = blockIdx.x >> 1;
   // item i: row block rb0 + i / nseg, tiles i % nseg, i % nseg + nseg, ...
   auto tiles_of = [&](int64_t rb) -> const int32_t* {
+    if (LIMITED) return p.tile_order + (rb - p.rb0) * p.tstride;
     return p.tile_order
                ? p.tile_order + (p.rb_cluster ? (int64_t)p.rb_cluster[rb] : rb) * p.tstride
                : nullptr;
   };
   auto walk_of = [&](int64_t rb) -> int64_t {
-    return p.walk_len ? (int64_t)p.walk_len[rb] : p.nwalk;
+    return LIMITED ? (int64_t)p.walk_len[rb - p.rb0] : p.nwalk;
   };
+  constexpr int MASK_BITS = LIMITED ? 8 : 0;  // of a list entry
 
   if (warp == 0) {
     // ---------------- TMA producer (of each CTA) ----------------
@@ -335,7 +342,7 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
         const int64_t nwalk = walk_of(rb);
         int64_t tn = tl ? tl[seg] : seg;  // tile index, read one tile ahead
         for (int64_t i = seg; i < nwalk && ok; i += nseg) {
-          const int j0 = (int)(tn * BN + rank * (BN / 2));
+          const int j0 = (int)((tn >> MASK_BITS) * BN + rank * (BN / 2));
           if (i + nseg < nwalk) tn = tl ? tl[i + nseg] : i + nseg;
           for (int kc = 0; kc < spt; ++kc) {
             ok = mbar_wait(smem_u32(s_empty + s), ph ^ 1, abort_flag);
@@ -551,7 +558,9 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
         ts = fmaxf(ts, t2);
       };
       for (int64_t i = seg; i < nwalk; i += nseg) {
-        const int32_t j0 = (int32_t)(tn * BN);
+        const int32_t j0 = (int32_t)((tn >> MASK_BITS) * BN);
+        // columns that these rows do not visit (bit c: the half c)
+        const uint32_t skip = LIMITED ? ~((uint32_t)tn >> (4 * rank + 2 * h)) & 3u : 0u;
         if (i + nseg < nwalk) tn = tl ? tl[i + nseg] : i + nseg;
         // with shares: the other shares' thresholds, read while the tile is computed
         uint32_t other = 0u;
@@ -579,6 +588,7 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(my_empty + (c >> 1) * (uint32_t)sizeof(uint64_t));
           }
+          if (LIMITED && ((skip >> (STREAM ? c >> 1 : c & 1)) & 1u)) continue;
           // resident rows: a column half is 64 columns of each CTA's 128
           const int32_t jc = j0 + (STREAM ? c * 64 : (c >> 1) * 64 + (c & 1) * (BN / 2));
           if (jc + 64 > p.nb) {  // the last tile's padding columns are never admitted
@@ -992,11 +1002,11 @@ struct TcMaps {
   CUtensorMap a, b, a_aug, b_aug;
 };
 
-template <int C, bool STREAM>
+template <int C, bool STREAM, bool LIMITED>
 void launch_tc(const TcMaps& m, TcArgs& a, size_t smem, cudaStream_t st) {
-  ensure_smem((const void*)k_knn_pair<C, STREAM>, smem);
+  ensure_smem((const void*)k_knn_pair<C, STREAM, LIMITED>, smem);
   const int64_t pairs = std::min<int64_t>(a.nrb * a.nseg, num_sms() / 2);
-  SSG_LAUNCH((k_knn_pair<C, STREAM>), (unsigned)(2 * pairs), THREADS, smem, st, m.a, m.b, m.a_aug,
+  SSG_LAUNCH((k_knn_pair<C, STREAM, LIMITED>), (unsigned)(2 * pairs), THREADS, smem, st, m.a, m.b, m.a_aug,
              m.b_aug, a);
 }
 
@@ -1072,7 +1082,13 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
   // same: the query rows are the base rows (a self-join); with ex.qid the query rows are a
   // gathered subset of the base and only the self column is excluded
   const bool same = self && !ex.qid;
-  SSG_REQUIRE(max_tiles == 0 || (same && knn_order_fits(na, API_TILE)), SSG_EINVAL,
+  // A limited walk's lists set what each row is compared with: max_tiles 128-point tiles for each
+  // block of 256 rows, or (rows longer than 128 values) as many points in 256-point tiles for each
+  // block of 128.  A work item walks the tiles of all its blocks' lists, and each block's rows
+  // take only those of their own.
+  const int list_rows = max_tiles == 0 ? BM : stream ? 128 : 256;
+  const int list_tile = max_tiles == 0 || stream ? BN : API_TILE;
+  SSG_REQUIRE(max_tiles == 0 || (same && knn_order_fits(na, list_tile)), SSG_EINVAL,
               "a tile limit needs a self-join whose cluster order fits");
   // (not for streamed rows: their tiles are long enough that the appends a slowly falling
   // threshold costs matter less than L2 reuse, which needs every cluster to walk the columns in
@@ -1081,15 +1097,9 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
   const bool ordered =
       max_tiles > 0 || (!stream && same && na >= (1 << 16) && K >= 16 && knn_order_fits(na, BN));
   if (ordered) {
-    // A limited walk's lists are those of 256 rows and 128-point tiles, which set what each row
-    // is compared with; a work item takes the tiles of both its 256-row blocks.
     const float* on = ex.order_norm ? ex.order_norm : a_norm;
-    if (max_tiles > 0) {
-      knn_cluster_order(A, lda, d, na, BM / 2, API_TILE, st, ord, max_tiles, on);
-      knn_pair_tiles(na, BM / 2, st, ord);
-    } else {
-      knn_cluster_order(A, lda, d, na, BM, BN, st, ord, 0, on);
-    }
+    knn_cluster_order(A, lda, d, na, list_rows, list_tile, st, ord,
+                      ceil_div((int64_t)max_tiles * API_TILE, list_tile), on);
     norm_p.alloc((size_t)na, st);
   }
   const int32_t* perm = ordered ? (const int32_t*)ord.perm.p : nullptr;
@@ -1130,7 +1140,8 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
   a.na = na;
   a.nb = nb;
   a.nwalk = ntiles;
-  a.tstride = max_tiles > 0 ? 2 * ord.tstride : (ordered ? ord.tstride : ntiles);
+  a.tstride = max_tiles > 0 ? std::min<int64_t>(BM / list_rows * ord.tstride, ntiles)
+                            : (ordered ? ord.tstride : ntiles);
   a.nseg = max_tiles > 0 ? 1 : pick_shares(nrb, a.nwalk, C, KS, num_sms() / 2);
   a.kchunks = kchunks;
   a.dp_chunks = dp / 64;
@@ -1140,9 +1151,8 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
   a.err = err.p;
   if (ordered) {
     a.perm = ord.perm.p;
-    a.tile_order = max_tiles > 0 ? ord.pair_tiles.p : ord.tile_order.p;
-    a.rb_cluster = max_tiles > 0 ? nullptr : ord.rb_cluster.p;
-    a.walk_len = max_tiles > 0 ? ord.pair_len.p : nullptr;
+    a.tile_order = ord.tile_order.p;
+    a.rb_cluster = ord.rb_cluster.p;
   }
   // Near-first full walks may be preceded by one over each block's prepass_tiles nearest tiles
   // that only records each row's KS-th largest accumulator there, from which the full walk
@@ -1173,6 +1183,15 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
   Scratch<int> cnt((size_t)per_launch * BM * a.nseg, st);
   a.rowbuf = rowbuf.p;
   a.cnt = cnt.p;
+  // a limited walk's lists of one launch's items
+  Scratch<int32_t> item_tiles, item_len;
+  if (max_tiles > 0) {
+    item_tiles.alloc((size_t)(per_launch * a.tstride), st);
+    item_len.alloc((size_t)per_launch, st);
+    a.tile_order = item_tiles.p;
+    a.rb_cluster = nullptr;
+    a.walk_len = item_len.p;
+  }
   FinArgs f{};
   f.err = err.p;
   f.rowbuf = rowbuf.p;
@@ -1199,13 +1218,24 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
     for (int64_t rb = 0; rb < nrb; rb += per_launch) {
       args.rb0 = rb;
       args.nrb = std::min<int64_t>(per_launch, nrb - rb);
+      if (max_tiles > 0)
+        knn_item_tiles(ord, na, list_rows, list_tile, rb, args.nrb, args.tstride, item_tiles.p,
+                       item_len.p, st);
+      auto launch = [&](auto size) {
+        constexpr int S = decltype(size)::value;
+        if (max_tiles > 0)
+          stream ? launch_tc<S, true, true>(maps, args, smem, st)
+                 : launch_tc<S, false, true>(maps, args, smem, st);
+        else
+          stream ? launch_tc<S, true, false>(maps, args, smem, st)
+                 : launch_tc<S, false, false>(maps, args, smem, st);
+      };
       if (C == 256)
-        stream ? launch_tc<256, true>(maps, args, smem, st) : launch_tc<256, false>(maps, args, smem, st);
+        launch(std::integral_constant<int, 256>());
       else if (C == 512)
-        stream ? launch_tc<512, true>(maps, args, smem, st) : launch_tc<512, false>(maps, args, smem, st);
+        launch(std::integral_constant<int, 512>());
       else
-        stream ? launch_tc<1024, true>(maps, args, smem, st)
-               : launch_tc<1024, false>(maps, args, smem, st);
+        launch(std::integral_constant<int, 1024>());
       fin.row0 = rb * BM;
       fin.rows = std::min<int64_t>(args.nrb * BM, na - fin.row0);
       SSG_LAUNCH(k_knn_finish, (unsigned)ceil_div(fin.rows, 4), 128, fsm, st, fin);
