@@ -69,6 +69,8 @@ constexpr int STOP_BAND = -2;       // the band list overflowed
 constexpr int STOP_ROW = -3;        // u's kNN row settles nothing: the full scan takes u
 constexpr int STOP_BFS = -4;        // u is linked, its traversal outgrew the block
 constexpr int STOP_KNN = -5;        // unreached nodes remain, k_repair_knn is next
+constexpr int STOP_RESCAN = -6;     // the band is taken again against hi_bits as it stands
+constexpr int FIRST_BAND = 2048;    // band entries up to which that is not needed
 
 __global__ void k_mark(uint32_t* __restrict__ bm, int32_t* __restrict__ frontier,
                        RepairState* __restrict__ s, int32_t root) {
@@ -426,7 +428,10 @@ __device__ __forceinline__ void block_argmin(double& best, int& bid, double* bd,
 // then (its block's at most, so a superset of the band that can hold the minimum; a warp each);
 // then, in block 0, the (d2, id)-smallest of them, re-taken in coordinate order among those
 // within fp64_order_rel of the smallest.  Two grid barriers per repair; a host round trip and
-// seven launches took 60 us (30,011 x 100, 172 repairs: 12.7 -> 5.0 ms).
+// seven launches took 60 us (30,011 x 100, 172 repairs: 12.7 -> 5.0 ms).  Where the superset is
+// large (distances that take few values: every block may hold thousands of ties at its own
+// smallest one), the band is taken again from the stored fp32 distances, against the smallest
+// bound of the whole grid, and only that band counts towards the list's room.
 __global__ void __launch_bounds__(512) k_connect(ConnArgs a) {
   __shared__ double bd[32];
   __shared__ int bi[32];
@@ -461,31 +466,37 @@ __global__ void __launch_bounds__(512) k_connect(ConnArgs a) {
     if (!grid_barrier(s, phase)) return;
     const int64_t u = (int64_t)*(volatile unsigned long long*)&s->u;
     const int what = *(volatile int*)&s->best;
-    if (u >= a.n || (what != STOP_BFS && what != STOP_ROW)) return;
+    if (u >= a.n || (what != STOP_BFS && what != STOP_ROW && what != STOP_RESCAN)) return;
     if (what == STOP_BFS) {
       if (!grid_bfs(a, phase)) return;
       if (blockIdx.x == 0 && warp == 0) next_node();
       continue;
     }
     const float* xu = a.X + u * a.ld;
-    if (threadIdx.x == 0) bmin = 0x7f800000u;
-    __syncthreads();
-    float best = __int_as_float(0x7f800000);
-    for (int64_t v0 = gw * 4; v0 < a.n; v0 += nwarps * 4) {
-      const int64_t v = v0 + team;
-      const bool cand =
-          v < a.n && ((__ldcg(a.bm + (v >> 5)) >> (v & 31)) & 1u) && __ldcg(a.deg + v) < a.R;
-      const float e = team8_dist(a.X + (cand ? v : 0) * a.ld, xu, a.ld >> 2, tl, cand);
-      if (tl == 0 && v < a.n) a.d32[v] = cand ? e : -1.f;
-      if (cand) best = fminf(best, e);
+    const int room = what == STOP_RESCAN ? a.cap : min(a.cap, FIRST_BAND);
+    float hi;
+    if (what == STOP_RESCAN) {
+      hi = __uint_as_float(*(volatile unsigned*)&s->hi_bits);
+    } else {
+      if (threadIdx.x == 0) bmin = 0x7f800000u;
+      __syncthreads();
+      float best = __int_as_float(0x7f800000);
+      for (int64_t v0 = gw * 4; v0 < a.n; v0 += nwarps * 4) {
+        const int64_t v = v0 + team;
+        const bool cand =
+            v < a.n && ((__ldcg(a.bm + (v >> 5)) >> (v & 31)) & 1u) && __ldcg(a.deg + v) < a.R;
+        const float e = team8_dist(a.X + (cand ? v : 0) * a.ld, xu, a.ld >> 2, tl, cand);
+        if (tl == 0 && v < a.n) a.d32[v] = cand ? e : -1.f;
+        if (cand) best = fminf(best, e);
+      }
+      for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+      if (lane == 0 && best < __int_as_float(0x7f800000))
+        atomicMin(&bmin, __float_as_uint(best * (1.f + 2.f * a.rel) + 1e-30f));
+      __syncthreads();
+      if (threadIdx.x == 0 && bmin != 0x7f800000u) bmin = min(bmin, atomicMin(&s->hi_bits, bmin));
+      __syncthreads();
+      hi = __uint_as_float(bmin);
     }
-    for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if (lane == 0 && best < __int_as_float(0x7f800000))
-      atomicMin(&bmin, __float_as_uint(best * (1.f + 2.f * a.rel) + 1e-30f));
-    __syncthreads();
-    if (threadIdx.x == 0 && bmin != 0x7f800000u) bmin = min(bmin, atomicMin(&s->hi_bits, bmin));
-    __syncthreads();
-    const float hi = __uint_as_float(bmin);
     for (int64_t v0 = gw * 4; v0 < a.n; v0 += nwarps * 32) {
       // this warp's own distances: four nodes of each of eight rounds
       const int64_t v1 = v0 + (int64_t)(lane >> 2) * nwarps * 4 + (lane & 3);
@@ -498,7 +509,7 @@ __global__ void __launch_bounds__(512) k_connect(ConnArgs a) {
         int p = 0;
         if (lane == 0) p = atomicAdd(&s->band, 1);
         p = __shfl_sync(0xffffffffu, p, 0);
-        if (p >= a.cap) break;
+        if (p >= room) break;
         const double x = warp_dist2_f64(a.X + v * a.ld, xu, a.d);
         if (lane == 0) {
           a.band_ids[p] = (int32_t)v;
@@ -510,8 +521,11 @@ __global__ void __launch_bounds__(512) k_connect(ConnArgs a) {
     if (blockIdx.x != 0) continue;
     // block 0 links the smallest, expands u, and finds the next node
     const int m = *(volatile int*)&s->band;
-    if (m == 0 || m > a.cap) {
-      if (threadIdx.x == 0) s->best = m == 0 ? STOP_NONE : STOP_BAND;
+    if (m == 0 || m > room) {
+      if (threadIdx.x == 0) {
+        s->best = m == 0 ? STOP_NONE : what == STOP_RESCAN ? STOP_BAND : STOP_RESCAN;
+        s->band = 0;
+      }
       continue;
     }
     double b1 = INF;
