@@ -380,8 +380,9 @@ struct Pool {
 
 struct SearchLayout {
   int Ls, RP, ld, log2h;  // Ls: the largest pool, even; RP: a multiple of 32, at least R
+  int qb;                 // bytes for the query packed to bytes (float rows: none)
   __host__ __device__ size_t per_warp() const {
-    return (size_t)Ls * 8 + (size_t)(RP + 32) * 8 + (size_t)ld * 4 + (((size_t)ld + 15) & ~(size_t)15) + ((size_t)4 << log2h);
+    return (size_t)Ls * 8 + (size_t)(RP + 32) * 8 + (size_t)ld * 4 + (size_t)qb + ((size_t)4 << log2h);
   }
 };
 
@@ -418,7 +419,7 @@ __global__ void __launch_bounds__(256, MIN_BLOCKS)
   uint64_t* tmp = newk + lay.RP;                         // [32]
   float* qs = (float*)(tmp + 32);                        // [ld]
   uint32_t* qw = (uint32_t*)(qs + ld);                   // the query's bytes, if integer 0..255
-  int32_t* cache = (int32_t*)((unsigned char*)qw + (((size_t)ld + 15) & ~(size_t)15));
+  int32_t* cache = (int32_t*)((unsigned char*)qw + lay.qb);
   const int hcap = 1 << lay.log2h;
 
   for (int64_t qi = (int64_t)blockIdx.x * wpb + warp; qi < nq; qi += (int64_t)gridDim.x * wpb) {
@@ -601,37 +602,48 @@ void rows_to_u8(const float* X, int ld, int d, int64_t n, uint8_t* out, cudaStre
              (const float4*)X, n4, (uchar4*)out);
 }
 
+// A launch of k_search<T, NR, MIN_BLOCKS>: warps per block, shared memory, blocks per SM.
+struct SearchPlan {
+  SearchLayout lay;
+  int wpb, per_sm;
+  size_t smem;
+  int warps() const { return wpb * per_sm; }  // per SM
+};
+
 // ls: the pool size, or the largest one of qls.  Warps per block: eight, fewer where there are
 // too few queries to give every SM a block of eight (a query alone on an SM runs without the
 // others' instructions in its way).
 template <typename T, int NR, int MIN_BLOCKS>
-static bool launch_rows(const T* X, int ld, int d, const int32_t* adj, const int32_t* deg, int R,
-                          const int32_t* nav, int n_nav, const float* Q, int ldq, int64_t nq, int k,
-                          int ls, const int32_t* qk, const int32_t* qls, const int32_t* from,
-                          int ldo, int log2h, int32_t* out_ids, float* out_d2,
-                          unsigned long long* work, cudaStream_t st,
-                          bool one_wave = false) {
-  auto kernel = k_search<T, NR, MIN_BLOCKS>;
-  SearchLayout lay;
-  lay.Ls = (ls + 1) & ~1;
-  lay.RP = (R + 31) & ~31;
-  lay.ld = ld;
-  lay.log2h = log2h;
-  int wpb = work ? 2 : 8;
-  wpb = (int)std::min<int64_t>(wpb, std::max<int64_t>(1, ceil_div(nq, num_sms())));
-  while (lay.per_warp() * wpb > 200 * 1024 && lay.log2h > 8) --lay.log2h;
-  while (lay.per_warp() * wpb > 200 * 1024 && wpb > 1) wpb >>= 1;
-  const size_t smem = lay.per_warp() * wpb;
-  SSG_REQUIRE(smem <= 220 * 1024, SSG_EINVAL, "search: L_search and d too large for shared memory");
-  ensure_smem((const void*)kernel, smem);
-  int blocks_per_sm = 0;
-  SSG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, kernel, wpb * 32, smem));
-  const int64_t want = ceil_div(nq, wpb);
-  if (one_wave && want > (int64_t)blocks_per_sm * num_sms()) return false;
-  const int grid = (int)std::min<int64_t>(want, (int64_t)std::max(1, blocks_per_sm) * num_sms());
-  SSG_LAUNCH(kernel, grid, wpb * 32, smem, st, X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k,
-             ls, qk, qls, from, ldo, lay, out_ids, out_d2, work);
-  return true;
+static SearchPlan plan_rows(int ld, int R, int64_t nq, int ls, int log2h, bool work) {
+  const void* kernel = (const void*)k_search<T, NR, MIN_BLOCKS>;
+  SearchPlan p;
+  p.lay.Ls = (ls + 1) & ~1;
+  p.lay.RP = (R + 31) & ~31;
+  p.lay.ld = ld;
+  p.lay.qb = std::is_same<T, uint8_t>::value ? (ld + 15) & ~15 : 0;
+  p.lay.log2h = log2h;
+  p.wpb = work ? 2 : 8;
+  p.wpb = (int)std::min<int64_t>(p.wpb, std::max<int64_t>(1, ceil_div(nq, num_sms())));
+  while (p.lay.per_warp() * p.wpb > 200 * 1024 && p.lay.log2h > 8) --p.lay.log2h;
+  while (p.lay.per_warp() * p.wpb > 200 * 1024 && p.wpb > 1) p.wpb >>= 1;
+  p.smem = p.lay.per_warp() * p.wpb;
+  SSG_REQUIRE(p.smem <= 220 * 1024, SSG_EINVAL, "search: L_search and d too large for shared memory");
+  ensure_smem(kernel, p.smem);
+  p.per_sm = 0;
+  SSG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p.per_sm, kernel, p.wpb * 32, p.smem));
+  p.per_sm = std::max(1, p.per_sm);
+  return p;
+}
+
+template <typename T, int NR, int MIN_BLOCKS>
+static void launch_rows(const SearchPlan& p, const T* X, int ld, int d, const int32_t* adj,
+                        const int32_t* deg, int R, const int32_t* nav, int n_nav, const float* Q,
+                        int ldq, int64_t nq, int k, int ls, const int32_t* qk, const int32_t* qls,
+                        const int32_t* from, int ldo, int32_t* out_ids, float* out_d2,
+                        unsigned long long* work, cudaStream_t st) {
+  const int grid = (int)std::min<int64_t>(ceil_div(nq, p.wpb), (int64_t)p.per_sm * num_sms());
+  SSG_LAUNCH((k_search<T, NR, MIN_BLOCKS>), grid, p.wpb * 32, p.smem, st, X, ld, d, adj, deg, R, nav,
+             n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo, p.lay, out_ids, out_d2, work);
 }
 
 static void launch_search(const uint8_t* X, int ld, int d, const int32_t* adj, const int32_t* deg,
@@ -639,8 +651,9 @@ static void launch_search(const uint8_t* X, int ld, int d, const int32_t* adj, c
                           int k, int ls, const int32_t* qk, const int32_t* qls, const int32_t* from,
                           int ldo, int log2h, int32_t* out_ids, float* out_d2,
                           unsigned long long* work, cudaStream_t st) {
-  launch_rows<uint8_t, 2, 3>(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo,
-                             log2h, out_ids, out_d2, work, st);
+  launch_rows<uint8_t, 2, 3>(plan_rows<uint8_t, 2, 3>(ld, R, nq, ls, log2h, work != nullptr), X, ld, d,
+                             adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo, out_ids,
+                             out_d2, work, st);
 }
 // Float rows: while every warp of the batch fits two blocks of eight per SM, 16 rows in flight
 // per warp and 16 warps per SM; above, 8 rows and 24 warps.  50,000 x 128, us at L_search 40 and
@@ -648,24 +661,35 @@ static void launch_search(const uint8_t* X, int ld, int d, const int32_t* adj, c
 // 3,834 / 3,080; 10,000 over 100,000 x 96: 588 / 462 and 2,446 / 1,832.  Between 24 and 32 queries
 // per SM 32 warps of 64 registers take them all at once where shared memory lets them: 4,000
 // queries, L_search 200, 50,000 x 61 and x 128 2,307 -> 1,848 and 2,111 -> 1,786, 100,000 x 96
-// 1,035 -> 977.
+// 1,035 -> 977.  Rows of more than 512 values that leave shared memory for no more than those 16
+// warps anyway take 16 rows in flight at any batch size: 10,000 queries over 20,000 x 1,500, L_search
+// 10, 1,223 -> 1,008 us, x 2,500, L_search 40, 6,239 -> 5,325 (shorter rows under large pools gain
+// nothing: x 200, L_search 1,024, 23.6 / 24.1 ms).
 static void launch_search(const float* X, int ld, int d, const int32_t* adj, const int32_t* deg,
                           int R, const int32_t* nav, int n_nav, const float* Q, int ldq, int64_t nq,
                           int k, int ls, const int32_t* qk, const int32_t* qls, const int32_t* from,
                           int ldo, int log2h, int32_t* out_ids, float* out_d2,
                           unsigned long long* work, cudaStream_t st) {
   const int64_t sms = num_sms();
-  if (nq <= 16 * sms) {
-    launch_rows<float, 4, 2>(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo,
-                             log2h, out_ids, out_d2, work, st);
-    return;
+  const bool w = work != nullptr;
+  if (nq > 16 * sms) {
+    const SearchPlan p3 = plan_rows<float, 2, 3>(ld, R, nq, ls, log2h, w);
+    if (p3.warps() > 16 || ld <= 512) {
+      if (nq > 24 * sms && nq <= 32 * sms) {
+        const SearchPlan p4 = plan_rows<float, 2, 4>(ld, R, nq, ls, log2h, w);
+        if (nq <= p4.warps() * sms) {
+          launch_rows<float, 2, 4>(p4, X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls,
+                                   from, ldo, out_ids, out_d2, work, st);
+          return;
+        }
+      }
+      launch_rows<float, 2, 3>(p3, X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from,
+                               ldo, out_ids, out_d2, work, st);
+      return;
+    }
   }
-  if (nq > 24 * sms && nq <= 32 * sms &&
-      launch_rows<float, 2, 4>(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from,
-                               ldo, log2h, out_ids, out_d2, work, st, true))
-    return;
-  launch_rows<float, 2, 3>(X, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo,
-                           log2h, out_ids, out_d2, work, st);
+  launch_rows<float, 4, 2>(plan_rows<float, 4, 2>(ld, R, nq, ls, log2h, w), X, ld, d, adj, deg, R, nav,
+                           n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo, out_ids, out_d2, work, st);
 }
 
 // A 1,024-entry visited cache: its size only sets how often a distance is taken again, and a
@@ -709,6 +733,7 @@ bool search_from(const float* X, int ld, int d, const int32_t* adj, const int32_
   lay.Ls = Ls + 1;
   lay.RP = (R + 31) & ~31;
   lay.ld = ld;
+  lay.qb = 0;
   lay.log2h = 8;
   if (lay.per_warp() > 200 * 1024) return false;
   launch_search(X, ld, d, adj, deg, R, from, 1, Q, ldq, nq, 1, Ls, (const int32_t*)nullptr,
