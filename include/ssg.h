@@ -300,7 +300,9 @@ ssg_status ssg_connect_noalloc(const float* base, int64_t n, int32_t d, int32_t*
  * of at most L_search entries sorted by (d2, id); expand the first unchecked entry, add
  * every neighbour not visited before, re-sort, cut to L_search; stop when all entries are
  * checked; return the first k (padded with -1 / +inf).  out_d2 may be NULL.
- * EINVAL if k < 1, k > L_search or L_search > 1024. */
+ * EINVAL if k < 1, k > L_search or L_search > 1024, or where L_search and d are too large for
+ * the kernel's shared memory: 18 L_search + 8 max(32, R to a power of two) + 5 d + 1,024 bytes
+ * (parts rounded up to 16) may be at most 28,160 (ssg_search_work: 112,640). */
 ssg_status ssg_search_adj(const float* base, int64_t n, int32_t d, const int32_t* adj,
                           const int32_t* deg, int32_t R, const int32_t* nav, int32_t n_nav,
                           const float* queries, int64_t nq, int32_t k, int32_t L_search,

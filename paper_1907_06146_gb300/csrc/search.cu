@@ -692,6 +692,17 @@ static void launch_search(const float* X, int ld, int d, const int32_t* adj, con
                            n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo, out_ids, out_d2, work, st);
 }
 
+// The sizes a call may have: those of which eight queries' (a counting call: two) pools, each twice
+// and with a byte per entry, rows and smallest caches fit 220 KB.  The kernel needs less and takes
+// fewer warps per block where they do not fit; the limit is the interface's.
+static void require_sizes(int ls, int R, int ld, bool work) {
+  const auto up16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+  const size_t per = up16((size_t)ls * 16 + up16((size_t)ls * 2) +
+                          (size_t)std::max(32, next_pow2(R)) * 8 + (size_t)ld * 4 + 1024 + up16(ld));
+  SSG_REQUIRE(per * (work ? 2 : 8) <= 220 * 1024, SSG_EINVAL,
+              "search: L_search and d too large for shared memory");
+}
+
 // A 1,024-entry visited cache: its size only sets how often a distance is taken again, and a
 // larger one costs warps per SM.
 constexpr int CACHE_LOG2 = 10;
@@ -701,6 +712,7 @@ void search_run_mixed(const float* X, const uint8_t* X8, int ld, int d, const in
                       int ldq, int64_t nq, const int32_t* qk, const int32_t* qls, int ls_max,
                       int ldo, int32_t* out_ids, float* out_d2, cudaStream_t st) {
   if (nq == 0) return;
+  require_sizes(ls_max, R, ld, false);
   if (X8)
     launch_search(X8, ld, d, adj, deg, R, nav, n_nav, Q, ldq, nq, 0, ls_max, qk, qls, nullptr, ldo,
                   CACHE_LOG2, out_ids, out_d2, (unsigned long long*)nullptr, st);
@@ -715,6 +727,7 @@ void search_run(const float* X, const uint8_t* X8, int ld, int d, int64_t n, con
                 cudaStream_t st, unsigned long long* work) {
   (void)n;
   if (nq == 0) return;
+  require_sizes(Ls, R, ld, work != nullptr);
   // a call that counts the work takes a 16,384-entry cache, so that its distance count is
   // Alg. 1's (each node once) and not inflated by recomputations after cache evictions
   const int log2h = work ? 14 : CACHE_LOG2;
