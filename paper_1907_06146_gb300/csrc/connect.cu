@@ -446,6 +446,34 @@ __device__ __forceinline__ bool grid_bfs(const ConnArgs& a, unsigned& phase) {
   }
 }
 
+// Distances of U rows to b by a team of 8 lanes, each summed as team8_dist sums it; a step's loads
+// are all issued before its first product.
+template <int U>
+__device__ __forceinline__ void team8_dists(const float* const (&a)[U], const float* __restrict__ b,
+                                            int ld4, int tl, const bool (&valid)[U], float (&s)[U]) {
+#pragma unroll
+  for (int r = 0; r < U; ++r) s[r] = 0.f;
+  for (int f = tl; f < ld4; f += 8) {
+    const float4 y = __ldg((const float4*)b + f);
+    float4 x[U];
+#pragma unroll
+    for (int r = 0; r < U; ++r) x[r] = valid[r] ? __ldg((const float4*)a[r] + f) : y;
+#pragma unroll
+    for (int r = 0; r < U; ++r) {
+      float u;
+      u = x[r].x - y.x; s[r] = fmaf(u, u, s[r]);
+      u = x[r].y - y.y; s[r] = fmaf(u, u, s[r]);
+      u = x[r].z - y.z; s[r] = fmaf(u, u, s[r]);
+      u = x[r].w - y.w; s[r] = fmaf(u, u, s[r]);
+    }
+  }
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) {
+#pragma unroll
+    for (int r = 0; r < U; ++r) s[r] += __shfl_xor_sync(0xffffffffu, s[r], o);
+  }
+}
+
 // (d2, id)-smallest over the block (every thread returns it); bd / bi: 32 entries each.
 __device__ __forceinline__ void block_argmin(double& best, int& bid, double* bd, int* bi) {
   for (int o = 16; o > 0; o >>= 1) {
@@ -483,7 +511,7 @@ __device__ __forceinline__ void block_argmin(double& best, int& bid, double* bd,
 // large (distances that take few values: every block may hold thousands of ties at its own
 // smallest one), the band is taken again from the stored fp32 distances, against the smallest
 // bound of the whole grid, and only that band counts towards the list's room.
-__global__ void __launch_bounds__(512) k_connect(ConnArgs a) {
+__global__ void __launch_bounds__(512, 2) k_connect(ConnArgs a) {
   __shared__ double bd[32];
   __shared__ int bi[32];
   __shared__ int nties;
@@ -532,13 +560,26 @@ __global__ void __launch_bounds__(512) k_connect(ConnArgs a) {
       if (threadIdx.x == 0) bmin = 0x7f800000u;
       __syncthreads();
       float best = __int_as_float(0x7f800000);
-      for (int64_t v0 = gw * 4; v0 < a.n; v0 += nwarps * 4) {
-        const int64_t v = v0 + team;
-        const bool cand =
-            v < a.n && ((__ldcg(a.bm + (v >> 5)) >> (v & 31)) & 1u) && __ldcg(a.deg + v) < a.R;
-        const float e = team8_dist(a.X + (cand ? v : 0) * a.ld, xu, a.ld >> 2, tl, cand);
-        if (tl == 0 && v < a.n) a.d32[v] = cand ? e : -1.f;
-        if (cand) best = fminf(best, e);
+      constexpr int U = 4;
+      for (int64_t v0 = gw * 4; v0 < a.n; v0 += nwarps * 4 * U) {
+        const float* row[U];
+        bool cand[U];
+        float e[U];
+#pragma unroll
+        for (int r = 0; r < U; ++r) {
+          const int64_t v = v0 + r * nwarps * 4 + team;
+          const uint32_t word = v < a.n ? __ldcg(a.bm + (v >> 5)) : 0u;
+          const int dg = v < a.n ? __ldcg(a.deg + v) : a.R;
+          cand[r] = ((word >> (v & 31)) & 1u) && dg < a.R;
+          row[r] = a.X + (cand[r] ? v : 0) * a.ld;
+        }
+        team8_dists<U>(row, xu, a.ld >> 2, tl, cand, e);
+#pragma unroll
+        for (int r = 0; r < U; ++r) {
+          const int64_t v = v0 + r * nwarps * 4 + team;
+          if (tl == 0 && v < a.n) a.d32[v] = cand[r] ? e[r] : -1.f;
+          if (cand[r]) best = fminf(best, e[r]);
+        }
       }
       for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
       if (lane == 0 && best < __int_as_float(0x7f800000))
