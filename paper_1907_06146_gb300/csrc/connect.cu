@@ -151,6 +151,51 @@ __device__ __forceinline__ void warp_expand(const ConnArgs& a, uint32_t* bits, i
   }
 }
 
+// A level of a traversal that a whole block of k_repair_knn expands (block_level): the leading warp
+// sets it, the others wait for it at REPAIR_BAR.
+constexpr int REPAIR_THREADS = 512;
+struct BlockLevel {
+  const int32_t* fr;  // its nodes
+  int32_t* nx;        // those reached from it
+  int fc, count;      // their numbers; fc = 0: no more levels come
+};
+__device__ __forceinline__ void repair_bar() {
+  __syncwarp();
+  asm volatile("barrier.sync 1, %0;" ::"n"(REPAIR_THREADS) : "memory");
+}
+// All warps: a node each at a time, the next one's row and degree loading meanwhile.
+__device__ __forceinline__ void block_level(const ConnArgs& a, uint32_t* bits, BlockLevel* b) {
+  constexpr int NW = REPAIR_THREADS / 32;
+  const int lane = lane_id(), fc = b->fc;
+  int64_t node;
+  int32_t v = -1;
+  int dg = 0;
+  auto fetch = [&](int w) {
+    node = __ldcg(b->fr + w);
+    v = lane < a.R ? __ldcg(a.adj + node * a.R + lane) : -1;
+    dg = __ldcg(a.deg + node);
+  };
+  int w = threadIdx.x >> 5;
+  if (w < fc) fetch(w);
+  for (; w < fc; w += NW) {
+    const int64_t here = node;
+    const int32_t first = v;
+    const int n = dg;
+    if (w + NW < fc) fetch(w + NW);
+    for (int c = 0; c < n; c += 32) {
+      const int t = c + lane;
+      const int32_t x = t >= n ? 0 : c == 0 ? first : __ldcg(a.adj + here * a.R + t);
+      const uint32_t bit = 1u << (x & 31);
+      const bool fresh = t < n && !(peek(bits + (x >> 5)) & bit) && !(atomicOr(bits + (x >> 5), bit) & bit);
+      const unsigned bal = __ballot_sync(0xffffffffu, fresh);
+      int base = 0;
+      if (lane == 0 && bal) base = atomicAdd(&b->count, __popc(bal));
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (fresh) b->nx[base + __popc(bal & lanemask_lt())] = x;
+    }
+  }
+}
+
 // Repairs that kNN rows settle, back to back by one warp.  A row lists u's K nearest nodes in
 // exact (d2, id) order, so when some of them is reached and has a free slot the first such one
 // is the (d2, id)-smallest of all reached nodes with a free slot: the same choice as the
@@ -162,6 +207,10 @@ __device__ __forceinline__ void warp_expand(const ConnArgs& a, uint32_t* bits, i
 // latencies, so the rows, out-edges and degrees of the next two unreached nodes (which no repair
 // before their own changes) load while the current one is settled, and the degrees of the next
 // one's row entries too (a repair changes one degree, the one it links from).
+// Traversals: levels of up to four nodes by this warp, larger ones by its block (level, not null:
+// up to 4,096 nodes) or, within k_connect, by the grid, which also takes over after 64 levels (its
+// other blocks wait meanwhile).  60 islands of 640 nodes, each entered by a row: 25 ms where this
+// warp took levels of up to 256 nodes alone, now 3.1.
 struct RepairRow {
   static constexpr int PIECES = 4;  // of 32 entries, kept in registers
   int64_t u;
@@ -190,8 +239,8 @@ struct RepairRow {
   }
 };
 __device__ __noinline__ int64_t warp_knn_repairs(const ConnArgs& a, uint32_t* bits, int64_t start,
-                                                 int most, int* why) {
-  constexpr int LIMIT = 256;  // frontier nodes one warp expands itself
+                                                 int most, BlockLevel* level, int* why) {
+  constexpr int ALONE = 4;  // frontier nodes that this warp expands itself
   constexpr int P = RepairRow::PIECES;
   const int lane = lane_id();
   RepairState* s = a.s;
@@ -275,9 +324,16 @@ __device__ __noinline__ int64_t warp_knn_repairs(const ConnArgs& a, uint32_t* bi
     for (int c = P * 32; c < now.dg; c += 32)
       reach(c + lane < now.dg ? __ldcg(a.adj + u * a.R + c + lane) : -1, fr, fc);
     __syncwarp();
-    while (fc > 0 && fc <= LIMIT) {
+    for (int levels = 0; fc > 0 && (level ? fc <= 4096 : fc <= ALONE && levels < 64); ++levels) {
       int nc = 0;
-      for (int w = 0; w < fc; ++w) {
+      if (fc > ALONE) {
+        if (lane == 0) *level = BlockLevel{fr, nx, fc, 0};
+        repair_bar();
+        block_level(a, bits, level);
+        repair_bar();
+        nc = level->count;
+      }
+      for (int w = 0; fc <= ALONE && w < fc; ++w) {
         const int32_t node = __ldcg(fr + w);
         const int dg = __ldcg(a.deg + node);
         for (int c = 0; c < dg; c += 32)
@@ -320,9 +376,11 @@ __device__ __noinline__ int64_t warp_knn_repairs(const ConnArgs& a, uint32_t* bi
 
 // warp_knn_repairs with the bitmap in shared memory where it fits (up to 1.6M nodes): a chain
 // of dependent reads, each a shared-memory or an L2 latency.  200,000 nodes, 4,500 repairs:
-// 7.6 ms; one block that met at about ten barriers per repair took 15.5 ms.
-__global__ void __launch_bounds__(256) k_repair_knn(ConnArgs a, int shared_bits) {
+// 7.6 ms; one block that met at about ten barriers per repair took 15.5 ms.  The other warps only
+// take part in traversals.
+__global__ void __launch_bounds__(REPAIR_THREADS, 1) k_repair_knn(ConnArgs a, int shared_bits) {
   extern __shared__ uint32_t sbits[];
+  __shared__ BlockLevel level;
   uint32_t* bits = a.bm;
   if (shared_bits) {
     for (int64_t w = threadIdx.x; w < a.nw; w += blockDim.x) sbits[w] = a.bm[w];
@@ -331,10 +389,19 @@ __global__ void __launch_bounds__(256) k_repair_knn(ConnArgs a, int shared_bits)
   __syncthreads();
   if (threadIdx.x < 32) {
     int why;
-    const int64_t u = warp_knn_repairs(a, bits, a.start, INT_MAX, &why);
+    const int64_t u = warp_knn_repairs(a, bits, a.start, INT_MAX, &level, &why);
     if (threadIdx.x == 0) {
       a.s->u = (unsigned long long)u;
       a.s->best = u < a.n ? why : STOP_NONE;
+      level.fc = 0;
+    }
+    repair_bar();
+  } else {
+    for (;;) {
+      repair_bar();
+      if (level.fc == 0) break;
+      block_level(a, bits, &level);
+      repair_bar();
     }
   }
   __syncthreads();
@@ -528,7 +595,7 @@ __global__ void __launch_bounds__(512, 2) k_connect(ConnArgs a) {
     int why = STOP_ROW;
     int64_t u;
     if (a.knn && !a.stop_at_knn)
-      u = warp_knn_repairs(a, a.bm, start, 16, &why);
+      u = warp_knn_repairs(a, a.bm, start, 16, nullptr, &why);
     else
       u = warp_first_unreached(a.bm, a.nw, a.n, start);
     start = u >> 5;
@@ -736,7 +803,7 @@ static void connect_root(ConnArgs a, int32_t root, cudaStream_t st, F on_band) {
       const size_t smem = (size_t)a.nw * sizeof(uint32_t);
       const bool shared = smem <= 200 * 1024;
       if (shared) ensure_smem((const void*)k_repair_knn, smem);
-      SSG_LAUNCH(k_repair_knn, 1, 256, shared ? smem : 0, st, a, shared ? 1 : 0);
+      SSG_LAUNCH(k_repair_knn, 1, REPAIR_THREADS, shared ? smem : 0, st, a, shared ? 1 : 0);
       SSG_CUDA(cudaMemcpyAsync(&h, a.s, sizeof(h), cudaMemcpyDeviceToHost, st));
       SSG_CUDA(cudaStreamSynchronize(st));
       if ((int64_t)h.u >= a.n) break;
