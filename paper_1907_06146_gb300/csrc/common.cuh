@@ -93,6 +93,21 @@ inline void keep_pool_memory() {
   cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
 }
 
+// Device memory that the scratch pool can still take: the device's free memory and what the pool
+// holds unused.
+inline size_t scratch_room() {
+  int dev = 0;
+  cudaMemPool_t pool;
+  size_t free_b = 0, total_b = 0;
+  uint64_t held = 0, used = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+      cudaDeviceGetDefaultMemPool(&pool, dev) != cudaSuccess ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+    return free_b;
+  return free_b + (size_t)(held > used ? held - used : 0);
+}
+
 template <typename T>
 struct Scratch {
   T* p = nullptr;
@@ -103,7 +118,7 @@ struct Scratch {
   void alloc(size_t n, cudaStream_t st) {
     if (!try_alloc(n, st)) throw Fail{SSG_ENOMEM};
   }
-  // False, with the error's text set, where the device has no room.
+  // False, with the error's text set, where the device has no room (or a test injects that).
   bool try_alloc(size_t n, cudaStream_t st) {
     release();
     s = st;
@@ -111,14 +126,15 @@ struct Scratch {
     if (n == 0) return true;
     if (alloc_fault_injected()) {
       set_error("scratch allocation of %zu bytes failed: injected", n * sizeof(T));
-      throw Fail{SSG_ENOMEM};
+      return false;
     }
     keep_pool_memory();
     cudaError_t e = cudaMallocAsync((void**)&p, n * sizeof(T), st);
     if (e != cudaSuccess) {
       p = nullptr;
       set_error("scratch allocation of %zu bytes failed: %s", n * sizeof(T), cudaGetErrorString(e));
-      if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+      if (e != cudaErrorMemoryAllocation) throw Fail{SSG_ENOMEM};
+      cudaGetLastError();
       return false;
     }
     return true;

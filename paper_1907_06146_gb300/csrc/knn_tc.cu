@@ -1166,19 +1166,27 @@ void knn_exact_tc(const float* A, int64_t na, int lda, const float* a_norm, cons
     SSG_LAUNCH(k_ts_init, (unsigned)ceil_div(na, 256), 256, 0, st, ex.tau_in, a_norm, na, ts.p);
     a.ts_g = ts.p;
   }
-  // the row buffers of one launch take up to 2 GB; more rows go in several launches, whole
-  // rounds of the clusters each
-  const size_t block_bytes = (size_t)BM * a.nseg * C * sizeof(uint2);
+  // The row buffers of one launch take up to 2 GB, or an eighth of the memory that is left where
+  // that is less; more rows go in several launches, whole rounds of the clusters each.
   const int64_t round = std::max<int64_t>(1, num_sms() / 2);
-  int64_t rounds = std::max<int64_t>(1, (int64_t)((2ull << 30) / block_bytes) / round);
-  rounds = std::min(rounds, ceil_div(nrb, round));
+  int64_t rounds = ceil_div(nrb, round);
+  if (rounds > 1) {
+    const size_t round_bytes = (size_t)round * BM * a.nseg * C * sizeof(uint2);
+    const size_t room = std::min<size_t>(2ull << 30, scratch_room() / 8);
+    rounds = std::min(rounds, std::max<int64_t>(1, (int64_t)(room / round_bytes)));
+  }
   int64_t per_launch = std::min<int64_t>(nrb, rounds * round);
   Scratch<uint2> rowbuf;
   while (!rowbuf.try_alloc((size_t)per_launch * BM * a.nseg * C, st)) {
-    // where the device has less room, fewer rounds a launch, down to one (about 160 MB at C = 512)
-    if (rounds == 1) throw Fail{SSG_ENOMEM};
-    rounds = ceil_div(rounds, 2);
-    per_launch = rounds * round;
+    // where the device has less room: fewer rounds, then fewer shares, down to one round of rows
+    // whose columns are not shared out (SMs / 2 x 512 rows x C entries: 160 MB at C = 512)
+    if (rounds > 1)
+      rounds = ceil_div(rounds, 2);
+    else if (a.nseg > 1)
+      a.nseg = (a.nseg + 1) / 2;
+    else
+      throw Fail{SSG_ENOMEM};
+    per_launch = std::min<int64_t>(nrb, rounds * round);
   }
   Scratch<int> cnt((size_t)per_launch * BM * a.nseg, st);
   a.rowbuf = rowbuf.p;
