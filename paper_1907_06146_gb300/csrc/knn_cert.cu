@@ -29,27 +29,19 @@
 
 namespace ssg {
 
-// Column sums: block (32, 8), column blockIdx.x * 32 + tx, rows strided over y, four loads in
-// flight.  Each thread's running sum is a compensated fp32 pair (two-sum: 48 bits), joined in
-// fp64 at the end: GB300 adds fp64 at 1/64 of the fp32 rate, and with fp64 running sums the
-// 200,000 x 128 columns took 98 us against less than 30 (the read alone: 15).
+// Column sums in fp64: block (32, 8), column blockIdx.x * 32 + tx, rows strided over y.  Bound by the
+// fp64 additions (GB300 adds fp64 at 1/64 of the fp32 rate): 200,000 x 128 in 99 us, of which the read
+// alone is 15.  (Compensated fp32 pairs take less than 30, but hold 48 bits.)
 __global__ void k_col_sum(const float* __restrict__ X, int64_t n, int d, int ld,
                           double* __restrict__ sum) {
   __shared__ double part[8][33];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int c = blockIdx.x * 32 + tx;
-  float s = 0.f, e = 0.f;
-  if (c < d) {
-    const int64_t step = (int64_t)gridDim.y * 8;
-    for (int64_t r = (int64_t)blockIdx.y * 8 + ty; r < n; r += 4 * step) {
-      float v[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = r + u * step < n ? __ldg(X + (r + u * step) * ld + c) : 0.f;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) two_sum_acc(s, e, v[u]);
-    }
-  }
-  part[ty][tx] = (double)s + (double)e;
+  double s = 0.0;
+  if (c < d)
+    for (int64_t r = (int64_t)blockIdx.y * 8 + ty; r < n; r += (int64_t)gridDim.y * 8)
+      s += (double)X[r * ld + c];
+  part[ty][tx] = s;
   __syncthreads();
   if (ty == 0 && c < d) {
     double t = 0.0;
@@ -544,7 +536,7 @@ CertResult knn_bf16_certified(const float* A, int64_t na, int ld, const float* a
   // centre on the base's column mean; centred squared norms and their maximum
   Scratch<double> csum((size_t)d, st);
   SSG_CUDA(cudaMemsetAsync(csum.p, 0, sizeof(double) * d, st));
-  const unsigned gy = (unsigned)std::min<int64_t>(ceil_div(nb, 32), 4 * num_sms());
+  const unsigned gy = (unsigned)std::min<int64_t>(ceil_div(nb, 8), 4 * num_sms());
   SSG_LAUNCH(k_col_sum, dim3((unsigned)ceil_div(d, 32), gy), dim3(32, 8), 0, st, B, nb, d, ld, csum.p);
   Scratch<float> mu((size_t)d, st);
   SSG_LAUNCH(k_col_mean, (unsigned)ceil_div(d, 128), 128, 0, st, csum.p, d, nb, mu.p);
