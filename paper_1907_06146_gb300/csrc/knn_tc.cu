@@ -424,10 +424,10 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
       auto advance = [&](Half& u, int h) -> bool {
         if (u.it >= nitems) return false;
         bool ready = mbar_test(smem_u32(s_full + u.s), u.ph);
-        if (!STREAM) ready = ready && mbar_test(smem_u32(t_empty + 2 * h + u.sub), u.tph);
+        if (!STREAM) ready = ready && mbar_test_cluster(smem_u32(t_empty + 2 * h + u.sub), u.tph);
         if (STREAM && u.sub == 0)
-          ready = ready && mbar_test(smem_u32(t_empty + 2 * h), u.tph) &&
-                  mbar_test(smem_u32(t_empty + 2 * h + 1), u.tph);
+          ready = ready && mbar_test_cluster(smem_u32(t_empty + 2 * h), u.tph) &&
+                  mbar_test_cluster(smem_u32(t_empty + 2 * h + 1), u.tph);
         if (u.fresh) ready = ready && mbar_test(smem_u32(a_full), u.aph);
         if (!__all_sync(0xffffffffu, ready)) return false;
         tc_fence_after();
@@ -584,8 +584,10 @@ k_knn_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
           tmem_wait_ld(v[0]);
           tmem_dep(v[1]);
           if (c & 1) {
+            // every lane's loads, then (behind the warp's barrier) lane 0's arrival for all of them
             tc_fence_before();
             __syncwarp();
+            tc_fence_before();
             if (lane == 0) mbar_arrive_cluster(my_empty + (c >> 1) * (uint32_t)sizeof(uint64_t));
           }
           if (LIMITED && ((skip >> (STREAM ? c >> 1 : c & 1)) & 1u)) continue;

@@ -193,9 +193,10 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
                    : "memory");
 }
-// Arrival on a barrier of either CTA that orders nothing but the tcgen05 operations fenced
-// before it: a release at cluster scope would wait until the thread's global stores are
-// performed, about 1,000 cycles each time a row was appended to.
+// Arrival on a barrier of either CTA that orders nothing but the tcgen05 operations fenced before it
+// (tcgen05.fence::before_thread_sync orders them before the arrival, ::after_thread_sync behind the
+// test that sees it; the signal itself may be relaxed): a release at cluster scope would wait until
+// the thread's global stores are performed, about 1,000 cycles each time a row was appended to.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar)
                : "memory");
@@ -206,6 +207,20 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// The same for a barrier that threads of the other CTA arrive on by mbar_arrive_cluster: to be
+// followed by tc_fence_after (an acquire at cluster scope in the issuer's polling loop: 257 -> 267 ms
+// for a build of 1M x 128).
+__device__ __forceinline__ bool mbar_test_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}\n"
       : "=r"(ok)
       : "r"(bar), "r"(parity)
