@@ -421,7 +421,7 @@ ssg_status ssg_connect(const float* base, int64_t n, int32_t d, int32_t* adj, in
       SSG_REQUIRE(h[t] >= 0 && h[t] < n, SSG_EINVAL, "navigating node id %d out of range", h[t]);
     Ingested g;
     ingest_all(base, n, d, st, g, false);
-    const int64_t rep = connect_run(g.rows.p, g.rows.ld, d, n, adj, deg, R, nav, h.data(), n_nav, st);
+    const int64_t rep = connect_run(g.rows.p, g.rows.ld, d, n, adj, deg, R, h.data(), n_nav, st);
     if (n_repair_host) *n_repair_host = rep;
   });
 }
@@ -611,7 +611,7 @@ static void build_front(BuildCtx& c) {
     SSG_CUDA(cudaMalloc(&g->rows_u8, (size_t)n * in.rows.ld));
     g->rows_ld = in.rows.ld;
     g->rows_src = c.base;
-    rows_to_u8(in.rows.p, in.rows.ld, d, n, g->rows_u8, st);
+    rows_to_u8(in.rows.p, in.rows.ld, n, g->rows_u8, st);
   }
   c.t_ing->stop();
   c.ctr.alloc(1, st);
@@ -730,8 +730,8 @@ static void build_back(BuildCtx& c) {
 
   // a5: connectivity from the navigating nodes
   c.t_con->start();
-  c.n_repair = connect_run(in.rows.p, in.rows.ld, d, n, g->adj, g->deg, R, g->nav_dev,
-                           c.nav.data(), c.opts.n_nav, st, c.knn_id.p, c.knn_id.p ? c.K : 0, &c.n_repair_knn);
+  c.n_repair = connect_run(in.rows.p, in.rows.ld, d, n, g->adj, g->deg, R, c.nav.data(),
+                           c.opts.n_nav, st, c.knn_id.p, c.knn_id.p ? c.K : 0, &c.n_repair_knn);
   c.knn_id.release();
   c.t_con->stop();
   if (c.opts.debug_checks) debug_check(check_adj(g->adj, g->deg, n, R, st), "connectivity");

@@ -847,9 +847,8 @@ static std::vector<char> roots_reach_first(const ConnArgs& a, const int32_t* nav
 }
 
 int64_t connect_run(const float* X, int ld, int d, int64_t n, int32_t* adj, int32_t* deg,
-                    int R, const int32_t* nav_dev, const int32_t* nav_host, int n_nav,
+                    int R, const int32_t* nav_host, int n_nav,
                     cudaStream_t st, const int32_t* knn, int K, int64_t* knn_repairs) {
-  (void)nav_dev;
   const int64_t nw = ceil_div(n, 32);
   const int cap = 1 << 16;
   Scratch<uint32_t> bm((size_t)nw, st);
@@ -938,9 +937,8 @@ static unsigned char* noalloc_scratch() {
 }
 
 static int64_t connect_run_noalloc(const float* X, int ld, int d, int64_t n, int32_t* adj,
-                                   int32_t* deg, int R, const int32_t* nav_dev,
-                                   const int32_t* nav_host, int n_nav, cudaStream_t st) {
-  (void)nav_dev;
+                                   int32_t* deg, int R, const int32_t* nav_host, int n_nav,
+                                   cudaStream_t st) {
   unsigned char* base = noalloc_scratch();
   RepairState* S = (RepairState*)(base + OFF_STATE);
   SSG_CUDA(cudaMemsetAsync(S, 0, sizeof(RepairState), st));
@@ -985,7 +983,7 @@ extern "C" ssg_status ssg_connect_noalloc(const float* base, int64_t n, int32_t 
     SSG_CUDA(cudaStreamSynchronize(st));
     for (int t = 0; t < n_nav; ++t)
       SSG_REQUIRE(h[t] >= 0 && h[t] < n, SSG_EINVAL, "navigating node id %d out of range", h[t]);
-    const int64_t rep = connect_run_noalloc(base, d, d, n, adj, deg, R, nav, h.data(), n_nav, st);
+    const int64_t rep = connect_run_noalloc(base, d, d, n, adj, deg, R, h.data(), n_nav, st);
     if (n_repair_host) *n_repair_host = rep;
     return SSG_OK;
   } catch (const Fail& e) {

@@ -244,7 +244,7 @@ int reverse_run(const float* X, const uint8_t* X8, int ld, int d, int64_t n,
 // the exact kNN graph [n][K] in (d2, id) order, which settles most repairs without a pass
 // over all nodes (same result).
 int64_t connect_run(const float* X, int ld, int d, int64_t n, int32_t* adj, int32_t* deg,
-                    int R, const int32_t* nav_dev, const int32_t* nav_host, int n_nav,
+                    int R, const int32_t* nav_host, int n_nav,
                     cudaStream_t st, const int32_t* knn = nullptr, int K = 0,
                     int64_t* knn_repairs = nullptr);
 
@@ -270,7 +270,7 @@ bool search_from(const float* X, int ld, int d, const int32_t* adj, const int32_
 
 // Byte copy [n][ld] of rows that hold integers 0..255 (ld: the float rows' stride, a
 // multiple of 4; padding bytes 0).
-void rows_to_u8(const float* X, int ld, int d, int64_t n, uint8_t* out, cudaStream_t st);
+void rows_to_u8(const float* X, int ld, int64_t n, uint8_t* out, cudaStream_t st);
 
 // Invariant checks (csrc/check.cu).  row = -1: every row passed; else the smallest failing
 // row and its code.

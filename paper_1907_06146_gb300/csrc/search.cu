@@ -595,8 +595,7 @@ __global__ void k_rows_u8(const float4* __restrict__ X, int64_t n4, uchar4* __re
   }
 }
 
-void rows_to_u8(const float* X, int ld, int d, int64_t n, uint8_t* out, cudaStream_t st) {
-  (void)d;
+void rows_to_u8(const float* X, int ld, int64_t n, uint8_t* out, cudaStream_t st) {
   const int64_t n4 = n * ld / 4;
   SSG_LAUNCH(k_rows_u8, (unsigned)std::min<int64_t>(ceil_div(n4, 256), 16 * num_sms()), 256, 0, st,
              (const float4*)X, n4, (uchar4*)out);

@@ -155,17 +155,6 @@ __device__ __forceinline__ uint64_t sdesc_sw32(uint32_t saddr) {
   return d;
 }
 
-// TMA gather of four rows (y0..y3) of a 2-D tensor map whose box is one row high: the
-// rows land one after another at dst (128-byte swizzle applied by address).
-__device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* map, uint32_t bar,
-                                            int c0, int y0, int y1, int y2, int y3) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(dst),
-      "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(y0), "r"(y1), "r"(y2), "r"(y3)
-      : "memory");
-}
-
 // ---- CTA pairs (cta_group::2): clusters of two CTAs, the even one (the leader) issues the
 // MMAs for both.  Every tcgen05 instruction of such a kernel names the same group. ----
 __device__ __forceinline__ uint32_t cluster_rank() {
