@@ -18,12 +18,14 @@
 // The kept vectors sit in the block's shared memory (the first `cap` of them; the rest in
 // a device slot of the block, which stays in L2).  So the eight warps run eight independent
 // chains of dot products and meet once per window without a survivor, else four times.  Bound
-// by the latencies of those chains (a window's load, a round of four dot products, a barrier):
-// rows of up to 256 values take four blocks per SM and load a window ahead, the lengths' square
-// roots are taken once per vector, and the cosine's quotient is a product.  200,000 x 128, L =
-// 200, R = 32: 26.9 -> 19.2 ms; 100,000 x 960, L = 500, R = 70: 102 -> 90 ms, and the reverse
-// merge's short lists, most of which survive, 31 -> 21 ms (warp 0 used to take the survivors'
-// dot products alone, one after another).
+// by the latencies of those chains (a window's load, a round of four dot products, a barrier): as
+// many blocks per SM as registers and shared memory allow (wide_kernel), the lengths' square roots
+// taken once per vector, and the cosine's quotient a product.  200,000 x 128, L = 200, R = 32: 26.9
+// -> 17.5 ms; 100,000 x 960, L = 500, R = 70: 102 -> 90 ms, and the reverse merge's short lists, most
+// of which survive, 31 -> 21 ms (warp 0 used to take the survivors' dot products alone, one after
+// another).  Loading the next window's rows ahead (rows of up to 256 values) costs registers that
+// spill, and here more than it hides: without it 20,000 x 128, L = 200, R = 32 2.56 -> 2.39 ms,
+// 20,000 x 200, L = 60, R = 50 1.46 -> 0.92 (1.26 before rows were loaded ahead).
 // The decisions are those of the warp prune: the fp32 cosine decides outside a margin that
 // bounds its rounding error for any summation order; the rest, and zero-length edges, are
 // re-taken in fp64 from the original vectors.  Those fp64 dot products are summed by the
@@ -120,7 +122,7 @@ __device__ __forceinline__ int angle_test32(float g, float sj, float sk, float h
 // One node i of a (a.len, a.cand, ...) by the whole block.  NVR: float4 columns of the
 // candidate vector each lane holds (rows of up to 128 NVR values).  spill: this block's
 // device slot for kept vectors beyond a.cap.  n64 / nb: this thread's fp64 re-test counts.
-template <int NVR>
+template <int NVR, bool AHEAD>
 __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, unsigned char* smw,
                                                  float* spill, unsigned long long& n64,
                                                  unsigned long long& nb) {
@@ -153,10 +155,10 @@ __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, u
     __syncthreads();
     int kept = 0;  // the same in every thread
     const float hi = a.cosA32 + a.margin, lo = a.cosA32 - a.margin;
-    // short rows: the warp's next candidate's row loads while the current window is tested, its
-    // id a window before that (rows of more than 256 values have no registers to spare for it)
-    constexpr bool AHEAD = NVR <= 2;
-    float4 ahead[AHEAD ? NVR : 1];
+    // the warp's next two candidates (one window ahead: 100,000 x 960, L = 500, 90 -> 110 ms)
+    int32_t j1 = warp < len ? cand[warp] : -1;
+    int32_t j2 = warp + PW_WARPS < len ? cand[warp + PW_WARPS] : -1;
+    float4 ahead[AHEAD ? NVR : 1];  // AHEAD: the next one's row
     auto fetch = [&](int32_t j, float4* o) {
       const float4* c4 = (const float4*)(a.X + (int64_t)j * a.ld);
 #pragma unroll
@@ -165,8 +167,6 @@ __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, u
         o[r] = f < nq4 ? __ldg(c4 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     };
-    int32_t j1 = warp < len ? cand[warp] : -1;
-    int32_t j2 = warp + PW_WARPS < len ? cand[warp + PW_WARPS] : -1;
     if (AHEAD && j1 >= 0) fetch(j1, ahead);
     for (int t0 = 0; t0 < len && kept < a.R; t0 += PW_WARPS) {
       // ---- step 1: warp w takes candidate t0 + w against the kept vectors 0 .. kept-1
@@ -358,20 +358,23 @@ __device__ __forceinline__ void block_prune_node(const WideArgs& a, int64_t i, u
   }
 }
 
-template <int NVR>
-__global__ void __launch_bounds__(PW_THREADS, NVR <= 2 ? 4 : 2) k_prune_wide(WideArgs a) {
+// BLOCKS: per SM, as the registers allow (wide_kernel).
+template <int NVR, int BLOCKS>
+__global__ void __launch_bounds__(PW_THREADS, BLOCKS) k_prune_wide(WideArgs a) {
   extern __shared__ __align__(16) unsigned char smw[];
   const int d4 = (a.d + 3) & ~3;
   float* spill = a.Vg ? a.Vg + (size_t)blockIdx.x * (a.R + PW_WARPS - a.cap) * d4 : nullptr;
   unsigned long long n64 = 0, nb = 0;
   for (int64_t i = blockIdx.x; i < a.n; i += gridDim.x)
-    block_prune_node<NVR>(a, i, smw, spill, n64, nb);
+    block_prune_node<NVR, false>(a, i, smw, spill, n64, nb);
   if ((threadIdx.x & 31) == 0 && n64) atomicAdd(a.n64, n64);
   if ((threadIdx.x & 31) == 0 && nb) atomicAdd(a.nborder, nb);
 }
 
 // The same over the (index, node) work items of a batch, handed out from one counter in
-// the order of items (longest pools first); each block's spill slot holds vg_stride floats.
+// the order of items (longest pools first); each block's spill slot holds vg_stride floats.  Here
+// the next window's rows load ahead (rows of up to 256 values): a block's nodes come from indices of
+// different shapes, and without it six mixed indices take 28 ms in place of 17.
 template <int NVR>
 __global__ void __launch_bounds__(PW_THREADS, NVR <= 2 ? 4 : 2)
     k_prune_wide_batched(const WideArgs* __restrict__ jobs, const int2* __restrict__ items,
@@ -389,7 +392,7 @@ __global__ void __launch_bounds__(PW_THREADS, NVR <= 2 ? 4 : 2)
     const int2 w = items[it];
     const WideArgs a = jobs[w.x];
     unsigned long long n64 = 0, nb = 0;
-    block_prune_node<NVR>(a, w.y, smw, spill, n64, nb);
+    block_prune_node<NVR, NVR <= 2>(a, w.y, smw, spill, n64, nb);
     if ((threadIdx.x & 31) == 0 && n64) atomicAdd(a.n64, n64);
     if ((threadIdx.x & 31) == 0 && nb) atomicAdd(a.nborder, nb);
   }
@@ -410,6 +413,24 @@ static void wide_switch(int nvr, F f) {
     f(std::integral_constant<int, 4>());
   else
     f(std::integral_constant<int, 8>());
+}
+
+// Launch of k_prune_wide: four blocks per SM (64 registers) for rows of up to 256 values, three (80)
+// for rows of up to 512 where their shared memory leaves room for three, else two (128).  20,000 x
+// 300, L = 200: R = 32 3 / 2 blocks 3.55 / 4.31 ms; R = 70, whose kept vectors fill two blocks, 5.17
+// / 4.88.
+template <class F>
+static void wide_kernel(int nvr, size_t smem, F f) {
+  if (nvr == 1)
+    f(k_prune_wide<1, 4>);
+  else if (nvr == 2)
+    f(k_prune_wide<2, 4>);
+  else if (nvr == 4 && 3 * (smem + 1024) <= 228 * 1024)
+    f(k_prune_wide<4, 3>);
+  else if (nvr == 4)
+    f(k_prune_wide<4, 2>);
+  else
+    f(k_prune_wide<8, 2>);
 }
 
 bool prune_wide_available(int d) { return ((d + 3) & ~3) <= 1024; }
@@ -480,7 +501,7 @@ void prune_run_wide(const float* X, int ld, int d, int64_t n, const int32_t* can
   const size_t smem = wide_layout(d, R, cap).total;
   const int nv = wide_nvr(d4);
   const void* fn = nullptr;
-  wide_switch(nv, [&](auto nvr) { fn = (const void*)k_prune_wide<decltype(nvr)::value>; });
+  wide_kernel(nv, smem, [&](auto kernel) { fn = (const void*)kernel; });
   ensure_smem(fn, smem);
   int per_sm = 0;
   SSG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, PW_THREADS, smem));
@@ -491,8 +512,8 @@ void prune_run_wide(const float* X, int ld, int d, int64_t n, const int32_t* can
   WideArgs a{X, ld, d, n, cand, len, stride, R, (float)cos_a,
              angle_margin_fp32(d) + (float)border, cos_a, border, adj, deg, Vg.p, cap,
              &dctr->angle_fp64, &dctr->angle_border};
-  wide_switch(nv, [&](auto nvr) {
-    SSG_LAUNCH(k_prune_wide<decltype(nvr)::value>, (unsigned)grid, PW_THREADS, smem, st, a);
+  wide_kernel(nv, smem, [&](auto kernel) {
+    SSG_LAUNCH(kernel, (unsigned)grid, PW_THREADS, smem, st, a);
   });
 }
 
