@@ -136,16 +136,18 @@ typedef struct {
                                certify, 0.5..1), knn_prepass_tiles (tiles of the first,
                                threshold-only walk of the tensor-core kNN, 0..4096, 0 = none),
                                knn_stream_rows (1: rows of up to 128 values also take the
-                               K-chunked 128 x 256-tile kernel), prune_warps (warps per
+                               kernel that streams both sides in 64-value chunks),
+                               prune_warps (warps per
                                block of the batched prune, 0 = automatic, up to 16),
                                prune_bucket_width (pool lengths per bucket of the batched
                                prune's longest-first order, 1..1024), knn_bf16_pairs (the
                                certified bf16 kNN's operands as bf16 pairs: 1 always, 0
                                never, -1 = automatic: where the sized single-bf16 band
                                does not fit or is estimated dearer), prune_wide_blocks
-                               (blocks per SM of the block prune of rows of 330 to 1,024
-                               values, 0 = automatic (2), up to 4; fewer blocks hold more
-                               kept vectors in shared memory) */
+                               (blocks per SM whose shared memory the block prune, for
+                               rows of up to 1,024 values, is laid out for: 0 = automatic
+                               (2), up to 4; fewer blocks hold more kept vectors in shared
+                               memory) */
 } ssg_build_opts;
 
 /* Per-build measurements (all times from CUDA events on the build stream). */

@@ -965,7 +965,7 @@ ssg_status ssg_autotune_batched(int32_t count, const float* const* bases, const 
       build_setup(c, bases[i], n[i], d[i], K[i], L[i], R[i], alpha_deg[i], opts, st);
       if (knn_tc_available(d[i]) && d[i] <= 128 && c.opts.gemm_prec != SSG_PREC_FP32 &&
           c.opts.pool_tiles == 0) {
-        // the kNN kernel: resident 256 x 128 tiles against streamed 128 x 256 tiles
+        // the kNN kernel: resident query rows against streamed ones
         for (int w = 0; w < 2; ++w) {
           Ingested in;
           ingest_all(bases[i], n[i], d[i], st, in, true);

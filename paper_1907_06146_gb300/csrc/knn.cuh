@@ -76,8 +76,8 @@ struct TcExtra {
   const int32_t* qid = nullptr;       // self with A a gathered subset of B: query row r is
                                       // base row qid[r]; outputs go to row r
   const float* order_norm = nullptr;  // norms of A as given, for the cluster order
-  int stream_rows = 0;                // 1: the K-chunked kernel (128 x 256 tiles, N = 256)
-                                      // also for rows that fit the resident one
+  int stream_rows = 0;                // 1: both sides streamed in 64-value chunks (N = 256
+                                      // MMAs) also for rows that fit the resident kernel
   int pairs = 0;                      // 1: each centred value v goes in as the bf16 pair
                                       // hi = bf16(v), lo = bf16(v - hi); A rows are laid out
                                       // [hi | lo | hi] and B rows [lo | hi | hi] (each part
