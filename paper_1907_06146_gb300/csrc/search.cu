@@ -176,14 +176,14 @@ __device__ __forceinline__ float team8_dist_q(const float* __restrict__ qs,
 // packed four to a word (qw) and q2 = |q|^2, d2 = q2 + |x|^2 - 2 q.x from byte dot products
 // (dp4a), all in exact integer arithmetic.  Every value and partial sum of the float path
 // is an integer below 2^24 in that case, so the float path's sums are exact too and the two
-// give the same distances.  Rows of a multiple of 16 bytes load in 16-byte pieces, others in words;
-// either way a step's loads are all issued before the first product (words loaded and used one by
-// one: 50,000 x 100, L_search 10, 10,000 queries 355 us, teams of eight with all loads first 256,
+// give the same distances.  Rows of a multiple of 16 bytes load in 16-byte pieces, others (WORDS) in
+// words; either way a step's loads are all issued before the first product (words loaded and used one
+// by one: 50,000 x 100, L_search 10, 10,000 queries 355 us, teams of eight with all loads first 256,
 // now 214).
 __device__ __forceinline__ int sum_dp4a(uint32_t q, uint32_t x, int s) {
   return s + (int)__dp4a(x, x, 0u) - 2 * (int)__dp4a(q, x, 0u);
 }
-template <int NR>
+template <int NR, bool WORDS>
 __device__ __forceinline__ void team4_dist_qi(const uint32_t* __restrict__ qw,
                                               const uint8_t* __restrict__ X, int ld,
                                               const int32_t (&ids)[NR], const bool (&valid)[NR],
@@ -191,7 +191,7 @@ __device__ __forceinline__ void team4_dist_qi(const uint32_t* __restrict__ qw,
   int s[NR];
 #pragma unroll
   for (int r = 0; r < NR; ++r) s[r] = 0;
-  if ((ld & 15) == 0) {
+  if constexpr (!WORDS) {
     const int np = ld >> 4;
     for (int c0 = tl; c0 < np; c0 += 8) {
       uint4 raw[NR][2];
@@ -398,7 +398,9 @@ struct SearchLayout {
 // 723 us, one query 172 -> 122 (teams of four: 796 and 181; 32 warps per SM with spills 738).  A
 // pool in registers with an insertion per accepted neighbour was slower (0.93 ms): on the way to
 // the query about half the neighbours are accepted.
-template <typename T, int NR, int MIN_BLOCKS>
+// WORDS: byte rows of no multiple of 16 bytes, a kernel of their own: with both loads in one, rows of 128
+// bytes took 1-2% longer (one query over 200,000 x 128 91.4 us, now 89.8; 10,000 over 1M 550 / 545).
+template <typename T, int NR, int MIN_BLOCKS, bool WORDS>
 __global__ void __launch_bounds__(256, MIN_BLOCKS)
     k_search(const T* __restrict__ X, int ld, int d, const int32_t* __restrict__ adj,
              const int32_t* __restrict__ deg, int R, const int32_t* __restrict__ nav, int n_nav,
@@ -548,7 +550,7 @@ __global__ void __launch_bounds__(256, MIN_BLOCKS)
         if constexpr (BYTES) {
           float dd[NR];
           if (qint)
-            team4_dist_qi<NR>(qw, X, ld, ir, vr, tl, q2, dd);
+            team4_dist_qi<NR, WORDS>(qw, X, ld, ir, vr, tl, q2, dd);
           else
             team4_dist_q<T, NR>(qs, X, ld, ir, vr, tl, dd);
           __syncwarp();
@@ -601,7 +603,7 @@ void rows_to_u8(const float* X, int ld, int64_t n, uint8_t* out, cudaStream_t st
              (const float4*)X, n4, (uchar4*)out);
 }
 
-// A launch of k_search<T, NR, MIN_BLOCKS>: warps per block, shared memory, blocks per SM.
+// A launch of k_search<T, NR, MIN_BLOCKS, WORDS>: warps per block, shared memory, blocks per SM.
 struct SearchPlan {
   SearchLayout lay;
   int wpb, per_sm;
@@ -612,9 +614,9 @@ struct SearchPlan {
 // ls: the pool size, or the largest one of qls.  Warps per block: eight, fewer where there are
 // too few queries to give every SM a block of eight (a query alone on an SM runs without the
 // others' instructions in its way).
-template <typename T, int NR, int MIN_BLOCKS>
+template <typename T, int NR, int MIN_BLOCKS, bool WORDS = false>
 static SearchPlan plan_rows(int ld, int R, int64_t nq, int ls, int log2h, bool work) {
-  const void* kernel = (const void*)k_search<T, NR, MIN_BLOCKS>;
+  const void* kernel = (const void*)k_search<T, NR, MIN_BLOCKS, WORDS>;
   SearchPlan p;
   p.lay.Ls = (ls + 1) & ~1;
   p.lay.RP = (R + 31) & ~31;
@@ -634,14 +636,14 @@ static SearchPlan plan_rows(int ld, int R, int64_t nq, int ls, int log2h, bool w
   return p;
 }
 
-template <typename T, int NR, int MIN_BLOCKS>
+template <typename T, int NR, int MIN_BLOCKS, bool WORDS = false>
 static void launch_rows(const SearchPlan& p, const T* X, int ld, int d, const int32_t* adj,
                         const int32_t* deg, int R, const int32_t* nav, int n_nav, const float* Q,
                         int ldq, int64_t nq, int k, int ls, const int32_t* qk, const int32_t* qls,
                         const int32_t* from, int ldo, int32_t* out_ids, float* out_d2,
                         unsigned long long* work, cudaStream_t st) {
   const int grid = (int)std::min<int64_t>(ceil_div(nq, p.wpb), (int64_t)p.per_sm * num_sms());
-  SSG_LAUNCH((k_search<T, NR, MIN_BLOCKS>), grid, p.wpb * 32, p.smem, st, X, ld, d, adj, deg, R, nav,
+  SSG_LAUNCH((k_search<T, NR, MIN_BLOCKS, WORDS>), grid, p.wpb * 32, p.smem, st, X, ld, d, adj, deg, R, nav,
              n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo, p.lay, out_ids, out_d2, work);
 }
 
@@ -650,9 +652,14 @@ static void launch_search(const uint8_t* X, int ld, int d, const int32_t* adj, c
                           int k, int ls, const int32_t* qk, const int32_t* qls, const int32_t* from,
                           int ldo, int log2h, int32_t* out_ids, float* out_d2,
                           unsigned long long* work, cudaStream_t st) {
-  launch_rows<uint8_t, 2, 3>(plan_rows<uint8_t, 2, 3>(ld, R, nq, ls, log2h, work != nullptr), X, ld, d,
-                             adj, deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo, out_ids,
-                             out_d2, work, st);
+  const bool w = work != nullptr;
+  if (ld & 15)
+    launch_rows<uint8_t, 2, 3, true>(plan_rows<uint8_t, 2, 3, true>(ld, R, nq, ls, log2h, w), X, ld, d, adj,
+                                     deg, R, nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo, out_ids,
+                                     out_d2, work, st);
+  else
+    launch_rows<uint8_t, 2, 3>(plan_rows<uint8_t, 2, 3>(ld, R, nq, ls, log2h, w), X, ld, d, adj, deg, R,
+                               nav, n_nav, Q, ldq, nq, k, ls, qk, qls, from, ldo, out_ids, out_d2, work, st);
 }
 // Float rows: while every warp of the batch fits two blocks of eight per SM, 16 rows in flight
 // per warp and 16 warps per SM; above, 8 rows and 24 warps.  50,000 x 128, us at L_search 40 and
