@@ -244,15 +244,14 @@ __global__ void k_tile_order(const int32_t* __restrict__ order, const int32_t* _
 // The tile list of each work item of a limited walk: the 256-column tiles that hold those of its
 // `per` row blocks' lists (list entries taken in turn, so nearest first for all), each once, with
 // the mask of who visits what (knn_item_tiles).  All threads mark the lists in a bitmap per row
-// block; then one walks the lists with a bitmap of the tiles already listed.
+// block; then one walks the lists and unmarks the tiles that it has listed.
 __global__ void k_item_tiles(const int32_t* __restrict__ tile_order, const int32_t* __restrict__ rbc,
                              int64_t nrb, int per, int wide, int64_t tstride, int words, int64_t item0,
                              int64_t stride, int32_t* __restrict__ out, int32_t* __restrict__ len) {
-  extern __shared__ uint32_t marks[];  // [per][words] of the lists' tiles, then [words] of those seen
-  uint32_t* seen = marks + per * words;
+  extern __shared__ uint32_t marks[];  // [per][words] of the lists' tiles still to list
   const int64_t b0 = (item0 + blockIdx.x) * per;
   const int blocks = (int)min((int64_t)per, nrb - b0);
-  for (int w = threadIdx.x; w < (per + 1) * words; w += blockDim.x) marks[w] = 0u;
+  for (int w = threadIdx.x; w < per * words; w += blockDim.x) marks[w] = 0u;
   __syncthreads();
   for (int b = 0; b < blocks; ++b)
     for (int64_t i = threadIdx.x; i < tstride; i += blockDim.x) {
@@ -267,17 +266,18 @@ __global__ void k_item_tiles(const int32_t* __restrict__ tile_order, const int32
     for (int b = 0; b < blocks; ++b) {
       int32_t t = tile_order[(int64_t)rbc[b0 + b] * tstride + i];
       if (!wide) t >>= 1;
-      const uint32_t bit = 1u << (t & 31);
-      if (seen[t >> 5] & bit) continue;
-      seen[t >> 5] |= bit;
+      // the tile's bits in a bitmap: one, or those of its two 128-column tiles
+      const int w = wide ? t >> 5 : t >> 4, at = wide ? t & 31 : 2 * (t & 15);
+      const uint32_t bits = wide ? 1u : 3u;
       uint32_t mask = 0u;
       for (int v = 0; v < blocks; ++v) {
-        const uint32_t* m = marks + v * words;
-        const uint32_t cols = wide ? ((m[t >> 5] >> (t & 31)) & 1u) * 3u
-                                   : (m[t >> 4] >> (2 * (t & 15))) & 3u;
+        uint32_t* m = marks + v * words + w;
+        const uint32_t in = (*m >> at) & bits;
+        *m &= ~(bits << at);
+        const uint32_t cols = wide ? in * 3u : in;
         mask |= per == 2 ? (cols * 5u) << (4 * v) : cols << (2 * v);
       }
-      o[k++] = t << 8 | (int32_t)mask;
+      if (mask) o[k++] = t << 8 | (int32_t)mask;
     }
   }
   len[blockIdx.x] = k;
@@ -286,7 +286,8 @@ __global__ void k_item_tiles(const int32_t* __restrict__ tile_order, const int32
 void knn_item_tiles(const KnnOrder& o, int64_t n, int BM, int BN, int64_t item0, int64_t items,
                     int64_t stride, int32_t* out, int32_t* len, cudaStream_t st) {
   const int per = 512 / BM, words = (int)((o.ntiles + 31) >> 5);
-  const size_t smem = (size_t)(per + 1) * words * sizeof(uint32_t);
+  // at most 4 x 48 KB: knn_order_fits
+  const size_t smem = (size_t)per * words * sizeof(uint32_t);
   ensure_smem((const void*)k_item_tiles, smem);
   SSG_LAUNCH(k_item_tiles, (unsigned)items, 128, smem, st, o.tile_order.p, o.rb_cluster.p,
              ceil_div(n, BM), per, BN == 256 ? 1 : 0, o.tstride, words, item0, stride, out, len);
